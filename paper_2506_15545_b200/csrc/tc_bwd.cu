@@ -345,7 +345,8 @@ struct DqMaps {
 };
 
 __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, int n_items, int n_qt) {
-  int kc = 0, n = 0, co = 0;                               // ring uses, items, o_done completions so far
+  int kc = 0, n = 0, co = 0;                               // ring uses, items, o_done completions of the items so far
+  int co_window = 0;                                       // the completion that ends the previous item's window products
   for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++n) {
     const DqItem it = dq_item(a, idx, n_qt);
     auto ring_wait = [&]() -> bool {                       // the slot's previous user has been consumed
@@ -363,9 +364,14 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
       WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);      // and its dQ, staged there, has left
     }
     load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->qg_full, it.q0, it.bh_q);
-    // g_s: its one buffer is free once every product of the previous item has completed
-    // (o_done completes twice for an item with a residual part, once otherwise)
-    if (n >= 1) WAIT_OR_RETURN_W(bars->o_done, (co - 1) & 1);
+    // g_s: its one buffer is free once the previous item's window products have completed (the residual part
+    // reads g_r).  o_done completes twice for an item with a residual part, after the window products and at the
+    // end, once otherwise; it is the first of them that is awaited here.  Awaiting the second alone would not be
+    // safe: a parity wait tells a completion only from the one right before it, and while the first is still
+    // outstanding the parity of the second reads as already reached.  (The completions before the first are
+    // known to be over: acc_free of item n - 2 above follows them.)
+    if (n >= 1) WAIT_OR_RETURN_W(bars->o_done, co_window & 1);
+    co_window = co;
     co += it.has_rla ? 2 : 1;
     load_tile(smem + DQ_OFF_G, &tm.gs, &bars->qg_full, it.q0, it.bh_q);
     for (int i = 0; i < it.n_kt; ++i, ++kc) {
