@@ -1,18 +1,23 @@
-"""ctypes binding of librattn.so: argument marshalling only.
+"""Binding of librattn.so: argument marshalling only.
 
 Every function has the name of the C entry point it calls (include/rattn.h) and does
-nothing but turn torch tensors into device pointers, sizes and a stream handle.  There
-is no fallback: if the library has not been built, loading it raises.
+nothing but turn torch tensors into device pointers, sizes and a stream handle.  The calls
+that enqueue work are marshalled by the extension csrc/native.cpp (a decode step is over
+before ctypes has filled its parameter block); queries go through ctypes.  There is no
+fallback: if the library or the extension has not been built, loading it raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librattn.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 RATTN_BF16, RATTN_F32 = 0, 1
 MODE_RATTN, MODE_SWA_ONLY, MODE_FULL_CAUSAL = 0, 1, 2
@@ -143,6 +148,30 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+_native = None
+
+# in the order of native.cpp's table of entry points
+_ENTRIES = ("rattn_forward", "rattn_forward_static", "rattn_forward_ex", "rattn_backward", "rattn_backward_ex",
+            "rattn_decode_step", "rattn_decode_step_ex", "rattn_qk_prologue", "rattn_qk_prologue_backward",
+            "rattn_qk_prologue_workspace_bytes")
+
+
+def native():
+    """The marshalling extension, bound to the entry points of the loaded library."""
+    global _native
+    if _native is None:
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(
+                f"{NATIVE_PATH} is missing: build it with `python -m paper_2506_15545_b200.build`")
+        L = lib()
+        loader = importlib.machinery.ExtensionFileLoader(__package__ + "._native", NATIVE_PATH)
+        m = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
+        loader.exec_module(m)
+        m.bind(RattnError, *(ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in _ENTRIES))
+        _native = m
+    return _native
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -163,12 +192,6 @@ def _dtype_code(t: torch.Tensor) -> int:
 def _check(code: int, where: str):
     if code != 0:
         raise RattnError(code, where)
-
-
-def _dense(*ts):
-    for t in ts:
-        if t is not None and not (t.is_cuda and t.is_contiguous()):
-            raise ValueError("tensors must be contiguous CUDA tensors")
 
 
 def rattn_workspace_bytes(B, H_q, H_kv, T, d, w, dtype=RATTN_BF16) -> int:
@@ -208,6 +231,7 @@ def alloc_workspace(q, k, w, mode=None, flags=None, layout=LAYOUT_BHTD) -> torch
 
 def _params(q, k, v, out, w, scale, eps, gamma_swa, gamma_rla, mode, workspace, flags, phi=PHI_SOFTMAX,
             layout=LAYOUT_BHTD):
+    """The parameter block of an _ex entry point, for callers that go to a library of their own through ctypes."""
     p = RattnParams()
     p.feature_map = phi
     p.layout = layout
@@ -237,24 +261,14 @@ def _params(q, k, v, out, w, scale, eps, gamma_swa, gamma_rla, mode, workspace, 
 
 def rattn_forward(q, k, v, w, out=None, stream=None):
     """rattn_forward: bf16, scale 1, unit gains, eps 1e-6."""
-    _dense(q, k, v, out)
-    B, H_q, T, d = q.shape
-    out = torch.empty_like(q) if out is None else out
-    _check(lib().rattn_forward(_ptr(q), _ptr(k), _ptr(v), B, H_q, k.shape[1], T, d, w, _ptr(out),
-                               _stream(stream)), "rattn_forward")
-    return out
+    return (_native or native()).forward(q, k, v, w, out, stream)
 
 
 def rattn_forward_static(q, k, v, w, scale=1.0, out=None, stream=None):
     """rattn_forward_static: the forward that allocates nothing on the library side (its
     scratch is a fixed array inside the library).  `out` may be passed in so that the call
     allocates nothing on the Python side either."""
-    _dense(q, k, v, out)
-    B, H_q, T, d = q.shape
-    out = torch.empty_like(q) if out is None else out
-    _check(lib().rattn_forward_static(_ptr(q), _ptr(k), _ptr(v), B, H_q, k.shape[1], T, d, w, scale,
-                                      _ptr(out), _stream(stream)), "rattn_forward_static")
-    return out
+    return (_native or native()).forward_static(q, k, v, w, scale, out, stream)
 
 
 def rattn_forward_ex(q, k, v, w, *, scale=1.0, eps=1e-6, gamma_swa=None, gamma_rla=None,
@@ -262,75 +276,35 @@ def rattn_forward_ex(q, k, v, w, *, scale=1.0, eps=1e-6, gamma_swa=None, gamma_r
                      k_ring_out=None, v_ring_out=None, out=None, flags=0, phi=PHI_SOFTMAX, state_in=None,
                      k_ring_in=None, v_ring_in=None, pos0=0, seq_lens=None, layout=LAYOUT_BHTD, stream=None):
     """layout=LAYOUT_BTHD: q, out are [B, T, H_q, d] and k, v [B, T, H_kv, d]."""
-    _dense(q, k, v, out, gamma_swa, gamma_rla, workspace, state_out, k_ring_out, v_ring_out, state_in,
-           k_ring_in, v_ring_in, seq_lens)
-    out = torch.empty_like(q) if out is None else out
-    if save_residuals:
-        flags |= FLAG_SAVE_RESIDUALS
-    p = _params(q, k, v, out, w, scale, eps, gamma_swa, gamma_rla, mode, workspace, flags, phi, layout)
-    p.state_out = None if state_out is None else state_out.data_ptr()
-    p.k_ring_out = None if k_ring_out is None else k_ring_out.data_ptr()
-    p.v_ring_out = None if v_ring_out is None else v_ring_out.data_ptr()
-    p.state_in = None if state_in is None else state_in.data_ptr()
-    p.k_ring_in = None if k_ring_in is None else k_ring_in.data_ptr()
-    p.v_ring_in = None if v_ring_in is None else v_ring_in.data_ptr()
-    p.pos0 = pos0
-    p.seq_lens = None if seq_lens is None else seq_lens.data_ptr()
-    _check(lib().rattn_forward_ex(ctypes.byref(p), _stream(stream)), "rattn_forward_ex")
-    return out
+    return (_native or native()).forward_ex(
+        q, k, v, w, scale, eps, gamma_swa, gamma_rla, mode, workspace, save_residuals, state_out, k_ring_out,
+        v_ring_out, out, flags, phi, state_in, k_ring_in, v_ring_in, pos0, seq_lens, layout, stream)
 
 
 def rattn_backward(q, k, v, dout, workspace, w, dq=None, dk=None, dv=None, stream=None):
     """rattn_backward: bf16, scale 1, unit gains, eps 1e-6."""
-    _dense(q, k, v, dout, workspace, dq, dk, dv)
-    B, H_q, T, d = q.shape
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    _check(lib().rattn_backward(_ptr(q), _ptr(k), _ptr(v), _ptr(dout), _ptr(workspace),
-                                workspace.numel(), B, H_q, k.shape[1], T, d, w, _ptr(dq),
-                                _ptr(dk), _ptr(dv), _stream(stream)), "rattn_backward")
-    return dq, dk, dv
+    return (_native or native()).backward(q, k, v, dout, workspace, w, dq, dk, dv, stream)
 
 
 def rattn_backward_ex(q, k, v, dout, w, workspace, *, scale=1.0, eps=1e-6, gamma_swa=None,
                       gamma_rla=None, mode=MODE_RATTN, dq=None, dk=None, dv=None,
                       dgamma_swa=None, dgamma_rla=None, flags=0, phi=PHI_SOFTMAX, layout=LAYOUT_BHTD, stream=None):
-    _dense(q, k, v, dout, workspace, gamma_swa, gamma_rla, dq, dk, dv, dgamma_swa, dgamma_rla)
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    p = _params(q, k, v, dq, w, scale, eps, gamma_swa, gamma_rla, mode, workspace, flags, phi, layout)
-    p.dout, p.dq, p.dk, p.dv = dout.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr()
-    p.dgamma_swa = None if dgamma_swa is None else dgamma_swa.data_ptr()
-    p.dgamma_rla = None if dgamma_rla is None else dgamma_rla.data_ptr()
-    _check(lib().rattn_backward_ex(ctypes.byref(p), _stream(stream)), "rattn_backward_ex")
-    return dq, dk, dv
+    return (_native or native()).backward_ex(
+        q, k, v, dout, w, workspace, scale, eps, gamma_swa, gamma_rla, mode, dq, dk, dv, dgamma_swa, dgamma_rla,
+        flags, phi, layout, stream)
 
 
 def rattn_decode_step(q, k, v, k_ring, v_ring, state, pos, out=None, stream=None):
     """rattn_decode_step: bf16, scale 1, unit gains, eps 1e-6.  Ring and state in place."""
-    _dense(q, k, v, k_ring, v_ring, state, out)
-    B, H_q, d = q.shape
-    out = torch.empty_like(q) if out is None else out
-    _check(lib().rattn_decode_step(_ptr(q), _ptr(k), _ptr(v), _ptr(k_ring), _ptr(v_ring),
-                                   _ptr(state), pos, B, H_q, k.shape[1], d, k_ring.shape[2],
-                                   _ptr(out), _stream(stream)), "rattn_decode_step")
-    return out
+    return (_native or native()).decode_step(q, k, v, k_ring, v_ring, state, pos, out, stream)
 
 
 def rattn_decode_step_ex(q, k, v, k_ring, v_ring, state, pos, *, scale=1.0, eps=1e-6,
                          gamma_swa=None, gamma_rla=None, out=None, phi=PHI_SOFTMAX, pos_dev=None, flags=0,
                          stream=None):
     """pos_dev: optional int32 device tensor [B], one position per batch entry (then `pos` is ignored)."""
-    _dense(q, k, v, k_ring, v_ring, state, out, gamma_swa, gamma_rla, pos_dev)
-    out = torch.empty_like(q) if out is None else out
-    p = _params(q, k, v, out, k_ring.shape[2], scale, eps, gamma_swa, gamma_rla, MODE_RATTN,
-                None, flags, phi)
-    p.pos = None if pos_dev is None else pos_dev.data_ptr()
-    _check(lib().rattn_decode_step_ex(ctypes.byref(p), _ptr(k_ring), _ptr(v_ring), _ptr(state),
-                                      pos, _stream(stream)), "rattn_decode_step_ex")
-    return out
+    return (_native or native()).decode_step_ex(
+        q, k, v, k_ring, v_ring, state, pos, scale, eps, gamma_swa, gamma_rla, out, phi, pos_dev, flags, stream)
 
 
 def rattn_read_status(workspace, stream=None) -> int:
@@ -372,25 +346,6 @@ def rattn_timing_read() -> dict:
     return out
 
 
-def _qk_params(q, k, q_out, k_out, q_gain, k_gain, theta, eps, pos0, pos, layout=LAYOUT_BHTD):
-    p = RattnQkParams()
-    _dense(q, k, q_out, k_out, q_gain, k_gain, pos)
-    p.q, p.q_out = q.data_ptr(), None if q_out is None else q_out.data_ptr()
-    hd = 2 if layout == LAYOUT_BTHD else 1              # which dimension counts the heads
-    p.layout = layout
-    p.B, p.d = q.shape[0], q.shape[3]
-    p.H_q, p.T = q.shape[hd], q.shape[3 - hd]
-    if k is not None:
-        p.k, p.k_out = k.data_ptr(), None if k_out is None else k_out.data_ptr()
-        p.H_kv = k.shape[hd]
-    p.q_gain = None if q_gain is None else q_gain.data_ptr()
-    p.k_gain = None if k_gain is None else k_gain.data_ptr()
-    p.dtype = _dtype_code(q)
-    p.eps, p.theta, p.pos0 = eps, 0.0 if theta is None else theta, pos0
-    p.pos = None if pos is None else pos.data_ptr()
-    return p
-
-
 def rattn_qk_prologue_workspace_bytes(B, H_q, H_kv, T, d) -> int:
     return int(lib().rattn_qk_prologue_workspace_bytes(B, H_q, H_kv, T, d))
 
@@ -412,30 +367,12 @@ def rattn_qk_prologue(q, k, *, q_gain=None, k_gain=None, theta=5.0e5, eps=1e-6, 
                       inplace=False, layout=LAYOUT_BHTD, stream=None):
     """rattn_qk_prologue: qk-norm then rotary embedding of q [B,H_q,T,d] and k [B,H_kv,T,d] (k may be
     None).  theta None or <= 0: no rotation.  Returns (q_out, k_out); the inputs themselves if inplace."""
-    q_out = q if inplace else torch.empty_like(q)
-    k_out = None if k is None else (k if inplace else torch.empty_like(k))
-    p = _qk_params(q, k, q_out, k_out, q_gain, k_gain, theta, eps, pos0, pos, layout)
-    _check(lib().rattn_qk_prologue(ctypes.byref(p), _stream(stream)), "rattn_qk_prologue")
-    return q_out, k_out
+    return (_native or native()).qk_prologue(q, k, q_gain, k_gain, theta, eps, pos0, pos, layout, inplace, stream)
 
 
 def rattn_qk_prologue_backward(q, k, dq_out, dk_out, *, q_gain=None, k_gain=None, theta=5.0e5, eps=1e-6,
                                pos0=0, pos=None, gain_grads=True, workspace=None, layout=LAYOUT_BHTD, stream=None):
     """rattn_qk_prologue_backward: gradients with respect to q, k (inputs as they were before the
     forward pass) and, with gain_grads, to the two gains.  Returns (dq, dk, dq_gain, dk_gain)."""
-    _dense(dq_out, dk_out)
-    dq = torch.empty_like(q)
-    dk = None if k is None else torch.empty_like(k)
-    dqg = dkg = None
-    p = _qk_params(q, k, None, None, q_gain, k_gain, theta, eps, pos0, pos, layout)
-    if gain_grads:
-        dqg = torch.empty(q.shape[-1], dtype=torch.float32, device=q.device)
-        dkg = None if k is None else torch.empty(q.shape[-1], dtype=torch.float32, device=q.device)
-        if workspace is None:
-            n = rattn_qk_prologue_workspace_bytes(p.B, p.H_q, p.H_kv, p.T, p.d)
-            workspace = torch.empty(n, dtype=torch.uint8, device=q.device)
-    nbytes = 0 if workspace is None else workspace.numel()
-    _check(lib().rattn_qk_prologue_backward(ctypes.byref(p), _ptr(dq_out), _ptr(dk_out), _ptr(dq), _ptr(dk),
-                                            _ptr(dqg), _ptr(dkg), _ptr(workspace), nbytes, _stream(stream)),
-           "rattn_qk_prologue_backward")
-    return dq, dk, dqg, dkg
+    return (_native or native()).qk_prologue_backward(
+        q, k, dq_out, dk_out, q_gain, k_gain, theta, eps, pos0, pos, layout, gain_grads, workspace, stream)

@@ -18,6 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "librattn.so")
 LIB_DEBUG = os.path.join(HERE, "librattn_dbg.so")      # same sources with -DRATTN_DEBUG_KNOBS (include/rattn_debug.h)
+NATIVE = os.path.join(HERE, "_native.so")              # CPython extension of binding.py (csrc/native.cpp)
 LIB_TIMELINE = os.path.join(HERE, "librattn_tl.so")    # same sources with -DRATTN_TIMELINE (bench.py --case timeline)
 
 SOURCES = ["rattn_api.cu", "generic_fwd.cu", "generic_bwd.cu", "decode.cu", "tc_fwd.cu",
@@ -65,6 +66,8 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False, timel
     """Compile every source and link librattn.so (debug: librattn_dbg.so; timeline: librattn_tl.so,
     the forward kernel with its per-role clock stamps compiled in); returns its path."""
     lib = LIB_DEBUG if debug else LIB_TIMELINE if timeline else LIB
+    if lib == LIB:
+        build_native(force)
     sources = [s for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
     if not force and os.path.exists(lib) and os.path.getmtime(lib) >= _newest_dep_mtime():
         return lib
@@ -78,6 +81,31 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False, timel
     return lib
 
 
+def build_native(force: bool = False) -> str:
+    """Compile the marshalling extension against the installed torch; returns its path."""
+    src = os.path.join(CSRC, "native.cpp")
+    newest = max(os.path.getmtime(f) for f in (src, os.path.join(ROOT, "include", "rattn.h"), __file__))
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) >= newest:
+        return NATIVE
+    import sysconfig
+
+    import torch
+    base = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    inc = [os.path.join(base, "include"), os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(ROOT, "include")]
+    lib = os.path.join(base, "lib")
+    # the libraries are the ones `import torch` has loaded already
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", src, "-o", NATIVE,
+           *["-I" + d for d in inc], f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for native.cpp:\n{r.stdout}\n{r.stderr}")
+    return NATIVE
+
+
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
     print(build(force="--force" in sys.argv, debug=True))
+    print(NATIVE)
