@@ -172,13 +172,13 @@ typedef struct rattn_params {
  * device memory on its own: where the tensor-core path applies (d = 128, w % 128 == 0)
  * it needs scratch for the chunk states of the linear branch
  * (rattn_workspace_bytes_ex(..., RATTN_MODE_RATTN, 0) bytes) and obtains it with
- * cudaMallocAsync / cudaFreeAsync on `stream` (the device's stream-ordered pool; no
- * synchronisation).  Callers that must control every allocation use rattn_forward_ex
- * with their own workspace.  That scratch, and the status word in it, are gone when the call
- * returns, so the word is latched into the library before the scratch is freed:
- * rattn_forward_status (synchronises the stream) returns RATTN_ERR_TIMEOUT if a bounded
- * device-side wait has expired in any rattn_forward call on the current device since it was
- * last asked, else RATTN_OK.
+ * cudaMallocFromPoolAsync / cudaFreeAsync on `stream` from a stream-ordered pool of its own (one per
+ * device; no synchronisation).  The pool keeps up to 256 MiB of freed scratch for the calls that
+ * follow; rattn_forward_status gives it back to the device.  Callers that must control every
+ * allocation use rattn_forward_ex with their own workspace.  The scratch is gone when the call
+ * returns, so its kernels report to a word inside the library: rattn_forward_status (synchronises
+ * the stream) returns RATTN_ERR_TIMEOUT if a bounded device-side wait has expired in any
+ * rattn_forward call on the current device since it was last asked, else RATTN_OK.
  */
 int rattn_forward(const void* q, const void* k, const void* v,
                   int B, int H_q, int H_kv, int T, int d, int w,

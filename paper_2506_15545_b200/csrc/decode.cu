@@ -344,8 +344,7 @@ template <typename TIO, int D>
 cudaError_t launch_dec(const DecodeArgs& a, cudaStream_t s) {
   const size_t smem = decode_smem_floats<D>(a.group, a.w) * sizeof(float);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(decode_kernel<TIO, D>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem<decode_kernel<TIO, D>>((int)smem);
   if (e != cudaSuccess) return e;
   { KernelTimer kt("decode_step", s); decode_kernel<TIO, D><<<a.B * a.H_kv, DEC_THREADS, smem, s>>>(a); }
   count_launches(1);
@@ -423,31 +422,37 @@ __global__ void __launch_bounds__(256) handoff_state_kernel(const TIO* __restric
   for (int c = 0; c < D / 32; ++c) state[((size_t)bh * D + r0 + row) * D + cl + 32 * c] = acc[c];
 }
 
-// ring[b,hk, j % w] = x[b,hk, j] for the last min(w,T) tokens; other slots zero.
-template <typename TIO>
-__global__ void handoff_ring_kernel(const TIO* __restrict__ k, const TIO* __restrict__ v,
-                                    TIO* __restrict__ kr, TIO* __restrict__ vr, int T, int w, int D,
-                                    const int* __restrict__ len, int H_kv, int pos_shift, int layout) {
+// ring[b,hk, j % w] = x[b,hk, j] for the last min(w,T) tokens; other slots zero.  A copy bound by HBM: one 16-byte
+// vector of K and of V per thread (as single elements, a block per slot, it ran at a tenth of the copy rate: 19 us
+// for 64 heads at w = 512).  zero_state: no token has left the window yet, so the head's state is all zeros.
+__global__ void __launch_bounds__(256) handoff_ring_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v,
+                                                           uint4* __restrict__ kr, uint4* __restrict__ vr, int T, int w,
+                                                           int vec_shift, const int* __restrict__ len, int H_kv,
+                                                           int pos_shift, int layout, float4* __restrict__ zero_state,
+                                                           int state_vecs) {
   const int bh = blockIdx.y;
-  const size_t head0 = layout ? ((size_t)(bh / H_kv) * T * H_kv + bh % H_kv) * D : (size_t)bh * T * D;
-  const size_t pitch = layout ? (size_t)H_kv * D : (size_t)D;
-  const int slot = blockIdx.x;
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (zero_state) {
+    for (int e = i; e < state_vecs; e += gridDim.x * 256)
+      zero_state[(size_t)bh * state_vecs + e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  const int slot = i >> vec_shift, c = i & ((1 << vec_shift) - 1);
+  if (slot >= w) return;
+  const size_t head0 = layout ? ((size_t)(bh / H_kv) * T * H_kv + bh % H_kv) << vec_shift : ((size_t)bh * T) << vec_shift;
+  const size_t pitch = (size_t)(layout ? H_kv : 1) << vec_shift;
   // Row j of k, v is the token at sequence position j + pos_shift (a resumed sequence's rows start
   // before the chunk); the ring keeps position p at slot p % w.  The newest row that maps to this slot:
   const int Tb = len ? min(T, len[bh / H_kv]) : T;
   const int last = Tb - 1;
   const int j = last - ((last + pos_shift - slot) % w + w) % w;
-  const bool valid = j >= 0 && j >= Tb - w;
-  for (int c = threadIdx.x; c < D; c += blockDim.x) {
-    const size_t dst = ((size_t)bh * w + slot) * D + c;
-    if (valid) {
-      kr[dst] = k[head0 + (size_t)j * pitch + c];
-      vr[dst] = v[head0 + (size_t)j * pitch + c];
-    } else {
-      kr[dst] = from_f<TIO>(0.f);
-      vr[dst] = from_f<TIO>(0.f);
-    }
+  uint4 kk = make_uint4(0u, 0u, 0u, 0u), vv = kk;
+  if (j >= 0 && j >= Tb - w) {
+    kk = k[head0 + (size_t)j * pitch + c];
+    vv = v[head0 + (size_t)j * pitch + c];
   }
+  const size_t dst = (((size_t)bh * w) << vec_shift) + i;
+  kr[dst] = kk;
+  vr[dst] = vv;
 }
 
 template <typename TIO, int D>
@@ -462,13 +467,13 @@ cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too) {
     count_launches(1);
   }
   if (a.k_ring_out && a.v_ring_out) {
-    dim3 grid(a.w, BH);
+    constexpr int vec_shift = (D == 128 ? 4 : 3) + (sizeof(TIO) == 4 ? 1 : 0);      // 16-byte vectors per row: 1 << shift
+    dim3 grid((unsigned)((((size_t)a.w << vec_shift) + 255) / 256), BH);
     KernelTimer kt("handoff_ring", s);
-    handoff_ring_kernel<TIO><<<grid, 64, 0, s>>>(reinterpret_cast<const TIO*>(a.k),
-                                                 reinterpret_cast<const TIO*>(a.v),
-                                                 reinterpret_cast<TIO*>(a.k_ring_out),
-                                                 reinterpret_cast<TIO*>(a.v_ring_out), a.Tk, a.w, D, a.seq_lens,
-                                                 a.H_kv, a.pos_shift, a.kv_layout);
+    handoff_ring_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const uint4*>(a.k), reinterpret_cast<const uint4*>(a.v),
+                                             reinterpret_cast<uint4*>(a.k_ring_out), reinterpret_cast<uint4*>(a.v_ring_out),
+                                             a.Tk, a.w, vec_shift, a.seq_lens, a.H_kv, a.pos_shift, a.kv_layout,
+                                             a.zero_state ? reinterpret_cast<float4*>(a.state_out) : nullptr, D * D / 4);
     count_launches(1);
   }
   return cudaGetLastError();

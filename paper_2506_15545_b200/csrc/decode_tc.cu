@@ -488,7 +488,7 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
 
 template <int G>
 cudaError_t launch_g(const DecodeTcArgs& a, const DecodeTcMaps& m, int smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(decode_tc_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem<decode_tc_kernel<G>>(smem);
   if (e != cudaSuccess) return e;
   { KernelTimer kt("decode_step", s); decode_tc_kernel<G><<<a.B * a.H_kv, DT_THREADS, smem, s>>>(a, m); }
   count_launches(1);

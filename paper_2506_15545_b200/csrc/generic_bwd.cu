@@ -386,9 +386,9 @@ cudaError_t launch_bwd(const Args& a, cudaStream_t s) {
   constexpr int LD = D + PAD;
   constexpr size_t smem_dq = (size_t)(4 * 32 * LD + 3 * 64 * LD + 32 * (64 + PAD) + 64) * sizeof(float);
   constexpr size_t smem_dkv = (size_t)(4 * 32 * LD + 3 * 64 * LD + 64 * (32 + PAD) + 64) * sizeof(float);
-  e = cudaFuncSetAttribute(bwd_dq_kernel<TIO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_dq);
+  e = allow_smem<bwd_dq_kernel<TIO, D>>((int)smem_dq);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(bwd_dkv_kernel<TIO, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_dkv);
+  e = allow_smem<bwd_dkv_kernel<TIO, D>>((int)smem_dkv);
   if (e != cudaSuccess) return e;
   dim3 gq((a.T + 31) / 32, a.B * a.H_q);
   { KernelTimer kt("generic_bwd_dq", s); bwd_dq_kernel<TIO, D><<<gq, NT, smem_dq, s>>>(a, do_s, do_r, delta); }

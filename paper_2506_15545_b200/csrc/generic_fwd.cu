@@ -196,8 +196,7 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
 template <typename TIO, int D>
 cudaError_t launch_fwd(const Args& a, cudaStream_t s) {
   constexpr size_t smem = (size_t)(5 * BM * (D + PAD) + BM * (BN + PAD)) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(generic_fwd_kernel<TIO, D>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem<generic_fwd_kernel<TIO, D>>((int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.T + BM - 1) / BM, a.B * a.H_q);
   { KernelTimer kt("generic_fwd", s); generic_fwd_kernel<TIO, D><<<grid, NT, smem, s>>>(a); }

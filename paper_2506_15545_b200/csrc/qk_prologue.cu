@@ -514,15 +514,22 @@ void fill(const rattn_qk_params* p, QkArgs* a, Freqs* f) {
   a->partial = nullptr;
   a->dy[0] = a->dy[1] = nullptr;
   a->y[0] = a->y[1] = nullptr;
-  for (int i = 0; i < 64; ++i)
-    f->inv[i] = a->rotate && i < p->d / 2 ? std::pow((double)p->theta, -2.0 * i / p->d) : 0.0;
+  if (!a->rotate) return;                  // the kernels then read no frequency
+  // The frequencies depend on theta and d alone, which a model never changes: 64 powers (2.5 us of host time) are
+  // formed when a thread meets another pair of them.
+  thread_local struct { float theta = 0.f; int d = 0; Freqs f; } known;
+  if (known.theta != p->theta || known.d != p->d) {
+    for (int i = 0; i < 64; ++i) known.f.inv[i] = i < p->d / 2 ? std::pow((double)p->theta, -2.0 * i / p->d) : 0.0;
+    known.theta = p->theta;
+    known.d = p->d;
+  }
+  *f = known.f;
 }
 
 // CTAs of a launch: every resident slot of the device, fewer when there are fewer chunks
 cudaError_t grid_size(const QkArgs& a, int per_sm, int* n_cta) {
-  int dev = 0, n_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  int n_sm = 0;
+  const cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
   long long n = (long long)a.n_chunks[0] + a.n_chunks[1];
   if (n > (long long)n_sm * per_sm) n = (long long)n_sm * per_sm;
@@ -534,7 +541,7 @@ cudaError_t grid_size(const QkArgs& a, int per_sm, int* n_cta) {
 template <typename T, int D, bool BWD, bool BTHD>
 cudaError_t launch_layout(const QkArgs& a, const Freqs& f, int n_cta, cudaStream_t s) {
   const int smem = Ring<T, BWD>::kBytes + 2 * a.tbl_tokens * (D / 2) * (int)sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(qk_prologue_kernel<T, D, BWD, BTHD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem<qk_prologue_kernel<T, D, BWD, BTHD>>(smem);
   if (e != cudaSuccess) return e;
   KernelTimer kt(BWD ? "qk_prologue_bwd" : "qk_prologue", s);
   qk_prologue_kernel<T, D, BWD, BTHD><<<n_cta, QK_THREADS, smem, s>>>(a, f);

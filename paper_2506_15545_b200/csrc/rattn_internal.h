@@ -7,6 +7,9 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <mutex>
+
 #include "rattn.h"
 
 namespace rattn {
@@ -74,8 +77,8 @@ struct Args {
   float* lse2p;
   float* dscp;
   int n_chunks;
-  int* status;                 // device status block (may be null when no workspace): word 0 status,
-                               // word 1 detail, word 2 the forward's work counter
+  int* status;                 // device status word (may be null when no workspace)
+  int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin)
   int* state_ready;            // [B*H_kv], zero at launch: chunk states the chunk-state kernel has stored so far
                                // (null: the main kernel waits for that whole kernel instead)
   bool training;               // the backward will read every chunk state
@@ -83,6 +86,7 @@ struct Args {
   float* state_out;
   void* k_ring_out;
   void* v_ring_out;
+  bool zero_state;             // the ring hand-off also clears state_out (no token has left the window)
   // backward
   const void* dout;
   void* dq;
@@ -148,6 +152,27 @@ int debug_skip_arrive();                    // always 0 outside the debug build
 int tuning(int knob);                       // current value of a rattn_knob
 void count_launches(int n);
 void set_last_cuda_error(int cuda_error);   // what rattn_last_cuda_error() reports for this thread
+
+// Multiprocessors of the current device, asked of the driver once per device.
+cudaError_t sm_count(int* n_sm);
+constexpr int kMaxDevices = 64;
+// Lets the kernel use `bytes` of dynamic shared memory on the current device.  The driver is called only when a
+// device meets a larger size than before: as a call per launch it cost small launches a microsecond of host time.
+template <auto Kernel>
+cudaError_t allow_smem(int bytes) {
+  static std::atomic<int> granted[kMaxDevices];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (granted[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
+  static std::mutex mu;                    // of two threads the one with the larger size must come last
+  std::lock_guard<std::mutex> lk(mu);
+  if (granted[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) granted[dev].store(bytes, std::memory_order_relaxed);
+  return e;
+}
 
 // Records a CUDA event pair around one kernel launch on its stream while per-kernel
 // timing is enabled (rattn_timing_enable); free otherwise.

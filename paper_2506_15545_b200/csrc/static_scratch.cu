@@ -23,7 +23,6 @@ constexpr size_t kStateBytes = kMatrices * 128 * 128 * sizeof(__nv_bfloat16);
 // [status block, 256 B | progress words, 256 B | chunk states, bf16]
 static __device__ __align__(256) unsigned char g_static_scratch[kStatusBytes + kStateBytes];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 unsigned char* g_scratch_addr[kMaxDevices] = {};
 
@@ -85,6 +84,7 @@ extern "C" int rattn_forward_static(const void* q, const void* k, const void* v,
   e = scratch_address(&base);
   if (e != cudaSuccess) return cuda_failure(e);
   a.status = reinterpret_cast<int*>(base);
+  a.work_counter = a.status + 2;
   a.state_ready = reinterpret_cast<int*>(base + 256);
   a.chunk_state = reinterpret_cast<__nv_bfloat16*>(base + kStatusBytes);
   a.n_chunks = n_chunks;

@@ -1214,7 +1214,9 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   const bool rla_on = (a.mode == RATTN_MODE_RATTN);
   const int n_qt = (a.T + TILE - 1) / TILE;
   const int wt = a.w / TILE;
-  cudaError_t e;
+  int n_sm = 0;
+  cudaError_t e = sm_count(&n_sm);
+  if (e != cudaSuccess) return e;
   if (a.dgamma_swa) {
     e = cudaMemsetAsync(a.dgamma_swa, 0, sizeof(float) * a.H_q * 128, s);
     if (e != cudaSuccess) return e;
@@ -1235,10 +1237,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     pa.status = a.status;
     pa.n_heads = a.B * a.H_q; pa.T = a.T; pa.t_pad = t_pad; pa.H_q = a.H_q; pa.rla_on = rla_on ? 1 : 0;
     pa.eps = a.eps; pa.scale = a.scale;
-    int dev = 0, n_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_bwd_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PREP_SMEM);
+    e = allow_smem<tc_bwd_prep_kernel>(PREP_SMEM);
     if (e != cudaSuccess) return e;
     const long long n_chunks_all = (long long)pa.n_heads * (t_pad / PREP_ROWS);
     const int grid = (int)(n_chunks_all < 2ll * n_sm ? n_chunks_all : 2ll * n_sm);
@@ -1287,18 +1286,13 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   t.T = a.T; t.w = a.w; t.H_q = a.H_q; t.group = a.group; t.mode = a.mode; t.n_chunks = a.n_chunks;
   t.scale = a.scale; t.scale_log2 = a.scale * LOG2E;
   t.phi = a.phi;
-  e = cudaFuncSetAttribute(tc_bwd_dq_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DQ_SMEM);
+  e = allow_smem<tc_bwd_dq_kernel>(DQ_SMEM);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(tc_bwd_dkv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, KV_SMEM);
+  e = allow_smem<tc_bwd_dkv_kernel>(KV_SMEM);
   if (e != cudaSuccess) return e;
   {
     DqMaps dm;
     dm.q = tm_q; dm.k = tm_k; dm.v = tm_v; dm.gs = tm_gs; dm.gr = tm_gr; dm.st = tm_st; dm.dq = tm_dq;
-    int dev = 0, n_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
     const int n_items = n_qt * (int)nq;
     KernelTimer kt("tc_bwd_dq", s);
     tc_bwd_dq_kernel<<<n_items < n_sm ? n_items : n_sm, DQ_THREADS, DQ_SMEM, s>>>(dm, t, n_items, n_qt);
@@ -1309,11 +1303,6 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
       !make_map(&km.grh, g_r, a.T, nq, 64))
     return cudaErrorInvalidValue;
   {
-    int dev = 0, n_sm = 0;
-    e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
     const int n_items = n_qt * (int)nkv;
     KernelTimer kt("tc_bwd_dkv", s);
     tc_bwd_dkv_kernel<<<n_items < n_sm ? n_items : n_sm, KV_THREADS, KV_SMEM, s>>>(km, t, n_items);

@@ -33,12 +33,12 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
   bool progress = a.state_ready != nullptr;
   if (progress) {
     const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
-    int dev = 0, n_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n_sm = 0;
+    int n_sm = 0;
+    const cudaError_t e = sm_count(&n_sm);
+    if (e != cudaSuccess) return e;
     progress = knob == 1 || (knob == 0 && 4 * n_kv <= n_sm && n_kt >= 48 && wt <= 4);
   }
-  if (want_state && a.Tk <= a.w && !a.seq_lens) {
+  if (want_state && a.Tk <= a.w && !a.seq_lens && !a.zero_state) {
     // nothing has left the window yet
     cudaError_t e = cudaMemsetAsync(a.state_out, 0, sizeof(float) * (size_t)n_kv * 128 * 128, s);
     if (e != cudaSuccess) return e;

@@ -888,10 +888,8 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
       !make_map(&tm.o_swa, a.o_swa ? (const void*)a.o_swa : a.out, a.T, (uint64_t)a.B * a.H_q) ||
       !make_map(&tm.o_rla, a.o_rla ? (const void*)a.o_rla : a.out, a.T, (uint64_t)a.B * a.H_q))
     return cudaErrorInvalidValue;
-  int dev = 0, n_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  int n_sm = 0;
+  cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
   FArgs t;
   t.lse = a.lse;
@@ -923,8 +921,8 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   // have put the units without a state first anyway (few K/V heads, many SMs free beside the chain)
   t.ascending = (t.state_ready && t.n_stateless > 0) ? 1 : 0;
   t.debug_skip_arrive = debug_skip_arrive();
-  t.work_counter = (a.status && order != 3) ? a.status + 2 : nullptr;
-  e = cudaFuncSetAttribute(tc_fwd2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, F_SMEM);
+  t.work_counter = order != 3 ? a.work_counter : nullptr;
+  e = allow_smem<tc_fwd2_kernel>(F_SMEM);
   if (e != cudaSuccess) return e;
   if (tuning(RATTN_TUNE_GRID) > 0 && tuning(RATTN_TUNE_GRID) < n_sm) n_sm = tuning(RATTN_TUNE_GRID);
   const int grid = t.n_units < n_sm ? t.n_units : n_sm;

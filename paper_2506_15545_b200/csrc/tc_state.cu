@@ -300,7 +300,7 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   a.seq_lens = L.seq_lens; a.kv_per_batch = L.kv_per_batch > 0 ? L.kv_per_batch : 1;
   a.phi = L.phi;
   a.ready = (L.dir > 0 && L.group == 1) ? L.ready : nullptr;
-  cudaError_t e = cudaFuncSetAttribute(tc_state_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
+  cudaError_t e = allow_smem<tc_state_scan_kernel>(ST_SMEM);
   if (e != cudaSuccess) return e;
   {
     KernelTimer kt(L.name, s);
