@@ -124,6 +124,7 @@ WorkspaceLayout workspace_layout(int B, int H_q, int H_kv, int T, int d, int w, 
   L.delta = take(train, rows * sizeof(float));
   L.chunk_state = take(tc && rla, states * sizeof(__nv_bfloat16));
   L.rstate = take(tc && rla && train, states * sizeof(__nv_bfloat16));
+  L.rdelta = take(tc && rla && train && (long long)B * H_kv * L.n_chunks <= kMaxParallelTerms, states * sizeof(float));
   L.lse2p = take(tc && train, rows_pad * sizeof(float));
   L.dscp = take(tc && train, rows_pad * sizeof(float));
   const size_t io_elem = dtype == RATTN_F32 ? sizeof(float) : sizeof(__nv_bfloat16);
@@ -190,6 +191,7 @@ static int bind_workspace(const rattn_params* p, Args* a, bool required, unsigne
   a->delta = reinterpret_cast<float*>(at(L.delta));
   a->chunk_state = reinterpret_cast<__nv_bfloat16*>(at(L.chunk_state));
   a->rstate = reinterpret_cast<__nv_bfloat16*>(at(L.rstate));
+  a->rdelta = reinterpret_cast<float*>(at(L.rdelta));
   a->lse2p = reinterpret_cast<float*>(at(L.lse2p));
   a->dscp = reinterpret_cast<float*>(at(L.dscp));
   a->n_chunks = L.n_chunks;

@@ -28,6 +28,7 @@ struct WorkspaceLayout {
   size_t delta;         // fp32 [B,H_q,T]      backward scratch
   size_t chunk_state;   // bf16 [B,H_kv,n_chunks,d,d]  exclusive prefix over chunks
   size_t rstate;        // bf16 [B,H_kv,n_chunks,d,d]  backward: suffix sums of phi(Q)^T g_r
+  size_t rdelta;        // fp32 [B,H_kv,n_chunks,d,d]  backward: their terms, where these are formed in parallel
   size_t lse2p;         // fp32 [B*H_q, n_chunks*128]  backward: lse * log2(e), +inf in the padding
   size_t dscp;          // fp32 [B*H_q, n_chunks*128]  backward: D_t * scale, 0 in the padding
   size_t k_ext;         // I/O type [B,H_kv,w+T,d]  chunked prefill: history + chunk keys, in time order
@@ -35,6 +36,12 @@ struct WorkspaceLayout {
   size_t total;
   int n_chunks;         // ceil(T / 128)
 };
+
+// The reverse states of the backward are a running sum over the query tiles of each K/V head.  Walked by one CTA per
+// head (tc_state.cu) the chain takes a microsecond per tile and query head of the group on as few SMs as there are
+// heads.  Up to this many terms (64 KB each) they are formed by a CTA each and summed by a second kernel instead; with
+// more of them the chain runs beside the dq kernel, which hides it.
+constexpr long long kMaxParallelTerms = 512;
 
 // Offset of a region the call does not use.
 constexpr size_t kAbsent = ~(size_t)0;
@@ -74,11 +81,13 @@ struct Args {
   // tensor-path scratch
   __nv_bfloat16* chunk_state;
   __nv_bfloat16* rstate;
+  float* rdelta;
   float* lse2p;
   float* dscp;
   int n_chunks;
   int* status;                 // device status word (may be null when no workspace)
-  int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin)
+  int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin);
+                               // the backward's two kernels use the two words behind it
   int* state_ready;            // [B*H_kv], zero at launch: chunk states the chunk-state kernel has stored so far
                                // (null: the main kernel waits for that whole kernel instead)
   bool training;               // the backward will read every chunk state
@@ -140,6 +149,9 @@ struct StateLaunch {
   int phi;                  // rattn_feature_map applied to x
   int* status;
   int* ready;               // optional [n_kv] (forward chain): matrices stored so far, published after each store
+  float* delta;             // optional fp32 scratch, n_kv * n_steps matrices: the terms are formed in parallel and
+                            // summed by a second kernel (store_every = 1, no hand-off, no incoming state)
+  bool after_independent;   // the kernel before on the stream neither feeds this one nor is fed by it: they may overlap
   const char* name;         // label of the timing record
 };
 cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s);

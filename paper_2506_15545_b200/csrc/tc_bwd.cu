@@ -48,10 +48,61 @@ struct BwdArgs {
   const float* dscp;    // [B*H_q, t_pad]  D_t * scale, 0 beyond T
   int t_pad;
   int* status;
-  int T, w, H_q, group, mode, n_chunks;
+  int* counter;         // next item of the launch (device memory, zero at launch)
+  int wait_before;      // 1: the kernel ahead (the reverse states' chain) may still be running; not to end before it
+  int T, w, H_q, group, mode, n_chunks, n_bh;   // n_bh: query heads (dq), K/V heads (dk/dv) over the batch
   int phi;              // rattn_feature_map
   float scale, scale_log2;
 };
+
+// ------------------------------------------------------------------------ work items
+// Both main kernels are persistent; a CTA's next item comes from a device-wide counter, so that CTAs that start late
+// (the SM was still running another kernel) or meet heavy items simply take fewer.  The loader warp draws it and
+// publishes it in a small ring that the other roles read in order; a slot is rewritten once every reader has read it.
+constexpr int SCHED_SLOTS = 4;
+struct SchedRing {
+  uint64_t full[SCHED_SLOTS], free_[SCHED_SLOTS];
+  int item[SCHED_SLOTS];
+};
+__device__ __forceinline__ void sched_init(SchedRing* r, int readers) {
+  for (int i = 0; i < SCHED_SLOTS; ++i) {
+    mbar_init(&r->full[i], 1);
+    mbar_init(&r->free_[i], readers);
+  }
+}
+// the loader warp's side: item n of this CTA, -1 when there is none left
+__device__ __forceinline__ bool sched_draw(SchedRing* r, int* counter, int n_items, int n, volatile int* abort, int* out) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (use >= 1) { if (!mbar_wait_warp(&r->free_[slot], (use - 1) & 1, abort)) return false; }
+  int i = 0;
+  if ((threadIdx.x & 31) == 0) i = atomicAdd(counter, 1);
+  i = __shfl_sync(0xffffffffu, i, 0);
+  if (i >= n_items) i = -1;
+  if ((threadIdx.x & 31) == 0) {
+    r->item[slot] = i;
+    mbar_arrive(&r->full[slot]);
+  }
+  __syncwarp();
+  *out = i;
+  return true;
+}
+// a reading thread's side
+__device__ __forceinline__ bool sched_read(SchedRing* r, int n, volatile int* abort, int* out) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (!mbar_wait(&r->full[slot], use & 1, abort)) return false;
+  *out = r->item[slot];
+  mbar_arrive(&r->free_[slot]);
+  return true;
+}
+// ... and a whole warp's (one of its lanes is counted)
+__device__ __forceinline__ bool sched_read_warp(SchedRing* r, int n, volatile int* abort, int* out) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (!mbar_wait_warp(&r->full[slot], use & 1, abort)) return false;
+  *out = r->item[slot];
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&r->free_[slot]);
+  return true;
+}
 
 #define WAIT_OR_RETURN(bar, parity) \
   do { if (!mbar_wait(&(bar), (parity), &bars->abort)) return false; } while (0)
@@ -83,6 +134,7 @@ struct PrepArgs {
   float* delta; float* dgamma_s; float* dgamma_r;
   const float* lse; float* lse2p; float* dscp;
   int* status;
+  int* counters;        // work counters of the two main kernels: cleared here
   int n_heads, T, t_pad, H_q, rla_on;
   float eps, scale;
 };
@@ -113,6 +165,7 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
     for (int i = 0; i < PREP_STAGES; ++i) mbar_init(&full[i], 1);
     *abort = 0;
     fence_mbar_init();
+    if (blockIdx.x == 0) a.counters[0] = a.counters[1] = 0;
   }
   __syncthreads();
 
@@ -308,14 +361,17 @@ constexpr int DQ_OFF_K = 2 * TILE_BYTES;   // 2 stages
 constexpr int DQ_OFF_V = 4 * TILE_BYTES;   // 2 stages
 constexpr int DQ_OFF_Q1 = 6 * TILE_BYTES;  // Q buffer 1
 constexpr int DQ_OFF_BAR = 7 * TILE_BYTES;
-constexpr int DQ_SMEM = DQ_OFF_BAR + 256;
+constexpr int DQ_SMEM = DQ_OFF_BAR + 384;
 constexpr int DQ_THREADS = 320;            // 2 row groups, MMA warp, loader warp
 
 struct DqBars {
   uint64_t qg_full, kv_full[2], kv_free[2], s_full, ds_full, phik_ready, o_done, acc_free, q_read, drain;
+  SchedRing sched;
   uint32_t tmem_base;
   int abort;
 };
+
+static_assert(sizeof(DqBars) <= DQ_SMEM - DQ_OFF_BAR, "barriers");
 
 struct DqItem {
   int q0, bh_q, bh_kv, n_kt, st_index;
@@ -324,8 +380,9 @@ struct DqItem {
 
 __device__ __forceinline__ DqItem dq_item(const BwdArgs& a, int idx, int n_qt) {
   DqItem it;
-  it.bh_q = idx / n_qt;
-  const int qt = n_qt - 1 - idx % n_qt;                    // long bands first within a head
+  const int rank = idx / a.n_bh;                           // long bands first
+  it.bh_q = idx - rank * a.n_bh;
+  const int qt = n_qt - 1 - rank;
   it.q0 = qt * TILE;
   const int b = it.bh_q / a.H_q, h = it.bh_q % a.H_q;
   it.bh_kv = b * (a.H_q / a.group) + h / a.group;
@@ -347,7 +404,10 @@ struct DqMaps {
 __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, int n_items, int n_qt) {
   int kc = 0, n = 0, co = 0;                               // ring uses, items, o_done completions of the items so far
   int co_window = 0;                                       // the completion that ends the previous item's window products
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++n) {
+  for (;; ++n) {
+    int idx;
+    if (!sched_draw(&bars->sched, a.counter, n_items, n, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     auto ring_wait = [&]() -> bool {                       // the slot's previous user has been consumed
       const int st = kc & 1, use = kc >> 1;
@@ -393,12 +453,15 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
   return true;
 }
 
-__device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int n_items, int n_qt) {
+__device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int n_qt) {
   const uint32_t sG = smem_u32(smem + DQ_OFF_G), sK = smem_u32(smem + DQ_OFF_K), sV = smem_u32(smem + DQ_OFF_V);
   const uint32_t tS = tmem, tP = tmem + 128, tQ = tmem + 256, tF = tmem + 384;
   constexpr uint32_t idesc_ts = instr_desc(128, 128, 0, 1);
   int kc = 0, n = 0, cs = 0, cr = 0;                       // ring uses, items, score hand-overs, residual items
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++n) {
+  for (;; ++n) {
+    int idx;
+    if (!sched_read_warp(&bars->sched, n, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     const uint32_t sQ = smem_u32(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q));
     WAIT_OR_RETURN_W(bars->qg_full, n & 1);
@@ -446,13 +509,16 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
 }
 
 __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int g, int r,
-                        int n_items, int n_qt) {
+                        int n_qt) {
   const uint32_t lane_off = (uint32_t)((r & ~31) << 16);
   const uint32_t tS = tmem + lane_off, tP = tmem + 128 + lane_off, tQ = tmem + 256 + lane_off,
                  tF = tmem + 384 + lane_off;
   int kc = 0, n = 0, cs = 0, co = 0;                       // ring uses, items, score hand-overs, o_done completions
   bool store_pending = false;                              // this thread issued a dQ store whose read-out it has not confirmed
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++n) {
+  for (;; ++n) {
+    int idx;
+    if (!sched_read(&bars->sched, n, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     const int n_kt = it.n_kt;
     unsigned char* sQ = smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q);
@@ -638,11 +704,14 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   extern __shared__ __align__(1024) unsigned char smem[];
   DqBars* bars = reinterpret_cast<DqBars*>(smem + DQ_OFF_BAR);
   const int tid = threadIdx.x, warp = tid >> 5;
+  // a kernel that does not read dq may take the SMs that run out of items
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0 && a.status) atomicExch(a.status, 2);
     return;
   }
   if (tid == 0) {
+    sched_init(&bars->sched, 256 + 1);
     mbar_init(&bars->qg_full, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->kv_full[i], 1);
@@ -678,9 +747,9 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
 
   bool ok = true;
   if (warp < 8) {
-    ok = dq_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127, n_items, n_qt);
+    ok = dq_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127, n_qt);
   } else if (warp == 8) {
-    ok = dq_mma(a, smem, bars, tmem, n_items, n_qt);
+    ok = dq_mma(a, smem, bars, tmem, n_qt);
     if (!ok) {
       mma_commit(&bars->drain);
       for (int it = 0; it < (1 << 16) && !mbar_try_wait(&bars->drain, 0); ++it) {}
@@ -689,6 +758,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     ok = dq_loader(tm, a, smem, bars, n_items, n_qt);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
+  if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   if (warp == 8) {
@@ -720,15 +790,18 @@ constexpr int KV_OFF_OUT = 3 * TILE_BYTES;                 // stages dV at the e
 constexpr int KV_OFF_STAGE = 4 * TILE_BYTES;               // KV_NS x [Q_h 16 KB | g_h 16 KB]
 constexpr int KV_OFF_STAT = KV_OFF_STAGE + KV_NS * TILE_BYTES;   // KV_NS x (lse2[64], D*scale[64]) fp32
 constexpr int KV_OFF_BAR = KV_OFF_STAT + KV_NS * 512;
-constexpr int KV_SMEM = KV_OFF_BAR + 256;
+constexpr int KV_SMEM = KV_OFF_BAR + 384;
 constexpr int KV_THREADS = 352;                            // 2 row groups, score warp, loader warp, accumulate warp
 
 struct KvBars {
   uint64_t kv_full, kphi_ready, full[KV_NS], acc_done[KV_NS], s_full[2], p_ready[2], phiq_ready[2],
       r_acc_done, fold_done, all_done, acc_free, out_read, drain, drain2;
+  SchedRing sched;
   uint32_t tmem_base;
   int abort;
 };
+
+static_assert(sizeof(KvBars) <= KV_SMEM - KV_OFF_BAR, "barriers");
 
 struct KvMaps {
   UMap k, v, qh, dk, dv;        // the caller's tensors (either head layout)
@@ -750,8 +823,8 @@ struct KvPlan {
 __device__ __forceinline__ KvPlan kv_plan(const BwdArgs& a, int idx) {
   KvPlan pl;
   pl.n_qt = (a.T + TILE - 1) / TILE;
-  pl.bh_kv = idx / pl.n_qt;
-  pl.j = idx % pl.n_qt;
+  pl.j = idx / a.n_bh;                                     // most query tiles first
+  pl.bh_kv = idx - pl.j * a.n_bh;
   pl.rs_index = pl.bh_kv * a.n_chunks + pl.j;
   pl.wt = a.w / TILE;
   pl.group = a.group;
@@ -773,7 +846,10 @@ struct KvCount {
 
 __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* smem, KvBars* bars, int n_items) {
   KvCount c = {0, 0, 0, 0};
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++c.it) {
+  for (;; ++c.it) {
+    int idx;
+    if (!sched_draw(&bars->sched, a.counter, n_items, c.it, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const KvPlan pl = kv_plan(a, idx);
     const int j0 = pl.j * TILE;
     // K_j, V_j replace the previous key tile's once every product that read them has completed
@@ -828,7 +904,7 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
 // group -> accumulate on its TMEM slot, of which there are two.  Order between the two warps:
 //   scores(n) -> row group -> p_ready -> accumulate(n)        (existing barriers)
 //   accumulate(n - 2) complete -> scores(n) may overwrite the TMEM slot they share   (acc_done of n - 2's stage)
-__device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int n_items) {
+__device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem) {
   const uint32_t sK = smem_u32(smem + KV_OFF_K), sV = smem_u32(smem + KV_OFF_V), sKphi = smem_u32(smem + KV_OFF_KPHI);
   const uint32_t sStage = smem_u32(smem + KV_OFF_STAGE);
   // slot s: [S^T | dP^T] at columns 256 + 128 s and 320 + 128 s (computed, not looked up: an array
@@ -837,7 +913,10 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
   KvCount c = {0, 0, 0, 0};
   int cq0 = 0, cq1 = 0;                                    // phi(Q_h) hand-overs per TMEM slot
 
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++c.it) {
+  for (;; ++c.it) {
+    int idx;
+    if (!sched_read_warp(&bars->sched, c.it, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const KvPlan pl = kv_plan(a, idx);
     // K_j, V_j have landed (which also means every product of the previous key tile has completed)
     WAIT_OR_RETURN_W(bars->kv_full, c.it & 1);
@@ -868,14 +947,17 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
   return true;
 }
 
-__device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int n_items) {
+__device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem) {
   const uint32_t sV = smem_u32(smem + KV_OFF_V), sKphi = smem_u32(smem + KV_OFF_KPHI);
   const uint32_t sStage = smem_u32(smem + KV_OFF_STAGE);
   const uint32_t tV = tmem, tK = tmem + 128;
   const uint32_t tS0 = tmem + 256, tP0 = tmem + 320;
   KvCount c = {0, 0, 0, 0};
 
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x, ++c.it) {
+  for (;; ++c.it) {
+    int idx;
+    if (!sched_read_warp(&bars->sched, c.it, &bars->abort, &idx)) return false;
+    if (idx < 0) break;
     const KvPlan pl = kv_plan(a, idx);
     bool accV = false, accK = false;
     // the previous key tile's epilogue has read the two accumulators
@@ -916,7 +998,7 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
 }
 
 __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int gg,
-                        int r, int n_items) {
+                        int r) {
   // two groups of 128 threads (thread = key row = TMEM lane), one per TMEM slot; a thread takes
   // all 64 query columns of its item, 32 at a time (more row groups per slot measured no faster
   // and cost registers)
@@ -927,7 +1009,10 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   const unsigned char* sKphi = smem + KV_OFF_KPHI;
   KvCount cnt = {0, 0, 0, 0};
 
-  for (int idx = blockIdx.x; idx < n_items; idx += gridDim.x) {
+  for (;;) {
+  int idx;
+  if (!sched_read(&bars->sched, cnt.it, &bars->abort, &idx)) return false;
+  if (idx < 0) break;
   const KvPlan pl = kv_plan(a, idx);
   const int bh_kv = pl.bh_kv;
   if (gg < 2) {
@@ -1144,6 +1229,7 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     return;
   }
   if (tid == 0) {
+    sched_init(&bars->sched, 256 + 2);
     mbar_init(&bars->kv_full, 1);
     mbar_init(&bars->kphi_ready, 256);
     for (int i = 0; i < KV_NS; ++i) {
@@ -1186,9 +1272,9 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
 
   bool ok = true;
   if (warp < 8) {
-    ok = kv_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127, n_items);
+    ok = kv_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127);
   } else if (warp == 8 || warp == 10) {
-    ok = warp == 8 ? kv_mma_scores(a, smem, bars, tmem, n_items) : kv_mma_accum(a, smem, bars, tmem, n_items);
+    ok = warp == 8 ? kv_mma_scores(a, smem, bars, tmem) : kv_mma_accum(a, smem, bars, tmem);
     if (!ok) {                                             // let this warp's products in flight finish
       uint64_t* drain = warp == 8 ? &bars->drain : &bars->drain2;
       mma_commit(drain);
@@ -1234,7 +1320,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     pa.g_s = g_s; pa.g_r = g_r;
     pa.delta = a.delta; pa.dgamma_s = a.dgamma_swa; pa.dgamma_r = a.dgamma_rla;
     pa.lse = a.lse; pa.lse2p = a.lse2p; pa.dscp = a.dscp;
-    pa.status = a.status;
+    pa.status = a.status; pa.counters = a.work_counter + 1;
     pa.n_heads = a.B * a.H_q; pa.T = a.T; pa.t_pad = t_pad; pa.H_q = a.H_q; pa.rla_on = rla_on ? 1 : 0;
     pa.eps = a.eps; pa.scale = a.scale;
     e = allow_smem<tc_bwd_prep_kernel>(PREP_SMEM);
@@ -1259,24 +1345,6 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
       !make_state_map(&tm_st, a.chunk_state, a.k, nkv * a.n_chunks) || !make_state_map(&tm_rs, a.rstate, a.k, nkv * a.n_chunks))
     return cudaErrorInvalidValue;
 
-  // reverse states of the residual branch: chunks c with a query tile beyond c + wt
-  const int n_r = rla_on && a.mode != RATTN_MODE_FULL_CAUSAL ? n_qt - wt - 1 : 0;
-  // R_c for c = 0 .. n_r-1: walk the query tiles from the last one down to wt+1
-  {
-    StateLaunch L;
-    L.ready = nullptr;
-    L.x = a.q; L.y = g_r; L.out = a.rstate;
-    L.x_heads = a.H_q; L.x_layout = a.layout; L.y_heads = 0; L.y_layout = 0;
-    L.T = a.T; L.n_kv = (int)nkv; L.group = a.group; L.n_chunks = a.n_chunks;
-    L.n_steps = n_r; L.first = n_qt - 1; L.dir = -1; L.out_first = n_qt - wt - 2;
-    L.store_every = 1; L.store_phase = 0; L.handoff = 0; L.w = a.w; L.final_out = nullptr;
-    L.state_in = nullptr; L.seq_lens = nullptr; L.kv_per_batch = 1;
-    L.phi = a.phi;
-    L.status = a.status; L.name = "tc_state_bwd";
-    e = launch_tc_states(L, s);
-  }
-  if (e != cudaSuccess) return e;
-
   BwdArgs t;
   t.dq = reinterpret_cast<__nv_bfloat16*>(a.dq);
   t.dk = reinterpret_cast<__nv_bfloat16*>(a.dk);
@@ -1290,12 +1358,60 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   e = allow_smem<tc_bwd_dkv_kernel>(KV_SMEM);
   if (e != cudaSuccess) return e;
+
+  // Reverse states of the residual branch: R_c for c = 0 .. n_r-1 (chunks with a query tile beyond c + wt), a running
+  // sum that walks the query tiles from the last one down to wt+1.  The dq kernel does not read them, so the two share
+  // the GPU.  A serial chain (one CTA per K/V head) goes first, and the dq kernel runs beside it on the other SMs; that
+  // costs least as long as the chain is over by then (1.4 us per tile and query head, measured, against about
+  // 2 us per key tile + 5 us for a dq item; up to 15 % longer is still cheaper than the other way).  Where it would
+  // outlast the dq kernel, its terms are formed in parallel behind that kernel, on the SMs it runs out of items on: at
+  // 1 x 16/4 heads, T = 1111, w = 128 the chain took 46 us on four SMs beside a dq kernel of 16 us, the terms and their
+  // sum end 11 us behind it.  With a chain on more than half of the SMs there is nothing to share.
+  const int n_r = rla_on && a.mode != RATTN_MODE_FULL_CAUSAL ? n_qt - wt - 1 : 0;
+  const long long chain_ns = 1400ll * n_r * a.group, dq_ns = 1000ll * n_qt * (long long)nq * (2 * (wt + 1) + 5) / n_sm;
+  const bool few_heads = 2 * (int)nkv <= n_sm;
+  const bool parallel_terms = n_r > 0 && a.rdelta != nullptr && few_heads && 100 * chain_ns > 115 * dq_ns;
+  const bool chain_beside = n_r > 0 && !parallel_terms && few_heads;
+  StateLaunch L;
+  L.ready = nullptr;
+  L.x = a.q; L.y = g_r; L.out = a.rstate;
+  L.x_heads = a.H_q; L.x_layout = a.layout; L.y_heads = 0; L.y_layout = 0;
+  L.T = a.T; L.n_kv = (int)nkv; L.group = a.group; L.n_chunks = a.n_chunks;
+  L.n_steps = n_r; L.first = n_qt - 1; L.dir = -1; L.out_first = n_qt - wt - 2;
+  L.store_every = 1; L.store_phase = 0; L.handoff = 0; L.w = a.w; L.final_out = nullptr;
+  L.state_in = nullptr; L.seq_lens = nullptr; L.kv_per_batch = 1;
+  L.phi = a.phi;
+  L.status = a.status; L.name = "tc_state_bwd";
+  L.delta = parallel_terms ? a.rdelta : nullptr;
+  L.after_independent = parallel_terms;
+  if (!parallel_terms) {
+    e = launch_tc_states(L, s);
+    if (e != cudaSuccess) return e;
+  }
   {
     DqMaps dm;
     dm.q = tm_q; dm.k = tm_k; dm.v = tm_v; dm.gs = tm_gs; dm.gr = tm_gr; dm.st = tm_st; dm.dq = tm_dq;
     const int n_items = n_qt * (int)nq;
+    t.n_bh = (int)nq;
+    t.counter = a.work_counter + 1;
+    t.wait_before = chain_beside ? 1 : 0;
     KernelTimer kt("tc_bwd_dq", s);
-    tc_bwd_dq_kernel<<<n_items < n_sm ? n_items : n_sm, DQ_THREADS, DQ_SMEM, s>>>(dm, t, n_items, n_qt);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n_items < n_sm ? n_items : n_sm));
+    cfg.blockDim = dim3(DQ_THREADS);
+    cfg.dynamicSmemBytes = DQ_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = chain_beside ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, tc_bwd_dq_kernel, dm, t, n_items, n_qt);
+    if (e != cudaSuccess) return e;
+  }
+  if (parallel_terms) {
+    e = launch_tc_states(L, s);
+    if (e != cudaSuccess) return e;
   }
   KvMaps km;
   km.k = tm_k; km.v = tm_v; km.rs = tm_rs; km.dk = tm_dk; km.dv = tm_dv;
@@ -1304,6 +1420,9 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     return cudaErrorInvalidValue;
   {
     const int n_items = n_qt * (int)nkv;
+    t.n_bh = (int)nkv;
+    t.counter = a.work_counter + 2;
+    t.wait_before = 0;
     KernelTimer kt("tc_bwd_dkv", s);
     tc_bwd_dkv_kernel<<<n_items < n_sm ? n_items : n_sm, KV_THREADS, KV_SMEM, s>>>(km, t, n_items);
   }

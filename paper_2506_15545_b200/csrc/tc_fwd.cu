@@ -63,6 +63,8 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.phi = a.phi;
     L.status = a.status; L.name = "tc_state_fwd";
     L.ready = progress ? a.state_ready : nullptr;
+    L.delta = nullptr;
+    L.after_independent = false;
     cudaError_t e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;
     chained = true;

@@ -50,6 +50,10 @@ struct StateArgs {
   int phi;          // rattn_feature_map
   int* status;
   int* ready;       // optional [n_kv]: number of leading output matrices stored so far (forward chain)
+  float* delta;     // optional: the CTA forms the term of one step alone and leaves it here in fp32, matrix
+                    // (kv * n_split + step), its float4 columns outermost ([32][128 rows][4])
+  int n_split;      // steps that the grid is split into (delta)
+  int wait_before;  // 1: the kernel ahead may still be running; not to end before it
 };
 
 struct StBars {
@@ -63,7 +67,7 @@ __device__ __forceinline__ bool stored_step(const StateArgs& a, int s) {
   return o >= 0 && (o % a.store_every) == a.store_phase;
 }
 __device__ __forceinline__ bool flushed_step(const StateArgs& a, int s, int n_steps) {
-  return stored_step(a, s) || (a.final_out != nullptr && s == n_steps - 1);
+  return a.delta != nullptr || stored_step(a, s) || (a.final_out != nullptr && s == n_steps - 1);
 }
 
 __global__ void __launch_bounds__(ST_THREADS, 1)
@@ -72,7 +76,8 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   extern __shared__ __align__(1024) unsigned char smem[];
   StBars* bars = reinterpret_cast<StBars*>(smem + ST_OFF_BAR);
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int kv = blockIdx.x;
+  const int kv = a.delta ? blockIdx.x / a.n_split : blockIdx.x;
+  const int first = a.delta ? a.first + a.dir * (int)(blockIdx.x - kv * a.n_split) : a.first;
   // the kernel that follows may start its own prologue (and whatever does not read the states)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((smem_u32(smem) & 1023u) != 0) {
@@ -105,8 +110,8 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   const uint32_t tmem = bars->tmem_base;
   // this head's chain: the caller's step count, or -- variable-length batches -- what the entry's own
   // length asks for; with the hand-off the tokens from len - w on are still inside the window
-  int n_steps = a.n_steps, row_limit = INT_MAX;
-  {
+  int n_steps = a.delta ? 1 : a.n_steps, row_limit = INT_MAX;
+  if (!a.delta) {
     const int len = a.seq_lens ? min(a.T, a.seq_lens[kv / a.kv_per_batch]) : a.T;
     if (a.seq_lens) {
       const int nd = max(0, (len + TILE - 1) / TILE - 1 - a.w / TILE);
@@ -126,7 +131,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       if (!ok) break;
       unsigned char* xh = smem + st * ST_STAGE + (tid & 1) * HALF_BYTES;
       const int row = tid >> 1;
-      const int token = (a.first + a.dir * (it / a.group)) * TILE + row;
+      const int token = (first + a.dir * (it / a.group)) * TILE + row;
       // every lane maps its row (the softmax map exchanges partial results between the two lanes
       // of a row with full-warp shuffles, so no lane may skip it); rows past the limit are then cleared
       feature_map_pair_any(xh, xh, row, a.phi);
@@ -162,7 +167,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       const int s = it / a.group, hh = it - s * a.group;
       if (use >= 1) ok = mbar_wait_warp(&bars->free_[st], (use - 1) & 1, &bars->abort);
       if (!ok) break;
-      const int row = (a.first + a.dir * s) * TILE, z = kv * a.group + hh;
+      const int row = (first + a.dir * s) * TILE, z = kv * a.group + hh;
       unsigned char* dst = smem + st * ST_STAGE;
       mbar_arrive_expect_tx(&bars->full[st], ST_STAGE);
       load_tile(dst, &tm_x, &bars->full[st], row, z);
@@ -258,6 +263,15 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       tmem_wait_ld();
       tc_fence_before();
       mbar_arrive(&bars->acc_free);                            // the next step may accumulate
+      if (a.delta) {                                           // rows are neighbours in memory: whole 512-byte runs per store
+        float4* dst = reinterpret_cast<float4*>(a.delta) + (size_t)blockIdx.x * 4096 + r;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            dst[(8 * c + e) * 128] = make_float4(x[c][4 * e], x[c][4 * e + 1], x[c][4 * e + 2], x[c][4 * e + 3]);
+        continue;
+      }
       if (stored_step(a, s)) store_row(x, a.out_first + a.dir * s);
       if (a.final_out != nullptr && s == n_steps - 1) write_final(x);
     }
@@ -267,11 +281,37 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     }
   }
   if (!ok && a.status) atomicExch(a.status, 1);
+  if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   if (warp == 8) {
     tc_fence_after();
     tmem_dealloc(tmem, 128);
+  }
+}
+
+// Running sums of the terms left by the kernel above: state(s) = sum of the terms 0 .. s, as bf16, row-major.  A pure
+// stream (64 KB in and 32 KB out per matrix): a thread owns one float4 of the matrix and walks the steps with four loads
+// in flight.  A warp covers 8 rows x 4 float4 columns, so that it reads 128-byte runs of the column-major terms and
+// writes whole 32-byte sectors of the row-major states.
+__global__ void __launch_bounds__(256) tc_state_sum_kernel(const float4* __restrict__ delta, uint2* __restrict__ out,
+                                                           int n_split, int n_chunks, int out_first, int dir) {
+  const int kv = blockIdx.x >> 4, part = blockIdx.x & 15;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = 32 * (part & 3) + 8 * (warp & 3) + (lane & 7), c4 = 8 * (part >> 2) + 4 * (warp >> 2) + (lane >> 3);
+  const float4* src = delta + (size_t)kv * n_split * 4096 + c4 * 128 + row;
+  uint2* dst = out + ((size_t)kv * n_chunks + out_first) * 4096 + row * 32 + c4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < n_split; s0 += 4) {
+    float4 d[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = s0 + k < n_split ? __ldcg(src + (size_t)(s0 + k) * 4096) : acc;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (s0 + k >= n_split) break;
+      acc.x += d[k].x; acc.y += d[k].y; acc.z += d[k].z; acc.w += d[k].w;
+      dst[(ptrdiff_t)dir * (s0 + k) * 4096] = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+    }
   }
 }
 
@@ -300,13 +340,33 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   a.seq_lens = L.seq_lens; a.kv_per_batch = L.kv_per_batch > 0 ? L.kv_per_batch : 1;
   a.phi = L.phi;
   a.ready = (L.dir > 0 && L.group == 1) ? L.ready : nullptr;
+  a.delta = L.delta;
+  a.n_split = L.delta ? L.n_steps : 1;
+  a.wait_before = L.after_independent ? 1 : 0;
   cudaError_t e = allow_smem<tc_state_scan_kernel>(ST_SMEM);
   if (e != cudaSuccess) return e;
   {
     KernelTimer kt(L.name, s);
-    tc_state_scan_kernel<<<L.n_kv, ST_THREADS, ST_SMEM, s>>>(tm_x, tm_y, tm_out, a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(L.n_kv * a.n_split));
+    cfg.blockDim = dim3(ST_THREADS);
+    cfg.dynamicSmemBytes = ST_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = L.after_independent ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, tc_state_scan_kernel, tm_x, tm_y, tm_out, a);
+    if (e != cudaSuccess) return e;
   }
   count_launches(1);
+  if (L.delta) {
+    KernelTimer kt("tc_state_sum", s);
+    tc_state_sum_kernel<<<L.n_kv * 16, 256, 0, s>>>(reinterpret_cast<const float4*>(L.delta), reinterpret_cast<uint2*>(L.out),
+                                                    L.n_steps, L.n_chunks, L.out_first, L.dir);
+    count_launches(1);
+  }
   return cudaGetLastError();
 }
 
