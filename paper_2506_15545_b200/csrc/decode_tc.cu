@@ -3,14 +3,22 @@
 //
 // The step reads the K ring, the V ring and the fp32 state of a K/V head once and writes the
 // state back (Section 2.1: a cache of at most w+1 tokens; Eq. 4: the state), so it is bound by
-// HBM traffic.  One CTA per (batch entry, K/V head), two CTAs per SM.  Everything it will read
-// is requested up front as 16 KB pieces (64 ring slots, or 32 state rows) that pass through a
-// ring of stages (as many as let two CTAs share an SM, five at w = 512 with four heads), so the memory system always has the next pieces in flight, whatever the
-// warps are doing.  The two ring products are small matrix products with the group's query heads
-// as rows (q K^T, then P V), issued as warp-level mma on the pieces in shared memory (the K and V
-// pieces arrive 128-byte swizzled, so the fragment loads are conflict-free); with at most 8 rows
-// they are far too small for tcgen05's 64-row minimum.  The attention weights enter P V as a
-// bf16 pair (value + remainder), which keeps 16 bits of them.  The state is read out and updated
+// HBM traffic, or, for few sequences, by the latency of one CTA's share of it.  A (batch entry, K/V head) is therefore
+// shared by a cluster of 1, 2, 4 or 8 CTAs: each takes a run of ring pieces and of state rows, forms the partial
+// softmax sums and read-outs of them, and the cluster combines these through distributed shared memory.  Everything a
+// CTA will read is requested up front as 16 KB pieces (64 ring slots, or up to 32 state rows) that pass through a
+// ring of stages (as many as let two CTAs share an SM), refilled by whichever warp reads a stage last, so the memory
+// system always has the next pieces in flight, whatever the warps are doing.
+//
+// The ring is one pass over K and V pieces together: four warps take the even pieces and four the odd ones, 16 slots
+// each, with an online softmax of their own (maximum, sum and output per warp), so no barrier falls between the first
+// K piece and the last V piece; the warps' outputs meet once at the end.  The two groups of warps have half of the
+// stages each, and nothing of the other's passes through them: a stage's barrier tells only whether the last or the
+// last but one of its uses has landed, so everyone who waits on it must have waited for all uses before.  Both products are warp-level mma with the
+// group's query heads as rows (q K^T, then P V; the pieces arrive 128-byte swizzled, so the fragment loads are
+// conflict-free): with at most 8 rows they are far too small for tcgen05's 64-row minimum.  The weights stay in
+// registers, where the fragment of q K^T is the fragment P V wants; they enter as a bf16 pair, the leading part in rows
+// 0-7 and the remainder in rows 8-15, so one product keeps 16 bits of them.  The state is read out and updated
 // in fp32 on the CUDA cores.
 #include "rattn_internal.h"
 #include "tc_common.cuh"
@@ -35,7 +43,7 @@ struct DecodeTcArgs {
   __nv_bfloat16* k_ring; __nv_bfloat16* v_ring; float* state; __nv_bfloat16* out;
   const float* gamma_swa; const float* gamma_rla;
   const int* pos_dev;
-  int B, H_q, H_kv, w, pos, group, phi, stages;
+  int B, H_q, H_kv, w, pos, group, phi, stages, cluster;
   float scale, eps;
 };
 
@@ -78,6 +86,9 @@ __device__ __forceinline__ void warp_feature_map(float* dst, const float* src, i
   for (int i = 0; i < 4; ++i) dst[lane + 32 * i] = x[i];
 }
 
+__device__ __forceinline__ void ldmatrix_x2(uint32_t addr, uint32_t (&r)[2]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+}
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
@@ -102,36 +113,53 @@ __device__ __forceinline__ uint32_t keep_valid(uint32_t pair, int s, int live) {
 
 // Shared-memory plan (bytes, after the 1024-byte aligned stages).
 struct Plan {
-  int stages, q_b, zero, p_hi, p_lo, logit, q_f, fq, vec, o_swa, o_rla, stat, red, bars, total;
+  int stages, q_b, zero, q_f, fq, vec, o_warp, o_swa, o_rla, w_stat, stat, bars, total;
 };
-__host__ __device__ inline Plan plan_with(int g, int w, int stages) {
+__host__ __device__ inline Plan plan_with(int g, int stages) {
   Plan p;
   p.stages = stages;
   int off = stages * DT_PIECE;
   auto take = [&](int bytes) { const int at = off; off += (bytes + 15) & ~15; return at; };
   p.q_b = take(8 * QB_STRIDE * 2);         // bf16 [8][136]: the group's queries, rows >= g zero
-  p.zero = take(16);                       // what the fragment rows 8..15 point at
-  p.p_hi = take(g * (w + 8) * 2);          // bf16 [g][w + 8]: attention weights, leading part
-  p.p_lo = take(g * (w + 8) * 2);          //                  remainder
-  p.logit = take(g * (w + 4) * 4);         // fp32 [g][w + 4]: scaled logits, then un-normalised weights
   p.q_f = take(g * D * 4);                 // fp32 raw q
   p.fq = take(g * D * 4);                  // phi(q)
   p.vec = take(5 * D * 4);                 // k_new, v_new, k_old, v_old, phi(k_old)
+  p.o_warp = take(DT_WARPS * g * D * 4);   // per warp: un-normalised output over its slots
   p.o_swa = take(g * D * 4);
-  p.o_rla = take(g * D * 4);
-  p.stat = take(4 * 8 * 4);                // per head: 1 / sum, weight of the incoming token, incoming logit
-  p.red = take(2 * DT_WARPS * 8 * 4);       // per warp and head: maximum, then sum, of its share of the logits
-  p.bars = take(8 * DT_MAX_STAGES + 16);
+  p.o_rla = take(2 * g * D * 4);           // per group of warps
+  p.w_stat = take(2 * DT_WARPS * 8 * 4);   // per warp and head: maximum, sum
+  p.stat = take(3 * 8 * 4);                // per head: this CTA's maximum and sum, logit of the incoming token
+  p.bars = take(8 * DT_MAX_STAGES + 4 * DT_MAX_STAGES + 4 * DT_MAX_STAGES + 16);
   p.total = off + 1024;                    // room to align the stages
   return p;
 }
-// As many stages as let two CTAs share an SM (each may use (227 KB - 2 KB) / 2), at least three.
-__host__ __device__ inline Plan plan(int g, int w, int forced = 0) {
-  if (forced >= 3 && forced <= DT_MAX_STAGES && plan_with(g, w, forced).total <= 227 * 1024) return plan_with(g, w, forced);
-  int stages = 6;
-  while (stages > 3 && plan_with(g, w, stages).total > (227 * 1024 - 2048) / 2) --stages;
-  return plan_with(g, w, stages);
+// As many stages (an even number) as let two CTAs share an SM (each may use (227 KB - 2 KB) / 2), at least four.
+__host__ __device__ inline Plan plan(int g, int forced = 0) {
+  forced &= ~1;
+  if (forced >= 4 && forced <= DT_MAX_STAGES && plan_with(g, forced).total <= 227 * 1024) return plan_with(g, forced);
+  return plan_with(g, plan_with(g, 6).total <= (227 * 1024 - 2048) / 2 ? 6 : 4);
 }
+
+// ---- cluster: barrier halves, and a read from another CTA's shared memory
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+// pieces of the ring that one CTA of a cluster of cs takes, of np
+__host__ __device__ inline int pieces_per_rank(int np, int cs) { return (np + cs - 1) / cs; }
 
 template <int G>
 __global__ void __launch_bounds__(DT_THREADS, 2)
@@ -139,12 +167,10 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int g = a.group, w = a.w;
-  const Plan P = plan(g, w, a.stages);
-  const int NS = P.stages;
+  const int CS = a.cluster, rank = CS > 1 ? (int)(blockIdx.x % CS) : 0;
+  const Plan P = plan(g, a.stages);
+  const int NS = P.stages, NG = NS / 2;                         // stages in all, and of each group of warps
   __nv_bfloat16* q_b = reinterpret_cast<__nv_bfloat16*>(sm + P.q_b);
-  __nv_bfloat16* p_hi = reinterpret_cast<__nv_bfloat16*>(sm + P.p_hi);
-  __nv_bfloat16* p_lo = reinterpret_cast<__nv_bfloat16*>(sm + P.p_lo);
-  float* logit = reinterpret_cast<float*>(sm + P.logit);
   float* q_f = reinterpret_cast<float*>(sm + P.q_f);
   float* fq_s = reinterpret_cast<float*>(sm + P.fq);
   float* k_new = reinterpret_cast<float*>(sm + P.vec);
@@ -154,23 +180,43 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   float* fk_old = v_old + D;
   float* o_swa = reinterpret_cast<float*>(sm + P.o_swa);
   float* o_rla = reinterpret_cast<float*>(sm + P.o_rla);
-  float* inv_sum = reinterpret_cast<float*>(sm + P.stat);      // [8]
-  float* p_new = inv_sum + 8;                                  // [8] un-normalised weight of the incoming token
-  float* l_new = p_new + 8;                                    // [8] its scaled logit
-  float* w_max = reinterpret_cast<float*>(sm + P.red);         // [8 warps][8 heads]
+  float* o_warp = reinterpret_cast<float*>(sm + P.o_warp);     // [8 warps][g][128]
+  float* st_max = reinterpret_cast<float*>(sm + P.stat);       // [8] maximum over this CTA's logits
+  float* st_sum = st_max + 8;                                  // [8] sum of its weights
+  float* l_new = st_sum + 8;                                   // [8] scaled logit of the incoming token
+  float* w_max = reinterpret_cast<float*>(sm + P.w_stat);      // [8 warps][8 heads]
   float* w_sum = w_max + DT_WARPS * 8;
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + P.bars);
-  volatile int* abort = reinterpret_cast<volatile int*>(full + DT_MAX_STAGES);
-  const int LS = w + 4, PS = w + 8;
+  int* readers = reinterpret_cast<int*>(full + DT_MAX_STAGES); // per stage: warps that have read its piece
+  int* issued = readers + DT_MAX_STAGES;                       // per stage: pieces requested so far
+  volatile int* abort = issued + DT_MAX_STAGES;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int z = blockIdx.x, b = z / a.H_kv, hk = z % a.H_kv;
+  const int z = blockIdx.x / CS, b = z / a.H_kv, hk = z % a.H_kv;
+  // The next kernel on the stream may be set up; what this one reads may still be on its way from the one before.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid == 0) {
+    prefetch_tensormap(&maps.k);
+    prefetch_tensormap(&maps.v);
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&full[i], 1);
+      readers[i] = issued[i] = 0;
+    }
+    *abort = 0;
+    fence_mbar_init();
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int pos = a.pos_dev ? a.pos_dev[b] : a.pos;
   const bool evict = pos - w >= 0;
   const int slot = pos % w;
   const int n_valid = pos < w ? pos : w;
-  const int np = (n_valid + 63) >> 6;                          // K (and V) pieces that hold valid slots
-  const int n_pieces = 2 * np + 4;
+  const int np_all = (n_valid + 63) >> 6;                      // K (and V) pieces that hold valid slots
+  const int ppr = pieces_per_rank(np_all, CS), piece0 = min(rank * ppr, np_all);
+  const int np = min(ppr, np_all - piece0);                    // ... this CTA's
+  const int live_all = max(0, min(n_valid - 64 * piece0, 64 * np));   // its slots that hold a token
+  const int st_rows = D / CS, st_piece = st_rows < 64 ? st_rows / 2 : 32, row0 = rank * st_rows;   // its state rows
+  // this group's pieces: K and V of the ring pieces grp, grp + 2, ..., then the state pieces grp, grp + 2, ...
+  const int grp = warp >> 2, n_kv = 2 * ((np - grp + 1) >> 1), n_pieces = n_kv + (st_rows / st_piece) / 2;
 
   const __nv_bfloat16* qg = a.q + ((size_t)b * a.H_q + (size_t)hk * g) * D;
   const __nv_bfloat16* kg = a.k + (size_t)z * D;
@@ -183,10 +229,6 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   // The step's small operands are requested before any bulk traffic: behind 20 MB of ring pieces
   // they would wait microseconds.  They go to registers here and to shared memory once the pieces
   // have been asked for.
-  if (tid == 0) {
-    prefetch_tensormap(&maps.k);
-    prefetch_tensormap(&maps.v);
-  }
   uint4 q_reg = make_uint4(0u, 0u, 0u, 0u);                      // thread (row, 16-byte chunk) of the group's queries
   if (tid < g * 16) q_reg = reinterpret_cast<const uint4*>(qg)[tid];
   __nv_bfloat16 kn = __float2bfloat16_rn(0.f), vn = kn, ko = kn, vo_ = kn;
@@ -198,29 +240,40 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
       vo_ = vr[(size_t)slot * D + tid];
     }
   }
-  if (tid == 0) {
-    for (int i = 0; i < NS; ++i) mbar_init(&full[i], 1);
-    *abort = 0;
-    fence_mbar_init();
-  }
   __syncthreads();
 
-  // piece p of the step's stream into stage p % NS (warp 0, all lanes)
+  // piece p of the group's stream into its stage p % NG (one whole warp)
+  auto stage_of = [&](int p) { return grp * NG + p % NG; };
   auto issue = [&](int p) {
-    unsigned char* dst = sm + (p % NS) * DT_PIECE;
-    uint64_t* bar = &full[p % NS];
-    mbar_arrive_expect_tx(bar, DT_PIECE);
-    if (p < 2 * np) {
-      const CUtensorMap* m = p < np ? &maps.k : &maps.v;
-      const int row = (p < np ? p : p - np) * 64;
+    const int st = stage_of(p);
+    unsigned char* dst = sm + st * DT_PIECE;
+    uint64_t* bar = &full[st];
+    if (lane == 0) ++issued[st];
+    if (p < n_kv) {
+      const CUtensorMap* m = (p & 1) ? &maps.v : &maps.k;
+      const int row = (piece0 + grp + 2 * (p >> 1)) * 64;
+      mbar_arrive_expect_tx(bar, DT_PIECE);
       tma_load_3d(dst, m, bar, 0, row, z);
       tma_load_3d(dst + DT_PIECE / 2, m, bar, 64, row, z);
     } else {
-      bulk_load_1d(dst, S + (size_t)(p - 2 * np) * 32 * D, DT_PIECE, bar);
+      const uint32_t bytes = (uint32_t)st_piece * D * 4;
+      mbar_arrive_expect_tx(bar, bytes);
+      bulk_load_1d(dst, S + (size_t)(row0 + (grp + 2 * (p - n_kv)) * st_piece) * D, bytes, bar);
     }
   };
-  if (warp == 0)
-    for (int p = 0; p < NS && p < n_pieces; ++p) issue(p);
+  auto wait_piece = [&](int p) { return mbar_wait_warp(&full[stage_of(p)], (uint32_t)(p / NG) & 1u, abort); };
+  // this warp has read piece p; the last of the group's four to do so requests the piece that takes its stage
+  auto release = [&](int p) {
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) {
+      last = atomicAdd(&readers[stage_of(p)], 1) == 3;
+      if (last) readers[stage_of(p)] = 0;
+    }
+    if (__shfl_sync(0xffffffffu, last, 0) && p + NG < n_pieces) issue(p + NG);
+  };
+  if ((warp & 3) == 0)
+    for (int p = 0; p < NG && p < n_pieces; ++p) issue(p);
 
   // queries: bf16 rows for the fragments (rows beyond the group zero), fp32 for phi and the new logit
   if (tid < 128) {
@@ -236,29 +289,20 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
       }
     }
   }
-  if (tid < 4) reinterpret_cast<uint32_t*>(sm + P.zero)[tid] = 0u;
   if (tid < D) {
     k_new[tid] = __bfloat162float(kn);
     v_new[tid] = __bfloat162float(vn);
     k_old[tid] = __bfloat162float(ko);
     v_old[tid] = __bfloat162float(vo_);
   }
-  // weights of slots that hold no token yet
-  for (int r = 0; r < g; ++r)
-    for (int c = n_valid + tid; c < PS; c += DT_THREADS) p_hi[r * PS + c] = p_lo[r * PS + c] = __float2bfloat16_rn(0.f);
   __syncthreads();
+  if (CS > 1) cluster_arrive();                                  // the evicted slot has been read (every CTA needs it)
 
-  // query fragments: rows 0..7 from q_b, rows 8..15 are zero
-  const uint32_t zero_addr = smem_u32(sm + P.zero);
-  uint32_t qa[8][4];
-  {
-    const bool upper = (lane >> 3) & 1;
+  // query fragments: rows 0..7 from q_b (rows 8..15 of the 16-row product are zero)
+  uint32_t qa[8][2];
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const uint32_t addr = upper ? zero_addr : smem_u32(q_b + (lane & 7) * QB_STRIDE + (kk * 2 + (lane >> 4)) * 8);
-      ldmatrix_x4(addr, qa[kk]);
-    }
-  }
+  for (int kk = 0; kk < 8; ++kk)
+    ldmatrix_x2(smem_u32(q_b + (lane & 7) * QB_STRIDE + (kk * 2 + ((lane >> 3) & 1)) * 8), qa[kk]);
 
   // phi(q), phi(k_old) and the incoming token's logit (Section 2.1), while the first pieces are on their way
   for (int r = warp; r <= g; r += DT_WARPS) {
@@ -275,132 +319,129 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
     }
   }
 
-  int pc = 0;                                                    // pieces consumed so far
+  // ---- one pass over the ring: this warp's pieces, 16 slots of each -----------------------------------
   bool ok = true;
-  // ---- q K^T over the ring: piece = 64 slots, warp = 8 of them --------------------------------
-  float my_max = -INFINITY;                                      // over this thread's logits (head lane / 4)
-  for (int j = 0; j < np && ok; ++j, ++pc) {
-    const bool got = mbar_wait_warp(&full[pc % NS], (uint32_t)(pc / NS) & 1u, abort);
-    if (got) {
-      const uint32_t base = smem_u32(sm + (pc % NS) * DT_PIECE);
-      const int row = 8 * warp + (lane & 7);
-      float c[4] = {0.f, 0.f, 0.f, 0.f}, c2[4] = {0.f, 0.f, 0.f, 0.f};
+  float m_run = -INFINITY, l_run = 0.f;                          // head lane / 4: maximum (quad-wide), sum (this thread's columns)
+  float o[16][4];                                                // feature tile, fragment: rows 0-7 leading parts, 8-15 remainders
 #pragma unroll
-      for (int kk0 = 0; kk0 < 8; kk0 += 2) {
-        const int chunk = (kk0 + (lane >> 4)) * 2 + ((lane >> 3) & 1);
+  for (int i = 0; i < 64; ++i) o[i >> 2][i & 3] = 0.f;
+  const int slot0 = 16 * (warp & 3);                             // of the piece's 64
+  for (int pk = 0; pk < n_kv; pk += 2) {
+    const int pv = pk + 1, j = grp + pk;                         // ring piece j of this CTA's
+    ok = wait_piece(pk);
+    if (!ok) break;
+    float c[2][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i >> 2][i & 3] = 0.f;
+    {
+      const uint32_t base = smem_u32(sm + stage_of(pk) * DT_PIECE);
+      const int row = slot0 + (lane & 7) + ((lane >> 4) << 3);   // slots 0-7, 8-15 for the two column tiles
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        const int chunk = kk * 2 + ((lane >> 3) & 1);
         uint32_t kb[4];
         ldmatrix_x4(base + (chunk >> 3) * (DT_PIECE / 2) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4), kb);
-        mma_16816(c, qa[kk0], kb[0], kb[1]);
-        mma_16816(c2, qa[kk0 + 1], kb[2], kb[3]);
-      }
-      const int hh = lane >> 2, s = j * 64 + 8 * warp + 2 * (lane & 3);
-      if (hh < g) {
-        const float l0 = (c[0] + c2[0]) * a.scale, l1 = (c[1] + c2[1]) * a.scale;
-        logit[hh * LS + s] = l0;
-        logit[hh * LS + s + 1] = l1;
-        if (s < n_valid) my_max = fmaxf(my_max, l0);             // a slot without a token may hold anything
-        if (s + 1 < n_valid) my_max = fmaxf(my_max, l1);
+        const uint32_t qf[4] = {qa[kk][0], 0u, qa[kk][1], 0u};
+        mma_16816(c[0], qf, kb[0], kb[1]);
+        mma_16816(c[1], qf, kb[2], kb[3]);
       }
     }
-    ok = __syncthreads_and(got) != 0;
-    if (ok && warp == 0 && pc + NS < n_pieces) issue(pc + NS);
-  }
-  my_max = fmaxf(my_max, __shfl_xor_sync(0xffffffffu, my_max, 1));
-  my_max = fmaxf(my_max, __shfl_xor_sync(0xffffffffu, my_max, 2));
-  if ((lane & 3) == 0) w_max[warp * 8 + (lane >> 2)] = my_max;
-  __syncthreads();
-
-  // ---- softmax over the window: thread = slot, all heads; weights as a bf16 pair ------------------
-  {
-    float m[G], l[G];
+    release(pk);
+    const int live = live_all - 64 * j - slot0;                  // of this warp's 16 slots, those below hold a token
+    const int s0 = 2 * (lane & 3);
+    float p[4];                                                  // slots s0, s0 + 1, s0 + 8, s0 + 9
 #pragma unroll
-    for (int hh = 0; hh < G; ++hh) {
-      l[hh] = 0.f;
-      m[hh] = hh < g ? l_new[hh] : 0.f;
+    for (int i = 0; i < 4; ++i) p[i] = s0 + (i & 1) + 8 * (i >> 1) < live ? c[i >> 1][i & 1] * a.scale : -INFINITY;
+    float mx = fmaxf(fmaxf(p[0], p[1]), fmaxf(p[2], p[3]));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float m_new = fmaxf(m_run, mx), m_safe = m_new == -INFINITY ? 0.f : m_new;
+    if (__any_sync(0xffffffffu, m_new > m_run)) {
+      const float f = __expf(m_run - m_safe);
+      l_run *= f;
 #pragma unroll
-      for (int wv = 0; wv < DT_WARPS; ++wv) m[hh] = fmaxf(m[hh], w_max[wv * 8 + hh]);
+      for (int i = 0; i < 64; ++i) o[i >> 2][i & 3] *= f;
+      m_run = m_new;
     }
-    for (int s = tid; s < n_valid; s += DT_THREADS) {
+    uint32_t pa[4];
+    {
+      float lo[4];
+      uint32_t hi[2];
 #pragma unroll
-      for (int hh = 0; hh < G; ++hh) {
-        if (hh < g) {
-          const float e = __expf(logit[hh * LS + s] - m[hh]);
-          l[hh] += e;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(e);
-          p_hi[hh * PS + s] = hi;
-          p_lo[hh * PS + s] = __float2bfloat16_rn(e - __bfloat162float(hi));
-        }
+      for (int i = 0; i < 4; ++i) {
+        p[i] = __expf(p[i] - m_safe);
+        l_run += p[i];
       }
+      hi[0] = pack_bf16(p[0], p[1]);
+      hi[1] = pack_bf16(p[2], p[3]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        lo[i] = p[i] - __uint_as_float((i & 1) ? hi[i >> 1] & 0xffff0000u : hi[i >> 1] << 16);
+      pa[0] = hi[0]; pa[1] = pack_bf16(lo[0], lo[1]); pa[2] = hi[1]; pa[3] = pack_bf16(lo[2], lo[3]);
     }
+    ok = wait_piece(pv);
+    if (!ok) break;
+    if (live > 0) {
+      const uint32_t base = smem_u32(sm + stage_of(pv) * DT_PIECE);
+      const int row = slot0 + (lane & 15);
 #pragma unroll
-    for (int hh = 0; hh < G; ++hh) {
-      l[hh] = warp_sum(l[hh]);
-      if (lane == 0) w_sum[warp * 8 + hh] = l[hh];
-    }
-    __syncthreads();
-    if (tid < g) {
-      float tot = 0.f;
-#pragma unroll
-      for (int wv = 0; wv < DT_WARPS; ++wv) tot += w_sum[wv * 8 + tid];
-      float mm = l_new[tid];
-#pragma unroll
-      for (int wv = 0; wv < DT_WARPS; ++wv) mm = fmaxf(mm, w_max[wv * 8 + tid]);
-      const float en = __expf(l_new[tid] - mm);
-      p_new[tid] = en;
-      inv_sum[tid] = 1.f / (tot + en);
-    }
-    __syncthreads();
-  }
-
-  // ---- P V: piece = 64 slots of V, warp = 16 of the 128 value features.  Rows 0..7 of the weight
-  // fragment carry the leading parts, rows 8..15 the remainders: one product gives both.
-  float o[2][2][4];                                              // [slot-step parity][feature tile][fragment]
-#pragma unroll
-  for (int i = 0; i < 16; ++i) o[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
-  for (int j = 0; j < np && ok; ++j, ++pc) {
-    const bool got = mbar_wait_warp(&full[pc % NS], (uint32_t)(pc / NS) & 1u, abort);
-    if (got) {
-      unsigned char* piece = sm + (pc % NS) * DT_PIECE;
-      const uint32_t base = smem_u32(piece);
-      const bool upper = (lane >> 3) & 1;
-      const int chunk = 2 * warp + (lane >> 4);
-      const int live = n_valid - j * 64;                         // slots of this piece that hold a token
-      const __nv_bfloat16* p_part = (upper ? p_lo : p_hi) + (lane & 7) * PS + j * 64 + (lane >> 4) * 8;
-#pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        if (ks * 16 >= live) break;                              // nothing but zero weights from here on
-        const int row = ks * 16 + (lane & 7) + (upper ? 8 : 0);
-        uint32_t vb[4], pa[4];
+      for (int t = 0; t < 8; ++t) {
+        const int chunk = 2 * t + (lane >> 4);
+        uint32_t vb[4];
         ldmatrix_x4_trans(base + (chunk >> 3) * (DT_PIECE / 2) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4), vb);
-        if (live < 64) {
+        if (live < 16) {
           // a slot without a token may hold anything; its weight is zero, but 0 * NaN is not
-          const int s0 = ks * 16 + 2 * (lane & 3);
           vb[0] = keep_valid(vb[0], s0, live);
           vb[2] = keep_valid(vb[2], s0, live);
           vb[1] = keep_valid(vb[1], s0 + 8, live);
           vb[3] = keep_valid(vb[3], s0 + 8, live);
         }
-        ldmatrix_x4((lane & 7) >= g ? zero_addr : smem_u32(p_part + ks * 16), pa);
-        mma_16816(o[ks & 1][0], pa, vb[0], vb[1]);
-        mma_16816(o[ks & 1][1], pa, vb[2], vb[3]);
+        mma_16816(o[2 * t], pa, vb[0], vb[1]);
+        mma_16816(o[2 * t + 1], pa, vb[2], vb[3]);
       }
     }
-    ok = __syncthreads_and(got) != 0;
-    if (ok && warp == 0 && pc + NS < n_pieces) issue(pc + NS);
+    release(pv);
   }
-  if (ok) {
+  l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+  l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+  {
     const int hh = lane >> 2;
+    if ((lane & 3) == 0) {
+      w_max[warp * 8 + hh] = m_run;
+      w_sum[warp * 8 + hh] = l_run;
+    }
     if (hh < g) {
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int c = 16 * warp + 8 * nt + 2 * (lane & 3);
-        const float x0 = o[0][nt][0] + o[0][nt][2] + o[1][nt][0] + o[1][nt][2];
-        const float x1 = o[0][nt][1] + o[0][nt][3] + o[1][nt][1] + o[1][nt][3];
-        o_swa[hh * D + c] = (x0 + p_new[hh] * v_new[c]) * inv_sum[hh];
-        o_swa[hh * D + c + 1] = (x1 + p_new[hh] * v_new[c + 1]) * inv_sum[hh];
-      }
+      for (int t = 0; t < 16; ++t)
+        *reinterpret_cast<float2*>(o_warp + (warp * g + hh) * D + 8 * t + 2 * (lane & 3)) =
+            make_float2(o[t][0] + o[t][2], o[t][1] + o[t][3]);
     }
-    // the incoming token takes the evicted token's slot: every piece of the ring has been consumed
+  }
+  ok = __syncthreads_and(ok) != 0;
+  // the warps' shares meet; the incoming token is rank 0's
+  for (int i = tid; i < g * D; i += DT_THREADS) {
+    const int hh = i >> 7, c = i & (D - 1);
+    float m = rank == 0 ? l_new[hh] : -INFINITY;
+#pragma unroll
+    for (int wv = 0; wv < DT_WARPS; ++wv) m = fmaxf(m, w_max[wv * 8 + hh]);
+    const float ms = m == -INFINITY ? 0.f : m, en = rank == 0 ? __expf(l_new[hh] - ms) : 0.f;
+    float x = en * v_new[c], l = en;
+#pragma unroll
+    for (int wv = 0; wv < DT_WARPS; ++wv) {
+      const float f = __expf(w_max[wv * 8 + hh] - ms);           // 0 for a warp without a valid slot
+      x += f * o_warp[(wv * g + hh) * D + c];
+      l += f * w_sum[wv * 8 + hh];
+    }
+    o_swa[i] = x;
+    if (c == 0) {
+      st_max[hh] = m;
+      st_sum[hh] = l;
+    }
+  }
+  if (CS > 1) cluster_wait();
+  // the incoming token takes the evicted token's slot: the CTA whose piece that is has consumed it (a slot
+  // beyond the valid pieces is read by nobody), and every CTA has read the evicted token
+  if (ok && rank == min((slot >> 6) / max(ppr, 1), CS - 1)) {
     if (tid < D) {
       kr[(size_t)slot * D + tid] = kn;
       vr[(size_t)slot * D + tid] = vn;
@@ -408,81 +449,127 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   }
 
   // ---- the state: read-out phi(q) S and the update S += phi(k_old)^T v_old (Eq. 4), fp32 -----------
-  // thread = one float4 column group (c4) and one of 8 row lanes (rl) that sit in the same warp
+  // thread = two float4 column groups (c4, c4 + 16) and one of 8 row lanes (rl) that sit in the same warp; a piece
+  // belongs to one group of four warps
   {
-    const int rl = (lane >> 2) & 7, c4 = (lane & 3) | (warp << 2);
-    float4 ar[G];
+    const int rl = (lane >> 2) & 7, c4 = (lane & 3) | ((warp & 3) << 2);
+    float4 ar[G][2], vo[2];
 #pragma unroll
-    for (int hh = 0; hh < G; ++hh) ar[hh] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const float4 vo = *reinterpret_cast<const float4*>(v_old + c4 * 4);
-    for (int i = 0; i < 4 && ok; ++i, ++pc) {
-      const bool got = mbar_wait_warp(&full[pc % NS], (uint32_t)(pc / NS) & 1u, abort);
-      if (got) {
-        const float* piece = reinterpret_cast<const float*>(sm + (pc % NS) * DT_PIECE);
+    for (int hh = 0; hh < G; ++hh) ar[hh][0] = ar[hh][1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const int rp = rl + 8 * m, r = 32 * i + rp;
-          float4 s4 = *reinterpret_cast<const float4*>(piece + rp * D + c4 * 4);
+    for (int u = 0; u < 2; ++u) vo[u] = *reinterpret_cast<const float4*>(v_old + (c4 + 16 * u) * 4);
+    for (int p = n_kv; p < n_pieces && ok; ++p) {
+      ok = wait_piece(p);
+      if (!ok) break;
+      const float* piece = reinterpret_cast<const float*>(sm + stage_of(p) * DT_PIECE);
+      const int r0 = row0 + (grp + 2 * (p - n_kv)) * st_piece;
 #pragma unroll
-          for (int hh = 0; hh < G; ++hh) {
-            const float f = hh < g ? fq_s[hh * D + r] : 0.f;
-            ar[hh].x += f * s4.x; ar[hh].y += f * s4.y; ar[hh].z += f * s4.z; ar[hh].w += f * s4.w;
+      for (int m = 0; m < 4; ++m) {
+        const int rp = rl + 8 * m, r = r0 + rp;
+        if (rp >= st_piece) break;
+        const float fk = fk_old[r];
+        float4 s4[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) s4[u] = *reinterpret_cast<const float4*>(piece + rp * D + (c4 + 16 * u) * 4);
+#pragma unroll
+        for (int hh = 0; hh < G; ++hh) {
+          const float f = hh < g ? fq_s[hh * D + r] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            ar[hh][u].x += f * s4[u].x; ar[hh][u].y += f * s4[u].y; ar[hh][u].z += f * s4[u].z; ar[hh][u].w += f * s4[u].w;
           }
-          if (evict) {
-            const float fk = fk_old[r];
-            s4.x += fk * vo.x; s4.y += fk * vo.y; s4.z += fk * vo.z; s4.w += fk * vo.w;
-            *reinterpret_cast<float4*>(S + (size_t)r * D + c4 * 4) = s4;
+        }
+        if (evict) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            s4[u].x += fk * vo[u].x; s4[u].y += fk * vo[u].y; s4[u].z += fk * vo[u].z; s4[u].w += fk * vo[u].w;
+            *reinterpret_cast<float4*>(S + (size_t)r * D + (c4 + 16 * u) * 4) = s4[u];
           }
         }
       }
-      ok = __syncthreads_and(got) != 0;
-      if (ok && warp == 0 && pc + NS < n_pieces) issue(pc + NS);
+      release(p);
     }
 #pragma unroll
     for (int hh = 0; hh < G; ++hh) {
 #pragma unroll
-      for (int off = 4; off < 32; off <<= 1) {
-        ar[hh].x += __shfl_xor_sync(0xffffffffu, ar[hh].x, off);
-        ar[hh].y += __shfl_xor_sync(0xffffffffu, ar[hh].y, off);
-        ar[hh].z += __shfl_xor_sync(0xffffffffu, ar[hh].z, off);
-        ar[hh].w += __shfl_xor_sync(0xffffffffu, ar[hh].w, off);
+      for (int u = 0; u < 2; ++u) {
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+          ar[hh][u].x += __shfl_xor_sync(0xffffffffu, ar[hh][u].x, off);
+          ar[hh][u].y += __shfl_xor_sync(0xffffffffu, ar[hh][u].y, off);
+          ar[hh][u].z += __shfl_xor_sync(0xffffffffu, ar[hh][u].z, off);
+          ar[hh][u].w += __shfl_xor_sync(0xffffffffu, ar[hh][u].w, off);
+        }
+        if (rl == 0 && hh < g) *reinterpret_cast<float4*>(o_rla + (grp * g + hh) * D + (c4 + 16 * u) * 4) = ar[hh][u];
       }
-      if (rl == 0 && hh < g) *reinterpret_cast<float4*>(o_rla + hh * D + c4 * 4) = ar[hh];
     }
   }
-  __syncthreads();
-
-  if (!ok) {
-    // a wait ran out: give what is still in flight a bounded time to land, report, leave the caches alone
-    if (tid == 0) {
-      for (int p = pc; p < n_pieces && p < pc + NS; ++p)
-        for (int it = 0; it < kWaitPolls && !mbar_try_wait(&full[p % NS], (uint32_t)(p / NS) & 1u); ++it) {}
-      g_decode_status = RATTN_ERR_TIMEOUT;
-    }
-    return;
+  ok = __syncthreads_and(ok) != 0;
+  if (CS > 1) {
+    cluster_arrive();                                              // partial sums of every CTA are in place
+    cluster_wait();
   }
 
-  // ---- Section 3.2: two RMS norms and the sum -----------------------------------------------------
-  if (warp < g) {
-    const int h = hk * g + warp;
-    float x[4], y[4], ss = 0.f, sr = 0.f;
+  // ---- combine, Section 3.2: two RMS norms and the sum: one warp per head, heads spread over the cluster -----
+  const int hh = CS > 1 ? rank + CS * warp : warp;
+  if (ok && hh < g) {
+    const int h = hk * g + hh, c0 = 4 * lane;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+    if (CS == 1) {
+      const float inv = 1.f / st_sum[hh];
+      const float4 p = *reinterpret_cast<const float4*>(o_swa + hh * D + c0);
+      x = make_float4(p.x * inv, p.y * inv, p.z * inv, p.w * inv);
+      const float4 ya = *reinterpret_cast<const float4*>(o_rla + hh * D + c0);
+      const float4 yb = *reinterpret_cast<const float4*>(o_rla + (g + hh) * D + c0);
+      y = make_float4(ya.x + yb.x, ya.y + yb.y, ya.z + yb.z, ya.w + yb.w);
+    } else {
+      // lane r has rank r's maximum and sum
+      float m_r = -INFINITY, l_r = 0.f;
+      if (lane < CS) {
+        m_r = ld_cluster(cluster_addr(st_max + hh, lane));
+        l_r = ld_cluster(cluster_addr(st_sum + hh, lane));
+      }
+      float4 p[8], r4[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      x[i] = o_swa[warp * D + lane + 32 * i];
-      y[i] = o_rla[warp * D + lane + 32 * i];
-      ss += x[i] * x[i];
-      sr += y[i] * y[i];
+      for (int r = 0; r < 8; ++r) {
+        if (r < CS) {
+          p[r] = ld_cluster4(cluster_addr(o_swa + hh * D + c0, r));
+          const float4 ya = ld_cluster4(cluster_addr(o_rla + hh * D + c0, r));
+          const float4 yb = ld_cluster4(cluster_addr(o_rla + (g + hh) * D + c0, r));
+          r4[r] = make_float4(ya.x + yb.x, ya.y + yb.y, ya.z + yb.z, ya.w + yb.w);
+        }
+      }
+      const float m = warp_max(m_r), f = __expf(m_r - m);          // a CTA without a valid slot: exp(-inf) = 0
+      const float inv = 1.f / warp_sum(f * l_r);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        if (r < CS) {
+          const float fr = __shfl_sync(0xffffffffu, f, r) * inv;
+          x.x += fr * p[r].x; x.y += fr * p[r].y; x.z += fr * p[r].z; x.w += fr * p[r].w;
+          y.x += r4[r].x; y.y += r4[r].y; y.z += r4[r].z; y.w += r4[r].w;
+        }
+      }
     }
-    ss = warp_sum(ss);
-    sr = warp_sum(sr);
+    const float ss = warp_sum(x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w);
+    const float sr = warp_sum(y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w);
     const float is = rsqrtf(ss / D + a.eps), ir = rsqrtf(sr / D + a.eps);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int c = lane + 32 * i;
-      const float gs = a.gamma_swa ? a.gamma_swa[(size_t)h * D + c] : 1.f;
-      const float gr = a.gamma_rla ? a.gamma_rla[(size_t)h * D + c] : 1.f;
-      og[(size_t)warp * D + c] = __float2bfloat16_rn(gs * x[i] * is + gr * y[i] * ir);
-    }
+    const float4 one = make_float4(1.f, 1.f, 1.f, 1.f);
+    const float4 gs = a.gamma_swa ? *reinterpret_cast<const float4*>(a.gamma_swa + (size_t)h * D + c0) : one;
+    const float4 gr = a.gamma_rla ? *reinterpret_cast<const float4*>(a.gamma_rla + (size_t)h * D + c0) : one;
+    *reinterpret_cast<uint2*>(og + (size_t)hh * D + c0) =
+        make_uint2(pack_bf16(gs.x * x.x * is + gr.x * y.x * ir, gs.y * x.y * is + gr.y * y.y * ir),
+                   pack_bf16(gs.z * x.z * is + gr.z * y.z * ir, gs.w * x.w * is + gr.w * y.w * ir));
+  }
+  if (!ok && tid == 0) {
+    // a wait ran out: give what is still in flight a bounded time to land, report (the step's results are unspecified)
+    for (int i = 0; i < NS; ++i)
+      for (int it = 0; it < kWaitPolls && issued[i] > 0 && !mbar_try_wait(&full[i], (uint32_t)(issued[i] - 1) & 1u); ++it) {}
+    g_decode_status = RATTN_ERR_TIMEOUT;
+  }
+  if (CS > 1) {                                                    // nobody leaves while its sums are being read
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
   }
 }
 
@@ -490,15 +577,42 @@ template <int G>
 cudaError_t launch_g(const DecodeTcArgs& a, const DecodeTcMaps& m, int smem, cudaStream_t s) {
   cudaError_t e = allow_smem<decode_tc_kernel<G>>(smem);
   if (e != cudaSuccess) return e;
-  { KernelTimer kt("decode_step", s); decode_tc_kernel<G><<<a.B * a.H_kv, DT_THREADS, smem, s>>>(a, m); }
+  {
+    KernelTimer kt("decode_step", s);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.B * a.H_kv * a.cluster));
+    cfg.blockDim = dim3(DT_THREADS);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    // the kernel waits for its predecessor itself (griddepcontrol.wait), after its set-up
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.cluster > 1 ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, decode_tc_kernel<G>, a, m);
+    if (e != cudaSuccess) return e;
+  }
   count_launches(1);
   return cudaGetLastError();
+}
+
+// CTAs per (batch entry, K/V head): as many as still find room on the GPU at once (two per SM).  A second wave costs more
+// than the shorter shares save: at w = 512 and 64 heads clusters of 2 / 4 / 8 take 12.0 / 12.0 / 20.8 us a step, at 256
+// heads 1 / 2 / 4 take 23.6 / 35.7 / 54.6.
+int cluster_size(int n_heads, int n_sm) {
+  int cs = 1;
+  while (cs < 8 && cs * n_heads <= n_sm) cs *= 2;
+  return cs;
 }
 
 }  // namespace
 
 bool decode_tc_applies(const Args& p, int w) {
-  return p.dtype == RATTN_BF16 && p.d == 128 && w % 64 == 0 && p.group <= 8 && plan(p.group, w).total <= 227 * 1024;
+  return p.dtype == RATTN_BF16 && p.d == 128 && w % 64 == 0 && p.group <= 8;
 }
 
 cudaError_t launch_decode_tc(const Args& p, void* k_ring, void* v_ring, float* state, int pos, const int* pos_dev,
@@ -520,7 +634,11 @@ cudaError_t launch_decode_tc(const Args& p, void* k_ring, void* v_ring, float* s
       !tc::make_map(&m.v, v_ring, (uint64_t)p.w, (uint64_t)p.B * p.H_kv, 64))
     return cudaErrorInvalidValue;
   a.stages = tuning(RATTN_TUNE_DECODE_STAGES);
-  const int smem = plan(p.group, p.w, a.stages).total;
+  int n_sm = 0;
+  const cudaError_t e = sm_count(&n_sm);
+  if (e != cudaSuccess) return e;
+  a.cluster = cluster_size(p.B * p.H_kv, n_sm);
+  const int smem = plan(p.group, a.stages).total;
   if (p.group == 1) return launch_g<1>(a, m, smem, s);
   if (p.group == 2) return launch_g<2>(a, m, smem, s);
   if (p.group <= 4) return launch_g<4>(a, m, smem, s);
