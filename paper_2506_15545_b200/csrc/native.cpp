@@ -10,7 +10,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ATen.h>
-#include <ATen/core/LegacyTypeDispatch.h>
+#include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
 
 #include <cstring>
@@ -107,10 +107,12 @@ int dtype_code(const at::Tensor& t) {
   raise(PyExc_TypeError, "unsupported dtype: bfloat16 or float32 is expected");
 }
 
-at::Tensor like(const at::Tensor& t) {
-  at::AutoDispatchBelowADInplaceOrView below;
-  return at::empty_like(t);
+// An uninitialised contiguous tensor on t's device.  Straight to the CUDA factory: through the dispatcher each of a
+// step's three results cost 1.4 us.
+at::Tensor fresh(at::IntArrayRef sizes, at::ScalarType type, const at::Tensor& t) {
+  return at::Tensor(at::detail::empty_cuda(sizes, type, t.device(), c10::nullopt));
 }
+at::Tensor like(const at::Tensor& t) { return fresh(t.sizes(), t.scalar_type(), t); }
 at::Tensor or_like(at::Tensor given, const at::Tensor& t) { return given.defined() ? given : like(t); }
 
 PyObject* wrap(const at::Tensor& t) {
@@ -366,13 +368,11 @@ PyObject* qk_prologue_backward(Args a) {
   const at::Tensor dq = like(x.q), dk = x.k.defined() ? like(x.k) : at::Tensor();
   at::Tensor dqg, dkg;
   if (gain_grads) {
-    at::AutoDispatchBelowADInplaceOrView below;
-    const auto f32 = x.q.options().dtype(at::kFloat);
-    dqg = at::empty({x.q.size(3)}, f32);
-    if (x.k.defined()) dkg = at::empty({x.q.size(3)}, f32);
+    dqg = fresh({x.q.size(3)}, at::kFloat, x.q);
+    if (x.k.defined()) dkg = fresh({x.q.size(3)}, at::kFloat, x.q);
     if (!ws.defined()) {
       const size_t n = E.qk_prologue_workspace_bytes(x.p.B, x.p.H_q, x.p.H_kv, x.p.T, x.p.d);
-      ws = at::empty({(int64_t)n}, x.q.options().dtype(at::kByte));
+      ws = fresh({(int64_t)n}, at::kByte, x.q);
     }
   }
   const size_t nbytes = ws.defined() ? (size_t)ws.numel() : 0;
