@@ -127,43 +127,47 @@ __device__ __forceinline__ void flush_bf16_block(const unsigned char* stage, int
   }
 }
 
-// phi over the 128 features of one row by a pair of adjacent lanes: this lane owns the 64
-// columns of column half `half` (eight 16-byte chunks at src + row * 128 within that half's box).
-// src_half / dst_half point at the [rows x 64] box of this lane's column half.
-__device__ __forceinline__ void feature_map_pair(const unsigned char* src_half, unsigned char* dst_half, int row) {
-  float x[64];
-  float m = -INFINITY;
+// phi over the 128 features of one row by a pair of adjacent lanes: this lane (`ch` = its parity) owns the 64
+// columns of one column half (eight 16-byte chunks at src + row * 128 within that half's box).
+// src_half / dst_half point at the [rows x 64] box of this lane's column half.  The two lanes walk the chunks four
+// apart: the boxes lie a multiple of 8 KB from each other, and in the same order both lanes would meet in the same banks.
+__device__ __forceinline__ void feature_map_pair(const unsigned char* src_half, unsigned char* dst_half, int row, int ch) {
+  const int sw = (row & 7) ^ (ch << 2);
+  float x[64], m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const uint4 u = *reinterpret_cast<const uint4*>(src_half + row * 128 + ((c ^ (row & 7)) << 4));
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+    const uint4 u = *reinterpret_cast<const uint4*>(src_half + row * 128 + ((c ^ sw) << 4));
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float2 f = __bfloat1622float2(h[e]);
-      x[c * 8 + 2 * e] = f.x;
-      x[c * 8 + 2 * e + 1] = f.y;
-      m = fmaxf(m, fmaxf(f.x, f.y));
+      x[c * 8 + 2 * e] = __uint_as_float(w[e] << 16);
+      x[c * 8 + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+      m0 = fmaxf(m0, x[c * 8 + 2 * e]);
+      m1 = fmaxf(m1, x[c * 8 + 2 * e + 1]);
     }
   }
+  float m = fmaxf(m0, m1);
   m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
   const float ml = m * 1.4426950408889634f;
-  float sum = 0.f;
+  const float2 l2e = make_float2(1.4426950408889634f, 1.4426950408889634f), nml = make_float2(-ml, -ml);
+  float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < 64; ++i) {
-    x[i] = ex2(x[i] * 1.4426950408889634f - ml);
-    sum += x[i];
+  for (int i = 0; i < 64; i += 2) {
+    const float2 y = __ffma2_rn(make_float2(x[i], x[i + 1]), l2e, nml);
+    const float2 p = make_float2(ex2(y.x), ex2(y.y));
+    x[i] = p.x;
+    x[i + 1] = p.y;
+    if (i & 2) s1 = __fadd2_rn(s1, p);
+    else s0 = __fadd2_rn(s0, p);
   }
+  float sum = (s0.x + s0.y) + (s1.x + s1.y);
   sum += __shfl_xor_sync(0xffffffffu, sum, 1);
   const float inv = 1.f / sum;
 #pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    uint4 u;
-    u.x = pack_bf16(x[c * 8 + 0] * inv, x[c * 8 + 1] * inv);
-    u.y = pack_bf16(x[c * 8 + 2] * inv, x[c * 8 + 3] * inv);
-    u.z = pack_bf16(x[c * 8 + 4] * inv, x[c * 8 + 5] * inv);
-    u.w = pack_bf16(x[c * 8 + 6] * inv, x[c * 8 + 7] * inv);
-    *reinterpret_cast<uint4*>(dst_half + row * 128 + ((c ^ (row & 7)) << 4)) = u;
-  }
+  for (int c = 0; c < 8; ++c)
+    *reinterpret_cast<uint4*>(dst_half + row * 128 + ((c ^ sw) << 4)) =
+        make_uint4(pack_bf16(x[c * 8 + 0] * inv, x[c * 8 + 1] * inv), pack_bf16(x[c * 8 + 2] * inv, x[c * 8 + 3] * inv),
+                   pack_bf16(x[c * 8 + 4] * inv, x[c * 8 + 5] * inv), pack_bf16(x[c * 8 + 6] * inv, x[c * 8 + 7] * inv));
 }
 
 // The element-wise maps of the paper's ablation (Table 6) on packed bf16 pairs: ReLU; the
@@ -178,7 +182,7 @@ __device__ __forceinline__ uint4 relu_bf16x8(uint4 u) {
 // feature_map_pair for any map: softmax as above; ReLU / identity element-wise (src may differ from dst)
 __device__ __forceinline__ void feature_map_pair_any(const unsigned char* src_half, unsigned char* dst_half, int row, int phi) {
   if (phi == RATTN_PHI_SOFTMAX) {
-    feature_map_pair(src_half, dst_half, row);
+    feature_map_pair(src_half, dst_half, row, (int)(threadIdx.x & 1));
     return;
   }
   if (phi == RATTN_PHI_IDENTITY && src_half == dst_half) return;
