@@ -429,9 +429,13 @@ __global__ void __launch_bounds__(256) handoff_ring_kernel(const uint4* __restri
                                                            uint4* __restrict__ kr, uint4* __restrict__ vr, int T, int w,
                                                            int vec_shift, const int* __restrict__ len, int H_kv,
                                                            int pos_shift, int layout, float4* __restrict__ zero_state,
-                                                           int state_vecs) {
+                                                           int state_vecs, int* __restrict__ clear, int clear_ints) {
   const int bh = blockIdx.y;
   const int i = blockIdx.x * 256 + threadIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (bh == 0)
+    for (int e = i; e < clear_ints; e += gridDim.x * 256) clear[e] = 0;
   if (zero_state) {
     for (int e = i; e < state_vecs; e += gridDim.x * 256)
       zero_state[(size_t)bh * state_vecs + e] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -456,7 +460,7 @@ __global__ void __launch_bounds__(256) handoff_ring_kernel(const uint4* __restri
 }
 
 template <typename TIO, int D>
-cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too) {
+cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too, int* clear, int clear_ints) {
   const int BH = a.B * a.H_kv;
   if (a.state_out && state_too) {
     dim3 grid(D / 8, BH);
@@ -470,10 +474,21 @@ cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too) {
     constexpr int vec_shift = (D == 128 ? 4 : 3) + (sizeof(TIO) == 4 ? 1 : 0);      // 16-byte vectors per row: 1 << shift
     dim3 grid((unsigned)((((size_t)a.w << vec_shift) + 255) / 256), BH);
     KernelTimer kt("handoff_ring", s);
-    handoff_ring_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const uint4*>(a.k), reinterpret_cast<const uint4*>(a.v),
-                                             reinterpret_cast<uint4*>(a.k_ring_out), reinterpret_cast<uint4*>(a.v_ring_out),
-                                             a.Tk, a.w, vec_shift, a.seq_lens, a.H_kv, a.pos_shift, a.kv_layout,
-                                             a.zero_state ? reinterpret_cast<float4*>(a.state_out) : nullptr, D * D / 4);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];               // the kernel waits for its predecessor itself
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(
+        &cfg, handoff_ring_kernel, reinterpret_cast<const uint4*>(a.k), reinterpret_cast<const uint4*>(a.v),
+        reinterpret_cast<uint4*>(a.k_ring_out), reinterpret_cast<uint4*>(a.v_ring_out), a.Tk, a.w, vec_shift, a.seq_lens,
+        a.H_kv, a.pos_shift, a.kv_layout, a.zero_state ? reinterpret_cast<float4*>(a.state_out) : (float4*)nullptr, D * D / 4,
+        clear, clear_ints);
+    if (e != cudaSuccess) return e;
     count_launches(1);
   }
   return cudaGetLastError();
@@ -483,8 +498,10 @@ cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too) {
 __global__ void gather_history_kernel(const uint4* __restrict__ k_chunk, const uint4* __restrict__ v_chunk,
                                       const uint4* __restrict__ k_ring, const uint4* __restrict__ v_ring,
                                       uint4* __restrict__ k_ext, uint4* __restrict__ v_ext, int T, int w, int pos0,
-                                      int vec_per_row, int H_kv, int layout) {
+                                      int vec_per_row, int H_kv, int layout, int* __restrict__ clear, int clear_ints) {
   const int bh = blockIdx.y;
+  if (bh == 0)
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < clear_ints; e += gridDim.x * blockDim.x) clear[e] = 0;
   // the chunk is the caller's tensor: [B, H_kv, T, d] (layout 0) or [B, T, H_kv, d] (layout 1), in 16-byte vectors
   const size_t head0 = layout ? ((size_t)(bh / H_kv) * T * H_kv + bh % H_kv) * vec_per_row : (size_t)bh * T * vec_per_row;
   const size_t pitch = layout ? (size_t)H_kv * vec_per_row : (size_t)vec_per_row;
@@ -508,7 +525,8 @@ __global__ void gather_history_kernel(const uint4* __restrict__ k_chunk, const u
 }  // namespace
 
 cudaError_t launch_gather_history(const Args& a, const void* k_chunk, const void* v_chunk, const void* k_ring,
-                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, cudaStream_t s) {
+                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, int* clear, int clear_ints,
+                                  cudaStream_t s) {
   const int elem = a.dtype == RATTN_F32 ? 4 : 2;
   const int vec_per_row = a.d * elem / 16;
   const size_t n_ext = (size_t)(a.w + a.T) * vec_per_row;
@@ -517,7 +535,8 @@ cudaError_t launch_gather_history(const Args& a, const void* k_chunk, const void
   gather_history_kernel<<<grid, 256, 0, s>>>(
       reinterpret_cast<const uint4*>(k_chunk), reinterpret_cast<const uint4*>(v_chunk),
       reinterpret_cast<const uint4*>(k_ring), reinterpret_cast<const uint4*>(v_ring),
-      reinterpret_cast<uint4*>(k_ext), reinterpret_cast<uint4*>(v_ext), a.T, a.w, pos0, vec_per_row, a.H_kv, a.layout);
+      reinterpret_cast<uint4*>(k_ext), reinterpret_cast<uint4*>(v_ext), a.T, a.w, pos0, vec_per_row, a.H_kv, a.layout, clear,
+      clear_ints);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -537,11 +556,12 @@ cudaError_t launch_decode(const Args& p, void* k_ring, void* v_ring, float* stat
   return p.d == 64 ? launch_dec<__nv_bfloat16, 64>(a, s) : launch_dec<__nv_bfloat16, 128>(a, s);
 }
 
-cudaError_t launch_handoff(const Args& a, cudaStream_t s, bool state_too) {
+cudaError_t launch_handoff(const Args& a, cudaStream_t s, bool state_too, int* clear, int clear_ints) {
   if (a.dtype == RATTN_F32)
-    return a.d == 64 ? launch_handoff_t<float, 64>(a, s, state_too) : launch_handoff_t<float, 128>(a, s, state_too);
-  return a.d == 64 ? launch_handoff_t<__nv_bfloat16, 64>(a, s, state_too)
-                   : launch_handoff_t<__nv_bfloat16, 128>(a, s, state_too);
+    return a.d == 64 ? launch_handoff_t<float, 64>(a, s, state_too, clear, clear_ints)
+                     : launch_handoff_t<float, 128>(a, s, state_too, clear, clear_ints);
+  return a.d == 64 ? launch_handoff_t<__nv_bfloat16, 64>(a, s, state_too, clear, clear_ints)
+                   : launch_handoff_t<__nv_bfloat16, 128>(a, s, state_too, clear, clear_ints);
 }
 
 }  // namespace rattn

@@ -235,20 +235,42 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
   a.training = train;
   a.zero_state = tc && p->state_out && p->k_ring_out && !resume && !p->seq_lens && p->T <= p->w;
   cudaError_t e;
-  if (a.status) {
-    e = cudaMemsetAsync(a.status, 0, L.status_bytes, s);
-    if (e != cudaSuccess) return fail_cuda(e);
-    if (status_word) a.status = status_word;
-  }
+  // The status block (status word, work counters, progress words) has to be zero before the kernels that use it.  The
+  // first kernel of the call does that where it is one that none of them runs beside -- the gather of a resumed
+  // sequence, the ring hand-off (which then goes first: it reads the inputs only) -- and a memory set otherwise.
+  int* const block = a.status;
+  const int block_ints = (int)(L.status_bytes / sizeof(int));
+  const bool rings = want_handoff && p->k_ring_out;
+  bool cleared = block == nullptr;
+  if (block && status_word) a.status = status_word;
   if (resume) {
     char* base = reinterpret_cast<char*>(p->workspace);
     void* k_ext = base + L.k_ext;
     void* v_ext = base + L.v_ext;
-    e = launch_gather_history(a, p->k, p->v, p->k_ring_in, p->v_ring_in, k_ext, v_ext, p->pos0, s);
+    e = launch_gather_history(a, p->k, p->v, p->k_ring_in, p->v_ring_in, k_ext, v_ext, p->pos0, block, block_ints, s);
     if (e != cudaSuccess) return fail_cuda(e);
+    cleared = true;
     a.k = k_ext; a.v = v_ext;
     a.kv_layout = RATTN_LAYOUT_BHTD;                       // the gathered history + chunk is dense per head
     a.Tk = p->w + p->T; a.q_off = p->w; a.state_in = p->state_in; a.pos_shift = p->pos0 - p->w;
+  }
+  // the rings may be written over in place (a resumed sequence hands out where it came from): after the gather
+  const bool rings_first = rings && tc;
+  if (rings_first) {
+    e = launch_handoff(a, s, false, cleared ? nullptr : block, cleared ? 0 : block_ints);
+    if (e != cudaSuccess) return fail_cuda(e);
+    cleared = true;
+  }
+#ifdef RATTN_HAVE_TC
+  // a forward that is one kernel with one unit per CTA uses nothing but the status word, which it clears itself
+  if (!cleared && tc && tc_forward_clears_status(a)) {
+    if (a.status == block) a.clear_status = block;
+    cleared = true;
+  }
+#endif
+  if (!cleared) {
+    e = cudaMemsetAsync(block, 0, L.status_bytes, s);
+    if (e != cudaSuccess) return fail_cuda(e);
   }
 #ifdef RATTN_HAVE_TC
   if (tc) e = launch_tc_forward(a, s);
@@ -256,8 +278,8 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
 #endif
     e = launch_generic_forward(a, s);
   if (e != cudaSuccess) return fail_cuda(e);
-  if (want_handoff) {
-    e = launch_handoff(a, s, !tc);      // the tensor-core forward has left the state itself
+  if (want_handoff && !tc) {            // the tensor-core forward has left the state itself
+    e = launch_handoff(a, s, true);
     if (e != cudaSuccess) return fail_cuda(e);
   }
   return RATTN_OK;

@@ -86,6 +86,8 @@ struct Args {
   float* dscp;
   int n_chunks;
   int* status;                 // device status word (may be null when no workspace)
+  int* clear_status;           // the status word, where no kernel ahead of the forward's first one has cleared it
+  bool single_tiles;           // the forward's work units are single query tiles instead of pairs
   int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin);
                                // the backward's two kernels use the two words behind it
   int* state_ready;            // [B*H_kv], zero at launch: chunk states the chunk-state kernel has stored so far
@@ -119,9 +121,11 @@ bool decode_tc_applies(const Args& a, int w);
 cudaError_t launch_decode_tc(const Args& a, void* k_ring, void* v_ring, float* state, int pos, const int* pos_dev,
                              cudaStream_t s);
 int decode_tc_status(cudaStream_t s, cudaError_t* err);
-// prefill -> decode hand-off: the rings, and (state_too) the state by the portable kernel
-cudaError_t launch_handoff(const Args& a, cudaStream_t s, bool state_too);
+// prefill -> decode hand-off: the rings, and (state_too) the state by the portable kernel.  `clear` (clear_ints of them):
+// words to set to zero beside it
+cudaError_t launch_handoff(const Args& a, cudaStream_t s, bool state_too, int* clear = nullptr, int clear_ints = 0);
 cudaError_t launch_tc_forward(const Args& a, cudaStream_t s);        // chunk states, then the main kernel
+bool tc_forward_clears_status(const Args& a);   // one kernel, one unit per CTA: only Args::clear_status has to be set
 // after_states: a chunk-state kernel was launched just before on the same stream
 cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_states);
 // Running sums of phi(X_c)^T Y_c over the chunks first, first+dir, ... (n_steps of them) for every
@@ -158,7 +162,8 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s);
 cudaError_t launch_tc_backward(const Args& a, cudaStream_t s);
 // chunked prefill: k_ext/v_ext[b,hk] = the ring's tokens pos0-w .. pos0-1 in time order, then the chunk
 cudaError_t launch_gather_history(const Args& a, const void* k_chunk, const void* v_chunk, const void* k_ring,
-                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, cudaStream_t s);
+                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, int* clear, int clear_ints,
+                                  cudaStream_t s);
 
 int debug_skip_arrive();                    // always 0 outside the debug build
 int tuning(int knob);                       // current value of a rattn_knob

@@ -14,6 +14,32 @@
 
 namespace rattn {
 
+// Query tiles of a work unit.  Pairs share their K/V tiles and half of the stored states, but where they do not fill
+// the GPU a tile of its own per CTA ends sooner (1 x 16/4 heads, T = 1111: 80 pairs or 144 tiles on 148 SMs).  With
+// single tiles every tile reads a stored state, in bf16, where of a pair the second takes the chunk in between exactly.
+// The element-wise maps' signed sums feel that rounding (of the output's bound of 2e-2 the last rounding alone takes
+// 1.6e-2 above 4), so they keep pairs.
+static bool single_tiles(const Args& a) {
+  int n_sm = 0;
+  if (sm_count(&n_sm) != cudaSuccess) return false;
+  const int n_qt = (a.T + tc::TILE - 1) / tc::TILE;
+  const bool states = a.mode == RATTN_MODE_RATTN && (a.state_in || n_qt - 1 - a.w / tc::TILE > 0);
+  return (long long)((n_qt + 1) / 2) * a.B * a.H_q < n_sm && (a.phi == RATTN_PHI_SOFTMAX || !states);
+}
+// whether a chunk-state kernel runs ahead of the main kernel
+static bool has_chain(const Args& a) {
+  const int n_kt = (a.Tk + tc::TILE - 1) / tc::TILE;
+  const bool rla = a.mode == RATTN_MODE_RATTN, want_state = rla && a.state_out != nullptr;
+  const int n_delta = rla ? n_kt - 1 - a.w / tc::TILE : 0;
+  return n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
+}
+bool tc_forward_clears_status(const Args& a) {
+  int n_sm = 0;
+  if (sm_count(&n_sm) != cudaSuccess || has_chain(a)) return false;
+  const int n_qt = (a.T + tc::TILE - 1) / tc::TILE, per = single_tiles(a) ? 1 : 2;
+  return (long long)((n_qt + per - 1) / per) * a.B * a.H_q <= n_sm;
+}
+
 cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
   // key-space tiles: a resumed sequence carries its w-token history in front of the chunk
   const int n_kt = (a.Tk + tc::TILE - 1) / tc::TILE;
@@ -44,7 +70,8 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
   }
   const int n_steps = (want_state && (a.Tk > a.w || a.seq_lens)) ? n_delta + 1 : n_delta;
-  if (n_steps > 0 || (a.state_in && rla) || (a.seq_lens && want_state)) {
+  const bool single = single_tiles(a);
+  if (has_chain(a)) {
     StateLaunch L;
     L.x = a.k; L.y = a.v; L.out = a.chunk_state;
     L.x_heads = L.y_heads = a.H_kv; L.x_layout = L.y_layout = a.kv_layout;
@@ -52,7 +79,7 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.n_steps = n_steps > 0 ? n_steps : 0; L.first = 0; L.dir = +1; L.out_first = 1;
     // the main kernel reads S_[c] for c = off + 2p - wt only
     const int m = tuning(RATTN_TUNE_STATE_STRIDE);
-    const bool every = a.training || m == 1;
+    const bool every = a.training || m == 1 || single;
     L.store_every = every ? 1 : 2;
     L.store_phase = every ? 0 : ((off + wt) & 1);
     L.handoff = want_state ? 1 : 0;
@@ -70,6 +97,7 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     chained = true;
   }
   Args m = a;
+  m.single_tiles = single;
   if (!progress) m.state_ready = nullptr;            // the main kernel waits for the whole chain instead
   return launch_tc_forward_main(m, s, chained);
 }

@@ -60,8 +60,11 @@ struct FArgs {
   const float* gamma_swa;
   const float* gamma_rla;
   int* status;
+  int* clear_status;      // status word that nothing ahead of this kernel has cleared
   int* work_counter;      // next unit to hand out (device memory, zero at launch); null: static round-robin
   int T, w, H_q, group, mode, n_chunks, n_qt, n_pairs, n_units, n_bh;
+  int per_unit;           // query tiles of a unit: 2, or 1 where pairs would not fill the GPU (n_pairs then counts tiles)
+  int wait_first;         // the kernel ahead produces what this one reads: wait for it after the set-up
   int phi;                // rattn_feature_map
   int off;                // key tile of query tile 0 (a resumed sequence carries w/128 history tiles in front)
   int first_state;        // smallest chunk index whose state is stored: 1 (S_[0] = 0), or 0 with an incoming state
@@ -107,8 +110,8 @@ __device__ __forceinline__ Unit make_unit(const FArgs& a, int u) {
   un.windowed = (a.mode != RATTN_MODE_FULL_CAUSAL);
   // tile indices are key-space positions: query tile i of the call sits at key tile i + off
   const int n_qt = a.seq_lens ? (min(a.T, a.seq_lens[b]) + TILE - 1) / TILE : a.n_qt;
-  un.t[0] = (2 * p < n_qt) ? a.off + 2 * p : -1;             // a unit without tile A is empty
-  un.t[1] = (2 * p + 1 < n_qt) ? a.off + 2 * p + 1 : -1;
+  un.t[0] = (a.per_unit * p < n_qt) ? a.off + a.per_unit * p : -1;             // a unit without tile A is empty
+  un.t[1] = (a.per_unit == 2 && 2 * p + 1 < n_qt) ? a.off + 2 * p + 1 : -1;
   un.kt_hi = un.t[1] >= 0 ? un.t[1] : un.t[0];
   const int loA = un.windowed ? max(0, un.t[0] - un.wt) : 0;
   un.n = un.kt_hi - loA + 1;
@@ -836,6 +839,8 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
     prefetch_tensormap(&tm.o_swa);
     prefetch_tensormap(&tm.o_rla);
   }
+  if (a.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.clear_status && blockIdx.x == 0 && tid == 0) *a.clear_status = 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -898,7 +903,8 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   t.gamma_swa = a.gamma_swa; t.gamma_rla = a.gamma_rla; t.status = a.status;
   t.T = a.T; t.w = a.w; t.H_q = a.H_q; t.group = a.group; t.mode = a.mode; t.n_chunks = a.n_chunks;
   t.n_qt = (a.T + TILE - 1) / TILE;
-  t.n_pairs = (t.n_qt + 1) / 2;
+  t.per_unit = a.single_tiles ? 1 : 2;
+  t.n_pairs = (t.n_qt + t.per_unit - 1) / t.per_unit;
   t.n_bh = a.B * a.H_q;
   t.n_units = t.n_pairs * t.n_bh;
   t.scale_log2 = a.scale * LOG2E; t.eps = a.eps;
@@ -912,7 +918,7 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   const int order = tuning(RATTN_TUNE_UNIT_ORDER);
   const bool stateless_first = order == 1 || (order == 0 && 2 * a.B * a.H_kv <= n_sm);
   if (a.mode == RATTN_MODE_RATTN && after_states && !a.state_in && stateless_first) {
-    t.n_stateless = (a.w / TILE) / 2 + 1;
+    t.n_stateless = (a.w / TILE) / t.per_unit + 1;
     if (t.n_stateless > t.n_pairs) t.n_stateless = t.n_pairs;
   }
   t.wait_for_states = after_states ? 1 : 0;
@@ -921,7 +927,9 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   // have put the units without a state first anyway (few K/V heads, many SMs free beside the chain)
   t.ascending = (t.state_ready && t.n_stateless > 0) ? 1 : 0;
   t.debug_skip_arrive = debug_skip_arrive();
-  t.work_counter = order != 3 ? a.work_counter : nullptr;
+  t.work_counter = (order != 3 && t.n_units > n_sm) ? a.work_counter : nullptr;   // one unit per CTA needs no counter
+  t.clear_status = after_states ? nullptr : a.clear_status;
+  t.wait_first = after_states ? 0 : 1;
   e = allow_smem<tc_fwd2_kernel>(F_SMEM);
   if (e != cudaSuccess) return e;
   if (tuning(RATTN_TUNE_GRID) > 0 && tuning(RATTN_TUNE_GRID) < n_sm) n_sm = tuning(RATTN_TUNE_GRID);
@@ -930,7 +938,7 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
     KernelTimer kt("tc_fwd", s);
     // Programmatic dependent launch: when a chunk-state kernel precedes it on the stream, this
     // kernel may begin while that one is still running; its loader waits (griddepcontrol.wait)
-    // before the first state load.  Without a preceding state kernel the attribute changes nothing.
+    // before the first state load.  Behind any other kernel it waits right after its set-up.
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(F_THREADS);
@@ -938,7 +946,7 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = (after_states && tuning(RATTN_TUNE_OVERLAP)) ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = (!after_states || tuning(RATTN_TUNE_OVERLAP)) ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, tc_fwd2_kernel, tm, t);

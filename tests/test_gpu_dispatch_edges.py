@@ -1,0 +1,82 @@
+"""Kernel variants that are chosen by size, each side of every rule: clusters of 1 to 8 CTAs in the decode step, the
+per-vector and the chunked prologue, single-tile and pair units of the tensor-core forward."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rattn_oracle as O
+from paper_2506_15545_b200 import binding as R
+from paper_2506_15545_b200 import workloads as W
+from test_gpu_parity import check, np64, small
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hkv,g,w,pos", [
+    (1, 2, 4, 512, 1777),        # cluster of 8, one ring piece each
+    (2, 8, 2, 448, 200),         # 8 CTAs, seven pieces' room, four with tokens: some CTAs have no slot at all
+    (5, 8, 1, 64, 64),           # 4 CTAs on a single piece, exactly full
+    (11, 8, 3, 128, 100),        # 2 CTAs, the last piece partly filled
+    (19, 8, 8, 192, 1000),       # one CTA per head, an odd number of pieces
+    (40, 4, 2, 64, 0),           # one CTA per head, no token yet
+])
+def test_decode_clusters_against_the_portable_kernel(B, Hkv, g, w, pos):
+    gen = torch.Generator(device="cuda").manual_seed(77 + B)
+    rnd = lambda *s, dt=torch.bfloat16: torch.randn(s, generator=gen, device="cuda").to(dt)
+    q, k, v = rnd(B, Hkv * g, 128), rnd(B, Hkv, 128), rnd(B, Hkv, 128)
+    kr, vr, st = rnd(B, Hkv, w, 128), rnd(B, Hkv, w, 128), rnd(B, Hkv, 128, 128, dt=torch.float32)
+    kr[:, :, min(pos, w):] = float("nan")              # slots that hold no token yet
+    vr[:, :, min(pos, w):] = float("nan")
+    other = [t.clone() for t in (kr, vr, st)]
+    y = R.rattn_decode_step_ex(q, k, v, kr, vr, st, pos, scale=0.088)
+    z = R.rattn_decode_step_ex(q, k, v, *other, pos, scale=0.088, flags=R.FLAG_FORCE_GENERIC)
+    torch.cuda.synchronize()
+    assert R.rattn_decode_status() == 0
+    # both round y to bf16 once: one rounding step of values up to 8 in magnitude
+    assert (y.float() - z.float()).abs().max().item() <= 2.0 ** -5
+    assert (y.float() - z.float()).abs().mean().item() <= 5e-4
+    assert torch.equal(kr.nan_to_num(), other[0].nan_to_num()) and torch.equal(vr.nan_to_num(), other[1].nan_to_num())
+    # state: phi(k)^T v added in fp32 by both; phi from the fast exponential, 2^-21 relative per term of size up to 4
+    assert (st - other[2]).abs().max().item() <= 1e-5
+
+
+@pytest.mark.parametrize("layout", [R.LAYOUT_BHTD, R.LAYOUT_BTHD])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_prologue_per_vector_and_chunked_agree(layout, d, dtype):
+    """4096 head vectors take the one kernel, 4160 the other; the shared tokens must come out alike."""
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    B, Hq, Hkv, T = 1, 48, 16, 65                      # 65 tokens x 64 heads; the first 64 are 4096 vectors
+    make = lambda H: torch.randn(B, T, H, d, generator=gen, device="cuda").to(dtype)
+    q, k = make(Hq), make(Hkv)
+    gain = torch.rand(d, generator=gen, device="cuda") + 0.5
+    view = (lambda t: t) if layout == R.LAYOUT_BTHD else (lambda t: t.transpose(1, 2))
+    call = lambda n: [view(t) for t in R.rattn_qk_prologue(view(q[:, :n]).contiguous(), view(k[:, :n]).contiguous(),
+                                                            q_gain=gain, k_gain=gain, pos0=1000, layout=layout)]
+    for a, b in zip(call(65), call(64)):
+        a = a[:, :64].float()
+        # the same fp32 arithmetic with sums in another order, rounded once
+        assert (a - b.float()).abs().max().item() <= a.abs().max().item() * (2.0 ** -8 if dtype == torch.bfloat16 else 2e-6)
+    assert R.rattn_qk_prologue_status() == 0
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,T,w", [
+    (4, 18, 18, 384, 128),       # 144 pairs: single tiles, three per head
+    (10, 16, 4, 300, 128),       # 320 pairs, the second one half empty, one unit drawn after another
+    (1, 37, 37, 1000, 256),      # exactly 148 pairs: no single tiles, one pair per CTA
+    (1, 147, 49, 200, 128),      # 147 pairs: single tiles, two waves
+])
+def test_forward_single_tiles_and_pairs(B, Hq, Hkv, T, w):
+    wl = small("units", B, Hq, Hkv, T, 128, w, "bf16", 9500 + T, unit=True)
+    q, k, v = W.make_qkv(wl)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    ws = R.alloc_workspace(qd, kd, w, R.MODE_RATTN, 0)
+    ws.fill_(0xff)
+    y = R.rattn_forward_ex(qd, kd, vd, w, scale=wl.scale, workspace=ws)
+    torch.cuda.synchronize()
+    assert R.rattn_read_status(ws) == 0
+    g, heads = Hq // Hkv, sorted({0, Hq // 2, Hq - 1})
+    for h in heads:
+        ref = O.forward(np64(q[-1:, h:h + 1]), np64(k[-1:, h // g:h // g + 1]), np64(v[-1:, h // g:h // g + 1]), w, wl.scale)
+        check(y[-1:, h:h + 1], ref, "bf16", f"head {h}")
+    assert np.isfinite(np64(y)).all()
