@@ -280,8 +280,10 @@ int rattn_decode_status(void* stream);
  *                                      mode RATTN only;
  *   RATTN_FLAG_SAVE_RESIDUALS          in addition the residuals of Section 3.2's two branches
  *                                      (log-sum-exp, un-normalised o_swa and o_rla: bf16 on the
- *                                      tensor-core path, fp32 on the portable one) and the
- *                                      backward's scratch of the same shapes.
+ *                                      tensor-core path, fp32 on the portable one), the
+ *                                      backward's scratch of the same shapes and, on the portable
+ *                                      kernels in mode RATTN, fp32 chunk states of 64 tokens,
+ *                                      2 x [B,H_kv,ceil(T/64),d,d].
  * The backward needs the size of its forward (same sizes, mode, flags with
  * RATTN_FLAG_SAVE_RESIDUALS set).  A larger buffer is always accepted.
  */

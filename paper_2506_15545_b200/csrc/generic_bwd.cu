@@ -11,9 +11,13 @@
 //                        dphi_q_t += da phi(k_j); dphi_k_j += da phi(q_t); dv_j += a do_r_t
 //   feature map (Section 3.1):  dx = phi * (dphi - <dphi, phi>)
 //   GQA: dk, dv of a K/V head sum over the query heads of its group.
-// Three launches: a per-row preprocess, a dq kernel (one CTA per query tile) and a dk/dv
-// kernel (one CTA per key tile that loops over the group's heads), so no atomics are
-// needed for dq/dk/dv and the result is deterministic.
+// A per-row preprocess, a dq kernel (one CTA per query tile) and a dk/dv kernel (one CTA per
+// key tile that loops over the group's heads), so no atomics are needed for dq/dk/dv and the
+// result is deterministic.  Where the workspace has room for chunk states (generic_common.cuh) the
+// sums over whole chunks beyond the window are read from them: dphi_q += g_r S^T, dphi_k += V R^T,
+// dv += phi(k) R.
+#include <type_traits>
+
 #include "generic_common.cuh"
 
 namespace rattn {
@@ -105,6 +109,7 @@ __global__ void __launch_bounds__(NT) bwd_dq_kernel(Args a, const float* __restr
   float* del_s = lse_s + BQ;
 
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the dk/dv kernel does not read dq
   const int n_qt = (a.T + BQ - 1) / BQ;
   const int qt = n_qt - 1 - blockIdx.x;
   const int bh = blockIdx.y, b = bh / a.H_q, h = bh % a.H_q, hk = h / a.group;
@@ -138,10 +143,12 @@ __global__ void __launch_bounds__(NT) bwd_dq_kernel(Args a, const float* __restr
 
   const int q_last = min(q0 + BQ, T) - 1;
   const int n_kt = q_last / BK + 1;
+  static_assert(BK == GC, "chunks are key tiles");
+  const int whole = (rla_on && a.gstate && q0 > w) ? (q0 - w) / GC : 0;   // chunks wholly before every row's window
   for (int kt = 0; kt < n_kt; ++kt) {
     const int j0 = kt * BK;
     const bool need_swa = (j0 + BK - 1 >= q0 - w);
-    const bool need_rla = rla_on && (j0 < q_last - w);
+    const bool need_rla = rla_on && kt >= whole && (j0 < q_last - w);
     if (!need_swa && !need_rla) continue;
     __syncthreads();
     load_tile<TIO, D, BK>(Ks, kg, j0, T, tid, kv_pitch);
@@ -183,6 +190,10 @@ __global__ void __launch_bounds__(NT) bwd_dq_kernel(Args a, const float* __restr
       tile_pv<D, 2, BK>(dfq, Ps, Fk, ty, tx);
     }
   }
+  // the whole chunks: dphi_q += g_r S^T
+  if (whole > 0)
+    tile_matrix<D, 2>(dfq, Gr, a.gstate + (((size_t)b * a.H_kv + hk) * ((T + GC - 1) / GC) + whole) * D * D, true, Ks, Ps, tid,
+                      ty, tx);
   // dq += gradient through phi: phi(q) * (dphi_q - <dphi_q, phi(q)>) for the softmax map
   TIO* dqg = reinterpret_cast<TIO*>(a.dq) + head_base<D>(b, h, a.H_q, T, a.layout);
 #pragma unroll
@@ -215,11 +226,12 @@ __global__ void __launch_bounds__(NT) bwd_dq_kernel(Args a, const float* __restr
 }
 
 // ------------------------------------------------------------------------------ dk, dv
-template <typename TIO, int D>
+// BK: key rows per CTA (64, or 32 where tiles of 64 would leave most of the GPU idle)
+template <typename TIO, int D, int BK>
 __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __restrict__ do_s,
                                                      const float* __restrict__ do_r,
                                                      const float* __restrict__ delta) {
-  constexpr int BQ = 32, BK = 64, LD = D + PAD, LP = BQ + PAD;
+  constexpr int BQ = 32, NA = BK / 16, LD = D + PAD, LP = BQ + PAD;
   extern __shared__ __align__(16) float smem[];
   float* Ks = smem;                  // [BK][LD]
   float* Vs = Ks + BK * LD;
@@ -247,9 +259,9 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
   __syncthreads();
   if (rla_on) feature_map_tile<D, BK>(Fk, Ks, tid, a.phi);
 
-  float4 dk[4][D / 64], dv[4][D / 64], dfk[4][D / 64];
+  float4 dk[NA][D / 64], dv[NA][D / 64], dfk[NA][D / 64];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < NA; ++i)
 #pragma unroll
     for (int c = 0; c < D / 64; ++c) {
       dk[i][c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -258,6 +270,8 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
     }
 
   const int n_qt = (T + BQ - 1) / BQ;
+  // queries from this chunk of them on lie beyond the window of every key of the tile: they come through the reverse state
+  const int n_c = (T + GC - 1) / GC, c_far = (rla_on && a.grstate) ? (j0 + BK + w + GC - 1) / GC : n_c;
   for (int hh = 0; hh < a.group; ++hh) {
     const int h = hk * a.group + hh;
     const size_t row_base = ((size_t)b * a.H_q + h) * T;
@@ -265,7 +279,7 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
     for (int qt = j0 / BQ; qt < n_qt; ++qt) {
       const int q0 = qt * BQ, q_last = min(q0 + BQ, T) - 1;
       const bool need_swa = (j0 <= q_last) && (j0 + BK - 1 >= q0 - w);
-      const bool need_rla = rla_on && (j0 < q_last - w);
+      const bool need_rla = rla_on && qt < c_far * (GC / BQ) && (j0 < q_last - w);
       if (!need_swa && !need_rla) continue;
       __syncthreads();
       load_tile<TIO, D, BQ>(Qs, qg, q0, T, tid, q_pitch);
@@ -279,11 +293,11 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
       __syncthreads();
       if (need_rla) feature_map_tile<D, BQ>(Fq, Qs, tid, a.phi);
       if (need_swa) {
-        float s[4][2], dp[4][2];
-        tile_scores<D, 4, 2>(s, Ks, Qs, ty, tx);
-        tile_scores<D, 4, 2>(dp, Vs, Gs, ty, tx);
+        float s[NA][2], dp[NA][2];
+        tile_scores<D, NA, 2>(s, Ks, Qs, ty, tx);
+        tile_scores<D, NA, 2>(dp, Vs, Gs, ty, tx);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < NA; ++i) {
           const int jj = j0 + ty + 16 * i;
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -294,25 +308,25 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
           }
         }
         __syncthreads();
-        tile_pv<D, 4, BQ>(dv, Ps, Gs, ty, tx);
+        tile_pv<D, NA, BQ>(dv, Ps, Gs, ty, tx);
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < NA; ++i)
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             const int c = tx + 16 * j;
             Ps[(ty + 16 * i) * LP + c] = s[i][j] * (dp[i][j] - del_s[c]) * a.scale;
           }
         __syncthreads();
-        tile_pv<D, 4, BQ>(dk, Ps, Qs, ty, tx);
+        tile_pv<D, NA, BQ>(dk, Ps, Qs, ty, tx);
       }
       if (need_rla) {
         __syncthreads();
-        float at[4][2], da[4][2];
-        tile_scores<D, 4, 2>(at, Fk, Fq, ty, tx);
-        tile_scores<D, 4, 2>(da, Vs, Gr, ty, tx);
+        float at[NA][2], da[NA][2];
+        tile_scores<D, NA, 2>(at, Fk, Fq, ty, tx);
+        tile_scores<D, NA, 2>(da, Vs, Gr, ty, tx);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < NA; ++i) {
           const int jj = j0 + ty + 16 * i;
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -323,21 +337,26 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
           }
         }
         __syncthreads();
-        tile_pv<D, 4, BQ>(dv, Ps, Gr, ty, tx);
+        tile_pv<D, NA, BQ>(dv, Ps, Gr, ty, tx);
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < NA; ++i)
 #pragma unroll
           for (int j = 0; j < 2; ++j) Ps[(ty + 16 * i) * LP + tx + 16 * j] = da[i][j];
         __syncthreads();
-        tile_pv<D, 4, BQ>(dfk, Ps, Fq, ty, tx);
+        tile_pv<D, NA, BQ>(dfk, Ps, Fq, ty, tx);
       }
     }
+  }
+  if (c_far < n_c) {
+    const float* R = a.grstate + (((size_t)b * a.H_kv + hk) * n_c + c_far) * D * D;
+    tile_matrix<D, NA>(dfk, Vs, R, true, Qs, Gs, tid, ty, tx);           // dphi_k += V R^T
+    tile_matrix<D, NA>(dv, Fk, R, false, Qs, Gs, tid, ty, tx);           // dv     += phi(k) R
   }
   TIO* dkg = reinterpret_cast<TIO*>(a.dk) + kv_head;
   TIO* dvg = reinterpret_cast<TIO*>(a.dv) + kv_head;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NA; ++i) {
     const int r = ty + 16 * i, jj = j0 + r;
     float dot = 0.f;
     float4 f[D / 64];
@@ -364,6 +383,7 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
       }
     }
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");                   // not to end before the dq kernel beside it
 }
 
 template <typename TIO, int D>
@@ -383,18 +403,47 @@ cudaError_t launch_bwd(const Args& a, cudaStream_t s) {
   }
   { KernelTimer kt("generic_bwd_preprocess", s);
     bwd_preprocess_kernel<TIO, D><<<(unsigned)((n_rows + 7) / 8), 256, 0, s>>>(a, do_s, do_r, delta); }
+  count_launches(1);
+  if (a.grstate) {
+    e = launch_chunk_states<TIO, float, D>(static_cast<const TIO*>(a.q), do_r, a.grstate, a.B, a.T, a.H_kv, a.group, a.layout,
+                                           RATTN_LAYOUT_BHTD, a.phi, 1, s);
+    if (e != cudaSuccess) return e;
+  }
   constexpr int LD = D + PAD;
   constexpr size_t smem_dq = (size_t)(4 * 32 * LD + 3 * 64 * LD + 32 * (64 + PAD) + 64) * sizeof(float);
-  constexpr size_t smem_dkv = (size_t)(4 * 32 * LD + 3 * 64 * LD + 64 * (32 + PAD) + 64) * sizeof(float);
   e = allow_smem<bwd_dq_kernel<TIO, D>>((int)smem_dq);
-  if (e != cudaSuccess) return e;
-  e = allow_smem<bwd_dkv_kernel<TIO, D>>((int)smem_dkv);
   if (e != cudaSuccess) return e;
   dim3 gq((a.T + 31) / 32, a.B * a.H_q);
   { KernelTimer kt("generic_bwd_dq", s); bwd_dq_kernel<TIO, D><<<gq, NT, smem_dq, s>>>(a, do_s, do_r, delta); }
-  dim3 gk((a.T + 63) / 64, a.B * a.H_kv);
-  { KernelTimer kt("generic_bwd_dkv", s); bwd_dkv_kernel<TIO, D><<<gk, NT, smem_dkv, s>>>(a, do_s, do_r, delta); }
-  count_launches(3);
+  count_launches(1);
+  int n_sm = 0;
+  e = sm_count(&n_sm);
+  if (e != cudaSuccess) return e;
+  auto dkv = [&](auto bk_t) -> cudaError_t {
+    constexpr int BK = decltype(bk_t)::value;
+    constexpr int smem = (4 * 32 * LD + 3 * BK * LD + BK * (32 + PAD) + 64) * (int)sizeof(float);
+    const cudaError_t e2 = allow_smem<bwd_dkv_kernel<TIO, D, BK>>(smem);
+    if (e2 != cudaSuccess) return e2;
+    dim3 gk((a.T + BK - 1) / BK, a.B * a.H_kv);
+    KernelTimer kt("generic_bwd_dkv", s);
+    // Beside the dq kernel (small problems leave most SMs free under it): it starts once every CTA of that one has,
+    // and everything it reads was complete before that one began.
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = gk;
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e3 = cudaLaunchKernelEx(&cfg, bwd_dkv_kernel<TIO, D, BK>, a, (const float*)do_s, (const float*)do_r, (const float*)delta);
+    count_launches(1);
+    return e3;
+  };
+  e = (long long)((a.T + 63) / 64) * a.B * a.H_kv < n_sm ? dkv(std::integral_constant<int, 32>{}) : dkv(std::integral_constant<int, 64>{});
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 

@@ -163,5 +163,132 @@ __device__ __forceinline__ void tile_pv(float4 (&acc)[NA][D / 64], const float* 
   }
 }
 
+// ---- chunk states ------------------------------------------------------------------------------
+// Over whole chunks of 64 tokens the residual sums are read from running sums of d x d matrices (Eq. 2): S_c = sum over
+// the chunks before c of phi(K)^T V for the forward and dq, R_c = sum over the chunks from c on of phi(Q)^T g_r, over the
+// group's heads, for dk and dv.  Their terms are formed by a CTA each; a second kernel turns them into the running sums
+// in place.  In quadratic form the residual part is O(T^2): at T = 1024, w = 128 the last query tile of a head walked 16
+// key tiles, one after another, where it now walks five and a matrix.
+constexpr int GC = 64;        // tokens of a chunk
+
+// term[bh, c] = sum over the output's `group` heads of phi(X_c)^T Y_c; X (type TX) is mapped through phi, Y (type TY) taken
+// as it is; both have H_out * group heads per batch entry.
+template <typename TX, typename TY, int D>
+__global__ void __launch_bounds__(NT) chunk_term_kernel(const TX* __restrict__ x, const TY* __restrict__ y, float* __restrict__ out,
+                                                        int T, int H_out, int group, int x_layout, int y_layout, int phi) {
+  constexpr int LD = D + PAD, M = D / 16;
+  extern __shared__ __align__(16) float smem[];
+  float* Xs = smem;
+  float* Fs = Xs + GC * LD;
+  float* Ys = Fs + GC * LD;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int c = blockIdx.x, bh = blockIdx.y, b = bh / H_out, ho = bh - b * H_out, H = H_out * group;
+  float acc[M][M];
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M; ++j) acc[i][j] = 0.f;
+  for (int g = 0; g < group; ++g) {
+    const int h = ho * group + g;
+    __syncthreads();
+    load_tile<TX, D, GC>(Xs, x + head_base<D>(b, h, H, T, x_layout), c * GC, T, tid, row_pitch<D>(H, x_layout));
+    load_tile<TY, D, GC>(Ys, y + head_base<D>(b, h, H, T, y_layout), c * GC, T, tid, row_pitch<D>(H, y_layout));
+    __syncthreads();
+    feature_map_tile<D, GC>(Fs, Xs, tid, phi);          // a row beyond T maps to something, but its Y row is zero
+    __syncthreads();
+#pragma unroll 2
+    for (int t = 0; t < GC; ++t) {
+      float f[M], v[M];
+#pragma unroll
+      for (int i = 0; i < M; i += 4) {
+        *reinterpret_cast<float4*>(f + i) = *reinterpret_cast<const float4*>(Fs + t * LD + ty * 4 + 16 * i);
+        *reinterpret_cast<float4*>(v + i) = *reinterpret_cast<const float4*>(Ys + t * LD + tx * 4 + 16 * i);
+      }
+#pragma unroll
+      for (int i = 0; i < M; ++i)
+#pragma unroll
+        for (int j = 0; j < M; ++j) acc[i][j] += f[i] * v[j];
+    }
+  }
+  float* o = out + ((size_t)bh * gridDim.x + c) * D * D;
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int j = 0; j < M; j += 4)
+      *reinterpret_cast<float4*>(o + (size_t)(ty * 4 + 16 * (i & ~3) + (i & 3)) * D + tx * 4 + 16 * j) =
+          make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+}
+
+// In place along the chunks of each head: suffix = 0: slot c := sum of the slots before it; 1: sum of the slots from it on.
+// A thread walks one float4 of the matrix, eight loads in flight.
+static __global__ void __launch_bounds__(256) chunk_sum_kernel(float4* __restrict__ s, int n_chunks, int vecs, int suffix) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= vecs) return;
+  float4* p = s + (size_t)blockIdx.y * n_chunks * vecs + i + (suffix ? (size_t)(n_chunks - 1) * vecs : 0);
+  const ptrdiff_t step = suffix ? -(ptrdiff_t)vecs : (ptrdiff_t)vecs;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int c0 = 0; c0 < n_chunks; c0 += 8) {
+    float4 d[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (c0 + k < n_chunks) d[k] = p[(c0 + k) * step];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (c0 + k >= n_chunks) break;
+      if (!suffix) p[(c0 + k) * step] = acc;
+      acc.x += d[k].x; acc.y += d[k].y; acc.z += d[k].z; acc.w += d[k].w;
+      if (suffix) p[(c0 + k) * step] = acc;
+    }
+  }
+}
+
+template <typename TX, typename TY, int D>
+cudaError_t launch_chunk_states(const TX* x, const TY* y, float* out, int B, int T, int H_out, int group, int x_layout,
+                                int y_layout, int phi, int suffix, cudaStream_t s) {
+  constexpr int smem = 3 * GC * (D + PAD) * (int)sizeof(float);
+  const cudaError_t e = allow_smem<chunk_term_kernel<TX, TY, D>>(smem);
+  if (e != cudaSuccess) return e;
+  const int n = (T + GC - 1) / GC;
+  { KernelTimer kt("generic_terms", s);
+    chunk_term_kernel<TX, TY, D><<<dim3(n, B * H_out), NT, smem, s>>>(x, y, out, T, H_out, group, x_layout, y_layout, phi); }
+  { KernelTimer kt("generic_sums", s);
+    chunk_sum_kernel<<<dim3((D * D / 4 + 255) / 256, B * H_out), 256, 0, s>>>(reinterpret_cast<float4*>(out), n, D * D / 4, suffix); }
+  count_launches(2);
+  return cudaGetLastError();
+}
+
+// acc[i][c] += sum_f P[ty+16i][f] * M[f][tx*4 + 64c ..] over all D columns of the fp32 tile P (16*NA rows) and the D x D
+// matrix m in global memory (transposed: M[f][v] = m[v][f]), 64 rows of M at a time through `stage` ([64][D+PAD]) and the
+// column slice of P through `slice` ([16*NA][64+PAD]).
+template <int D, int NA>
+__device__ __forceinline__ void tile_matrix(float4 (&acc)[NA][D / 64], const float* P, const float* m, bool transposed,
+                                            float* stage, float* slice, int tid, int ty, int tx) {
+  constexpr int LD = D + PAD, LP = 64 + PAD;
+  for (int f0 = 0; f0 < D; f0 += 64) {
+    __syncthreads();
+    if (!transposed) {
+      for (int i = tid; i < 64 * (D / 4); i += NT) {
+        const int r = i / (D / 4), c = (i % (D / 4)) * 4;
+        *reinterpret_cast<float4*>(stage + r * LD + c) = *reinterpret_cast<const float4*>(m + (size_t)(f0 + r) * D + c);
+      }
+    } else {
+      for (int i = tid; i < D * 16; i += NT) {
+        const int r = i >> 4, c = (i & 15) * 4;          // row r of m, columns f0 + c ..: column r of the stage
+        const float4 v = *reinterpret_cast<const float4*>(m + (size_t)r * D + f0 + c);
+        stage[(c + 0) * LD + r] = v.x;
+        stage[(c + 1) * LD + r] = v.y;
+        stage[(c + 2) * LD + r] = v.z;
+        stage[(c + 3) * LD + r] = v.w;
+      }
+    }
+    for (int i = tid; i < 16 * NA * 64; i += NT) {
+      const int r = i >> 6, c = i & 63;
+      slice[r * LP + c] = P[r * LD + f0 + c];
+    }
+    __syncthreads();
+    tile_pv<D, NA, 64>(acc, slice, stage, ty, tx);
+  }
+}
+
 }  // namespace generic
 }  // namespace rattn

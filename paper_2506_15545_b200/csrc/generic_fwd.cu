@@ -10,11 +10,12 @@ namespace rattn {
 namespace {
 
 using namespace generic;
-constexpr int BM = 64;        // query rows per CTA
 constexpr int BN = 64;        // keys per tile
 
-template <typename TIO, int D>
+// BM: query rows per CTA (64, or 32 where tiles of 64 would leave most of the GPU idle)
+template <typename TIO, int D, int BM>
 __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
+  constexpr int NA = BM / 16;
   constexpr int LD = D + PAD;
   constexpr int LP = BN + PAD;
   extern __shared__ __align__(16) float smem[];
@@ -43,14 +44,14 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
   const TIO* kg = reinterpret_cast<const TIO*>(a.k) + head_base<D>(b, hk, a.H_kv, a.Tk, a.kv_layout);
   const TIO* vg = reinterpret_cast<const TIO*>(a.v) + head_base<D>(b, hk, a.H_kv, a.Tk, a.kv_layout);
 
-  load_tile<TIO, D, 64>(Qs, qg, q0, T, tid, q_pitch);
+  load_tile<TIO, D, BM>(Qs, qg, q0, T, tid, q_pitch);
   __syncthreads();
-  if (rla_on) feature_map_tile<D, 64>(Fq, Qs, tid, a.phi);
+  if (rla_on) feature_map_tile<D, BM>(Fq, Qs, tid, a.phi);
 
-  float m_run[4], l_run[4];
-  float4 acc_s[4][D / 64], acc_r[4][D / 64];
+  float m_run[NA], l_run[NA];
+  float4 acc_s[NA][D / 64], acc_r[NA][D / 64];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NA; ++i) {
     m_run[i] = -INFINITY;
     l_run[i] = 0.f;
 #pragma unroll
@@ -62,11 +63,13 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
 
   const int q_last = min(q0 + BM, T) - 1;
   const int n_kt = (q_last + off) / BN + 1;
+  static_assert(BN == GC, "chunks are key tiles");
+  const int whole = (rla_on && a.gstate && q0 > w) ? (q0 - w) / GC : 0;   // chunks wholly before every row's window
   for (int kt = 0; kt < n_kt; ++kt) {
     const int j0 = kt * BN;
     // some row t in [q0, q_last] has this tile's keys inside its window / residual set
     const bool need_swa = (j0 + BN - 1 >= q0 + off - w);
-    const bool need_rla = rla_on && (j0 < q_last + off - w);
+    const bool need_rla = rla_on && kt >= whole && (j0 < q_last + off - w);
     if (!need_swa && !need_rla) continue;
     __syncthreads();                              // previous tile fully consumed
     load_tile<TIO, D, 64>(Ks, kg, j0, Tk, tid, kv_pitch);
@@ -75,10 +78,10 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
     if (need_rla) feature_map_tile<D, 64>(Fk, Ks, tid, a.phi);
 
     if (need_swa) {
-      float s[4][4];
-      tile_scores<D, 4, 4>(s, Qs, Ks, ty, tx);
+      float s[NA][4];
+      tile_scores<D, NA, 4>(s, Qs, Ks, ty, tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < NA; ++i) {
         const int t = q0 + ty + 16 * i, tk = t + off;
         float mx = -INFINITY;
 #pragma unroll
@@ -107,14 +110,14 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
         }
       }
       __syncthreads();
-      tile_pv<D, 4, 64>(acc_s, Ps, Vs, ty, tx);
+      tile_pv<D, NA, 64>(acc_s, Ps, Vs, ty, tx);
     }
     if (need_rla) {
       __syncthreads();                            // Fk written, Ps free again
-      float s[4][4];
-      tile_scores<D, 4, 4>(s, Fq, Fk, ty, tx);
+      float s[NA][4];
+      tile_scores<D, NA, 4>(s, Fq, Fk, ty, tx);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < NA; ++i) {
         const int t = q0 + ty + 16 * i;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -123,34 +126,22 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
         }
       }
       __syncthreads();
-      tile_pv<D, 4, 64>(acc_r, Ps, Vs, ty, tx);
+      tile_pv<D, NA, 64>(acc_r, Ps, Vs, ty, tx);
     }
   }
 
-  // A resumed sequence: the tokens before the history reach every row through the incoming state,
-  // o_rla += phi(q) S_in (Eq. 4), 64 feature rows of S_in at a time.
-  if (rla_on && a.state_in) {
-    const float* Sg = a.state_in + ((size_t)b * a.H_kv + hk) * D * D;
-    for (int f0 = 0; f0 < D; f0 += 64) {
-      __syncthreads();
-      for (int i = tid; i < 64 * (D / 4); i += NT) {
-        const int r = i / (D / 4), c = (i % (D / 4)) * 4;
-        *reinterpret_cast<float4*>(Vs + r * LD + c) = *reinterpret_cast<const float4*>(Sg + (size_t)(f0 + r) * D + c);
-      }
-      for (int i = tid; i < 64 * 64; i += NT) {
-        const int r = i >> 6, c = i & 63;
-        Ps[r * LP + c] = Fq[r * LD + f0 + c];
-      }
-      __syncthreads();
-      tile_pv<D, 4, 64>(acc_r, Ps, Vs, ty, tx);
-    }
-  }
+  // The tokens before a resumed sequence's history reach every row through the incoming state, o_rla += phi(q) S_in
+  // (Eq. 4); of a fresh sequence's residual keys the whole chunks through their running sum.
+  if (rla_on && a.state_in) tile_matrix<D, NA>(acc_r, Fq, a.state_in + ((size_t)b * a.H_kv + hk) * D * D, false, Vs, Ps, tid, ty, tx);
+  if (whole > 0)
+    tile_matrix<D, NA>(acc_r, Fq, a.gstate + (((size_t)b * a.H_kv + hk) * ((a.T + GC - 1) / GC) + whole) * D * D, false, Vs, Ps,
+                       tid, ty, tx);
 
   // Section 3.2: two separate RMS norms, then the sum.
   TIO* og = reinterpret_cast<TIO*>(a.out) + head_base<D>(b, h, a.H_q, a.T, a.layout);
   const size_t row_base = ((size_t)b * a.H_q + h) * a.T;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NA; ++i) {
     const int t = q0 + ty + 16 * i;
     const float inv_l = (l_run[i] > 0.f) ? 1.f / l_run[i] : 0.f;
     float ss = 0.f, sr = 0.f;
@@ -193,15 +184,28 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
   }
 }
 
-template <typename TIO, int D>
-cudaError_t launch_fwd(const Args& a, cudaStream_t s) {
-  constexpr size_t smem = (size_t)(5 * BM * (D + PAD) + BM * (BN + PAD)) * sizeof(float);
-  cudaError_t e = allow_smem<generic_fwd_kernel<TIO, D>>((int)smem);
+template <typename TIO, int D, int BM>
+cudaError_t launch_tiles(const Args& a, cudaStream_t s) {
+  constexpr int smem = (2 * BM * (D + PAD) + 3 * BN * (D + PAD) + BM * (BN + PAD)) * (int)sizeof(float);
+  const cudaError_t e = allow_smem<generic_fwd_kernel<TIO, D, BM>>(smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.T + BM - 1) / BM, a.B * a.H_q);
-  { KernelTimer kt("generic_fwd", s); generic_fwd_kernel<TIO, D><<<grid, NT, smem, s>>>(a); }
+  { KernelTimer kt("generic_fwd", s); generic_fwd_kernel<TIO, D, BM><<<grid, NT, smem, s>>>(a); }
   count_launches(1);
   return cudaGetLastError();
+}
+
+template <typename TIO, int D>
+cudaError_t launch_fwd(const Args& a, cudaStream_t s) {
+  int n_sm = 0;
+  cudaError_t e = sm_count(&n_sm);
+  if (e != cudaSuccess) return e;
+  if (a.gstate) {
+    e = launch_chunk_states<TIO, TIO, D>(static_cast<const TIO*>(a.k), static_cast<const TIO*>(a.v), a.gstate, a.B, a.T, a.H_kv, 1,
+                                         a.kv_layout, a.kv_layout, a.phi, 0, s);
+    if (e != cudaSuccess) return e;
+  }
+  return (long long)((a.T + 63) / 64) * a.B * a.H_q < n_sm ? launch_tiles<TIO, D, 32>(a, s) : launch_tiles<TIO, D, 64>(a, s);
 }
 
 }  // namespace

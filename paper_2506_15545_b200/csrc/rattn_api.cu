@@ -125,6 +125,11 @@ WorkspaceLayout workspace_layout(int B, int H_q, int H_kv, int T, int d, int w, 
   L.chunk_state = take(tc && rla, states * sizeof(__nv_bfloat16));
   L.rstate = take(tc && rla && train, states * sizeof(__nv_bfloat16));
   L.rdelta = take(tc && rla && train && (long long)B * H_kv * L.n_chunks <= kMaxParallelTerms, states * sizeof(float));
+  // (not for a shape that is merely kept off the tensor-core kernels: that is for comparisons)
+  const bool gs = !tc && rla && train && !tensor_path(d, w, dtype, mode, 0);
+  const size_t gstates = (size_t)B * H_kv * ((T + 63) / 64) * d * d * sizeof(float);
+  L.gstate = take(gs, gstates);
+  L.grstate = take(gs, gstates);
   L.lse2p = take(tc && train, rows_pad * sizeof(float));
   L.dscp = take(tc && train, rows_pad * sizeof(float));
   const size_t io_elem = dtype == RATTN_F32 ? sizeof(float) : sizeof(__nv_bfloat16);
@@ -191,6 +196,8 @@ static int bind_workspace(const rattn_params* p, Args* a, bool required, unsigne
   a->delta = reinterpret_cast<float*>(at(L.delta));
   a->chunk_state = reinterpret_cast<__nv_bfloat16*>(at(L.chunk_state));
   a->rstate = reinterpret_cast<__nv_bfloat16*>(at(L.rstate));
+  a->gstate = reinterpret_cast<float*>(at(L.gstate));
+  a->grstate = reinterpret_cast<float*>(at(L.grstate));
   a->rdelta = reinterpret_cast<float*>(at(L.rdelta));
   a->lse2p = reinterpret_cast<float*>(at(L.lse2p));
   a->dscp = reinterpret_cast<float*>(at(L.dscp));

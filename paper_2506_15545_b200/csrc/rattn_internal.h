@@ -28,6 +28,8 @@ struct WorkspaceLayout {
   size_t delta;         // fp32 [B,H_q,T]      backward scratch
   size_t chunk_state;   // bf16 [B,H_kv,n_chunks,d,d]  exclusive prefix over chunks
   size_t rstate;        // bf16 [B,H_kv,n_chunks,d,d]  backward: suffix sums of phi(Q)^T g_r
+  size_t gstate;        // fp32 [B,H_kv,ceil(T/64),d,d]  portable training path: sums of phi(K)^T V over the chunks before
+  size_t grstate;       // fp32 [B,H_kv,ceil(T/64),d,d]  ... and of phi(Q)^T g_r over the chunks from this one on
   size_t rdelta;        // fp32 [B,H_kv,n_chunks,d,d]  backward: their terms, where these are formed in parallel
   size_t lse2p;         // fp32 [B*H_q, n_chunks*128]  backward: lse * log2(e), +inf in the padding
   size_t dscp;          // fp32 [B*H_q, n_chunks*128]  backward: D_t * scale, 0 in the padding
@@ -81,6 +83,8 @@ struct Args {
   // tensor-path scratch
   __nv_bfloat16* chunk_state;
   __nv_bfloat16* rstate;
+  float* gstate;               // portable path, training: see WorkspaceLayout (null: residual sums in quadratic form)
+  float* grstate;
   float* rdelta;
   float* lse2p;
   float* dscp;

@@ -80,3 +80,29 @@ def test_forward_single_tiles_and_pairs(B, Hq, Hkv, T, w):
         ref = O.forward(np64(q[-1:, h:h + 1]), np64(k[-1:, h // g:h // g + 1]), np64(v[-1:, h // g:h // g + 1]), w, wl.scale)
         check(y[-1:, h:h + 1], ref, "bf16", f"head {h}")
     assert np.isfinite(np64(y)).all()
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,T,d,w,dtype", [
+    (1, 2, 2, 193, 64, 1, "f32"),        # window of two keys: every chunk but one through the states, last chunk one row
+    (1, 2, 1, 320, 64, 63, "f32"),       # state boundary at a tile edge, group of two
+    (2, 3, 1, 400, 128, 100, "bf16"),    # d = 128 in two slices, ragged, group of three
+    (1, 40, 40, 256, 64, 64, "f32"),     # enough heads for tiles of 64 rows
+    (1, 2, 2, 130, 64, 65, "f32"),       # a window that leaves no whole chunk
+])
+def test_portable_chunk_states(B, Hq, Hkv, T, d, w, dtype):
+    wl = small("gst", B, Hq, Hkv, T, d, w, dtype, 9700 + T, unit=True)
+    q, k, v = W.make_qkv(wl)
+    dy = W.make_dout(wl)
+    qd, kd, vd, dyd = (t.cuda() for t in (q, k, v, dy))
+    ws = R.alloc_workspace(qd, kd, w, R.MODE_RATTN, R.FLAG_SAVE_RESIDUALS)
+    ws.fill_(0xff)
+    y = R.rattn_forward_ex(qd, kd, vd, w, scale=wl.scale, workspace=ws, save_residuals=True)
+    grads = R.rattn_backward_ex(qd, kd, vd, dyd, w, ws, scale=wl.scale, flags=R.FLAG_SAVE_RESIDUALS)
+    torch.cuda.synchronize()
+    heads = slice(None) if Hq < 8 else slice(Hq - 1, Hq)          # a wide case checks its last head
+    args = [np64(t[:, heads]) for t in (q, k, v)]
+    check(y[:, heads], O.forward(*args, w, wl.scale), dtype, "forward")
+    want = O.backward(*args, np64(dy[:, heads]), w, wl.scale)
+    for name, got, ref in zip(("dq", "dk", "dv"), grads, want):
+        got = np64(got[:, heads])
+        assert np.linalg.norm(got - ref) <= (1e-4 if dtype == "f32" else 5e-2) * np.linalg.norm(ref), name
