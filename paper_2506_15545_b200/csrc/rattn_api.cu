@@ -124,7 +124,10 @@ WorkspaceLayout workspace_layout(int B, int H_q, int H_kv, int T, int d, int w, 
   L.delta = take(train, rows * sizeof(float));
   L.chunk_state = take(tc && rla, states * sizeof(__nv_bfloat16));
   L.rstate = take(tc && rla && train, states * sizeof(__nv_bfloat16));
-  L.rdelta = take(tc && rla && train && (long long)B * H_kv * L.n_chunks <= kMaxParallelTerms, states * sizeof(float));
+  L.rdelta = take(tc && rla && train && (long long)B * H_kv * L.n_chunks <= kMaxParallelTerms,
+                  states * sizeof(float) * (size_t)head_split((long long)B * H_kv * L.n_chunks, H_q / H_kv));
+  const int parts = head_split((long long)B * H_kv * L.n_chunks, H_q / H_kv);
+  L.kvpart = take(tc && train && parts > 1, 2 * states * sizeof(float) * (size_t)parts);
   // (not for a shape that is merely kept off the tensor-core kernels: that is for comparisons)
   const bool gs = !tc && rla && train && !tensor_path(d, w, dtype, mode, 0);
   const size_t gstates = (size_t)B * H_kv * ((T + 63) / 64) * d * d * sizeof(float);
@@ -199,6 +202,7 @@ static int bind_workspace(const rattn_params* p, Args* a, bool required, unsigne
   a->gstate = reinterpret_cast<float*>(at(L.gstate));
   a->grstate = reinterpret_cast<float*>(at(L.grstate));
   a->rdelta = reinterpret_cast<float*>(at(L.rdelta));
+  a->kvpart = reinterpret_cast<float*>(at(L.kvpart));
   a->lse2p = reinterpret_cast<float*>(at(L.lse2p));
   a->dscp = reinterpret_cast<float*>(at(L.dscp));
   a->n_chunks = L.n_chunks;

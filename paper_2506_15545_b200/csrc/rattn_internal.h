@@ -9,6 +9,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <utility>
 
 #include "rattn.h"
 
@@ -30,7 +31,8 @@ struct WorkspaceLayout {
   size_t rstate;        // bf16 [B,H_kv,n_chunks,d,d]  backward: suffix sums of phi(Q)^T g_r
   size_t gstate;        // fp32 [B,H_kv,ceil(T/64),d,d]  portable training path: sums of phi(K)^T V over the chunks before
   size_t grstate;       // fp32 [B,H_kv,ceil(T/64),d,d]  ... and of phi(Q)^T g_r over the chunks from this one on
-  size_t rdelta;        // fp32 [B,H_kv,n_chunks,d,d]  backward: their terms, where these are formed in parallel
+  size_t rdelta;        // fp32 [B,H_kv,n_chunks,head_split,d,d]  backward: their terms, where these are formed in parallel
+  size_t kvpart;        // fp32 [B,H_kv,n_chunks,head_split,2,d,d]  backward: partial dK, dV of a share of a group's heads
   size_t lse2p;         // fp32 [B*H_q, n_chunks*128]  backward: lse * log2(e), +inf in the padding
   size_t dscp;          // fp32 [B*H_q, n_chunks*128]  backward: D_t * scale, 0 in the padding
   size_t k_ext;         // I/O type [B,H_kv,w+T,d]  chunked prefill: history + chunk keys, in time order
@@ -44,6 +46,15 @@ struct WorkspaceLayout {
 // heads.  Up to this many terms (64 KB each) they are formed by a CTA each and summed by a second kernel instead; with
 // more of them the chain runs beside the dq kernel, which hides it.
 constexpr long long kMaxParallelTerms = 512;
+
+// Grouped heads: where the (key tile, K/V head) items of the dk/dv kernel leave most of the GPU idle, an item is split
+// over the group's query heads, whose contributions (fp32) a second kernel adds.  The largest divisor of the group for
+// which the parts still run at once, one per SM of a B200.
+inline int head_split(long long items, int group) {
+  for (int n = group; n > 1; --n)
+    if (group % n == 0 && items * n <= 148) return n;
+  return 1;
+}
 
 // Offset of a region the call does not use.
 constexpr size_t kAbsent = ~(size_t)0;
@@ -86,6 +97,7 @@ struct Args {
   float* gstate;               // portable path, training: see WorkspaceLayout (null: residual sums in quadratic form)
   float* grstate;
   float* rdelta;
+  float* kvpart;
   float* lse2p;
   float* dscp;
   int n_chunks;
@@ -157,8 +169,9 @@ struct StateLaunch {
   int phi;                  // rattn_feature_map applied to x
   int* status;
   int* ready;               // optional [n_kv] (forward chain): matrices stored so far, published after each store
-  float* delta;             // optional fp32 scratch, n_kv * n_steps matrices: the terms are formed in parallel and
-                            // summed by a second kernel (store_every = 1, no hand-off, no incoming state)
+  float* delta;             // optional fp32 scratch, n_kv * n_steps * h_split matrices: the terms are formed in parallel
+                            // and summed by a second kernel (store_every = 1, no hand-off, no incoming state)
+  int h_split;              // ... each by this many CTAs, a share of the group's heads each
   bool after_independent;   // the kernel before on the stream neither feeds this one nor is fed by it: they may overlap
   const char* name;         // label of the timing record
 };
@@ -193,6 +206,24 @@ cudaError_t allow_smem(int bytes) {
   e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) granted[dev].store(bytes, std::memory_order_relaxed);
   return e;
+}
+
+// Launch with or without programmatic stream serialisation: with it the kernel may be set up while the one ahead of it on
+// the stream still runs, and has to wait for that one itself (griddepcontrol.wait) before it reads or overwrites anything
+// the other uses -- and in any case before it ends, so that whatever follows may rely on both.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // Records a CUDA event pair around one kernel launch on its stream while per-kernel

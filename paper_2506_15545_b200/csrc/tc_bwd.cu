@@ -49,8 +49,11 @@ struct BwdArgs {
   int t_pad;
   int* status;
   int* counter;         // next item of the launch (device memory, zero at launch)
+  int wait_first;       // 1: wait for the kernel ahead right after the set-up
   int wait_before;      // 1: the kernel ahead (the reverse states' chain) may still be running; not to end before it
-  int T, w, H_q, group, mode, n_chunks, n_bh;   // n_bh: query heads (dq), K/V heads (dk/dv) over the batch
+  int T, w, H_q, group, mode, n_chunks, n_bh;   // n_bh: query heads (dq), K/V heads times parts (dk/dv) over the batch
+  int split;            // dk/dv: parts that the group's heads are split into
+  float4* part;         // ... and where their dK, dV go in fp32 (null: one part, straight to the outputs)
   int phi;              // rattn_feature_map
   float scale, scale_log2;
 };
@@ -165,8 +168,10 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
     for (int i = 0; i < PREP_STAGES; ++i) mbar_init(&full[i], 1);
     *abort = 0;
     fence_mbar_init();
-    if (blockIdx.x == 0) a.counters[0] = a.counters[1] = 0;
   }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");        // the forward's residuals
+  if (blockIdx.x == 0 && tid == 0) a.counters[0] = a.counters[1] = 0;
   __syncthreads();
 
   // chunk i: head i / cph, rows t0 .. t0 + 31 of it; rows at or beyond T are padding (nothing is copied)
@@ -704,8 +709,6 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   extern __shared__ __align__(1024) unsigned char smem[];
   DqBars* bars = reinterpret_cast<DqBars*>(smem + DQ_OFF_BAR);
   const int tid = threadIdx.x, warp = tid >> 5;
-  // a kernel that does not read dq may take the SMs that run out of items
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0 && a.status) atomicExch(a.status, 2);
     return;
@@ -731,6 +734,10 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
+  if (a.wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // A kernel that does not read dq may take the SMs that run out of items.  (Behind the wait: the terms of the reverse
+  // states start on this signal alone, and what they read is complete only then.)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 288) {
     prefetch_map(&tm.q);
     prefetch_map(&tm.k);
@@ -812,7 +819,7 @@ struct KvMaps {
 // are numbered.  Counters that run on across key tiles (ring slots, TMEM slots, barrier
 // phases) are kept by every role in the same way.
 struct KvPlan {
-  int j, bh_kv, rs_index, n_qt, wt, group, n_R, n_s_tiles, N;
+  int j, bh_kv, head0, part_index, rs_index, n_qt, wt, group, n_R, n_s_tiles, N;
   bool windowed, has_inter;
   __device__ bool is_r(int n) const { return n < n_R; }
   __device__ int head(int n) const { return n < n_R ? (n >> 1) : (n - n_R) / (2 * n_s_tiles); }
@@ -824,17 +831,21 @@ __device__ __forceinline__ KvPlan kv_plan(const BwdArgs& a, int idx) {
   KvPlan pl;
   pl.n_qt = (a.T + TILE - 1) / TILE;
   pl.j = idx / a.n_bh;                                     // most query tiles first
-  pl.bh_kv = idx - pl.j * a.n_bh;
+  const int rem = idx - pl.j * a.n_bh;
+  pl.bh_kv = rem / a.split;
+  const int part = rem - pl.bh_kv * a.split;
+  pl.part_index = (pl.bh_kv * pl.n_qt + pl.j) * a.split + part;
   pl.rs_index = pl.bh_kv * a.n_chunks + pl.j;
   pl.wt = a.w / TILE;
-  pl.group = a.group;
+  pl.group = a.group / a.split;
+  pl.head0 = pl.bh_kv * a.group + part * pl.group;
   pl.windowed = (a.mode != RATTN_MODE_FULL_CAUSAL);
   const int i_hi = (pl.windowed && pl.j + pl.wt < pl.n_qt - 1) ? pl.j + pl.wt : pl.n_qt - 1;
   pl.n_s_tiles = i_hi - pl.j + 1;
   const bool r_tile = pl.windowed && (a.mode == RATTN_MODE_RATTN) && (pl.j + pl.wt <= pl.n_qt - 1);
-  pl.n_R = r_tile ? 2 * a.group : 0;
-  pl.has_inter = r_tile && (pl.j + pl.wt + 1 <= pl.n_qt - 1);
-  pl.N = pl.n_R + 2 * a.group * pl.n_s_tiles;
+  pl.n_R = r_tile ? 2 * pl.group : 0;
+  pl.has_inter = part == 0 && r_tile && (pl.j + pl.wt + 1 <= pl.n_qt - 1);
+  pl.N = pl.n_R + 2 * pl.group * pl.n_s_tiles;
   return pl;
 }
 
@@ -878,7 +889,7 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
       int st;
       if (!ring(st)) return false;
       unsigned char* dst = smem + KV_OFF_STAGE + st * TILE_BYTES;
-      const int z = pl.bh_kv * pl.group + pl.head(n);
+      const int z = pl.head0 + pl.head(n);
       const int row = pl.qtile(n) * TILE + 64 * pl.half(n);
       if (pl.is_r(n)) {
         mbar_arrive_expect_tx(&bars->full[st], 2 * HT_BYTES);
@@ -1179,35 +1190,50 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   if (gg < 2) {
     WAIT_OR_RETURN(bars->all_done, cnt.it & 1);
     tc_fence_after();
-    if (gg == 1 && r == 0) tma_store_wait_read();            // the previous dV has left the staging tile
-    if (gg == 1) group_sync(1);
-    unsigned char* sOut = gg == 0 ? smem + KV_OFF_STAGE + ((seq0 + pl.N + 2) % KV_NS) * TILE_BYTES : smem + KV_OFF_OUT;
     const uint32_t tOut = gg == 0 ? tK : tV;
+    if (a.part) {
+      // one of several parts: fp32, float4 columns outermost ([32][128 rows]), so that a warp's stores are whole runs
+      float4* dst = a.part + ((size_t)pl.part_index * 2 + gg) * 4096 + r;
 #pragma unroll 1
-    for (int cc = 0; cc < 4; cc += 2) {                        // two loads in flight
-      float x[2][32];
-      tmem_ld32(tOut + 32 * cc, x[0]);
-      tmem_ld32(tOut + 32 * (cc + 1), x[1]);
-      tmem_wait_ld();
+      for (int cc = 0; cc < 4; ++cc) {
+        float x[32];
+        tmem_ld32(tOut + 32 * cc, x);
+        tmem_wait_ld();
 #pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2)
+        for (int e = 0; e < 8; ++e) dst[(8 * cc + e) * 128] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+      }
+      tc_fence_before();
+      mbar_arrive(&bars->acc_free);
+    } else {
+      if (gg == 1 && r == 0) tma_store_wait_read();            // the previous dV has left the staging tile
+      if (gg == 1) group_sync(1);
+      unsigned char* sOut = gg == 0 ? smem + KV_OFF_STAGE + ((seq0 + pl.N + 2) % KV_NS) * TILE_BYTES : smem + KV_OFF_OUT;
+#pragma unroll 1
+      for (int cc = 0; cc < 4; cc += 2) {                        // two loads in flight
+        float x[2][32];
+        tmem_ld32(tOut + 32 * cc, x[0]);
+        tmem_ld32(tOut + 32 * (cc + 1), x[1]);
+        tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          uint4 u;
-          u.x = pack_bf16(x[h2][8 * e + 0], x[h2][8 * e + 1]);
-          u.y = pack_bf16(x[h2][8 * e + 2], x[h2][8 * e + 3]);
-          u.z = pack_bf16(x[h2][8 * e + 4], x[h2][8 * e + 5]);
-          u.w = pack_bf16(x[h2][8 * e + 6], x[h2][8 * e + 7]);
-          *reinterpret_cast<uint4*>(sOut + swz(r, 4 * (cc + h2) + e)) = u;
-        }
-    }
-    tc_fence_before();
-    mbar_arrive(&bars->acc_free);                              // the accumulators have been read
-    fence_proxy_async_smem();
-    group_sync(gg);
-    if (r == 0) {
-      store_tile(gg == 0 ? &tm.dk : &tm.dv, sOut, pl.j * TILE, bh_kv);
-      tma_store_commit();
+        for (int h2 = 0; h2 < 2; ++h2)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            uint4 u;
+            u.x = pack_bf16(x[h2][8 * e + 0], x[h2][8 * e + 1]);
+            u.y = pack_bf16(x[h2][8 * e + 2], x[h2][8 * e + 3]);
+            u.z = pack_bf16(x[h2][8 * e + 4], x[h2][8 * e + 5]);
+            u.w = pack_bf16(x[h2][8 * e + 6], x[h2][8 * e + 7]);
+            *reinterpret_cast<uint4*>(sOut + swz(r, 4 * (cc + h2) + e)) = u;
+          }
+      }
+      tc_fence_before();
+      mbar_arrive(&bars->acc_free);                              // the accumulators have been read
+      fence_proxy_async_smem();
+      group_sync(gg);
+      if (r == 0) {
+        store_tile(gg == 0 ? &tm.dk : &tm.dv, sOut, pl.j * TILE, bh_kv);
+        tma_store_commit();
+      }
     }
   }
   cnt.seq = seq0 + pl.N;
@@ -1255,6 +1281,8 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (tid == 288) {
     prefetch_map(&tm.k);
     prefetch_map(&tm.v);
@@ -1290,6 +1318,35 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
+}
+
+// dK, dV of an item = the sum of its parts, rounded once.  Mapping as in the sum of the chunk-state terms: a warp reads
+// 128-byte runs of the parts and writes whole 32-byte sectors of eight rows.
+struct KvSumArgs {
+  const float4* part;
+  __nv_bfloat16* out[2];
+  int split, n_qt, T, H_kv, layout;
+};
+__global__ void __launch_bounds__(256) tc_bwd_kv_sum_kernel(const KvSumArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int item = blockIdx.x >> 4, piece = blockIdx.x & 15, which = blockIdx.y;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = 32 * (piece & 3) + 8 * (warp & 3) + (lane & 7), c4 = 8 * (piece >> 2) + 4 * (warp >> 2) + (lane >> 3);
+  const int bh = item / a.n_qt, t = (item - bh * a.n_qt) * TILE + row;
+  if (t >= a.T) return;
+  const float4* src = a.part + ((size_t)item * a.split * 2 + which) * 4096 + c4 * 128 + row;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int p0 = 0; p0 < a.split; p0 += 4) {
+    float4 d[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) d[k] = p0 + k < a.split ? __ldcg(src + (size_t)(p0 + k) * 2 * 4096) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { acc.x += d[k].x; acc.y += d[k].y; acc.z += d[k].z; acc.w += d[k].w; }
+  }
+  const int b = bh / a.H_kv, h = bh - b * a.H_kv;
+  const size_t at = (a.layout == RATTN_LAYOUT_BTHD ? ((size_t)b * a.T + t) * a.H_kv + h : (size_t)bh * a.T + t) * 128 + 4 * c4;
+  *reinterpret_cast<uint2*>(a.out[which] + at) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
 }
 
 }  // namespace
@@ -1330,7 +1387,8 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     CUtensorMap dy_map;
     if (!make_row_map(&dy_map, a.dout, a.T, a.H_q, a.B, a.layout, PREP_ROWS)) return cudaErrorInvalidValue;
     KernelTimer kt("tc_bwd_prep", s);
-    tc_bwd_prep_kernel<<<grid, PREP_THREADS, PREP_SMEM, s>>>(pa, dy_map);
+    e = launch_pdl(tc_bwd_prep_kernel, dim3(grid), dim3(PREP_THREADS), PREP_SMEM, s, !a.dgamma_swa && !a.dgamma_rla, pa, dy_map);
+    if (e != cudaSuccess) return e;
   }
   count_launches(1);
 
@@ -1372,6 +1430,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   const bool few_heads = 2 * (int)nkv <= n_sm;
   const bool parallel_terms = n_r > 0 && a.rdelta != nullptr && few_heads && 100 * chain_ns > 115 * dq_ns;
   const bool chain_beside = n_r > 0 && !parallel_terms && few_heads;
+  const int parts = a.kvpart ? head_split((long long)n_qt * (long long)nkv, a.group) : 1;
   StateLaunch L;
   L.ready = nullptr;
   L.x = a.q; L.y = g_r; L.out = a.rstate;
@@ -1383,6 +1442,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   L.phi = a.phi;
   L.status = a.status; L.name = "tc_state_bwd";
   L.delta = parallel_terms ? a.rdelta : nullptr;
+  L.h_split = parts;
   L.after_independent = parallel_terms;
   if (!parallel_terms) {
     e = launch_tc_states(L, s);
@@ -1395,18 +1455,11 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     t.n_bh = (int)nq;
     t.counter = a.work_counter + 1;
     t.wait_before = chain_beside ? 1 : 0;
+    t.wait_first = chain_beside ? 0 : 1;
+    t.split = 1; t.part = nullptr;
     KernelTimer kt("tc_bwd_dq", s);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n_items < n_sm ? n_items : n_sm));
-    cfg.blockDim = dim3(DQ_THREADS);
-    cfg.dynamicSmemBytes = DQ_SMEM;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = chain_beside ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, tc_bwd_dq_kernel, dm, t, n_items, n_qt);
+    e = launch_pdl(tc_bwd_dq_kernel, dim3((unsigned)(n_items < n_sm ? n_items : n_sm)), dim3(DQ_THREADS), DQ_SMEM, s, true, dm, t,
+                   n_items, n_qt);
     if (e != cudaSuccess) return e;
   }
   if (parallel_terms) {
@@ -1419,12 +1472,26 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
       !make_map(&km.grh, g_r, a.T, nq, 64))
     return cudaErrorInvalidValue;
   {
-    const int n_items = n_qt * (int)nkv;
-    t.n_bh = (int)nkv;
+    const int n_items = n_qt * (int)nkv * parts;
+    t.n_bh = (int)nkv * parts;
+    t.split = parts;
+    t.part = parts > 1 ? reinterpret_cast<float4*>(a.kvpart) : nullptr;
     t.counter = a.work_counter + 2;
     t.wait_before = 0;
     KernelTimer kt("tc_bwd_dkv", s);
-    tc_bwd_dkv_kernel<<<n_items < n_sm ? n_items : n_sm, KV_THREADS, KV_SMEM, s>>>(km, t, n_items);
+    e = launch_pdl(tc_bwd_dkv_kernel, dim3((unsigned)(n_items < n_sm ? n_items : n_sm)), dim3(KV_THREADS), KV_SMEM, s, true, km, t,
+                   n_items);
+    if (e != cudaSuccess) return e;
+  }
+  if (parts > 1) {
+    KvSumArgs sa;
+    sa.part = reinterpret_cast<const float4*>(a.kvpart);
+    sa.out[0] = t.dk; sa.out[1] = t.dv;
+    sa.split = parts; sa.n_qt = n_qt; sa.T = a.T; sa.H_kv = a.H_kv; sa.layout = a.layout;
+    KernelTimer kt("tc_bwd_kv_sum", s);
+    e = launch_pdl(tc_bwd_kv_sum_kernel, dim3((unsigned)(n_qt * (int)nkv * 16), 2), dim3(256), 0, s, true, sa);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
   }
   count_launches(2);
   return cudaGetLastError();

@@ -91,6 +91,7 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.status = a.status; L.name = "tc_state_fwd";
     L.ready = progress ? a.state_ready : nullptr;
     L.delta = nullptr;
+    L.h_split = 1;
     L.after_independent = false;
     cudaError_t e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;

@@ -262,8 +262,6 @@ __device__ bool fwd_loader(const FMaps& tm, const FArgs& a, unsigned char* smem,
       ++cntX;
     }
   }
-  // not to end before the kernel whose states were taken as they appeared
-  if (a.state_ready && a.wait_for_states) asm volatile("griddepcontrol.wait;" ::: "memory");
   return true;
 }
 
@@ -794,6 +792,7 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   FBars* bars = reinterpret_cast<FBars*>(smem + F_OFF_BAR);
   const int tid = threadIdx.x, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");    // the next kernel may be set up in the tail
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0 && a.status) atomicExch(a.status, 2);
     return;
@@ -865,6 +864,9 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
     ok = fwd_convert(a, smem, bars, tid - 320);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
+  // Not to end before the chunk-state kernel, whether or not this CTA has read a state: what follows on the stream may
+  // wait for this kernel alone and read the decode state that the other one leaves.
+  if (a.wait_for_states) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   if (warp == 8) {

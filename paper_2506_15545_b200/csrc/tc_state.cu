@@ -53,6 +53,7 @@ struct StateArgs {
   float* delta;     // optional: the CTA forms the term of one step alone and leaves it here in fp32, matrix
                     // (kv * n_split + step), its float4 columns outermost ([32][128 rows][4])
   int n_split;      // steps that the grid is split into (delta)
+  int h_split;      // ... and the group's heads: term matrix ((kv * n_split + step) * h_split + part)
   int wait_before;  // 1: the kernel ahead may still be running; not to end before it
 };
 
@@ -76,8 +77,10 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   extern __shared__ __align__(1024) unsigned char smem[];
   StBars* bars = reinterpret_cast<StBars*>(smem + ST_OFF_BAR);
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int kv = a.delta ? blockIdx.x / a.n_split : blockIdx.x;
-  const int first = a.delta ? a.first + a.dir * (int)(blockIdx.x - kv * a.n_split) : a.first;
+  const int unit = a.delta ? (int)blockIdx.x / a.h_split : (int)blockIdx.x;      // (K/V head, step)
+  const int kv = a.delta ? unit / a.n_split : unit;
+  const int first = a.delta ? a.first + a.dir * (unit - kv * a.n_split) : a.first;
+  const int group = a.delta ? a.group / a.h_split : a.group, head0 = a.delta ? group * ((int)blockIdx.x - unit * a.h_split) : 0;
   // the kernel that follows may start its own prologue (and whatever does not read the states)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((smem_u32(smem) & 1023u) != 0) {
@@ -120,7 +123,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     if (a.handoff) row_limit = len - a.w;
   }
   const bool has_init = (a.state_in != nullptr);
-  const int n_items = n_steps * a.group;
+  const int n_items = n_steps * group;
   bool ok = true;
 
   if (warp < 8) {
@@ -131,7 +134,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       if (!ok) break;
       unsigned char* xh = smem + st * ST_STAGE + (tid & 1) * HALF_BYTES;
       const int row = tid >> 1;
-      const int token = (first + a.dir * (it / a.group)) * TILE + row;
+      const int token = (first + a.dir * (it / group)) * TILE + row;
       // every lane maps its row (the softmax map exchanges partial results between the two lanes
       // of a row with full-warp shuffles, so no lane may skip it); rows past the limit are then cleared
       feature_map_pair_any(xh, xh, row, a.phi);
@@ -147,7 +150,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     int n_wait = 0;                                          // hand-backs of the accumulator so far
     for (int it = 0; it < n_items && ok; ++it) {
       const int st = it % ST_NS, use = it / ST_NS;
-      const int s = it / a.group, hh = it - s * a.group;
+      const int s = it / group, hh = it - s * group;
       ok = mbar_wait_warp(&bars->phi_ready[st], use & 1, &bars->abort);
       // the flush warps hold the previous sum, or are still writing the incoming state into the accumulator
       if (ok && hh == 0 && ((s > 0 && flushed_step(a, s - 1, n_steps)) || (s == 0 && has_init))) {
@@ -158,16 +161,16 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       tc_fence_after();
       mma_mnmn(tmem, smem_u32(smem + st * ST_STAGE), smem_u32(smem + st * ST_STAGE + TILE_BYTES), it > 0 || has_init);
       mma_commit(&bars->free_[st]);
-      if (hh == a.group - 1 && flushed_step(a, s, n_steps)) mma_commit(&bars->done);
+      if (hh == group - 1 && flushed_step(a, s, n_steps)) mma_commit(&bars->done);
     }
   } else if (warp == 9) {
     // ---- loader ---------------------------------------------------------------------------
     for (int it = 0; it < n_items && ok; ++it) {
       const int st = it % ST_NS, use = it / ST_NS;
-      const int s = it / a.group, hh = it - s * a.group;
+      const int s = it / group, hh = it - s * group;
       if (use >= 1) ok = mbar_wait_warp(&bars->free_[st], (use - 1) & 1, &bars->abort);
       if (!ok) break;
-      const int row = (first + a.dir * s) * TILE, z = kv * a.group + hh;
+      const int row = (first + a.dir * s) * TILE, z = kv * a.group + head0 + hh;
       unsigned char* dst = smem + st * ST_STAGE;
       mbar_arrive_expect_tx(&bars->full[st], ST_STAGE);
       load_tile(dst, &tm_x, &bars->full[st], row, z);
@@ -290,27 +293,35 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   }
 }
 
-// Running sums of the terms left by the kernel above: state(s) = sum of the terms 0 .. s, as bf16, row-major.  A pure
-// stream (64 KB in and 32 KB out per matrix): a thread owns one float4 of the matrix and walks the steps with four loads
-// in flight.  A warp covers 8 rows x 4 float4 columns, so that it reads 128-byte runs of the column-major terms and
-// writes whole 32-byte sectors of the row-major states.
+// Running sums of the terms left by the kernel above: state(s) = sum of the terms 0 .. s (each h_split matrices), as
+// bf16, row-major.  A pure stream (64 KB in per term matrix, 32 KB out per state): a thread owns one float4 of the matrix
+// and walks the terms with four loads in flight.  A warp covers 8 rows x 4 float4 columns, so that it reads 128-byte runs
+// of the column-major terms and writes whole 32-byte sectors of the row-major states.
 __global__ void __launch_bounds__(256) tc_state_sum_kernel(const float4* __restrict__ delta, uint2* __restrict__ out,
-                                                           int n_split, int n_chunks, int out_first, int dir) {
+                                                           int n_split, int h_split, int n_chunks, int out_first, int dir) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int kv = blockIdx.x >> 4, part = blockIdx.x & 15;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row = 32 * (part & 3) + 8 * (warp & 3) + (lane & 7), c4 = 8 * (part >> 2) + 4 * (warp >> 2) + (lane >> 3);
-  const float4* src = delta + (size_t)kv * n_split * 4096 + c4 * 128 + row;
+  const int n = n_split * h_split;
+  const float4* src = delta + (size_t)kv * n * 4096 + c4 * 128 + row;
   uint2* dst = out + ((size_t)kv * n_chunks + out_first) * 4096 + row * 32 + c4;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s0 = 0; s0 < n_split; s0 += 4) {
+  int left = h_split;
+  for (int i0 = 0; i0 < n; i0 += 4) {
     float4 d[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) d[k] = s0 + k < n_split ? __ldcg(src + (size_t)(s0 + k) * 4096) : acc;
+    for (int k = 0; k < 4; ++k) d[k] = i0 + k < n ? __ldcg(src + (size_t)(i0 + k) * 4096) : acc;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (s0 + k >= n_split) break;
+      if (i0 + k >= n) break;
       acc.x += d[k].x; acc.y += d[k].y; acc.z += d[k].z; acc.w += d[k].w;
-      dst[(ptrdiff_t)dir * (s0 + k) * 4096] = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+      if (--left == 0) {
+        *dst = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+        dst += (ptrdiff_t)dir * 4096;
+        left = h_split;
+      }
     }
   }
 }
@@ -342,29 +353,22 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   a.ready = (L.dir > 0 && L.group == 1) ? L.ready : nullptr;
   a.delta = L.delta;
   a.n_split = L.delta ? L.n_steps : 1;
+  a.h_split = L.delta ? L.h_split : 1;
   a.wait_before = L.after_independent ? 1 : 0;
   cudaError_t e = allow_smem<tc_state_scan_kernel>(ST_SMEM);
   if (e != cudaSuccess) return e;
   {
     KernelTimer kt(L.name, s);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(L.n_kv * a.n_split));
-    cfg.blockDim = dim3(ST_THREADS);
-    cfg.dynamicSmemBytes = ST_SMEM;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = L.after_independent ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, tc_state_scan_kernel, tm_x, tm_y, tm_out, a);
+    e = launch_pdl(tc_state_scan_kernel, dim3((unsigned)(L.n_kv * a.n_split * a.h_split)), dim3(ST_THREADS), ST_SMEM, s,
+                   L.after_independent, tm_x, tm_y, tm_out, a);
     if (e != cudaSuccess) return e;
   }
   count_launches(1);
   if (L.delta) {
     KernelTimer kt("tc_state_sum", s);
-    tc_state_sum_kernel<<<L.n_kv * 16, 256, 0, s>>>(reinterpret_cast<const float4*>(L.delta), reinterpret_cast<uint2*>(L.out),
-                                                    L.n_steps, L.n_chunks, L.out_first, L.dir);
+    e = launch_pdl(tc_state_sum_kernel, dim3((unsigned)L.n_kv * 16), dim3(256), 0, s, true, reinterpret_cast<const float4*>(L.delta),
+                   reinterpret_cast<uint2*>(L.out), L.n_steps, a.h_split, L.n_chunks, L.out_first, L.dir);
+    if (e != cudaSuccess) return e;
     count_launches(1);
   }
   return cudaGetLastError();

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("B,Hq,Hkv,T,w,which", [
     (1, 4, 1, 385, 128, "terms: two"),
-    (1, 8, 2, 769, 128, "terms: five, the last query tile one row long"),
+    (1, 8, 2, 769, 128, "terms: five, four parts of a group, the last query tile one row long"),
     (2, 2, 1, 1152, 256, "terms: six of a two-head group"),
     (1, 8, 8, 1024, 640, "chain beside dq: two steps, one head per group"),
     (5, 16, 16, 400, 128, "chain on more than half of the SMs"),
