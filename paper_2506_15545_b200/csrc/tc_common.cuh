@@ -199,6 +199,16 @@ __device__ __forceinline__ uint32_t swz(int r, int c) {
   return (uint32_t)((c >> 3) * HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4));
 }
 
+// x[i] *= g[i] for 16 consecutive columns; every lane reads the same 64 bytes, as four 16-byte loads (gains are 16-byte
+// aligned and 16 columns are 64 bytes).
+__device__ __forceinline__ void apply_gain16(float (&x)[16], const float* __restrict__ g) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(g) + i);
+    x[4 * i] *= v.x; x[4 * i + 1] *= v.y; x[4 * i + 2] *= v.z; x[4 * i + 3] *= v.w;
+  }
+}
+
 // One [128 x 128] bf16 tile staged in shared memory (swizzled like a loaded tile) goes to
 // rows row0.. of matrix z of a tensor map: two 64-column boxes; rows past the end are clipped.
 __device__ __forceinline__ void store_tile(const UMap* tm, const unsigned char* tile, int row0, int z) {

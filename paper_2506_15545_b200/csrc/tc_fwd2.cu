@@ -730,27 +730,26 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
             tmem_ld16(tO + 16 * c, orl);
             tmem_wait_ld();
           }
-          uint32_t yk[8];
+          float y[16];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&stash[8 * c + e]));
-            const int col = 16 * c + 2 * e;
-            float y0 = f.x, y1 = f.y;
-            if constexpr (has_gains) {
-              y0 *= gs ? __ldg(gs + col) : 1.f;
-              y1 *= gs ? __ldg(gs + col + 1) : 1.f;
-            }
-            if constexpr (has_rla) {
-              float r0 = orl[2 * e] * rr, r1 = orl[2 * e + 1] * rr;
-              if constexpr (has_gains) {
-                r0 *= gr ? __ldg(gr + col) : 1.f;
-                r1 *= gr ? __ldg(gr + col + 1) : 1.f;
-              }
-              y0 += r0;
-              y1 += r1;
-            }
-            yk[e] = pack_bf16(y0, y1);
+            y[2 * e] = f.x;
+            y[2 * e + 1] = f.y;
           }
+          if constexpr (has_gains) {
+            if (gs) apply_gain16(y, gs + 16 * c);
+          }
+          if constexpr (has_rla) {
+            if constexpr (has_gains) {
+              if (gr) apply_gain16(orl, gr + 16 * c);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) y[e] += orl[e] * rr;
+          }
+          uint32_t yk[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) yk[e] = pack_bf16(y[2 * e], y[2 * e + 1]);
           *reinterpret_cast<uint4*>(sY + swz(r, 2 * c4)) = make_uint4(yk[0], yk[1], yk[2], yk[3]);
           *reinterpret_cast<uint4*>(sY + swz(r, 2 * c4 + 1)) = make_uint4(yk[4], yk[5], yk[6], yk[7]);
         }
