@@ -124,9 +124,10 @@ WorkspaceLayout workspace_layout(int B, int H_q, int H_kv, int T, int d, int w, 
   L.delta = take(train, rows * sizeof(float));
   L.chunk_state = take(tc && rla, states * sizeof(__nv_bfloat16));
   L.rstate = take(tc && rla && train, states * sizeof(__nv_bfloat16));
-  L.rdelta = take(tc && rla && train && (long long)B * H_kv * L.n_chunks <= kMaxParallelTerms,
-                  states * sizeof(float) * (size_t)head_split((long long)B * H_kv * L.n_chunks, H_q / H_kv));
-  const int parts = head_split((long long)B * H_kv * L.n_chunks, H_q / H_kv);
+  const long long terms = (long long)B * H_kv * L.n_chunks;
+  const int parts = head_split(terms, H_q / H_kv);
+  L.rdelta = take(tc && rla && ((train && terms <= kMaxParallelTerms) || (L.n_chunks >= kMinTermChunks && terms <= kMaxForwardTerms)),
+                  states * sizeof(float) * (size_t)parts);
   L.kvpart = take(tc && train && parts > 1, 2 * states * sizeof(float) * (size_t)parts);
   // (not for a shape that is merely kept off the tensor-core kernels: that is for comparisons)
   const bool gs = !tc && rla && train && !tensor_path(d, w, dtype, mode, 0);

@@ -47,6 +47,12 @@ struct WorkspaceLayout {
 // more of them the chain runs beside the dq kernel, which hides it.
 constexpr long long kMaxParallelTerms = 512;
 
+// The forward's chain, one CTA per K/V head, takes 2.6 us per chunk when every state is stored.  For long sequences of few
+// heads that is longer than everything else; the workspace then has room for the terms, so that they too can be formed in
+// parallel.  (From 64 chunks on: shorter chains hide under the main kernel.)
+constexpr int kMinTermChunks = 64;
+constexpr long long kMaxForwardTerms = 1024;
+
 // Grouped heads: where the (key tile, K/V head) items of the dk/dv kernel leave most of the GPU idle, an item is split
 // over the group's query heads, whose contributions (fp32) a second kernel adds.  The largest divisor of the group for
 // which the parts still run at once, one per SM of a B200.
@@ -103,7 +109,7 @@ struct Args {
   int n_chunks;
   int* status;                 // device status word (may be null when no workspace)
   int* clear_status;           // the status word, where no kernel ahead of the forward's first one has cleared it
-  bool single_tiles;           // the forward's work units are single query tiles instead of pairs
+  bool single_tiles;           // the pair kernel's work units are single query tiles
   int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin);
                                // the backward's two kernels use the two words behind it
   int* state_ready;            // [B*H_kv], zero at launch: chunk states the chunk-state kernel has stored so far
@@ -143,7 +149,8 @@ cudaError_t launch_handoff(const Args& a, cudaStream_t s, bool state_too, int* c
 cudaError_t launch_tc_forward(const Args& a, cudaStream_t s);        // chunk states, then the main kernel
 bool tc_forward_clears_status(const Args& a);   // one kernel, one unit per CTA: only Args::clear_status has to be set
 // after_states: a chunk-state kernel was launched just before on the same stream
-cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_states);
+cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_states);     // pairs of query tiles (tc_fwd2.cu)
+cudaError_t launch_tc_forward_single(const Args& a, cudaStream_t s, bool after_states);   // single tiles (tc_fwd1.cu)
 // Running sums of phi(X_c)^T Y_c over the chunks first, first+dir, ... (n_steps of them) for every
 // K/V head (tc_state.cu).  The sum after step s goes, as bf16, to matrix out_first + dir*s of the
 // head when that index is congruent to store_phase modulo store_every.  With `handoff` the chain
@@ -170,7 +177,7 @@ struct StateLaunch {
   int* status;
   int* ready;               // optional [n_kv] (forward chain): matrices stored so far, published after each store
   float* delta;             // optional fp32 scratch, n_kv * n_steps * h_split matrices: the terms are formed in parallel
-                            // and summed by a second kernel (store_every = 1, no hand-off, no incoming state)
+                            // and summed by a second kernel
   int h_split;              // ... each by this many CTAs, a share of the group's heads each
   bool after_independent;   // the kernel before on the stream neither feeds this one nor is fed by it: they may overlap
   const char* name;         // label of the timing record

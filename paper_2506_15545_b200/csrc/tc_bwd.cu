@@ -58,55 +58,6 @@ struct BwdArgs {
   float scale, scale_log2;
 };
 
-// ------------------------------------------------------------------------ work items
-// Both main kernels are persistent; a CTA's next item comes from a device-wide counter, so that CTAs that start late
-// (the SM was still running another kernel) or meet heavy items simply take fewer.  The loader warp draws it and
-// publishes it in a small ring that the other roles read in order; a slot is rewritten once every reader has read it.
-constexpr int SCHED_SLOTS = 4;
-struct SchedRing {
-  uint64_t full[SCHED_SLOTS], free_[SCHED_SLOTS];
-  int item[SCHED_SLOTS];
-};
-__device__ __forceinline__ void sched_init(SchedRing* r, int readers) {
-  for (int i = 0; i < SCHED_SLOTS; ++i) {
-    mbar_init(&r->full[i], 1);
-    mbar_init(&r->free_[i], readers);
-  }
-}
-// the loader warp's side: item n of this CTA, -1 when there is none left
-__device__ __forceinline__ bool sched_draw(SchedRing* r, int* counter, int n_items, int n, volatile int* abort, int* out) {
-  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
-  if (use >= 1) { if (!mbar_wait_warp(&r->free_[slot], (use - 1) & 1, abort)) return false; }
-  int i = 0;
-  if ((threadIdx.x & 31) == 0) i = atomicAdd(counter, 1);
-  i = __shfl_sync(0xffffffffu, i, 0);
-  if (i >= n_items) i = -1;
-  if ((threadIdx.x & 31) == 0) {
-    r->item[slot] = i;
-    mbar_arrive(&r->full[slot]);
-  }
-  __syncwarp();
-  *out = i;
-  return true;
-}
-// a reading thread's side
-__device__ __forceinline__ bool sched_read(SchedRing* r, int n, volatile int* abort, int* out) {
-  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
-  if (!mbar_wait(&r->full[slot], use & 1, abort)) return false;
-  *out = r->item[slot];
-  mbar_arrive(&r->free_[slot]);
-  return true;
-}
-// ... and a whole warp's (one of its lanes is counted)
-__device__ __forceinline__ bool sched_read_warp(SchedRing* r, int n, volatile int* abort, int* out) {
-  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
-  if (!mbar_wait_warp(&r->full[slot], use & 1, abort)) return false;
-  *out = r->item[slot];
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) mbar_arrive(&r->free_[slot]);
-  return true;
-}
-
 #define WAIT_OR_RETURN(bar, parity) \
   do { if (!mbar_wait(&(bar), (parity), &bars->abort)) return false; } while (0)
 // for roles run by a whole converged warp

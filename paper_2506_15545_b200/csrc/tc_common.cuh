@@ -127,16 +127,36 @@ __device__ __forceinline__ void flush_bf16_block(const unsigned char* stage, int
   }
 }
 
-// phi over the 128 features of one row by a pair of adjacent lanes: this lane (`ch` = its parity) owns the 64
-// columns of one column half (eight 16-byte chunks at src + row * 128 within that half's box).
-// src_half / dst_half point at the [rows x 64] box of this lane's column half.  The two lanes walk the chunks four
-// apart: the boxes lie a multiple of 8 KB from each other, and in the same order both lanes would meet in the same banks.
-__device__ __forceinline__ void feature_map_pair(const unsigned char* src_half, unsigned char* dst_half, int row, int ch) {
+// The element-wise maps of the paper's ablation (Table 6) on packed bf16 pairs: ReLU; the
+// identity needs no arithmetic at all.
+__device__ __forceinline__ uint4 relu_bf16x8(uint4 u) {
+  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
+  const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) h[e] = __hmax2(h[e], z);
+  return u;
+}
+// phi over the 128 features of one row by a pair of adjacent lanes, of which this one (`ch`, its parity) owns the 64
+// columns of one column half; `src` and `dst` point at that half of the row (128 bytes, chunks swizzled by row & 7) and may
+// be the same.  normalise = false: the softmax map leaves exp(x - max).  Returns 1 / sum (1 for the element-wise maps) for
+// callers that scale whatever is linear in the row afterwards.  The two lanes walk the chunks four apart: the halves lie
+// a multiple of 8 KB from each other, and in the same order both lanes would meet in the same banks.
+__device__ __forceinline__ float feature_map_half_row(const unsigned char* src, unsigned char* dst, int row, int ch, int phi,
+                                                      bool normalise) {
   const int sw = (row & 7) ^ (ch << 2);
+  if (phi != RATTN_PHI_SOFTMAX) {
+    if (phi == RATTN_PHI_IDENTITY && src == dst) return 1.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint4 u = *reinterpret_cast<const uint4*>(src + ((c ^ sw) << 4));
+      *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) = phi == RATTN_PHI_RELU ? relu_bf16x8(u) : u;
+    }
+    return 1.f;
+  }
   float x[64], m0 = -INFINITY, m1 = -INFINITY;
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
-    const uint4 u = *reinterpret_cast<const uint4*>(src_half + row * 128 + ((c ^ sw) << 4));
+    const uint4 u = *reinterpret_cast<const uint4*>(src + ((c ^ sw) << 4));
     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -162,36 +182,17 @@ __device__ __forceinline__ void feature_map_pair(const unsigned char* src_half, 
   }
   float sum = (s0.x + s0.y) + (s1.x + s1.y);
   sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-  const float inv = 1.f / sum;
+  const float inv = 1.f / sum, sc = normalise ? inv : 1.f;
 #pragma unroll
   for (int c = 0; c < 8; ++c)
-    *reinterpret_cast<uint4*>(dst_half + row * 128 + ((c ^ sw) << 4)) =
-        make_uint4(pack_bf16(x[c * 8 + 0] * inv, x[c * 8 + 1] * inv), pack_bf16(x[c * 8 + 2] * inv, x[c * 8 + 3] * inv),
-                   pack_bf16(x[c * 8 + 4] * inv, x[c * 8 + 5] * inv), pack_bf16(x[c * 8 + 6] * inv, x[c * 8 + 7] * inv));
+    *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) =
+        make_uint4(pack_bf16(x[c * 8 + 0] * sc, x[c * 8 + 1] * sc), pack_bf16(x[c * 8 + 2] * sc, x[c * 8 + 3] * sc),
+                   pack_bf16(x[c * 8 + 4] * sc, x[c * 8 + 5] * sc), pack_bf16(x[c * 8 + 6] * sc, x[c * 8 + 7] * sc));
+  return inv;
 }
-
-// The element-wise maps of the paper's ablation (Table 6) on packed bf16 pairs: ReLU; the
-// identity needs no arithmetic at all.
-__device__ __forceinline__ uint4 relu_bf16x8(uint4 u) {
-  __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
-  const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-  for (int e = 0; e < 4; ++e) h[e] = __hmax2(h[e], z);
-  return u;
-}
-// feature_map_pair for any map: softmax as above; ReLU / identity element-wise (src may differ from dst)
+// ... normalised; src_half / dst_half point at the [rows x 64] box of this lane's column half
 __device__ __forceinline__ void feature_map_pair_any(const unsigned char* src_half, unsigned char* dst_half, int row, int phi) {
-  if (phi == RATTN_PHI_SOFTMAX) {
-    feature_map_pair(src_half, dst_half, row, (int)(threadIdx.x & 1));
-    return;
-  }
-  if (phi == RATTN_PHI_IDENTITY && src_half == dst_half) return;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const int off = row * 128 + ((c ^ (row & 7)) << 4);
-    const uint4 u = *reinterpret_cast<const uint4*>(src_half + off);
-    *reinterpret_cast<uint4*>(dst_half + off) = phi == RATTN_PHI_RELU ? relu_bf16x8(u) : u;
-  }
+  feature_map_half_row(src_half + row * 128, dst_half + row * 128, row, (int)(threadIdx.x & 1), phi, true);
 }
 
 // byte offset of 16-byte chunk c (0..15) of row r inside a swizzled [128 x 128] bf16 tile
@@ -209,6 +210,16 @@ __device__ __forceinline__ void apply_gain16(float (&x)[16], const float* __rest
   }
 }
 
+// 64 threads bring a head's two gain vectors into L1 (16 bytes each): consecutive units of a CTA are units of other heads, and
+// by the epilogue's own loads, in sixteen batches, each an L2 latency, the gains took a tenth of a long prefill's time.
+__device__ __forceinline__ void prefetch_gains(const float* g_swa, const float* g_rla, int head, int i) {
+  const float* g = i < 32 ? g_swa : g_rla;
+  if (!g) return;
+  float4 v;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(g + (size_t)head * 128 + 4 * (i & 31)));
+}
+
 // One [128 x 128] bf16 tile staged in shared memory (swizzled like a loaded tile) goes to
 // rows row0.. of matrix z of a tensor map: two 64-column boxes; rows past the end are clipped.
 __device__ __forceinline__ void store_tile(const UMap* tm, const unsigned char* tile, int row0, int z) {
@@ -220,6 +231,9 @@ __device__ __forceinline__ void store_tile(const UMap* tm, const unsigned char* 
 __device__ __forceinline__ void store_half(const UMap* tm, const unsigned char* half, int x, int row0, int z) {
   const int b = z / tm->H, h = z - b * tm->H;
   tma_store_4d(&tm->m, half, x, row0, h, b);
+}
+__device__ __forceinline__ void store_half(const CUtensorMap* tm, const unsigned char* half, int x, int row0, int z) {
+  tma_store_3d(tm, half, x, row0, z);
 }
 __device__ __forceinline__ void store_tile(const CUtensorMap* tm, const unsigned char* tile, int row0, int z) {
   tma_store_3d(tm, tile, 0, row0, z);
@@ -430,6 +444,74 @@ __device__ __forceinline__ float feature_map_row_any(unsigned char* tile, int r,
   return 1.f;
 }
 
+// ------------------------------------------------------------------------ work items
+// Of persistent kernels: a CTA's next item comes from a device-wide counter, so that CTAs that start late
+// (the SM was still running another kernel) or meet heavy items simply take fewer.  The loader warp draws it and
+// publishes it in a small ring that the other roles read in order; a slot is rewritten once every reader has read it.
+constexpr int SCHED_SLOTS = 4;
+struct SchedRing {
+  uint64_t full[SCHED_SLOTS], free_[SCHED_SLOTS];
+  int item[SCHED_SLOTS];
+};
+__device__ __forceinline__ void sched_init(SchedRing* r, int readers) {
+  for (int i = 0; i < SCHED_SLOTS; ++i) {
+    mbar_init(&r->full[i], 1);
+    mbar_init(&r->free_[i], readers);
+  }
+}
+// the loader warp's side: item n of this CTA is i (-1: there is none left)
+__device__ __forceinline__ bool sched_publish(SchedRing* r, int n, int i, volatile int* abort) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (use >= 1) { if (!mbar_wait_warp(&r->free_[slot], (use - 1) & 1, abort)) return false; }
+  if ((threadIdx.x & 31) == 0) {
+    r->item[slot] = i;
+    mbar_arrive(&r->full[slot]);
+  }
+  __syncwarp();
+  return true;
+}
+// ... drawn from the counter
+__device__ __forceinline__ bool sched_draw(SchedRing* r, int* counter, int n_items, int n, volatile int* abort, int* out) {
+  int i = 0;
+  if ((threadIdx.x & 31) == 0) i = atomicAdd(counter, 1);
+  i = __shfl_sync(0xffffffffu, i, 0);
+  *out = i < n_items ? i : -1;
+  return sched_publish(r, n, *out, abort);
+}
+// a reading thread's side
+__device__ __forceinline__ bool sched_read(SchedRing* r, int n, volatile int* abort, int* out) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (!mbar_wait(&r->full[slot], use & 1, abort)) return false;
+  *out = r->item[slot];
+  mbar_arrive(&r->free_[slot]);
+  return true;
+}
+// ... and a whole warp's (one of its lanes is counted)
+__device__ __forceinline__ bool sched_read_warp(SchedRing* r, int n, volatile int* abort, int* out) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+  if (!mbar_wait_warp(&r->full[slot], use & 1, abort)) return false;
+  *out = r->item[slot];
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&r->free_[slot]);
+  return true;
+}
+
+// Bounded wait (whole warp) until a progress word of another kernel reaches `need`; the TMA loads
+// that follow are ordered behind the acquiring read.
+__device__ __forceinline__ bool wait_published(const int* word, int need, volatile int* abort) {
+#pragma unroll 1
+  for (int it = 0; it < (1 << 20); ++it) {
+    if (ld_acquire_gpu(word) >= need) {
+      fence_proxy_async_all();
+      return true;
+    }
+    if ((it & 15) == 15 && *abort) return false;
+    __nanosleep(200);
+  }
+  *abort = 1;
+  return false;
+}
+
 // ------------------------------------------------------------------------ host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -490,8 +572,8 @@ inline bool make_row_map(CUtensorMap* m, const void* base, uint64_t T, uint64_t 
 // [n_mats, 128, 128] bf16 chunk states.  Modes without a linear branch keep none: the kernels
 // then never use the map, which is encoded over one matrix of `any` (some valid bf16 buffer of
 // at least 128 x 128 elements) so that it is well formed.
-inline bool make_state_map(CUtensorMap* m, const void* states, const void* any, uint64_t n_mats) {
-  return states ? make_map(m, states, 128, n_mats) : make_map(m, any, 128, 1);
+inline bool make_state_map(CUtensorMap* m, const void* states, const void* any, uint64_t n_mats, uint32_t box_rows = 128) {
+  return states ? make_map(m, states, 128, n_mats, box_rows) : make_map(m, any, 128, 1, box_rows);
 }
 
 }  // namespace tc

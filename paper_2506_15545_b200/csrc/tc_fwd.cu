@@ -1,85 +1,99 @@
 // Tensor-core forward for bf16, d = 128, window a multiple of 128: the chunk states of the linear
-// branch first (tc_state.cu), then the main kernel (tc_fwd2.cu).
+// branch first (tc_state.cu), then the main kernel (tc_fwd1.cu: single query tiles, two CTAs per SM;
+// tc_fwd2.cu: pairs of tiles).
 //
 // Chunk states S_[c] = sum_{c' < c} phi(K_c')^T V_c' (Eq. 2): one CTA per K/V head walks the chunks
-// with the sum in TMEM.  The main kernel reads S_[c] only for c = 2p - w/128 (one stored state serves
-// a pair of query tiles), so an inference forward stores every second state -- the paper's "states
-// stored every m chunks" with m = 2; a training forward stores all of them, because the backward
-// reads one per query tile.  When the caller asks for the decode state, the chain runs one chunk
-// further (tokens up to T - w, the rest of that chunk masked) and leaves its fp32 sum there.
-// The main kernel is launched so that it may start while the chain still runs (programmatic
+// with the sum in TMEM.  The pair kernel reads S_[c] only for c = 2p - w/128 (one stored state serves
+// a pair of query tiles), so before it an inference forward stores every second state -- the paper's
+// "states stored every m chunks" with m = 2; a training forward stores all of them, because the backward
+// reads one per query tile, and so does the single-tile kernel.  When the caller asks for the decode state,
+// the chain runs one chunk further (tokens up to T - w, the rest of that chunk masked) and leaves its fp32
+// sum there.  The main kernel is launched so that it may start while the chain still runs (programmatic
 // dependent launch): its window loops need no state, and it waits for the chain only before its
 // first state load.
 #include "tc_common.cuh"
 
 namespace rattn {
 
-// Query tiles of a work unit.  Pairs share their K/V tiles and half of the stored states, but where they do not fill
-// the GPU a tile of its own per CTA ends sooner (1 x 16/4 heads, T = 1111: 80 pairs or 144 tiles on 148 SMs).  With
-// single tiles every tile reads a stored state, in bf16, where of a pair the second takes the chunk in between exactly.
-// The element-wise maps' signed sums feel that rounding (of the output's bound of 2e-2 the last rounding alone takes
-// 1.6e-2 above 4), so they keep pairs.
-static bool single_tiles(const Args& a) {
-  int n_sm = 0;
-  if (sm_count(&n_sm) != cudaSuccess) return false;
-  const int n_qt = (a.T + tc::TILE - 1) / tc::TILE;
-  const bool states = a.mode == RATTN_MODE_RATTN && (a.state_in || n_qt - 1 - a.w / tc::TILE > 0);
-  return (long long)((n_qt + 1) / 2) * a.B * a.H_q < n_sm && (a.phi == RATTN_PHI_SOFTMAX || !states);
-}
-// whether a chunk-state kernel runs ahead of the main kernel
-static bool has_chain(const Args& a) {
-  const int n_kt = (a.Tk + tc::TILE - 1) / tc::TILE;
+// How a forward is run.
+struct Plan {
+  bool chain;        // a chunk-state kernel runs ahead of the main kernel
+  bool terms;        // ... as terms formed in parallel and their sums
+  bool progress;     // the main kernel takes the states as the chain publishes them
+  bool single;       // tc_fwd1.cu instead of tc_fwd2.cu
+  bool single_tiles; // tc_fwd2.cu with units of one tile
+  int n_steps;       // chunks of the chain
+};
+static Plan make_plan(const Args& a, int n_sm) {
+  Plan p;
+  const int n_kt = (a.Tk + tc::TILE - 1) / tc::TILE, n_qt = (a.T + tc::TILE - 1) / tc::TILE, wt = a.w / tc::TILE;
   const bool rla = a.mode == RATTN_MODE_RATTN, want_state = rla && a.state_out != nullptr;
-  const int n_delta = rla ? n_kt - 1 - a.w / tc::TILE : 0;
-  return n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
-}
-bool tc_forward_clears_status(const Args& a) {
-  int n_sm = 0;
-  if (sm_count(&n_sm) != cudaSuccess || has_chain(a)) return false;
-  const int n_qt = (a.T + tc::TILE - 1) / tc::TILE, per = single_tiles(a) ? 1 : 2;
-  return (long long)((n_qt + per - 1) / per) * a.B * a.H_q <= n_sm;
-}
-
-cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
-  // key-space tiles: a resumed sequence carries its w-token history in front of the chunk
-  const int n_kt = (a.Tk + tc::TILE - 1) / tc::TILE;
-  const int wt = a.w / tc::TILE, off = a.q_off / tc::TILE;
-  const bool rla = (a.mode == RATTN_MODE_RATTN);
+  const int n_kv = a.B * a.H_kv, n_q = a.B * a.H_q;
   // S_[c] for c = 1 .. n_delta: the states some query tile reads (S_[0] is the incoming state, zero
   // for a fresh sequence, where it is never read)
   const int n_delta = rla ? n_kt - 1 - wt : 0;
-  const int n_kv = a.B * a.H_kv;
-  const bool want_state = rla && a.state_out != nullptr;
-  bool chained = false;
+  p.n_steps = (want_state && (a.Tk > a.w || a.seq_lens)) ? n_delta + 1 : n_delta;
+  if (p.n_steps < 0) p.n_steps = 0;
+  p.chain = n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
+  const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
+  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one), the main
+  // kernel 30 ns per query tile and 12 ns per tile and key tile with all SMs at work, and no less than 40 us as far as this
+  // matters.  Where the chain of a long sequence on few heads would outlast the main kernel, its terms are formed in
+  // parallel (1 x 8/1 heads, T = 16384, w = 512: 202 -> 113 us).
+  const long long chain_ns = 2600ll * p.n_steps;
+  long long main_ns = (long long)n_qt * n_q * (30 + 12 * (wt + 1));
+  if (main_ns < 40000) main_ns = 40000;
+  p.terms = p.chain && a.rdelta && knob == 0 && n_kt >= kMinTermChunks && (long long)n_kv * a.n_chunks <= kMaxForwardTerms &&
+            chain_ns > main_ns;
+  // The single-tile kernel wins where the window loop is not everything: 1.05 - 1.28 times at w <= 768 (8 x 32/8 heads,
+  // T = 4397, w = 128, training: 748 -> 610 us; 4 x 16/16, T = 4096, w = 512: 215 -> 201), in training, where all states are
+  // stored and three outputs leave per tile, up to w = 1536; at w = 1408 and 2048 the pair kernel is 8 - 10 % faster in
+  // inference.  It needs every state, in bf16, where of a pair the second tile takes the chunk in between exactly: a chain
+  // that outlasts the main kernel by far decides against it (16 heads, T = 16384, w = 128), and the element-wise maps'
+  // signed sums feel the rounding (of the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
+  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) &&
+             (p.terms || 2 * chain_ns <= 3 * main_ns);
+  // The pair kernel where pairs do not fill the GPU: a tile of its own per CTA ends sooner.
+  p.single_tiles = !p.single && !rla && (long long)((n_qt + 1) / 2) * n_q < n_sm;
   // The main kernel can take the chunk states as the chain publishes them instead of waiting for the whole
   // chain.  That pays where the chain is long and leaves most SMs to the main kernel, which otherwise runs out
-  // of work that needs no state (config 3: 16 chains of 64 chunks); elsewhere publishing only slows the chain.
-  // With wide windows the units without a state are many and heavy already, and taking the units in sequence
-  // order (light ones first) costs more at the tail than the earlier start gains (measured from w = 1024 on).
-  bool progress = a.state_ready != nullptr;
-  if (progress) {
-    const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
-    int n_sm = 0;
-    const cudaError_t e = sm_count(&n_sm);
-    if (e != cudaSuccess) return e;
-    progress = knob == 1 || (knob == 0 && 4 * n_kv <= n_sm && n_kt >= 48 && wt <= 4);
-  }
+  // of work that needs no state (2 x 32/8 heads, T = 8192, w = 512: 422 -> 357 us; 1 x 32/8, T = 2048: 64 -> 58); elsewhere
+  // publishing only slows the chain.  With wide windows the units without a state are many and heavy already, and taking
+  // the units in sequence order (light ones first) costs more at the tail than the earlier start gains.
+  const bool few = 4 * n_kv <= n_sm && n_kt >= 48 && wt <= (p.single ? 8 : 4);
+  const bool fewer = p.single && 8 * n_kv <= n_sm && n_kt >= 16;
+  p.progress = p.chain && !p.terms && a.state_ready && (knob == 1 || (knob == 0 && (few || fewer)));
+  return p;
+}
+bool tc_forward_clears_status(const Args& a) {
+  int n_sm = 0;
+  if (sm_count(&n_sm) != cudaSuccess) return false;
+  const Plan p = make_plan(a, n_sm);
+  const int n_qt = (a.T + tc::TILE - 1) / tc::TILE, per = p.single || p.single_tiles ? 1 : 2;
+  return !p.chain && (long long)((n_qt + per - 1) / per) * a.B * a.H_q <= (p.single ? 2 : 1) * n_sm;
+}
+
+cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
+  int n_sm = 0;
+  cudaError_t e = sm_count(&n_sm);
+  if (e != cudaSuccess) return e;
+  const Plan p = make_plan(a, n_sm);
+  const int wt = a.w / tc::TILE, off = a.q_off / tc::TILE;       // a resumed sequence carries its w-token history in front
+  const int n_kv = a.B * a.H_kv;
+  const bool want_state = a.mode == RATTN_MODE_RATTN && a.state_out != nullptr;
   if (want_state && a.Tk <= a.w && !a.seq_lens && !a.zero_state) {
     // nothing has left the window yet
-    cudaError_t e = cudaMemsetAsync(a.state_out, 0, sizeof(float) * (size_t)n_kv * 128 * 128, s);
+    e = cudaMemsetAsync(a.state_out, 0, sizeof(float) * (size_t)n_kv * 128 * 128, s);
     if (e != cudaSuccess) return e;
   }
-  const int n_steps = (want_state && (a.Tk > a.w || a.seq_lens)) ? n_delta + 1 : n_delta;
-  const bool single = single_tiles(a);
-  if (has_chain(a)) {
+  if (p.chain) {
     StateLaunch L;
     L.x = a.k; L.y = a.v; L.out = a.chunk_state;
     L.x_heads = L.y_heads = a.H_kv; L.x_layout = L.y_layout = a.kv_layout;
     L.T = a.Tk; L.n_kv = n_kv; L.group = 1; L.n_chunks = a.n_chunks;
-    L.n_steps = n_steps > 0 ? n_steps : 0; L.first = 0; L.dir = +1; L.out_first = 1;
-    // the main kernel reads S_[c] for c = off + 2p - wt only
-    const int m = tuning(RATTN_TUNE_STATE_STRIDE);
-    const bool every = a.training || m == 1 || single;
+    L.n_steps = p.n_steps; L.first = 0; L.dir = +1; L.out_first = 1;
+    // the pair kernel reads S_[c] for c = off + 2p - wt only
+    const bool every = a.training || p.single || tuning(RATTN_TUNE_STATE_STRIDE) == 1;
     L.store_every = every ? 1 : 2;
     L.store_phase = every ? 0 : ((off + wt) & 1);
     L.handoff = want_state ? 1 : 0;
@@ -89,18 +103,17 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.seq_lens = a.seq_lens; L.kv_per_batch = a.H_kv;
     L.phi = a.phi;
     L.status = a.status; L.name = "tc_state_fwd";
-    L.ready = progress ? a.state_ready : nullptr;
-    L.delta = nullptr;
+    L.ready = p.progress ? a.state_ready : nullptr;
+    L.delta = p.terms ? a.rdelta : nullptr;
     L.h_split = 1;
     L.after_independent = false;
-    cudaError_t e = launch_tc_states(L, s);
+    e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;
-    chained = true;
   }
   Args m = a;
-  m.single_tiles = single;
-  if (!progress) m.state_ready = nullptr;            // the main kernel waits for the whole chain instead
-  return launch_tc_forward_main(m, s, chained);
+  m.single_tiles = p.single_tiles;
+  if (!p.progress) m.state_ready = nullptr;          // the main kernel waits for the whole chain instead
+  return p.single ? launch_tc_forward_single(m, s, p.chain) : launch_tc_forward_main(m, s, p.chain);
 }
 
 }  // namespace rattn

@@ -41,14 +41,11 @@ constexpr int F_SMEM = F_OFF_BAR + 512;
 constexpr int F_THREADS = 384;
 constexpr float LOG2E = 1.4426950408889634f;
 
-constexpr int SCHED_SLOTS = 4;
-constexpr int SCHED_READERS = 256 + 1 + 64;      // row threads, the MMA warp's lane 0, the converter threads
 
 struct FBars {
   uint64_t q_full[2], q_free[2], k_full[2], v_full[2], v_ready[2], k_free[2], v_free[2], x_full, x_free;
   uint64_t s_full[2], p_ready[2], o_ready[2], stash_done[2], phiq_ready[2], phik_ready[2], o_free[2], y_done[2], drain;
-  uint64_t sched_full[SCHED_SLOTS], sched_free[SCHED_SLOTS];
-  int sched_unit[SCHED_SLOTS];
+  SchedRing sched;
   uint32_t tmem_base;
   int abort;
 };
@@ -162,61 +159,19 @@ __device__ __forceinline__ void mma_pv(uint32_t d, uint32_t p_tmem, uint32_t v_b
   for (int k = 0; k < 8; ++k) mma_bf16_ts(d, p_tmem + 8 * k, b0 + kstep_mn(k), idesc, (acc || k > 0) ? 1u : 0u);
 }
 
-// ------------------------------------------------------------------------------ work units
-// The loader warp draws the CTA's next unit (from a device-wide counter, so that CTAs that start
-// late -- their SM was still running the chunk-state kernel -- simply take fewer units) and
-// publishes it in a small ring; the other roles read the ring in order.  A slot is rewritten
-// only after every reader has read it.
-__device__ __forceinline__ bool sched_next_producer(const FArgs& a, FBars* bars, int n, int* u_out) {
-  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
-  if (use >= 1) { if (!mbar_wait_warp(&bars->sched_free[slot], (use - 1) & 1, &bars->abort)) return false; }
-  int u = 0;
-  if (a.work_counter) {
-    if ((threadIdx.x & 31) == 0) u = atomicAdd(a.work_counter, 1);
-    u = __shfl_sync(0xffffffffu, u, 0);
-  } else {
-    u = blockIdx.x + n * gridDim.x;
-  }
-  if (u >= a.n_units) u = -1;
-  if ((threadIdx.x & 31) == 0) {
-    bars->sched_unit[slot] = u;
-    mbar_arrive(&bars->sched_full[slot]);
-  }
-  __syncwarp();
-  *u_out = u;
-  return true;
-}
-// every reading thread calls this; `arrives` says whether this thread is one of the counted readers
-__device__ __forceinline__ bool sched_next(FBars* bars, int n, bool arrives, int* u_out) {
-  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
-  if (!mbar_wait(&bars->sched_full[slot], use & 1, &bars->abort)) return false;
-  *u_out = bars->sched_unit[slot];
-  if (arrives) mbar_arrive(&bars->sched_free[slot]);
-  return true;
-}
-
 // ----------------------------------------------------------------------------- loader
-// Bounded wait (whole warp) until a progress word of another kernel reaches `need`; the TMA loads
-// that follow are ordered behind the acquiring read.
-__device__ __forceinline__ bool wait_published(const int* word, int need, volatile int* abort) {
-#pragma unroll 1
-  for (int it = 0; it < (1 << 20); ++it) {
-    if (ld_acquire_gpu(word) >= need) {
-      fence_proxy_async_all();
-      return true;
-    }
-    if ((it & 15) == 15 && *abort) return false;
-    __nanosleep(200);
-  }
-  *abort = 1;
-  return false;
-}
 __device__ bool fwd_loader(const FMaps& tm, const FArgs& a, unsigned char* smem, FBars* bars) {
   int kv_count = 0, cntU[2] = {0, 0}, cntX = 0;
   bool states_ready = (a.wait_for_states == 0);
   for (int n = 0;; ++n) {
     int u;
-    if (!sched_next_producer(a, bars, n, &u)) return false;
+    if (a.work_counter) {
+      if (!sched_draw(&bars->sched, a.work_counter, a.n_units, n, &bars->abort, &u)) return false;
+    } else {                                     // dealt round-robin
+      u = blockIdx.x + n * gridDim.x;
+      if (u >= a.n_units) u = -1;
+      if (!sched_publish(&bars->sched, n, u, &bars->abort)) return false;
+    }
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t[0] < 0) continue;                    // beyond this batch entry's length
@@ -270,10 +225,11 @@ __device__ bool fwd_convert(const FArgs& a, unsigned char* smem, FBars* bars, in
   int kv_count = 0;
   for (int n = 0;; ++n) {
     int u;
-    if (!sched_next(bars, n, true, &u)) return false;
+    if (!sched_read(&bars->sched, n, &bars->abort, &u)) return false;
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t[0] < 0) continue;
+    prefetch_gains(a.gamma_swa, a.gamma_rla, un.h, cid);
     for (int i = 0; i < un.n; ++i, ++kv_count) {
       const int st = kv_count & 1, use = kv_count >> 1;
       WAIT_OR_RETURN(bars->v_full[st], use & 1);
@@ -304,8 +260,7 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
 
   for (int n = 0;; ++n) {
     int u;
-    if (!sched_next(bars, n, (threadIdx.x & 31) == 0, &u)) return false;
-    u = __shfl_sync(0xffffffffu, u, 0);
+    if (!sched_read_warp(&bars->sched, n, &bars->abort, &u)) return false;
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t[0] < 0) continue;
@@ -457,7 +412,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 
   for (int n = 0;; ++n) {
     int u;
-    if (!sched_next(bars, n, true, &u)) return false;
+    if (!sched_read(&bars->sched, n, &bars->abort, &u)) return false;
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t[0] < 0) continue;
@@ -817,10 +772,7 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
     mbar_init(&bars->x_full, 1);
     mbar_init(&bars->x_free, 1);
     mbar_init(&bars->drain, 1);
-    for (int i = 0; i < SCHED_SLOTS; ++i) {
-      mbar_init(&bars->sched_full[i], 1);
-      mbar_init(&bars->sched_free[i], SCHED_READERS);
-    }
+    sched_init(&bars->sched, 256 + 1 + 64);      // row threads, the MMA warp's lane 0, the converter threads
     bars->abort = 0;
     fence_mbar_init();
   }

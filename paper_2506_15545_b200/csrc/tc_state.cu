@@ -63,6 +63,16 @@ struct StBars {
   int abort;
 };
 
+// steps of a head's chain: the caller's count, or -- variable-length batches -- what the entry's own length asks for; with
+// the hand-off the tokens from len - w on are still inside the window
+__device__ __forceinline__ int head_len(const StateArgs& a, int kv) {
+  return a.seq_lens ? min(a.T, a.seq_lens[kv / a.kv_per_batch]) : a.T;
+}
+__device__ __forceinline__ int head_steps(const StateArgs& a, int kv) {
+  if (!a.seq_lens) return a.n_steps;
+  const int len = head_len(a, kv), nd = max(0, (len + TILE - 1) / TILE - 1 - a.w / TILE);
+  return (a.handoff && len > a.w) ? nd + 1 : nd;
+}
 __device__ __forceinline__ bool stored_step(const StateArgs& a, int s) {
   const int o = a.out_first + a.dir * s;
   return o >= 0 && (o % a.store_every) == a.store_phase;
@@ -111,18 +121,10 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
-  // this head's chain: the caller's step count, or -- variable-length batches -- what the entry's own
-  // length asks for; with the hand-off the tokens from len - w on are still inside the window
-  int n_steps = a.delta ? 1 : a.n_steps, row_limit = INT_MAX;
-  if (!a.delta) {
-    const int len = a.seq_lens ? min(a.T, a.seq_lens[kv / a.kv_per_batch]) : a.T;
-    if (a.seq_lens) {
-      const int nd = max(0, (len + TILE - 1) / TILE - 1 - a.w / TILE);
-      n_steps = (a.handoff && len > a.w) ? nd + 1 : nd;
-    }
-    if (a.handoff) row_limit = len - a.w;
-  }
-  const bool has_init = (a.state_in != nullptr);
+  int n_steps = head_steps(a, kv);
+  const int row_limit = a.handoff ? head_len(a, kv) - a.w : INT_MAX;
+  if (a.delta) n_steps = unit - kv * a.n_split < n_steps ? 1 : 0;     // one term, or none beyond this head's length
+  const bool has_init = (a.state_in != nullptr) && !a.delta;        // of terms the incoming state is none
   const int n_items = n_steps * group;
   bool ok = true;
 
@@ -231,7 +233,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
               make_float4(x[c][4 * e], x[c][4 * e + 1], x[c][4 * e + 2], x[c][4 * e + 3]);
       }
     };
-    if (has_init || (a.final_out != nullptr && n_steps == 0)) {
+    if (has_init || (a.final_out != nullptr && n_steps == 0 && !a.delta)) {
       // the chain starts from the incoming state (zero without one): into the accumulator, into the
       // matrix in front of the first step's, and -- when no token leaves the window -- straight out
       float x[4][32];
@@ -293,37 +295,46 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   }
 }
 
-// Running sums of the terms left by the kernel above: state(s) = sum of the terms 0 .. s (each h_split matrices), as
-// bf16, row-major.  A pure stream (64 KB in per term matrix, 32 KB out per state): a thread owns one float4 of the matrix
-// and walks the terms with four loads in flight.  A warp covers 8 rows x 4 float4 columns, so that it reads 128-byte runs
-// of the column-major terms and writes whole 32-byte sectors of the row-major states.
-__global__ void __launch_bounds__(256) tc_state_sum_kernel(const float4* __restrict__ delta, uint2* __restrict__ out,
-                                                           int n_split, int h_split, int n_chunks, int out_first, int dir) {
+// Running sums of the terms left by the kernel above: state(s) = incoming state + the terms 0 .. s (each h_split matrices),
+// as bf16, row-major, and the last one in fp32 where the decode state is asked for.  A pure stream (64 KB in per term
+// matrix, 32 KB out per state): a thread owns one float4 of the matrix and walks the terms with eight loads in flight.  A
+// warp covers 8 rows x 4 float4 columns, so that it reads 128-byte runs of the column-major terms and writes whole 32-byte
+// sectors of the row-major states.
+__global__ void __launch_bounds__(256) tc_state_sum_kernel(const StateArgs a, uint2* __restrict__ out) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int kv = blockIdx.x >> 4, part = blockIdx.x & 15;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row = 32 * (part & 3) + 8 * (warp & 3) + (lane & 7), c4 = 8 * (part >> 2) + 4 * (warp >> 2) + (lane >> 3);
-  const int n = n_split * h_split;
-  const float4* src = delta + (size_t)kv * n * 4096 + c4 * 128 + row;
-  uint2* dst = out + ((size_t)kv * n_chunks + out_first) * 4096 + row * 32 + c4;
+  const int n = head_steps(a, kv) * a.h_split;
+  const float4* src = reinterpret_cast<const float4*>(a.delta) + (size_t)kv * a.n_split * a.h_split * 4096 + c4 * 128 + row;
+  uint2* dst = out + (size_t)kv * a.n_chunks * 4096 + row * 32 + c4;
+  const size_t at = (size_t)kv * 4096 + row * 32 + c4;              // of a row-major fp32 matrix, in float4
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  int left = h_split;
-  for (int i0 = 0; i0 < n; i0 += 4) {
-    float4 d[4];
+  auto store = [&](int s) {
+    if (stored_step(a, s))
+      dst[(ptrdiff_t)(a.out_first + a.dir * s) * 4096] = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
+  };
+  if (a.state_in) {
+    acc = reinterpret_cast<const float4*>(a.state_in)[at];
+    store(-1);
+  }
+  int left = a.h_split, s = 0;
+  for (int i0 = 0; i0 < n; i0 += 8) {
+    float4 d[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) d[k] = i0 + k < n ? __ldcg(src + (size_t)(i0 + k) * 4096) : acc;
+    for (int k = 0; k < 8; ++k) d[k] = i0 + k < n ? __ldcg(src + (size_t)(i0 + k) * 4096) : acc;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 8; ++k) {
       if (i0 + k >= n) break;
       acc.x += d[k].x; acc.y += d[k].y; acc.z += d[k].z; acc.w += d[k].w;
       if (--left == 0) {
-        *dst = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
-        dst += (ptrdiff_t)dir * 4096;
-        left = h_split;
+        store(s++);
+        left = a.h_split;
       }
     }
   }
+  if (a.final_out) reinterpret_cast<float4*>(a.final_out)[at] = acc;
 }
 
 }  // namespace
@@ -366,8 +377,7 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   count_launches(1);
   if (L.delta) {
     KernelTimer kt("tc_state_sum", s);
-    e = launch_pdl(tc_state_sum_kernel, dim3((unsigned)L.n_kv * 16), dim3(256), 0, s, true, reinterpret_cast<const float4*>(L.delta),
-                   reinterpret_cast<uint2*>(L.out), L.n_steps, a.h_split, L.n_chunks, L.out_first, L.dir);
+    e = launch_pdl(tc_state_sum_kernel, dim3((unsigned)L.n_kv * 16), dim3(256), 0, s, true, a, reinterpret_cast<uint2*>(L.out));
     if (e != cudaSuccess) return e;
     count_launches(1);
   }
