@@ -321,7 +321,7 @@ constexpr int DQ_SMEM = DQ_OFF_BAR + 384;
 constexpr int DQ_THREADS = 320;            // 2 row groups, MMA warp, loader warp
 
 struct DqBars {
-  uint64_t qg_full, kv_full[2], kv_free[2], s_full, ds_full, phik_ready, o_done, acc_free, q_read, drain;
+  uint64_t qg_full, kv_full[2], kv_free[2], s_full, ds_full, phik_ready, o_done, g_free, acc_free, q_read, drain;
   SchedRing sched;
   uint32_t tmem_base;
   int abort;
@@ -358,8 +358,7 @@ struct DqMaps {
 };
 
 __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, int n_items, int n_qt) {
-  int kc = 0, n = 0, co = 0;                               // ring uses, items, o_done completions of the items so far
-  int co_window = 0;                                       // the completion that ends the previous item's window products
+  int kc = 0, n = 0;                                       // ring uses, items so far
   for (;; ++n) {
     int idx;
     if (!sched_draw(&bars->sched, a.counter, n_items, n, &bars->abort, &idx)) return false;
@@ -380,15 +379,12 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
       WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);      // and its dQ, staged there, has left
     }
     load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->qg_full, it.q0, it.bh_q);
-    // g_s: its one buffer is free once the previous item's window products have completed (the residual part
-    // reads g_r).  o_done completes twice for an item with a residual part, after the window products and at the
-    // end, once otherwise; it is the first of them that is awaited here.  Awaiting the second alone would not be
-    // safe: a parity wait tells a completion only from the one right before it, and while the first is still
-    // outstanding the parity of the second reads as already reached.  (The completions before the first are
-    // known to be over: acc_free of item n - 2 above follows them.)
-    if (n >= 1) WAIT_OR_RETURN_W(bars->o_done, co_window & 1);
-    co_window = co;
-    co += it.has_rla ? 2 : 1;
+    // g_s: its one buffer is free once the previous item's window products have completed (the residual part reads
+    // g_r).  A barrier of its own, one completion per item: a parity wait tells a completion only from the ones next to
+    // it, and of o_done, which completes twice for an item with a residual part, the loader may come too early for the
+    // second (the first still outstanding: the parity reads as reached) as well as too late for the first (the second
+    // over already: the wait would be for the next item's, which needs this load).
+    if (n >= 1) WAIT_OR_RETURN_W(bars->g_free, (n - 1) & 1);
     load_tile(smem + DQ_OFF_G, &tm.gs, &bars->qg_full, it.q0, it.bh_q);
     for (int i = 0; i < it.n_kt; ++i, ++kc) {
       if (!ring_wait()) return false;
@@ -440,6 +436,7 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
       if (!(it.has_rla && i == it.n_kt - 1)) mma_commit(&bars->kv_free[st]);
       // the next tile's scores follow these products in the tensor pipe, which runs in issue order
     }
+    mma_commit(&bars->g_free);                             // the window products are done with g_s
     if (it.has_rla) {
       const int xs = kc & 1;                               // slot of g_r and the stored state
       const uint32_t sG2 = sV + xs * TILE_BYTES, sSt = sK + xs * TILE_BYTES;
@@ -675,6 +672,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     mbar_init(&bars->ds_full, 256);
     mbar_init(&bars->phik_ready, 256);
     mbar_init(&bars->o_done, 1);
+    mbar_init(&bars->g_free, 1);
     mbar_init(&bars->acc_free, 128);
     mbar_init(&bars->q_read, 1);
     mbar_init(&bars->drain, 1);
