@@ -44,13 +44,15 @@ constexpr int F_NS = 5;                          // ring slots: a half tile of K
 constexpr int F_OFF_Q = 0;
 constexpr int F_OFF_RING = TILE_BYTES;
 constexpr int F_OFF_BAR = F_OFF_RING + F_NS * HT_BYTES;
-constexpr int F_OFF_EX = F_OFF_BAR + 320;        // one word per row, between its two threads
-constexpr int F_SMEM = F_OFF_EX + TILE * 4;      // 115,520 bytes: two CTAs share the SM's 228 KB
+constexpr int F_OFF_EX = F_OFF_BAR + 384;        // one word per row, between its two threads
+constexpr int F_SMEM = F_OFF_EX + TILE * 4;      // 115,584 bytes: two CTAs share the SM's 228 KB
 constexpr int F_THREADS = 384;                   // 8 row warps, MMA, loader, 2 converters
 constexpr float LOG2E = 1.4426950408889634f;
 
 struct FBars {
-  uint64_t full[F_NS], free_[F_NS], v_ready[F_NS];     // ring slots: landed, consumed; V re-encoded
+  // Ring slots: K or a state landed, V landed, consumed, V re-encoded.  V has a barrier of its own because the converters
+  // follow the V uses alone: a wait by parity cannot skip a phase (two loads in flight may land in either order).
+  uint64_t full[F_NS], v_full[F_NS], free_[F_NS], v_ready[F_NS];
   uint64_t q_full, q_free, s_full[2], p_ready[2], pv_done, o_ready, stash_done, phi_ready, o_free, drain;
   SchedRing sched;
   uint32_t tmem_base;
@@ -131,7 +133,16 @@ __device__ __forceinline__ int unit_uses(const Unit& un) { return 4 * un.n + (un
 struct Ring {
   int base = 0;                                  // uses of the units before
   __device__ __forceinline__ int slot(int pos) const { return (base + pos) % F_NS; }
-  __device__ __forceinline__ uint32_t phase(int pos) const { return (uint32_t)((base + pos) / F_NS) & 1u; }
+  __device__ __forceinline__ uint32_t phase(int pos) const { return (uint32_t)((base + pos) / F_NS) & 1u; }   // of free_
+};
+// full, v_full and v_ready complete once per use of their own kind: parity of the next such use of each slot
+struct UsePhase {
+  uint32_t bits = 0;
+  __device__ __forceinline__ uint32_t take(int st) {
+    const uint32_t p = (bits >> st) & 1u;
+    bits ^= 1u << st;
+    return p;
+  }
 };
 
 #define WAIT_OR_RETURN(bar, parity) \
@@ -177,24 +188,24 @@ __device__ bool fwd_loader(const FMaps& tm, const FArgs& a, unsigned char* smem,
       if (use >= 1) WAIT_OR_RETURN_W(bars->free_[ring.slot(pos)], (use - 1) & 1);
       return true;
     };
-    auto half_tile = [&](int pos, const UMap* map, int s) -> bool {
+    auto half_tile = [&](int pos, const UMap* map, uint64_t* landed, int s) -> bool {
       if (!slot_wait(pos)) return false;
       const int st = ring.slot(pos);
-      mbar_arrive_expect_tx(&bars->full[st], HT_BYTES);
-      load_half_tile(smem + F_OFF_RING + st * HT_BYTES, map, &bars->full[st], (un.t - (s >> 1)) * TILE + 64 * (s & 1), un.bh_kv);
+      mbar_arrive_expect_tx(&landed[st], HT_BYTES);
+      load_half_tile(smem + F_OFF_RING + st * HT_BYTES, map, &landed[st], (un.t - (s >> 1)) * TILE + 64 * (s & 1), un.bh_kv);
       return true;
     };
     // K0 may come while the previous unit's output still occupies the Q buffer
-    if (!half_tile(0, &tm.k, 0)) return false;
+    if (!half_tile(0, &tm.k, bars->full, 0)) return false;
     if (cu >= 1) WAIT_OR_RETURN_W(bars->q_free, (cu - 1) & 1);
     mbar_arrive_expect_tx(&bars->q_full, TILE_BYTES);
     load_tile(smem + F_OFF_Q, &tm.q, &bars->q_full, (un.t - a.off) * TILE, un.bh_q);
     ++cu;
-    if (!half_tile(1, &tm.k, 1)) return false;
+    if (!half_tile(1, &tm.k, bars->full, 1)) return false;
     for (int s = 0; s < L; ++s) {                // V(s) and K(s+2), in ring order
-      if (!(un.rla && s == L - 3) && !half_tile(pos_v(s, L, un.rla), &tm.v, s)) return false;
-      if (un.rla && s == L - 4 && !half_tile(pos_v(s + 1, L, un.rla), &tm.v, s + 1)) return false;
-      if (s + 2 < L && !half_tile(pos_k(s + 2, L, un.rla), &tm.k, s + 2)) return false;
+      if (!(un.rla && s == L - 3) && !half_tile(pos_v(s, L, un.rla), &tm.v, bars->v_full, s)) return false;
+      if (un.rla && s == L - 4 && !half_tile(pos_v(s + 1, L, un.rla), &tm.v, bars->v_full, s + 1)) return false;
+      if (s + 2 < L && !half_tile(pos_k(s + 2, L, un.rla), &tm.k, bars->full, s + 2)) return false;
     }
     if (un.has_state) {
       if (a.state_ready) {
@@ -220,6 +231,7 @@ __device__ bool fwd_loader(const FMaps& tm, const FArgs& a, unsigned char* smem,
 // -------------------------------------------------------------------------- V re-encoding
 __device__ bool fwd_convert(const FArgs& a, unsigned char* smem, FBars* bars, int cid) {
   Ring ring;
+  UsePhase vf;
   for (int n = 0;; ++n) {
     int u;
     if (!sched_read(&bars->sched, n, &bars->abort, &u)) return false;
@@ -229,8 +241,8 @@ __device__ bool fwd_convert(const FArgs& a, unsigned char* smem, FBars* bars, in
     prefetch_gains(a.gamma_swa, a.gamma_rla, un.h, cid);
     const int L = 2 * un.n;
     for (int s = 0; s < L; ++s) {
-      const int pos = pos_v(s, L, un.rla), st = ring.slot(pos);
-      WAIT_OR_RETURN(bars->full[st], ring.phase(pos));
+      const int st = ring.slot(pos_v(s, L, un.rla));
+      WAIT_OR_RETURN(bars->v_full[st], vf.take(st));
       unsigned char* tile = smem + F_OFF_RING + st * HT_BYTES;
 #pragma unroll 4
       for (int c = cid; c < HT_BYTES / 16; c += 64) {
@@ -250,21 +262,11 @@ __device__ bool fwd_convert(const FArgs& a, unsigned char* smem, FBars* bars, in
 }
 
 // ----------------------------------------------------------------------------- MMA warp
-// v_ready of a slot completes once per V use of it: its phase counts V uses only.
-struct VPhase {
-  uint32_t bits = 0;                             // parity of the next V use of each slot
-  __device__ __forceinline__ uint32_t take(int st) {
-    const uint32_t p = (bits >> st) & 1u;
-    bits ^= 1u << st;
-    return p;
-  }
-};
-
 __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32_t tmem) {
   const uint32_t sQ = smem_u32(smem + F_OFF_Q), sR = smem_u32(smem + F_OFF_RING);
   const uint32_t tS = tmem, tO = tmem + 128;
   Ring ring;
-  VPhase vp;
+  UsePhase kp, vp;                               // K and state uses, V uses
   int cu = 0, cs = 0, cr = 0;                    // units, score hand-overs per buffer, residual units so far
 
   for (int n = 0;; ++n) {
@@ -283,8 +285,8 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
     WAIT_OR_RETURN_W(bars->q_full, cu & 1);
 #pragma unroll
     for (int s = 0; s < 2; ++s) {                // a unit with a residual part has at least four steps
-      const int pos = pos_k(s, L, un.rla);
-      WAIT_OR_RETURN_W(bars->full[ring.slot(pos)], ring.phase(pos));
+      const int kst = ring.slot(pos_k(s, L, un.rla));
+      WAIT_OR_RETURN_W(bars->full[kst], kp.take(kst));
       tc_fence_after();
       scores(s, false);
     }
@@ -295,8 +297,8 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
       const int vst = ring.slot(pos_v(s, L, un.rla));
       WAIT_OR_RETURN_W(bars->v_ready[vst], vp.take(vst));
       if (s + 2 < L) {
-        const int pos = pos_k(s + 2, L, un.rla);
-        WAIT_OR_RETURN_W(bars->full[ring.slot(pos)], ring.phase(pos));
+        const int kst = ring.slot(pos_k(s + 2, L, un.rla));
+        WAIT_OR_RETURN_W(bars->full[kst], kp.take(kst));
       }
       if (s == 0 && cu >= 1) WAIT_OR_RETURN_W(bars->o_free, (cu - 1) & 1);   // the previous unit has read O
       WAIT_OR_RETURN_W(bars->p_ready[s & 1], (cs + (s >> 1)) & 1);
@@ -311,6 +313,7 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
     // ---- residual branch ---------------------------------------------------------------
     if (un.rla) {
       const int ka = ring.slot(2 * L - 4), kb = ring.slot(2 * L - 3), va = ring.slot(2 * L - 2), vb = ring.slot(2 * L - 1);
+      const int sa = ring.slot(2 * L), sb = ring.slot(2 * L + 1);
       WAIT_OR_RETURN_W(bars->phi_ready, cr & 1);
       tc_fence_after();
       mma_k_kh(tS, sQ, sR + ka * HT_BYTES);                                  // phi(Q) phi(K_c)^T, lower 64 keys
@@ -319,12 +322,12 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
       mma_k_kh(tS + 64, sQ, sR + kb * HT_BYTES);                             // upper 64 keys
       mma_commit(&bars->s_full[1]);
       mma_commit(&bars->free_[kb]);
-      if (un.has_state) WAIT_OR_RETURN_W(bars->full[ring.slot(2 * L)], ring.phase(2 * L));
+      if (un.has_state) WAIT_OR_RETURN_W(bars->full[sa], kp.take(sa));
       WAIT_OR_RETURN_W(bars->stash_done, cr & 1);
       tc_fence_after();
       if (un.has_state) {
-        mma_q_state(tO, sQ, 0, sR + ring.slot(2 * L) * HT_BYTES, false);     // phi(Q) S_[c], features 0 .. 63
-        mma_commit(&bars->free_[ring.slot(2 * L)]);
+        mma_q_state(tO, sQ, 0, sR + sa * HT_BYTES, false);     // phi(Q) S_[c], features 0 .. 63
+        mma_commit(&bars->free_[sa]);
       }
       WAIT_OR_RETURN_W(bars->p_ready[0], cs & 1);
       tc_fence_after();
@@ -335,10 +338,10 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
       mma_pv(tO, tS + 64, sR + vb * HT_BYTES, true);
       mma_commit(&bars->free_[vb]);
       if (un.has_state) {
-        WAIT_OR_RETURN_W(bars->full[ring.slot(2 * L + 1)], ring.phase(2 * L + 1));
+        WAIT_OR_RETURN_W(bars->full[sb], kp.take(sb));
         tc_fence_after();
-        mma_q_state(tO, sQ, 1, sR + ring.slot(2 * L + 1) * HT_BYTES, true);  // features 64 .. 127
-        mma_commit(&bars->free_[ring.slot(2 * L + 1)]);
+        mma_q_state(tO, sQ, 1, sR + sb * HT_BYTES, true);  // features 64 .. 127
+        mma_commit(&bars->free_[sb]);
       }
       mma_commit(&bars->o_ready);
       ++cs;
@@ -682,6 +685,7 @@ tc_fwd1_kernel(const __grid_constant__ FMaps tm, FArgs a) {
   if (tid == 0) {
     for (int i = 0; i < F_NS; ++i) {
       mbar_init(&bars->full[i], 1);
+      mbar_init(&bars->v_full[i], 1);
       mbar_init(&bars->free_[i], 1);
       mbar_init(&bars->v_ready[i], 64);
     }
