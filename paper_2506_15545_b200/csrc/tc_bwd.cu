@@ -373,11 +373,10 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
     // item the loader gets here while that item's Q and g_s are still in flight.
     if (n >= 1) WAIT_OR_RETURN_W(bars->qg_full, (n - 1) & 1);
     mbar_arrive_expect_tx(&bars->qg_full, 2 * TILE_BYTES);
-    // Q into the buffer last used two items ago: free once that item's epilogue has left it
-    if (n >= 2) {
-      WAIT_OR_RETURN_W(bars->acc_free, (n - 2) & 1);
-      WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);      // and its dQ, staged there, has left
-    }
+    // Q into the buffer last used two items ago: free once its dQ, staged there by that item's epilogue, has left.  (Not
+    // acc_free as well: the item in between may have completed that barrier a second time before this warp looks, and
+    // then the wait, which sees the parity alone, would be for a completion that needs this load.)
+    if (n >= 2) WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);
     load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->qg_full, it.q0, it.bh_q);
     // g_s: its one buffer is free once the previous item's window products have completed (the residual part reads
     // g_r).  A barrier of its own, one completion per item: a parity wait tells a completion only from the ones next to
@@ -886,6 +885,8 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
     for (int n = 0; n < pl.N; ++n) {
       const int st = (seq0 + n) % KV_NS, use = (seq0 + n) / KV_NS, slot = (gi0 + n) & 1;
       const uint32_t sQh = sStage + st * TILE_BYTES, sGh = sQh + HT_BYTES;
+      // the reverse state's use of this slot is over (this warp has not followed it, and may not skip a phase)
+      if (n == KV_NS - 1 && pl.has_inter) WAIT_OR_RETURN_W(bars->acc_done[st], (use - 1) & 1);
       WAIT_OR_RETURN_W(bars->full[st], use & 1);
       if (pl.is_r(n)) {
         WAIT_OR_RETURN_W(bars->phiq_ready[slot], (slot ? cq1 : cq0) & 1);
@@ -998,6 +999,9 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
     const bool is_r = pl.is_r(n);
     const int i = pl.qtile(n), hf = pl.half(n);
     unsigned char* sQh = smem + KV_OFF_STAGE + st * TILE_BYTES;
+    // A group sees every second item, so it follows a slot's uses with gaps, and a wait by parity cannot skip a phase:
+    // the previous use of the slot must be known to be over.
+    if (use >= 1) WAIT_OR_RETURN(bars->acc_done[st], (use - 1) & 1);
     WAIT_OR_RETURN(bars->full[st], use & 1);
     if (is_r) {
       // phi(Q_h) in place: 64 rows, two threads per row
