@@ -734,29 +734,29 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
 //                   after the row group has overwritten them with bf16 P^T and dS^T:
 //                   dV += P^T g_h, dK += dS^T Q_h with the A operand read from TMEM
 //   row group       P^T = exp2(S^T * scale_log2 - lse2[q]), dS^T = P^T (dP^T scale - D[q] scale)
-// The residual items run first and leave dphi_k in the dK accumulator; row group 0 then folds
+// The residual items run first and leave dphi_k in the dK accumulator; the row groups then fold
 // the feature-map Jacobian into it (dK := phi(k) (dphi_k - <dphi_k, phi(k)>)) and the window
 // items accumulate on top.
-constexpr int KV_NS = 3;                                   // item stages
+constexpr int KV_NS = 4;                                   // item stages (the last two of a key tile stage its dV and dK)
 constexpr int KV_OFF_K = 0;
 constexpr int KV_OFF_V = 1 * TILE_BYTES;
-constexpr int KV_OFF_KPHI = 2 * TILE_BYTES;                // phi(K_j); stages dK at the end of an item
-constexpr int KV_OFF_OUT = 3 * TILE_BYTES;                 // stages dV at the end of an item
-constexpr int KV_OFF_STAGE = 4 * TILE_BYTES;               // KV_NS x [Q_h 16 KB | g_h 16 KB]
+constexpr int KV_OFF_KPHI = 2 * TILE_BYTES;                // phi(K_j)
+constexpr int KV_OFF_STAGE = 3 * TILE_BYTES;               // KV_NS x [Q_h 16 KB | g_h 16 KB]
 constexpr int KV_OFF_STAT = KV_OFF_STAGE + KV_NS * TILE_BYTES;   // KV_NS x (lse2[64], D*scale[64]) fp32
 constexpr int KV_OFF_BAR = KV_OFF_STAT + KV_NS * 512;
-constexpr int KV_SMEM = KV_OFF_BAR + 384;
+constexpr int KV_OFF_EX = KV_OFF_BAR + 384;                // one word per row, between the two row groups
+constexpr int KV_SMEM = KV_OFF_EX + TILE * 4;              // 232,320 bytes of the 232,448 a CTA may have
 constexpr int KV_THREADS = 352;                            // 2 row groups, score warp, loader warp, accumulate warp
 
 struct KvBars {
   uint64_t kv_full, kphi_ready, full[KV_NS], acc_done[KV_NS], s_full[2], p_ready[2], phiq_ready[2],
-      r_acc_done, fold_done, all_done, acc_free, out_read, drain, drain2;
+      r_acc_done, fold_done, all_done, acc_free, kv_free, out_staged, drain, drain2;
   SchedRing sched;
   uint32_t tmem_base;
   int abort;
 };
 
-static_assert(sizeof(KvBars) <= KV_SMEM - KV_OFF_BAR, "barriers");
+static_assert(sizeof(KvBars) <= KV_OFF_EX - KV_OFF_BAR, "barriers");
 
 struct KvMaps {
   UMap k, v, qh, dk, dv;        // the caller's tensors (either head layout)
@@ -805,25 +805,39 @@ struct KvCount {
 
 __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* smem, KvBars* bars, int n_items) {
   KvCount c = {0, 0, 0, 0};
+  // dV and dK of a key tile are staged in the ring slots of its last two items, which the next key tile uses third and
+  // fourth.  This warp stores them, so that nobody else has to wait for the stores to have read the slots out: as soon as
+  // they are staged and before the first of the slots is refilled.
+  int out_row = 0, out_z = 0, out_seq = -1;                 // the key tile whose gradients are still to go
+  auto store_out = [&]() -> bool {
+    WAIT_OR_RETURN_W(bars->out_staged, (c.it - 1) & 1);
+    if ((threadIdx.x & 31) == 0) {
+      store_tile(&tm.dv, smem + KV_OFF_STAGE + out_seq % KV_NS * TILE_BYTES, out_row, out_z);
+      store_tile(&tm.dk, smem + KV_OFF_STAGE + (out_seq + 1) % KV_NS * TILE_BYTES, out_row, out_z);
+      tma_store_commit();
+      tma_store_wait_read();
+    }
+    __syncwarp();
+    out_seq = -1;
+    return true;
+  };
   for (;; ++c.it) {
     int idx;
     if (!sched_draw(&bars->sched, a.counter, n_items, c.it, &bars->abort, &idx)) return false;
     if (idx < 0) break;
     const KvPlan pl = kv_plan(a, idx);
     const int j0 = pl.j * TILE;
-    // K_j, V_j replace the previous key tile's once every product that read them has completed
-    if (c.it >= 1) WAIT_OR_RETURN_W(bars->all_done, (c.it - 1) & 1);
+    // K_j, V_j replace the previous key tile's once its last scores have been formed (the residual products that read V_j
+    // come before those): they arrive while its last items and its epilogue are still under way
+    if (c.it >= 1) WAIT_OR_RETURN_W(bars->kv_free, (c.it - 1) & 1);
     mbar_arrive_expect_tx(&bars->kv_full, 2 * TILE_BYTES);
     load_tile(smem + KV_OFF_K, &tm.k, &bars->kv_full, j0, pl.bh_kv);
     load_tile(smem + KV_OFF_V, &tm.v, &bars->kv_full, j0, pl.bh_kv);
-    // dK of the previous key tile left through the ring slot this tile uses third: its store must
-    // have read the slot out first
-    const int gate_seq = c.seq + 2;
     auto ring = [&](int& st) -> bool {                     // next ring slot, once its previous user is consumed
       st = c.seq % KV_NS;
       const int use = c.seq / KV_NS;
       if (use >= 1) WAIT_OR_RETURN_W(bars->acc_done[st], (use - 1) & 1);
-      if (c.it >= 1 && c.seq == gate_seq) WAIT_OR_RETURN_W(bars->out_read, (c.it - 1) & 1);
+      if (c.seq == out_seq + KV_NS && out_seq >= 0 && !store_out()) return false;
       ++c.seq;
       return true;
     };
@@ -852,7 +866,15 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
         bulk_load_1d(stat + 64, a.dscp + (size_t)z * a.t_pad + row, 256, &bars->full[st]);
       }
     }
+    if (out_seq >= 0 && !store_out()) return false;        // a key tile of two ring uses has not come to those slots
+    if (!a.part) {
+      out_row = j0;
+      out_z = pl.bh_kv;
+      out_seq = c.seq - 2;
+    }
   }
+  if (out_seq >= 0 && !store_out()) return false;
+  if ((threadIdx.x & 31) == 0) tma_store_wait();           // the last store has completed
   return true;
 }
 
@@ -871,13 +893,13 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
   const uint32_t tS0 = tmem + 256, tP0 = tmem + 320;
   KvCount c = {0, 0, 0, 0};
   int cq0 = 0, cq1 = 0;                                    // phi(Q_h) hand-overs per TMEM slot
+  int seq_m1 = -1, seq_m2 = -1;                            // ring uses of the last two items (the previous key tile's at first)
 
   for (;; ++c.it) {
     int idx;
     if (!sched_read_warp(&bars->sched, c.it, &bars->abort, &idx)) return false;
     if (idx < 0) break;
     const KvPlan pl = kv_plan(a, idx);
-    // K_j, V_j have landed (which also means every product of the previous key tile has completed)
     WAIT_OR_RETURN_W(bars->kv_full, c.it & 1);
     if (pl.n_R > 0) WAIT_OR_RETURN_W(bars->kphi_ready, c.cr & 1);
     if (pl.has_inter) ++c.seq;                             // the reverse state's ring slot (accumulate warp)
@@ -888,18 +910,18 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
       // the reverse state's use of this slot is over (this warp has not followed it, and may not skip a phase)
       if (n == KV_NS - 1 && pl.has_inter) WAIT_OR_RETURN_W(bars->acc_done[st], (use - 1) & 1);
       WAIT_OR_RETURN_W(bars->full[st], use & 1);
+      if (seq_m2 >= 0) WAIT_OR_RETURN_W(bars->acc_done[seq_m2 % KV_NS], (seq_m2 / KV_NS) & 1);   // the TMEM slot's previous item is over
+      seq_m2 = seq_m1;
+      seq_m1 = seq0 + n;
       if (pl.is_r(n)) {
         WAIT_OR_RETURN_W(bars->phiq_ready[slot], (slot ? cq1 : cq0) & 1);
         if (slot) ++cq1; else ++cq0;
-      }
-      if (n >= 2) {                                        // the slot's previous item has been accumulated
-        const int st2 = (seq0 + n - 2) % KV_NS, use2 = (seq0 + n - 2) / KV_NS;
-        WAIT_OR_RETURN_W(bars->acc_done[st2], use2 & 1);
       }
       tc_fence_after();
       mma_k_kh(tS0 + 128 * slot, pl.is_r(n) ? sKphi : sK, sQh);   // S^T  = K Q_h^T   (phi(K) phi(Q_h)^T)
       mma_k_kh(tP0 + 128 * slot, sV, sGh);                         // dP^T = V g_h^T
       mma_commit(&bars->s_full[slot]);
+      if (n == pl.N - 1) mma_commit(&bars->kv_free);
     }
     c.seq += pl.N;
     c.gi += pl.N;
@@ -975,21 +997,14 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   if (!sched_read(&bars->sched, cnt.it, &bars->abort, &idx)) return false;
   if (idx < 0) break;
   const KvPlan pl = kv_plan(a, idx);
-  const int bh_kv = pl.bh_kv;
-  if (gg < 2) {
+  if (pl.n_R > 0) {
+    // phi(K_j) into its own tile: 256 threads, two per row.  (Only here do these threads follow kv_full: without residual
+    // items the next key tile's K and V may land before they look.)
     WAIT_OR_RETURN(bars->kv_full, cnt.it & 1);
-    if (pl.n_R > 0) {
-      // phi(K_j) into its own tile: 256 threads, two per row
-      const int t2 = gg * 128 + r, row = t2 >> 1, hf = t2 & 1;
-      feature_map_pair_any(smem + KV_OFF_K + hf * HALF_BYTES, smem + KV_OFF_KPHI + hf * HALF_BYTES, row, a.phi);
-      fence_proxy_async_smem();
-      mbar_arrive(&bars->kphi_ready);
-    }
-    // the previous key tile's dK has long left its ring slot by now: tell the loader
-    if (gg == 0 && r == 0 && cnt.it >= 1) {
-      tma_store_wait_read();
-      mbar_arrive(&bars->out_read);
-    }
+    const int t2 = gg * 128 + r, row = t2 >> 1, hf = t2 & 1;
+    feature_map_pair_any(smem + KV_OFF_K + hf * HALF_BYTES, smem + KV_OFF_KPHI + hf * HALF_BYTES, row, a.phi);
+    fence_proxy_async_smem();
+    mbar_arrive(&bars->kphi_ready);
   }
   const int seq0 = cnt.seq + (pl.has_inter ? 1 : 0), gi0 = cnt.gi;
 
@@ -1079,68 +1094,62 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
     tc_fence_before();
     mbar_arrive(&bars->p_ready[g]);
 
-    if (gg == 0 && is_r && n + 2 >= pl.n_R) {                   // group 0's last residual item of this key tile
-      // end of the residual items: dK := dphi_k through the feature map's gradient
-      // (softmax map: phi(k) (dphi_k - <dphi_k, phi(k)>))
+    if (is_r && n + 2 >= pl.n_R) {                              // this group's last residual item of this key tile
+      // end of the residual items: dK := dphi_k through the feature map's gradient (softmax map:
+      // phi(k) (dphi_k - <dphi_k, phi(k)>)), each group half of the columns: every window item waits for it
       WAIT_OR_RETURN(bars->r_acc_done, cnt.cr & 1);
       tc_fence_after();
-      const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
-      float dot = 0.f;
-      if (soft) {
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          float df[32];
-          tmem_ld32(tK + 32 * c, df);
-          tmem_wait_ld();
-#pragma unroll
-          for (int cc = 0; cc < 4; ++cc) {
-            const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 4 * c + cc));
-            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float2 f = __bfloat1622float2(h2[e]);
-              dot += f.x * df[8 * cc + 2 * e] + f.y * df[8 * cc + 2 * e + 1];
-            }
-          }
-        }
-      }
       // the identity map leaves dphi_k as it is
       if (a.phi != RATTN_PHI_IDENTITY) {
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          float df[32];
-          tmem_ld32(tK + 32 * c, df);
-          tmem_wait_ld();
+        const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
+        float df[2][32];
+        tmem_ld32(tK + 64 * g, df[0]);
+        tmem_ld32(tK + 64 * g + 32, df[1]);
+        tmem_wait_ld();
+        float dot = 0.f;
+        if (soft) {
 #pragma unroll
-          for (int cc = 0; cc < 4; ++cc) {
-            const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 4 * c + cc));
+          for (int cc = 0; cc < 8; ++cc) {
+            const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 8 * g + cc));
             const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const float2 f = __bfloat1622float2(h2[e]);
-              if (soft) {
-                df[8 * cc + 2 * e] = f.x * (df[8 * cc + 2 * e] - dot);
-                df[8 * cc + 2 * e + 1] = f.y * (df[8 * cc + 2 * e + 1] - dot);
-              } else {                                   // ReLU: relu(k) > 0 exactly where k > 0
-                df[8 * cc + 2 * e] = f.x > 0.f ? df[8 * cc + 2 * e] : 0.f;
-                df[8 * cc + 2 * e + 1] = f.y > 0.f ? df[8 * cc + 2 * e + 1] : 0.f;
-              }
+              dot += f.x * df[cc >> 2][8 * (cc & 3) + 2 * e] + f.y * df[cc >> 2][8 * (cc & 3) + 2 * e + 1];
             }
           }
-          tmem_st32(tK + 32 * c, df);
+          // group 1 hands its half over, group 0 adds and hands the sum back (barriers of the two warps of these 32 rows)
+          float* ex = reinterpret_cast<float*>(smem + KV_OFF_EX) + r;
+          if (g) *ex = dot;
+          asm volatile("bar.sync %0, 64;" ::"r"(4 + (r >> 5)) : "memory");
+          if (!g) *ex = dot = dot + *ex;
+          asm volatile("bar.sync %0, 64;" ::"r"(4 + (r >> 5)) : "memory");
+          if (g) dot = *ex;
         }
+#pragma unroll
+        for (int cc = 0; cc < 8; ++cc) {
+          const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 8 * g + cc));
+          const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 f = __bfloat1622float2(h2[e]);
+            float &d0 = df[cc >> 2][8 * (cc & 3) + 2 * e], &d1 = df[cc >> 2][8 * (cc & 3) + 2 * e + 1];
+            d0 = soft ? f.x * (d0 - dot) : f.x > 0.f ? d0 : 0.f;             // ReLU: relu(k) > 0 exactly where k > 0
+            d1 = soft ? f.y * (d1 - dot) : f.y > 0.f ? d1 : 0.f;
+          }
+        }
+        tmem_st32(tK + 64 * g, df[0]);
+        tmem_st32(tK + 64 * g + 32, df[1]);
+        tmem_wait_st();
       }
-      tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->fold_done);
     }
   }
 
-  // every product has completed: group 1 stores dV, staged in its own tile; group 0 stores dK, staged
-  // in the ring slot that the next key tile uses third (its last user was this tile's last item), so
-  // that nobody has to wait for a store to read its source out: phi(K) of the next tile goes to its
-  // own tile at once, and the loader waits for out_read before it refills that slot
-  if (gg < 2) {
+  // every product has completed: group 1 stages dV and group 0 dK in the ring slots of this tile's last two items, from
+  // where the loader warp stores them
+  {
     WAIT_OR_RETURN(bars->all_done, cnt.it & 1);
     tc_fence_after();
     const uint32_t tOut = gg == 0 ? tK : tV;
@@ -1158,9 +1167,7 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
       tc_fence_before();
       mbar_arrive(&bars->acc_free);
     } else {
-      if (gg == 1 && r == 0) tma_store_wait_read();            // the previous dV has left the staging tile
-      if (gg == 1) group_sync(1);
-      unsigned char* sOut = gg == 0 ? smem + KV_OFF_STAGE + ((seq0 + pl.N + 2) % KV_NS) * TILE_BYTES : smem + KV_OFF_OUT;
+      unsigned char* sOut = smem + KV_OFF_STAGE + (seq0 + pl.N - 1 - gg) % KV_NS * TILE_BYTES;
 #pragma unroll 1
       for (int cc = 0; cc < 4; cc += 2) {                        // two loads in flight
         float x[2][32];
@@ -1182,11 +1189,7 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
       tc_fence_before();
       mbar_arrive(&bars->acc_free);                              // the accumulators have been read
       fence_proxy_async_smem();
-      group_sync(gg);
-      if (r == 0) {
-        store_tile(gg == 0 ? &tm.dk : &tm.dv, sOut, pl.j * TILE, bh_kv);
-        tma_store_commit();
-      }
+      mbar_arrive(&bars->out_staged);
     }
   }
   cnt.seq = seq0 + pl.N;
@@ -1194,7 +1197,6 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   if (pl.n_R > 0) ++cnt.cr;
   ++cnt.it;
   }
-  if (r == 0) tma_store_wait();                               // this thread's last store has completed
   return true;
 }
 
@@ -1221,10 +1223,11 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
       mbar_init(&bars->phiq_ready[i], 128);
     }
     mbar_init(&bars->r_acc_done, 1);
-    mbar_init(&bars->fold_done, 128);
+    mbar_init(&bars->fold_done, 256);
     mbar_init(&bars->all_done, 1);
     mbar_init(&bars->acc_free, 256);
-    mbar_init(&bars->out_read, 1);
+    mbar_init(&bars->kv_free, 1);
+    mbar_init(&bars->out_staged, 256);
     mbar_init(&bars->drain, 1);
     mbar_init(&bars->drain2, 1);
     bars->abort = 0;
