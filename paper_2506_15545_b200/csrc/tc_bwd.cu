@@ -28,6 +28,8 @@
 // accumulator row each (row = TMEM lane), a loader warp issues the TMA loads, an MMA warp the
 // tcgen05 products; all accumulation is fp32 in TMEM, and the weight matrices of each tile
 // pair (P, dS) are rounded to bf16 and handed to the tensor core through TMEM.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace rattn {
@@ -86,7 +88,7 @@ struct PrepArgs {
   const float* gamma_s; const float* gamma_r;
   __nv_bfloat16* g_s; __nv_bfloat16* g_r;
   float* delta; float* dgamma_s; float* dgamma_r;
-  const float* lse; float* lse2p; float* dscp;
+  const float* lse; float* lse2p; float* dscp;              // lse2p, dscp: -lse * log2(e) and -D * scale, padded
   int* status;
   int* counters;        // work counters of the two main kernels: cleared here
   int n_heads, T, t_pad, H_q, rla_on;
@@ -180,7 +182,7 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
     const int t = t0 + row;
     const size_t prow = (size_t)bq * a.t_pad + t;
     if (rows == 0) {                                                // padding only: statistics that make every weight zero
-      if (l == 0) { a.lse2p[prow] = INFINITY; a.dscp[prow] = 0.f; }
+      if (l == 0) { a.lse2p[prow] = -INFINITY; a.dscp[prow] = 0.f; }
       continue;
     }
     const int h = bq % a.H_q;
@@ -264,10 +266,10 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
           const size_t grow = (size_t)bq * a.T + t;
           const float dl = (As - cs * ss) * is;                     // D_t = g_s . o_swa
           a.delta[grow] = dl;
-          a.lse2p[prow] = lse_row * LOG2E;
-          a.dscp[prow] = dl * a.scale;
+          a.lse2p[prow] = -lse_row * LOG2E;
+          a.dscp[prow] = -dl * a.scale;
         } else {
-          a.lse2p[prow] = INFINITY;
+          a.lse2p[prow] = -INFINITY;
           a.dscp[prow] = 0.f;
         }
       }
@@ -744,9 +746,9 @@ constexpr int KV_OFF_KPHI = 2 * TILE_BYTES;                // phi(K_j)
 constexpr int KV_OFF_STAGE = 3 * TILE_BYTES;               // KV_NS x [Q_h 16 KB | g_h 16 KB]
 constexpr int KV_OFF_STAT = KV_OFF_STAGE + KV_NS * TILE_BYTES;   // KV_NS x (lse2[64], D*scale[64]) fp32
 constexpr int KV_OFF_BAR = KV_OFF_STAT + KV_NS * 512;
-constexpr int KV_OFF_EX = KV_OFF_BAR + 384;                // one word per row, between the two row groups
-constexpr int KV_SMEM = KV_OFF_EX + TILE * 4;              // 232,320 bytes of the 232,448 a CTA may have
-constexpr int KV_THREADS = 352;                            // 2 row groups, score warp, loader warp, accumulate warp
+constexpr int KV_SMEM = KV_OFF_BAR + 384;                  // 231,808 bytes of the 232,448 a CTA may have
+constexpr int KV_ROW_WARPS = 16;
+constexpr int KV_THREADS = 32 * (KV_ROW_WARPS + 4);        // 2 row groups; score, loader and accumulate warp (and one idle)
 
 struct KvBars {
   uint64_t kv_full, kphi_ready, full[KV_NS], acc_done[KV_NS], s_full[2], p_ready[2], phiq_ready[2],
@@ -756,7 +758,7 @@ struct KvBars {
   int abort;
 };
 
-static_assert(sizeof(KvBars) <= KV_OFF_EX - KV_OFF_BAR, "barriers");
+static_assert(sizeof(KvBars) <= KV_SMEM - KV_OFF_BAR, "barriers");
 
 struct KvMaps {
   UMap k, v, qh, dk, dv;        // the caller's tensors (either head layout)
@@ -980,16 +982,14 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
   return true;
 }
 
-__device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int gg,
-                        int r) {
-  // two groups of 128 threads (thread = key row = TMEM lane), one per TMEM slot; a thread takes
-  // all 64 query columns of its item, 32 at a time (more row groups per slot measured no faster
-  // and cost registers)
-  const int g = gg;
+__device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int g, int h, int r) {
+  // Two groups of 256 threads, one per TMEM slot.  A thread is key row r = TMEM lane and half h of its item's 64 query
+  // columns: with all 64 on one thread a warp had a scheduler almost to itself and an item's arithmetic took 1530 cycles of
+  // the 4400 from scores to scores on a slot.
   const uint32_t lane_off = (uint32_t)((r & ~31) << 16);
   const uint32_t tV = tmem + lane_off, tK = tmem + 128 + lane_off;
-  const uint32_t tS = tmem + 256 + 128 * g + lane_off, tP = tS + 64;
-  const unsigned char* sKphi = smem + KV_OFF_KPHI;
+  const uint32_t tS = tmem + 256 + 128 * g + 32 * h + lane_off, tP = tS + 64;
+  const int gt = h * 128 + r;                                  // thread of the group
   KvCount cnt = {0, 0, 0, 0};
 
   for (;;) {
@@ -998,11 +998,11 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   if (idx < 0) break;
   const KvPlan pl = kv_plan(a, idx);
   if (pl.n_R > 0) {
-    // phi(K_j) into its own tile: 256 threads, two per row.  (Only here do these threads follow kv_full: without residual
+    // phi(K_j) into its own tile, four threads per row.  (Only here do these threads follow kv_full: without residual
     // items the next key tile's K and V may land before they look.)
     WAIT_OR_RETURN(bars->kv_full, cnt.it & 1);
-    const int t2 = gg * 128 + r, row = t2 >> 1, hf = t2 & 1;
-    feature_map_pair_any(smem + KV_OFF_K + hf * HALF_BYTES, smem + KV_OFF_KPHI + hf * HALF_BYTES, row, a.phi);
+    const int row = (g * 256 + gt) >> 2;
+    feature_map_quad(smem + KV_OFF_K + row * 128, smem + KV_OFF_KPHI + row * 128, HALF_BYTES, row, gt & 3, a.phi);
     fence_proxy_async_smem();
     mbar_arrive(&bars->kphi_ready);
   }
@@ -1019,127 +1019,110 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
     if (use >= 1) WAIT_OR_RETURN(bars->acc_done[st], (use - 1) & 1);
     WAIT_OR_RETURN(bars->full[st], use & 1);
     if (is_r) {
-      // phi(Q_h) in place: 64 rows, two threads per row
-      const int row = r >> 1, ch = r & 1;
-      feature_map_pair_any(sQh + ch * HT_HALF, sQh + ch * HT_HALF, row, a.phi);
+      // phi(Q_h) in place: 64 rows, four threads per row
+      const int row = gt >> 2;
+      feature_map_quad(sQh + row * 128, sQh + row * 128, HT_HALF, row, gt & 3, a.phi);
       fence_proxy_async_smem();
       mbar_arrive(&bars->phiq_ready[g]);
     }
     WAIT_OR_RETURN(bars->s_full[g], ((gi0 + n) >> 1) & 1);
     tc_fence_after();
     const bool diag = !is_r && (i == pl.j), bound = !is_r && pl.windowed && (i == pl.j + pl.wt);
-    const float* l2 = reinterpret_cast<const float*>(smem + KV_OFF_STAT + st * 512);
-    const float* Ds = l2 + 64;
-#pragma unroll 1
-    for (int c = 0; c < 2; ++c) {                              // rolled: compact code
-      float s[32], dp[32];
-      tmem_ld32(tS + 32 * c, s);
-      tmem_ld32(tP + 32 * c, dp);
-      tmem_wait_ld();
-      const int rd = r - (64 * hf + 32 * c);                   // key row relative to this chunk's first query
-      uint32_t pk1[16], pk2[16];
-      if (is_r) {
-        const uint32_t keep = bits_gt(rd);                     // keep key r < query q
+    float s[32], dp[32];
+    tmem_ld32(tS, s);
+    tmem_ld32(tP, dp);
+    tmem_wait_ld();
+    const int rd = r - (64 * hf + 32 * h);                     // key row relative to this thread's first query
+    uint32_t pk1[16], pk2[16];
+    if (is_r) {
+      const uint32_t keep = bits_gt(rd);                       // keep key r < query q
 #pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          const bool k0 = (keep >> e) & 1u, k1 = (keep >> (e + 1)) & 1u;
-          pk1[e >> 1] = pack_bf16(k0 ? s[e] : 0.f, k1 ? s[e + 1] : 0.f);
-          pk2[e >> 1] = pack_bf16(k0 ? dp[e] : 0.f, k1 ? dp[e + 1] : 0.f);
-        }
-      } else {
-        // diagonal tile: queries q >= r; oldest tile of the band: queries q <= r
-        const uint32_t keep = (diag ? bits_ge(rd) : 0xffffffffu) & (bound ? bits_le(rd) : 0xffffffffu);
-        if (!diag && !bound) {                     // interior tiles of the band: no mask
-#pragma unroll
-          for (int e4 = 0; e4 < 32; e4 += 4) {
-            const float4 lv = *reinterpret_cast<const float4*>(l2 + 32 * c + e4);
-            const float4 dv = *reinterpret_cast<const float4*>(Ds + 32 * c + e4);
-            const float lq[4] = {lv.x, lv.y, lv.z, lv.w}, dq4[4] = {dv.x, dv.y, dv.z, dv.w};
-            float p[4], d[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              p[u] = ex2(s[e4 + u] * a.scale_log2 - lq[u]);
-              d[u] = p[u] * (dp[e4 + u] * a.scale - dq4[u]);
-            }
-            pk1[e4 >> 1] = pack_bf16(p[0], p[1]);
-            pk1[(e4 >> 1) + 1] = pack_bf16(p[2], p[3]);
-            pk2[e4 >> 1] = pack_bf16(d[0], d[1]);
-            pk2[(e4 >> 1) + 1] = pack_bf16(d[2], d[3]);
-          }
-        } else
+      for (int e = 0; e < 32; e += 2) {
+        const bool k0 = (keep >> e) & 1u, k1 = (keep >> (e + 1)) & 1u;
+        pk1[e >> 1] = pack_bf16(k0 ? s[e] : 0.f, k1 ? s[e + 1] : 0.f);
+        pk2[e >> 1] = pack_bf16(k0 ? dp[e] : 0.f, k1 ? dp[e + 1] : 0.f);
+      }
+    } else {
+      // the item's statistics, -lse2 and -D scale of its queries
+      const float* nl = reinterpret_cast<const float*>(smem + KV_OFF_STAT + st * 512) + 32 * h;
+      // diagonal tile: queries q >= r; oldest tile of the band: queries q <= r; no mask in between
+      const uint32_t keep = (diag ? bits_ge(rd) : 0xffffffffu) & (bound ? bits_le(rd) : 0xffffffffu);
+      const float2 sl2 = make_float2(a.scale_log2, a.scale_log2), sc2 = make_float2(a.scale, a.scale);
+      auto weights = [&](auto masked_t) {
+        constexpr bool masked = decltype(masked_t)::value;
 #pragma unroll
         for (int e4 = 0; e4 < 32; e4 += 4) {
-          const float4 lv = *reinterpret_cast<const float4*>(l2 + 32 * c + e4);
-          const float4 dv = *reinterpret_cast<const float4*>(Ds + 32 * c + e4);
-          const float lq[4] = {lv.x, lv.y, lv.z, lv.w}, dq4[4] = {dv.x, dv.y, dv.z, dv.w};
-          float p[4], d[4];
+          const float4 lv = *reinterpret_cast<const float4*>(nl + e4);
+          const float4 dv = *reinterpret_cast<const float4*>(nl + 64 + e4);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const bool ok = (keep >> (e4 + u)) & 1u;
-            const float pv = ex2(s[e4 + u] * a.scale_log2 - lq[u]);
-            p[u] = ok ? pv : 0.f;
-            d[u] = ok ? pv * (dp[e4 + u] * a.scale - dq4[u]) : 0.f;
+          for (int u = 0; u < 4; u += 2) {
+            const int e = e4 + u;
+            const float2 y = __ffma2_rn(make_float2(s[e], s[e + 1]), sl2, u ? make_float2(lv.z, lv.w) : make_float2(lv.x, lv.y));
+            const float2 p = make_float2(ex2(y.x), ex2(y.y));
+            const float2 d = __fmul2_rn(p, __ffma2_rn(make_float2(dp[e], dp[e + 1]), sc2, u ? make_float2(dv.z, dv.w) : make_float2(dv.x, dv.y)));
+            const bool k0 = !masked || ((keep >> e) & 1u), k1 = !masked || ((keep >> (e + 1)) & 1u);
+            pk1[e >> 1] = pack_bf16(k0 ? p.x : 0.f, k1 ? p.y : 0.f);
+            pk2[e >> 1] = pack_bf16(k0 ? d.x : 0.f, k1 ? d.y : 0.f);
           }
-          pk1[e4 >> 1] = pack_bf16(p[0], p[1]);
-          pk1[(e4 >> 1) + 1] = pack_bf16(p[2], p[3]);
-          pk2[e4 >> 1] = pack_bf16(d[0], d[1]);
-          pk2[(e4 >> 1) + 1] = pack_bf16(d[2], d[3]);
         }
-      }
-      // bf16 results (two per column) overwrite the first half of the chunk just consumed
-      tmem_st16(tS + 32 * c, pk1);
-      tmem_st16(tP + 32 * c, pk2);
+      };
+      if (diag || bound) weights(std::true_type{});
+      else weights(std::false_type{});
     }
+    // bf16 results (two per column) overwrite the first half of the columns just consumed
+    tmem_st16(tS, pk1);
+    tmem_st16(tP, pk2);
     tmem_wait_st();
     tc_fence_before();
     mbar_arrive(&bars->p_ready[g]);
 
     if (is_r && n + 2 >= pl.n_R) {                              // this group's last residual item of this key tile
       // end of the residual items: dK := dphi_k through the feature map's gradient (softmax map:
-      // phi(k) (dphi_k - <dphi_k, phi(k)>)), each group half of the columns: every window item waits for it
+      // phi(k) (dphi_k - <dphi_k, phi(k)>)), a quarter of the columns per thread: every window item waits for it
       WAIT_OR_RETURN(bars->r_acc_done, cnt.cr & 1);
       tc_fence_after();
       // the identity map leaves dphi_k as it is
       if (a.phi != RATTN_PHI_IDENTITY) {
         const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
-        float df[2][32];
-        tmem_ld32(tK + 64 * g, df[0]);
-        tmem_ld32(tK + 64 * g + 32, df[1]);
+        const int part = 2 * g + h;
+        unsigned char* sKphi = smem + KV_OFF_KPHI;
+        float df[32];
+        tmem_ld32(tK + 32 * part, df);
         tmem_wait_ld();
+        uint4 u[4];
+#pragma unroll
+        for (int cc = 0; cc < 4; ++cc) u[cc] = *reinterpret_cast<const uint4*>(sKphi + swz(r, 4 * part + cc));
         float dot = 0.f;
         if (soft) {
 #pragma unroll
-          for (int cc = 0; cc < 8; ++cc) {
-            const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 8 * g + cc));
-            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
+          for (int cc = 0; cc < 4; ++cc) {
+            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u[cc]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const float2 f = __bfloat1622float2(h2[e]);
-              dot += f.x * df[cc >> 2][8 * (cc & 3) + 2 * e] + f.y * df[cc >> 2][8 * (cc & 3) + 2 * e + 1];
+              dot += f.x * df[8 * cc + 2 * e] + f.y * df[8 * cc + 2 * e + 1];
             }
           }
-          // group 1 hands its half over, group 0 adds and hands the sum back (barriers of the two warps of these 32 rows)
-          float* ex = reinterpret_cast<float*>(smem + KV_OFF_EX) + r;
-          if (g) *ex = dot;
-          asm volatile("bar.sync %0, 64;" ::"r"(4 + (r >> 5)) : "memory");
-          if (!g) *ex = dot = dot + *ex;
-          asm volatile("bar.sync %0, 64;" ::"r"(4 + (r >> 5)) : "memory");
-          if (g) dot = *ex;
+          // the four parts of a row meet in its phi(k), which nothing reads any more
+          *reinterpret_cast<float*>(sKphi + swz(r, 4 * part)) = dot;
+          asm volatile("bar.sync %0, 128;" ::"r"(4 + (r >> 5)) : "memory");   // the four warps of these 32 rows
+          float d4[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) d4[k] = *reinterpret_cast<const float*>(sKphi + swz(r, 4 * k));
+          dot = (d4[0] + d4[1]) + (d4[2] + d4[3]);
         }
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
-          const uint4 u = *reinterpret_cast<const uint4*>(sKphi + swz(r, 8 * g + cc));
-          const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
+        for (int cc = 0; cc < 4; ++cc) {
+          const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u[cc]);
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float2 f = __bfloat1622float2(h2[e]);
-            float &d0 = df[cc >> 2][8 * (cc & 3) + 2 * e], &d1 = df[cc >> 2][8 * (cc & 3) + 2 * e + 1];
+            float &d0 = df[8 * cc + 2 * e], &d1 = df[8 * cc + 2 * e + 1];
             d0 = soft ? f.x * (d0 - dot) : f.x > 0.f ? d0 : 0.f;             // ReLU: relu(k) > 0 exactly where k > 0
             d1 = soft ? f.y * (d1 - dot) : f.y > 0.f ? d1 : 0.f;
           }
         }
-        tmem_st32(tK + 64 * g, df[0]);
-        tmem_st32(tK + 64 * g + 32, df[1]);
+        tmem_st32(tK + 32 * part, df);
         tmem_wait_st();
       }
       tc_fence_before();
@@ -1152,42 +1135,29 @@ __device__ bool kv_rows(const KvMaps& tm, const BwdArgs& a, unsigned char* smem,
   {
     WAIT_OR_RETURN(bars->all_done, cnt.it & 1);
     tc_fence_after();
-    const uint32_t tOut = gg == 0 ? tK : tV;
+    const uint32_t tOut = (g == 0 ? tK : tV) + 64 * h;
+    float x[2][32];
+    tmem_ld32(tOut, x[0]);
+    tmem_ld32(tOut + 32, x[1]);
+    tmem_wait_ld();
+    tc_fence_before();
+    mbar_arrive(&bars->acc_free);                              // the accumulators have been read
     if (a.part) {
       // one of several parts: fp32, float4 columns outermost ([32][128 rows]), so that a warp's stores are whole runs
-      float4* dst = a.part + ((size_t)pl.part_index * 2 + gg) * 4096 + r;
-#pragma unroll 1
-      for (int cc = 0; cc < 4; ++cc) {
-        float x[32];
-        tmem_ld32(tOut + 32 * cc, x);
-        tmem_wait_ld();
+      float4* dst = a.part + ((size_t)pl.part_index * 2 + g) * 4096 + 16 * h * 128 + r;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) dst[(8 * cc + e) * 128] = make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
+      for (int e = 0; e < 16; ++e) {
+        const float* y = &x[e >> 3][4 * (e & 7)];
+        dst[e * 128] = make_float4(y[0], y[1], y[2], y[3]);
       }
-      tc_fence_before();
-      mbar_arrive(&bars->acc_free);
     } else {
-      unsigned char* sOut = smem + KV_OFF_STAGE + (seq0 + pl.N - 1 - gg) % KV_NS * TILE_BYTES;
-#pragma unroll 1
-      for (int cc = 0; cc < 4; cc += 2) {                        // two loads in flight
-        float x[2][32];
-        tmem_ld32(tOut + 32 * cc, x[0]);
-        tmem_ld32(tOut + 32 * (cc + 1), x[1]);
-        tmem_wait_ld();
+      unsigned char* sOut = smem + KV_OFF_STAGE + (seq0 + pl.N - 1 - g) % KV_NS * TILE_BYTES;
 #pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            uint4 u;
-            u.x = pack_bf16(x[h2][8 * e + 0], x[h2][8 * e + 1]);
-            u.y = pack_bf16(x[h2][8 * e + 2], x[h2][8 * e + 3]);
-            u.z = pack_bf16(x[h2][8 * e + 4], x[h2][8 * e + 5]);
-            u.w = pack_bf16(x[h2][8 * e + 6], x[h2][8 * e + 7]);
-            *reinterpret_cast<uint4*>(sOut + swz(r, 4 * (cc + h2) + e)) = u;
-          }
+      for (int e = 0; e < 8; ++e) {
+        const float* y = &x[e >> 2][8 * (e & 3)];
+        *reinterpret_cast<uint4*>(sOut + swz(r, 8 * h + e)) =
+            make_uint4(pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]), pack_bf16(y[6], y[7]));
       }
-      tc_fence_before();
-      mbar_arrive(&bars->acc_free);                              // the accumulators have been read
       fence_proxy_async_smem();
       mbar_arrive(&bars->out_staged);
     }
@@ -1210,36 +1180,36 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     return;
   }
   if (tid == 0) {
-    sched_init(&bars->sched, 256 + 2);
+    sched_init(&bars->sched, 32 * KV_ROW_WARPS + 2);
     mbar_init(&bars->kv_full, 1);
-    mbar_init(&bars->kphi_ready, 256);
+    mbar_init(&bars->kphi_ready, 32 * KV_ROW_WARPS);
     for (int i = 0; i < KV_NS; ++i) {
       mbar_init(&bars->full[i], 1);
       mbar_init(&bars->acc_done[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->s_full[i], 1);
-      mbar_init(&bars->p_ready[i], 128);
-      mbar_init(&bars->phiq_ready[i], 128);
+      mbar_init(&bars->p_ready[i], 16 * KV_ROW_WARPS);
+      mbar_init(&bars->phiq_ready[i], 16 * KV_ROW_WARPS);
     }
     mbar_init(&bars->r_acc_done, 1);
-    mbar_init(&bars->fold_done, 256);
+    mbar_init(&bars->fold_done, 32 * KV_ROW_WARPS);
     mbar_init(&bars->all_done, 1);
-    mbar_init(&bars->acc_free, 256);
+    mbar_init(&bars->acc_free, 32 * KV_ROW_WARPS);
     mbar_init(&bars->kv_free, 1);
-    mbar_init(&bars->out_staged, 256);
+    mbar_init(&bars->out_staged, 32 * KV_ROW_WARPS);
     mbar_init(&bars->drain, 1);
     mbar_init(&bars->drain2, 1);
     bars->abort = 0;
     fence_mbar_init();
   }
-  if (warp == 8) {
+  if (warp == KV_ROW_WARPS) {
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (tid == 288) {
+  if (warp == KV_ROW_WARPS + 1 && (tid & 31) == 0) {
     prefetch_map(&tm.k);
     prefetch_map(&tm.v);
     prefetch_tensormap(&tm.rs);
@@ -1254,23 +1224,26 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
 
+  // registers follow the work: 512 x 104 + 128 x 64 = 640 x 96, the CTA's allocation
   bool ok = true;
-  if (warp < 8) {
-    ok = kv_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127);
-  } else if (warp == 8 || warp == 10) {
-    ok = warp == 8 ? kv_mma_scores(a, smem, bars, tmem) : kv_mma_accum(a, smem, bars, tmem);
+  if (warp < KV_ROW_WARPS) setmaxnreg_inc<104>();
+  else setmaxnreg_dec<64>();
+  if (warp < KV_ROW_WARPS) {
+    ok = kv_rows(a, smem, bars, tmem, warp >> 3, (warp >> 2) & 1, tid & 127);
+  } else if (warp == KV_ROW_WARPS || warp == KV_ROW_WARPS + 2) {
+    ok = warp == KV_ROW_WARPS ? kv_mma_scores(a, smem, bars, tmem) : kv_mma_accum(a, smem, bars, tmem);
     if (!ok) {                                             // let this warp's products in flight finish
-      uint64_t* drain = warp == 8 ? &bars->drain : &bars->drain2;
+      uint64_t* drain = warp == KV_ROW_WARPS ? &bars->drain : &bars->drain2;
       mma_commit(drain);
       for (int it = 0; it < (1 << 16) && !mbar_try_wait(drain, 0); ++it) {}
     }
-  } else if (warp == 9) {
+  } else if (warp == KV_ROW_WARPS + 1) {
     ok = kv_loader(tm, a, smem, bars, n_items);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == KV_ROW_WARPS) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }

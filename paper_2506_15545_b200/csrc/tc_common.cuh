@@ -195,6 +195,62 @@ __device__ __forceinline__ void feature_map_pair_any(const unsigned char* src_ha
   feature_map_half_row(src_half + row * 128, dst_half + row * 128, row, (int)(threadIdx.x & 1), phi, true);
 }
 
+// ... by four adjacent lanes per row, of which this one (q = lane & 3) owns 32 columns; `src` and `dst` point at the row in
+// the first column half's box, the second half's lies `half_stride` behind.  A quarter-warp (two rows) touches every bank
+// once: the lanes of the second half walk their chunks two apart from the first's.
+__device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsigned char* dst, int half_stride, int row, int q,
+                                                 int phi) {
+  const int sw = (row & 7) ^ ((q & 1) << 2) ^ (q & 2);
+  src += (q >> 1) * half_stride;
+  dst += (q >> 1) * half_stride;
+  if (phi != RATTN_PHI_SOFTMAX) {
+    if (phi == RATTN_PHI_IDENTITY && src == dst) return;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint4 u = *reinterpret_cast<const uint4*>(src + ((c ^ sw) << 4));
+      *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) = phi == RATTN_PHI_RELU ? relu_bf16x8(u) : u;
+    }
+    return;
+  }
+  float x[32], m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const uint4 u = *reinterpret_cast<const uint4*>(src + ((c ^ sw) << 4));
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      x[c * 8 + 2 * e] = __uint_as_float(w[e] << 16);
+      x[c * 8 + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+      m0 = fmaxf(m0, x[c * 8 + 2 * e]);
+      m1 = fmaxf(m1, x[c * 8 + 2 * e + 1]);
+    }
+  }
+  float m = fmaxf(m0, m1);
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+  const float ml = m * 1.4426950408889634f;
+  const float2 l2e = make_float2(1.4426950408889634f, 1.4426950408889634f), nml = make_float2(-ml, -ml);
+  float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < 32; i += 2) {
+    const float2 y = __ffma2_rn(make_float2(x[i], x[i + 1]), l2e, nml);
+    const float2 p = make_float2(ex2(y.x), ex2(y.y));
+    x[i] = p.x;
+    x[i + 1] = p.y;
+    if (i & 2) s1 = __fadd2_rn(s1, p);
+    else s0 = __fadd2_rn(s0, p);
+  }
+  float sum = (s0.x + s0.y) + (s1.x + s1.y);
+  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  const float sc = 1.f / sum;
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) =
+        make_uint4(pack_bf16(x[c * 8 + 0] * sc, x[c * 8 + 1] * sc), pack_bf16(x[c * 8 + 2] * sc, x[c * 8 + 3] * sc),
+                   pack_bf16(x[c * 8 + 4] * sc, x[c * 8 + 5] * sc), pack_bf16(x[c * 8 + 6] * sc, x[c * 8 + 7] * sc));
+}
+
 // byte offset of 16-byte chunk c (0..15) of row r inside a swizzled [128 x 128] bf16 tile
 __device__ __forceinline__ uint32_t swz(int r, int c) {
   return (uint32_t)((c >> 3) * HALF_BYTES + r * 128 + (((c & 7) ^ (r & 7)) << 4));
