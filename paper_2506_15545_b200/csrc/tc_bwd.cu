@@ -306,30 +306,38 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
 // Persistent: one CTA per SM walks a list of (query head, query tile) items, so that an item's
 // first loads are in flight while the previous item's epilogue drains (at w = 512 the fixed
 // cost per tile -- first TMA touch, output staging -- is larger than the band itself).
-//   loader warp   Q (two buffers, alternating), g_s, K/V tiles through a ring of two stages;
-//                 the residual operands (g_r, stored state) take one more slot of that ring
-//   MMA warp      per key tile S = Q K^T, dP = g_s V^T; after the row groups have overwritten S
+//   loader warp   Q (two buffers, alternating), K tiles through a ring of three slots, V tiles through one buffer, g_s;
+//                 for the residual part g_r follows in g_s's buffer and the stored state in the K ring
+//   MMA warp      per key tile S = Q K^T, dP = g_s V^T; after the row threads have overwritten S
 //                 with dS (bf16, in TMEM): dQ += dS K.  Then the residual part.
-//   row groups    two groups of 128 threads (thread = query row = TMEM lane), group g takes the
-//                 key columns 64g .. 64g+63 of every tile; group 0 runs the epilogue
+//   row threads   512: query row = TMEM lane, and a quarter of the 128 columns
+// TMEM holds S twice (the second buffer is dphi_q's, which only the residual part needs), so that S of the next key tile
+// is formed beside the row threads' work; dP of the next tile goes out the moment they are done, ahead of this tile's dQ.
+// V is read by dP alone, early in its step, K by S in the step before and by dQ at the end of it: three slots of K and one
+// of V keep the loads (1750 cycles each) off the path, two of each put one into every step (4150 cycles a step).
+// With one buffer, two threads per row and the epilogue on 128 of them, an item of 5 key tiles took 31k cycles.
 // All barriers run on with phase counters that every role advances in the same way.
 constexpr int DQ_OFF_Q = 0;                 // Q buffer 0
 constexpr int DQ_OFF_G = 1 * TILE_BYTES;
-constexpr int DQ_OFF_K = 2 * TILE_BYTES;   // 2 stages
-constexpr int DQ_OFF_V = 4 * TILE_BYTES;   // 2 stages
+constexpr int DQ_NK = 3;
+constexpr int DQ_OFF_K = 2 * TILE_BYTES;   // DQ_NK slots
+constexpr int DQ_OFF_V = 5 * TILE_BYTES;
 constexpr int DQ_OFF_Q1 = 6 * TILE_BYTES;  // Q buffer 1
 constexpr int DQ_OFF_BAR = 7 * TILE_BYTES;
-constexpr int DQ_SMEM = DQ_OFF_BAR + 384;
-constexpr int DQ_THREADS = 320;            // 2 row groups, MMA warp, loader warp
+constexpr int DQ_OFF_EX = DQ_OFF_BAR + 384;   // one word per row thread
+constexpr int DQ_ROW_WARPS = 16;
+constexpr int DQ_SMEM = DQ_OFF_EX + 32 * DQ_ROW_WARPS * 4;
+constexpr int DQ_THREADS = 32 * (DQ_ROW_WARPS + 4);   // row threads, MMA warp, loader warp (and two idle)
 
 struct DqBars {
-  uint64_t qg_full, kv_full[2], kv_free[2], s_full, ds_full, phik_ready, o_done, g_free, acc_free, q_read, drain;
+  uint64_t q_full, g_full, g_free, v_full, v_free, k_full[DQ_NK], k_free[DQ_NK], s_full, ds_full, phik_ready, o_done,
+      acc_free, q_read, drain;
   SchedRing sched;
   uint32_t tmem_base;
   int abort;
 };
 
-static_assert(sizeof(DqBars) <= DQ_SMEM - DQ_OFF_BAR, "barriers");
+static_assert(sizeof(DqBars) <= DQ_OFF_EX - DQ_OFF_BAR, "barriers");
 
 struct DqItem {
   int q0, bh_q, bh_kv, n_kt, st_index;
@@ -360,47 +368,58 @@ struct DqMaps {
 };
 
 __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, int n_items, int n_qt) {
-  int kc = 0, n = 0;                                       // ring uses, items so far
+  int kc = 0, vc = 0, gc = 0, n = 0;                       // uses of the K ring, the V and the g buffer; items so far
   for (;; ++n) {
     int idx;
     if (!sched_draw(&bars->sched, a.counter, n_items, n, &bars->abort, &idx)) return false;
     if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
-    auto ring_wait = [&]() -> bool {                       // the slot's previous user has been consumed
-      const int st = kc & 1, use = kc >> 1;
-      if (use >= 1) WAIT_OR_RETURN_W(bars->kv_free[st], (use - 1) & 1);
+    auto k_slot = [&](int& st) -> bool {                   // the next K slot, once its previous use is consumed
+      st = kc % DQ_NK;
+      const int use = kc / DQ_NK;
+      if (use >= 1) WAIT_OR_RETURN_W(bars->k_free[st], (use - 1) & 1);
+      ++kc;
+      return true;
+    };
+    auto load_k = [&](int i) -> bool {
+      int st;
+      if (!k_slot(st)) return false;
+      mbar_arrive_expect_tx(&bars->k_full[st], TILE_BYTES);
+      load_tile(smem + DQ_OFF_K + st * TILE_BYTES, &tm.k, &bars->k_full[st], it.q0 - i * TILE, it.bh_kv);
+      return true;
+    };
+    auto load_g = [&](const CUtensorMap* map) -> bool {
+      if (gc >= 1) WAIT_OR_RETURN_W(bars->g_free, (gc - 1) & 1);
+      mbar_arrive_expect_tx(&bars->g_full, TILE_BYTES);
+      load_tile(smem + DQ_OFF_G, map, &bars->g_full, it.q0, it.bh_q);
+      ++gc;
       return true;
     };
     // The barrier's previous phase must be over before this item arrives on it: after a short
-    // item the loader gets here while that item's Q and g_s are still in flight.
-    if (n >= 1) WAIT_OR_RETURN_W(bars->qg_full, (n - 1) & 1);
-    mbar_arrive_expect_tx(&bars->qg_full, 2 * TILE_BYTES);
+    // item the loader gets here while that item's Q is still in flight.
+    if (n >= 1) WAIT_OR_RETURN_W(bars->q_full, (n - 1) & 1);
+    mbar_arrive_expect_tx(&bars->q_full, TILE_BYTES);
     // Q into the buffer last used two items ago: free once its dQ, staged there by that item's epilogue, has left.  (Not
     // acc_free as well: the item in between may have completed that barrier a second time before this warp looks, and
     // then the wait, which sees the parity alone, would be for a completion that needs this load.)
     if (n >= 2) WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);
-    load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->qg_full, it.q0, it.bh_q);
-    // g_s: its one buffer is free once the previous item's window products have completed (the residual part reads
-    // g_r).  A barrier of its own, one completion per item: a parity wait tells a completion only from the ones next to
-    // it, and of o_done, which completes twice for an item with a residual part, the loader may come too early for the
-    // second (the first still outstanding: the parity reads as reached) as well as too late for the first (the second
-    // over already: the wait would be for the next item's, which needs this load).
-    if (n >= 1) WAIT_OR_RETURN_W(bars->g_free, (n - 1) & 1);
-    load_tile(smem + DQ_OFF_G, &tm.gs, &bars->qg_full, it.q0, it.bh_q);
-    for (int i = 0; i < it.n_kt; ++i, ++kc) {
-      if (!ring_wait()) return false;
-      const int st = kc & 1;
-      mbar_arrive_expect_tx(&bars->kv_full[st], 2 * TILE_BYTES);
-      load_tile(smem + DQ_OFF_K + st * TILE_BYTES, &tm.k, &bars->kv_full[st], it.q0 - i * TILE, it.bh_kv);
-      load_tile(smem + DQ_OFF_V + st * TILE_BYTES, &tm.v, &bars->kv_full[st], it.q0 - i * TILE, it.bh_kv);
+    load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->q_full, it.q0, it.bh_q);
+    // in the order in which their places become free: V_i behind dP_(i-1), K_(i+1) behind dQ_(i-2)
+    if (!load_k(0) || !load_g(&tm.gs)) return false;
+    for (int i = 0; i < it.n_kt; ++i, ++vc) {
+      if (vc >= 1) WAIT_OR_RETURN_W(bars->v_free, (vc - 1) & 1);
+      mbar_arrive_expect_tx(&bars->v_full, TILE_BYTES);
+      load_tile(smem + DQ_OFF_V, &tm.v, &bars->v_full, it.q0 - i * TILE, it.bh_kv);
+      if (i + 1 < it.n_kt && !load_k(i + 1)) return false;
     }
-    if (it.has_rla) {                                      // g_r in the V half of the slot, the state in the K half
-      if (!ring_wait()) return false;
-      const int st = kc & 1;
-      mbar_arrive_expect_tx(&bars->kv_full[st], (it.has_state ? 2 : 1) * TILE_BYTES);
-      load_tile(smem + DQ_OFF_V + st * TILE_BYTES, &tm.gr, &bars->kv_full[st], it.q0, it.bh_q);
-      if (it.has_state) load_tile(smem + DQ_OFF_K + st * TILE_BYTES, &tm.st, &bars->kv_full[st], 0, it.st_index);
-      ++kc;
+    if (it.has_rla) {
+      if (it.has_state) {
+        int st;
+        if (!k_slot(st)) return false;
+        mbar_arrive_expect_tx(&bars->k_full[st], TILE_BYTES);
+        load_tile(smem + DQ_OFF_K + st * TILE_BYTES, &tm.st, &bars->k_full[st], 0, it.st_index);
+      }
+      if (!load_g(&tm.gr)) return false;
     }
   }
   return true;
@@ -410,65 +429,107 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
   const uint32_t sG = smem_u32(smem + DQ_OFF_G), sK = smem_u32(smem + DQ_OFF_K), sV = smem_u32(smem + DQ_OFF_V);
   const uint32_t tS = tmem, tP = tmem + 128, tQ = tmem + 256, tF = tmem + 384;
   constexpr uint32_t idesc_ts = instr_desc(128, 128, 0, 1);
-  int kc = 0, n = 0, cs = 0, cr = 0;                       // ring uses, items, score hand-overs, residual items
+  int kc = 0, vc = 0, gc = 0, n = 0, cs = 0, cr = 0;       // K, V and g uses, items, score hand-overs, residual items
   for (;; ++n) {
     int idx;
     if (!sched_read_warp(&bars->sched, n, &bars->abort, &idx)) return false;
     if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     const uint32_t sQ = smem_u32(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q));
-    WAIT_OR_RETURN_W(bars->qg_full, n & 1);
-    int last_st = 0;
-    for (int i = 0; i < it.n_kt; ++i, ++kc, ++cs) {
-      const int st = kc & 1;
-      last_st = st;
-      WAIT_OR_RETURN_W(bars->kv_full[st], (kc >> 1) & 1);
-      tc_fence_after();
-      mma_kk(tS, sQ, sK + st * TILE_BYTES, false);         // S  = Q K^T
-      mma_kk(tP, sG, sV + st * TILE_BYTES, false);         // dP = g_s V^T
+    auto k_landed = [&](int use) -> bool {
+      WAIT_OR_RETURN_W(bars->k_full[use % DQ_NK], (use / DQ_NK) & 1);
+      return true;
+    };
+    // dP = g_s V^T of key tile i, with the releases behind it (the last tile's V is read once more by the residual part)
+    auto dp_products = [&](int i) {
+      mma_kk(tP, sG, sV, false);
       mma_commit(&bars->s_full);
+      if (!(it.has_rla && i + 1 == it.n_kt)) mma_commit(&bars->v_free);
+      if (i + 1 == it.n_kt) mma_commit(&bars->g_free);
+    };
+    WAIT_OR_RETURN_W(bars->q_full, n & 1);
+    if (!k_landed(kc)) return false;
+    tc_fence_after();
+    mma_kk(tS, sQ, sK + kc % DQ_NK * TILE_BYTES, false);   // S = Q K^T
+    WAIT_OR_RETURN_W(bars->g_full, gc & 1);
+    ++gc;
+    WAIT_OR_RETURN_W(bars->v_full, vc & 1);
+    ++vc;
+    tc_fence_after();
+    dp_products(0);
+    for (int i = 0; i < it.n_kt; ++i, ++kc, ++cs) {
+      const int st = kc % DQ_NK;
+      const uint32_t tSi = (i & 1) ? tF : tS, tSn = (i & 1) ? tS : tF;
+      const bool more = i + 1 < it.n_kt;
+      if (more && !k_landed(kc + 1)) return false;
+      if (i == 0 && n >= 1) WAIT_OR_RETURN_W(bars->acc_free, (n - 1) & 1);   // the previous item's epilogue has read dQ and dphi_q
+      if (more) {
+        tc_fence_after();
+        mma_kk(tSn, sQ, sK + (kc + 1) % DQ_NK * TILE_BYTES, false);   // the next tile's S, while the row threads work on this one's
+        WAIT_OR_RETURN_W(bars->v_full, vc & 1);
+        ++vc;
+      }
       WAIT_OR_RETURN_W(bars->ds_full, cs & 1);
-      if (i == 0 && n >= 1) WAIT_OR_RETURN_W(bars->acc_free, (n - 1) & 1);   // the previous item's epilogue has read dQ
       tc_fence_after();
+      if (more) dp_products(i + 1);                        // ahead of dQ: the row threads wait for it
 #pragma unroll
       for (int k = 0; k < 8; ++k)                          // dQ += dS K, dS read from TMEM
-        mma_bf16_ts(tQ, tS + (k < 4 ? 8 * k : 64 + 8 * (k - 4)), mnmajor_desc(sK + st * TILE_BYTES, k), idesc_ts, (i > 0 || k > 0) ? 1u : 0u);
+        mma_bf16_ts(tQ, tSi + 32 * (k >> 1) + 8 * (k & 1), mnmajor_desc(sK + st * TILE_BYTES, k), idesc_ts, (i > 0 || k > 0) ? 1u : 0u);
       // the last tile's K turns into phi(K) for the residual part: its slot is released there
-      if (!(it.has_rla && i == it.n_kt - 1)) mma_commit(&bars->kv_free[st]);
-      // the next tile's scores follow these products in the tensor pipe, which runs in issue order
+      if (!(it.has_rla && !more)) mma_commit(&bars->k_free[st]);
+      // the products that overwrite what these read follow them in the tensor pipe, which runs in issue order
     }
-    mma_commit(&bars->g_free);                             // the window products are done with g_s
     if (it.has_rla) {
-      const int xs = kc & 1;                               // slot of g_r and the stored state
-      const uint32_t sG2 = sV + xs * TILE_BYTES, sSt = sK + xs * TILE_BYTES;
+      const int last_st = (kc - 1) % DQ_NK, xs = kc % DQ_NK;   // K_cb; the stored state
       mma_commit(&bars->o_done);                           // (interim) every window product done: K_cb may be rewritten
-      WAIT_OR_RETURN_W(bars->kv_full[xs], (kc >> 1) & 1);
+      WAIT_OR_RETURN_W(bars->g_full, gc & 1);              // g_r
+      ++gc;
       tc_fence_after();
-      mma_kk(tS, sG2, sV + last_st * TILE_BYTES, false);   // dA = g_r V_cb^T
-      if (it.has_state) mma_kk(tF, sG2, sSt, false);       // g_r S_cb^T
+      mma_kk(tS, sG, sV, false);                           // dA = g_r V_cb^T
       mma_commit(&bars->s_full);
+      mma_commit(&bars->v_free);
+      if (it.has_state) {
+        if (!k_landed(kc)) return false;
+        tc_fence_after();
+        mma_kk(tF, sG, sK + xs * TILE_BYTES, false);       // g_r S_cb^T
+        mma_commit(&bars->k_free[xs]);
+        ++kc;
+      }
+      mma_commit(&bars->g_free);
       WAIT_OR_RETURN_W(bars->phik_ready, cr & 1);
       WAIT_OR_RETURN_W(bars->ds_full, cs & 1);
       tc_fence_after();
 #pragma unroll
       for (int k = 0; k < 8; ++k)                          // (dA masked) phi(K_cb)
-        mma_bf16_ts(tF, tS + (k < 4 ? 8 * k : 64 + 8 * (k - 4)), mnmajor_desc(sK + last_st * TILE_BYTES, k), idesc_ts, (it.has_state || k > 0) ? 1u : 0u);
-      mma_commit(&bars->kv_free[last_st]);
-      mma_commit(&bars->kv_free[xs]);
-      ++kc; ++cs; ++cr;
+        mma_bf16_ts(tF, tS + 32 * (k >> 1) + 8 * (k & 1), mnmajor_desc(sK + last_st * TILE_BYTES, k), idesc_ts, (it.has_state || k > 0) ? 1u : 0u);
+      mma_commit(&bars->k_free[last_st]);
+      ++cs; ++cr;
     }
     mma_commit(&bars->o_done);
   }
   return true;
 }
 
-__device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int g, int r,
+// Row thread (r, part): query row r = TMEM lane, columns 32 part .. 32 part + 31.
+__device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int part, int r,
                         int n_qt) {
-  const uint32_t lane_off = (uint32_t)((r & ~31) << 16);
+  const uint32_t lane_off = ((uint32_t)((r & ~31) << 16)) + 32 * part;
   const uint32_t tS = tmem + lane_off, tP = tmem + 128 + lane_off, tQ = tmem + 256 + lane_off,
                  tF = tmem + 384 + lane_off;
   int kc = 0, n = 0, cs = 0, co = 0;                       // ring uses, items, score hand-overs, o_done completions
   bool store_pending = false;                              // this thread issued a dQ store whose read-out it has not confirmed
+  const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
+  const float2 sl2 = make_float2(a.scale_log2, a.scale_log2), sc2 = make_float2(a.scale, a.scale);
+  // one value per thread, shared by the four threads of a row (the four warps of the same 32 rows meet; sync again before
+  // the words are used once more)
+  float* ex = reinterpret_cast<float*>(smem + DQ_OFF_EX);
+  auto row_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(4 + (r >> 5)) : "memory"); };
+  auto exchange = [&](float mine, float (&all)[4]) {
+    ex[part * TILE + r] = mine;
+    row_sync();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) all[k] = ex[k * TILE + r];
+  };
   for (;; ++n) {
     int idx;
     if (!sched_read(&bars->sched, n, &bars->abort, &idx)) return false;
@@ -479,39 +540,28 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
     const int t = it.q0 + r;
     const bool live = t < a.T;
     const size_t row = (size_t)it.bh_q * a.T + t;
-    const float l2 = live ? a.lse[row] * LOG2E : INFINITY;
-    const float Drs = live ? a.delta[row] * a.scale : 0.f;
+    const float nl2 = live ? -a.lse[row] * LOG2E : -INFINITY;
+    const float nD = live ? -a.delta[row] * a.scale : 0.f;
 
     for (int i = 0; i < n_kt; ++i, ++cs) {
       WAIT_OR_RETURN(bars->s_full, cs & 1);
       tc_fence_after();
       const bool diag = (i == 0), bound = it.has_boundary && (i == n_kt - 1);
-#pragma unroll 1
-      for (int c = 2 * g; c < 2 * g + 2; ++c) {                 // rolled: compact code
-        float s[32], dp[32];
-        tmem_ld32(tS + 32 * c, s);
-        tmem_ld32(tP + 32 * c, dp);
-        tmem_wait_ld();
-        uint32_t pk[16];
-        if (diag || bound) {                       // only the two edge tiles of the band need a mask
-          const uint32_t keep = keep_bits(r, c, diag, bound);
+      const uint32_t tSi = (i & 1) ? tF : tS;
+      float s[32], dp[32];
+      tmem_ld32(tSi, s);
+      tmem_ld32(tP, dp);
+      tmem_wait_ld();
+      if (diag || bound) mask32(s, keep_bits(r, part, diag, bound));   // the two edge tiles; exp2(-inf) = 0
+      uint32_t pk[16];
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float p0 = ex2(s[e] * a.scale_log2 - l2), p1 = ex2(s[e + 1] * a.scale_log2 - l2);
-            const float d0 = (keep >> e) & 1u ? p0 * (dp[e] * a.scale - Drs) : 0.f;
-            const float d1 = (keep >> (e + 1)) & 1u ? p1 * (dp[e + 1] * a.scale - Drs) : 0.f;
-            pk[e >> 1] = pack_bf16(d0, d1);
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const float p0 = ex2(s[e] * a.scale_log2 - l2), p1 = ex2(s[e + 1] * a.scale_log2 - l2);
-            pk[e >> 1] = pack_bf16(p0 * (dp[e] * a.scale - Drs), p1 * (dp[e + 1] * a.scale - Drs));
-          }
-        }
-        // dS (bf16, two per column) overwrites this group's own S columns already consumed
-        tmem_st16(tS + 64 * g + 16 * (c - 2 * g), pk);
+      for (int e = 0; e < 32; e += 2) {
+        const float2 y = __ffma2_rn(make_float2(s[e], s[e + 1]), sl2, make_float2(nl2, nl2));
+        const float2 d = __fmul2_rn(make_float2(ex2(y.x), ex2(y.y)),
+                                    __ffma2_rn(make_float2(dp[e], dp[e + 1]), sc2, make_float2(nD, nD)));
+        pk[e >> 1] = pack_bf16(d.x, d.y);
       }
+      tmem_st16(tSi, pk);                                    // dS (bf16, two per column) over this thread's own S columns
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->ds_full);
@@ -521,127 +571,117 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
         store_pending = false;
       }
     }
-    kc += n_kt;
+    const int last = (kc + n_kt - 1) % DQ_NK;                // the slot of K_cb
+    kc += n_kt + (it.has_state ? 1 : 0);
 
+    float ph[32];                                            // phi(q), this thread's columns
     if (it.has_rla) {
-      const int last = (kc - 1) & 1;
       WAIT_OR_RETURN(bars->o_done, co & 1);                    // every window product done: K_cb is no longer read raw
       ++co;
       {
-        const int t2 = g * 128 + r;                              // two threads per key row
-        unsigned char* kh = smem + DQ_OFF_K + last * TILE_BYTES + (t2 & 1) * HALF_BYTES;
-        feature_map_pair_any(kh, kh, t2 >> 1, a.phi);
+        const int t4 = part * TILE + r, krow = t4 >> 2;        // four threads per key row
+        unsigned char* kp = smem + DQ_OFF_K + last * TILE_BYTES + krow * 128;
+        feature_map_quad(kp, kp, HALF_BYTES, krow, t4 & 3, a.phi);
       }
       fence_proxy_async_smem();
       mbar_arrive(&bars->phik_ready);
       WAIT_OR_RETURN(bars->s_full, cs & 1);
       tc_fence_after();
-#pragma unroll 1
-      for (int c = 2 * g; c < 2 * g + 2; ++c) {
+      {
         float x[32];
-        tmem_ld32(tS + 32 * c, x);
+        tmem_ld32(tS, x);
         tmem_wait_ld();
-        const uint32_t keep = bits_lt(r - 32 * c);               // residual keys of row r in this chunk: j < r
+        const uint32_t keep = bits_lt(r - 32 * part);            // residual keys of row r in this chunk: j < r
         uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 32; e += 2)
           pk[e >> 1] = pack_bf16((keep >> e) & 1u ? x[e] : 0.f, (keep >> (e + 1)) & 1u ? x[e + 1] : 0.f);
-        tmem_st16(tS + 64 * g + 16 * (c - 2 * g), pk);
+        tmem_st16(tS, pk);
       }
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->ds_full);
       ++cs;
-      ++kc;
+      // phi(q), while the last products run (for the element-wise maps q itself)
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, 4 * part + cc));
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          ph[8 * cc + 2 * e] = __uint_as_float(w[e] << 16);
+          ph[8 * cc + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+        }
+      }
+      if (soft) {
+        float all[4];
+        exchange(max32(ph), all);
+        const float nml = -fmaxf(fmaxf(all[0], all[1]), fmaxf(all[2], all[3])) * LOG2E;
+        float2 s0 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          const float2 y = __ffma2_rn(make_float2(ph[e], ph[e + 1]), make_float2(LOG2E, LOG2E), make_float2(nml, nml));
+          ph[e] = ex2(y.x);
+          ph[e + 1] = ex2(y.y);
+          s0 = __fadd2_rn(s0, make_float2(ph[e], ph[e + 1]));
+        }
+        row_sync();
+        exchange(s0.x + s0.y, all);
+        const float inv = 1.f / ((all[0] + all[1]) + (all[2] + all[3]));
+#pragma unroll
+        for (int e = 0; e < 32; ++e) ph[e] *= inv;
+        row_sync();
+      }
     }
 
     // ---- dq = dQ + phi(q) * (dphi_q - <dphi_q, phi(q)>) -----------------------------------
-    const int co_final = co++;
-    if (g != 0) continue;                                      // group 0 alone runs the epilogue
-    WAIT_OR_RETURN(bars->o_done, co_final & 1);
+    WAIT_OR_RETURN(bars->o_done, co & 1);
+    ++co;
     tc_fence_after();
-    float m = 0.f, inv = 0.f, dot = 0.f;
-    const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
+    float dot = 0.f;
     if (it.has_rla && soft) {
-      m = -INFINITY;
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, c));
-        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 f = __bfloat1622float2(h[e]);
-          m = fmaxf(m, fmaxf(f.x, f.y));
-        }
-      }
-      const float ml = m * LOG2E;
-      float sum = 0.f, du = 0.f;
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        float df[32];
-        tmem_ld32(tF + 32 * c, df);
+      for (int c = 0; c < 2; ++c) {
+        float df[16];
+        tmem_ld16(tF + 16 * c, df);
         tmem_wait_ld();
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, 4 * c + cc));
-          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 f = __bfloat1622float2(h[e]);
-            const float e0 = ex2(f.x * LOG2E - ml), e1 = ex2(f.y * LOG2E - ml);
-            sum += e0 + e1;
-            du += e0 * df[8 * cc + 2 * e] + e1 * df[8 * cc + 2 * e + 1];
-          }
-        }
+        for (int e = 0; e < 16; ++e) dot += ph[16 * c + e] * df[e];
       }
-      inv = 1.f / sum;
-      dot = du * inv;
-      m = ml;
+      float all[4];
+      exchange(dot, all);
+      dot = (all[0] + all[1]) + (all[2] + all[3]);
     }
     // every product has completed: this item's Q buffer stages the output, each thread
-    // rewriting its own row in place, for one TMA store
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      float x[32], df[32];
-      tmem_ld32(tQ + 32 * c, x);
-      if (it.has_rla) tmem_ld32(tF + 32 * c, df);
-      tmem_wait_ld();
+    // rewriting its own columns in place, for one TMA store
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float x[16];
+      tmem_ld16(tQ + 16 * c, x);
       if (it.has_rla) {
+        float df[16];
+        tmem_ld16(tF + 16 * c, df);
+        tmem_wait_ld();
 #pragma unroll
-        for (int cc = 0; cc < 4; ++cc) {
-          const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, 4 * c + cc));
-          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 f = __bfloat1622float2(h[e]);
-            if (soft) {
-              const float e0 = ex2(f.x * LOG2E - m) * inv, e1 = ex2(f.y * LOG2E - m) * inv;
-              x[8 * cc + 2 * e] += e0 * (df[8 * cc + 2 * e] - dot);
-              x[8 * cc + 2 * e + 1] += e1 * (df[8 * cc + 2 * e + 1] - dot);
-            } else {
-              // element-wise maps: ReLU passes the gradient where q > 0, the identity everywhere
-              const bool relu = (a.phi == RATTN_PHI_RELU);
-              x[8 * cc + 2 * e] += (relu && !(f.x > 0.f)) ? 0.f : df[8 * cc + 2 * e];
-              x[8 * cc + 2 * e + 1] += (relu && !(f.y > 0.f)) ? 0.f : df[8 * cc + 2 * e + 1];
-            }
-          }
+        for (int e = 0; e < 16; ++e) {
+          // element-wise maps: ReLU passes the gradient where q > 0, the identity everywhere
+          if (soft) x[e] += ph[16 * c + e] * (df[e] - dot);
+          else x[e] += (a.phi == RATTN_PHI_RELU && !(ph[16 * c + e] > 0.f)) ? 0.f : df[e];
         }
+      } else {
+        tmem_wait_ld();
       }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint4 u;
-        u.x = pack_bf16(x[8 * e + 0], x[8 * e + 1]);
-        u.y = pack_bf16(x[8 * e + 2], x[8 * e + 3]);
-        u.z = pack_bf16(x[8 * e + 4], x[8 * e + 5]);
-        u.w = pack_bf16(x[8 * e + 6], x[8 * e + 7]);
-        *reinterpret_cast<uint4*>(sQ + swz(r, 4 * c + e)) = u;
-      }
+      for (int e = 0; e < 2; ++e)
+        *reinterpret_cast<uint4*>(sQ + swz(r, 4 * part + 2 * c + e)) =
+            make_uint4(pack_bf16(x[8 * e + 0], x[8 * e + 1]), pack_bf16(x[8 * e + 2], x[8 * e + 3]),
+                       pack_bf16(x[8 * e + 4], x[8 * e + 5]), pack_bf16(x[8 * e + 6], x[8 * e + 7]));
     }
     tc_fence_before();
     mbar_arrive(&bars->acc_free);          // the dQ / dphi_q columns have been read
     fence_proxy_async_smem();
-    rows_sync();
-    if (r == 0) {
+    asm volatile("bar.sync 1, 512;" ::: "memory");
+    if (part == 0 && r == 0) {
       // nobody waits for the store to read the Q buffer out: the loader refills that buffer two items
       // on, after q_read, which this thread confirms once the next item's first key tile is behind it
       store_tile(&tm.dq, sQ, it.q0, it.bh_q);
@@ -663,24 +703,27 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     return;
   }
   if (tid == 0) {
-    sched_init(&bars->sched, 256 + 1);
-    mbar_init(&bars->qg_full, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&bars->kv_full[i], 1);
-      mbar_init(&bars->kv_free[i], 1);
+    sched_init(&bars->sched, 32 * DQ_ROW_WARPS + 1);
+    mbar_init(&bars->q_full, 1);
+    mbar_init(&bars->g_full, 1);
+    mbar_init(&bars->g_free, 1);
+    mbar_init(&bars->v_full, 1);
+    mbar_init(&bars->v_free, 1);
+    for (int i = 0; i < DQ_NK; ++i) {
+      mbar_init(&bars->k_full[i], 1);
+      mbar_init(&bars->k_free[i], 1);
     }
     mbar_init(&bars->s_full, 1);
-    mbar_init(&bars->ds_full, 256);
-    mbar_init(&bars->phik_ready, 256);
+    mbar_init(&bars->ds_full, 32 * DQ_ROW_WARPS);
+    mbar_init(&bars->phik_ready, 32 * DQ_ROW_WARPS);
     mbar_init(&bars->o_done, 1);
-    mbar_init(&bars->g_free, 1);
-    mbar_init(&bars->acc_free, 128);
+    mbar_init(&bars->acc_free, 32 * DQ_ROW_WARPS);
     mbar_init(&bars->q_read, 1);
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
     fence_mbar_init();
   }
-  if (warp == 8) {
+  if (warp == DQ_ROW_WARPS) {
     tmem_alloc(&bars->tmem_base, 512);
     tmem_relinquish();
   }
@@ -688,7 +731,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   // A kernel that does not read dq may take the SMs that run out of items.  (Behind the wait: the terms of the reverse
   // states start on this signal alone, and what they read is complete only then.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (tid == 288) {
+  if (warp == DQ_ROW_WARPS + 1 && (tid & 31) == 0) {
     prefetch_map(&tm.q);
     prefetch_map(&tm.k);
     prefetch_map(&tm.v);
@@ -702,23 +745,26 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
 
+  // registers follow the work: 512 x 104 + 128 x 64 = 640 x 96, the CTA's allocation
   bool ok = true;
-  if (warp < 8) {
+  if (warp < DQ_ROW_WARPS) setmaxnreg_inc<104>();
+  else setmaxnreg_dec<64>();
+  if (warp < DQ_ROW_WARPS) {
     ok = dq_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127, n_qt);
-  } else if (warp == 8) {
+  } else if (warp == DQ_ROW_WARPS) {
     ok = dq_mma(a, smem, bars, tmem, n_qt);
     if (!ok) {
       mma_commit(&bars->drain);
       for (int it = 0; it < (1 << 16) && !mbar_try_wait(&bars->drain, 0); ++it) {}
     }
-  } else {
+  } else if (warp == DQ_ROW_WARPS + 1) {
     ok = dq_loader(tm, a, smem, bars, n_items, n_qt);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
   if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == DQ_ROW_WARPS) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
   }
