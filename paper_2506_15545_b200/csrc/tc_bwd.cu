@@ -306,23 +306,23 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
 // Persistent: one CTA per SM walks a list of (query head, query tile) items, so that an item's
 // first loads are in flight while the previous item's epilogue drains (at w = 512 the fixed
 // cost per tile -- first TMA touch, output staging -- is larger than the band itself).
-//   loader warp   Q (two buffers, alternating), K tiles through a ring of three slots, V tiles through one buffer, g_s;
-//                 for the residual part g_r follows in g_s's buffer and the stored state in the K ring
+//   loader warp   Q, g_s, K tiles through a ring of three slots, V tiles through two; for the residual part g_r follows in
+//                 g_s's buffer and the stored state in the K ring.  dQ leaves through the slot of the item's last K tile.
 //   MMA warp      per key tile S = Q K^T, dP = g_s V^T; after the row threads have overwritten S
 //                 with dS (bf16, in TMEM): dQ += dS K.  Then the residual part.
 //   row threads   512: query row = TMEM lane, and a quarter of the 128 columns
 // TMEM holds S twice (the second buffer is dphi_q's, which only the residual part needs), so that S of the next key tile
 // is formed beside the row threads' work; dP of the next tile goes out the moment they are done, ahead of this tile's dQ.
-// V is read by dP alone, early in its step, K by S in the step before and by dQ at the end of it: three slots of K and one
-// of V keep the loads (1750 cycles each) off the path, two of each put one into every step (4150 cycles a step).
+// K is read by S in the step before its own and by dQ at the end of it, V by dP early in its step: three slots of K and two
+// of V keep the loads (1750 cycles each) off the path; two of each, released together, put one into every step (4150 cycles
+// a step), and so did a single V (3800).  Q is read to the end of the window loop, phi(q) being kept in registers.
 // With one buffer, two threads per row and the epilogue on 128 of them, an item of 5 key tiles took 31k cycles.
 // All barriers run on with phase counters that every role advances in the same way.
-constexpr int DQ_OFF_Q = 0;                 // Q buffer 0
+constexpr int DQ_NK = 3, DQ_NV = 2;
+constexpr int DQ_OFF_Q = 0;
 constexpr int DQ_OFF_G = 1 * TILE_BYTES;
-constexpr int DQ_NK = 3;
 constexpr int DQ_OFF_K = 2 * TILE_BYTES;   // DQ_NK slots
-constexpr int DQ_OFF_V = 5 * TILE_BYTES;
-constexpr int DQ_OFF_Q1 = 6 * TILE_BYTES;  // Q buffer 1
+constexpr int DQ_OFF_V = 5 * TILE_BYTES;   // DQ_NV slots
 constexpr int DQ_OFF_BAR = 7 * TILE_BYTES;
 constexpr int DQ_OFF_EX = DQ_OFF_BAR + 384;   // one word per row thread
 constexpr int DQ_ROW_WARPS = 16;
@@ -330,8 +330,8 @@ constexpr int DQ_SMEM = DQ_OFF_EX + 32 * DQ_ROW_WARPS * 4;
 constexpr int DQ_THREADS = 32 * (DQ_ROW_WARPS + 4);   // row threads, MMA warp, loader warp (and two idle)
 
 struct DqBars {
-  uint64_t q_full, g_full, g_free, v_full, v_free, k_full[DQ_NK], k_free[DQ_NK], s_full, ds_full, phik_ready, o_done,
-      acc_free, q_read, drain;
+  uint64_t q_full, q_free, g_full, g_free, v_full[DQ_NV], v_free[DQ_NV], k_full[DQ_NK], k_free[DQ_NK], s_full, ds_full,
+      phik_ready, o_done, acc_free, out_staged, drain;
   SchedRing sched;
   uint32_t tmem_base;
   int abort;
@@ -368,7 +368,20 @@ struct DqMaps {
 };
 
 __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, int n_items, int n_qt) {
-  int kc = 0, vc = 0, gc = 0, n = 0;                       // uses of the K ring, the V and the g buffer; items so far
+  int kc = 0, vc = 0, gc = 0, n = 0;                       // uses of the K and V rings and of the g buffer; items so far
+  // dQ of an item is staged in the slot of its last K tile, from where this warp stores it before it refills that slot
+  int out_use = -1, out_row = 0, out_z = 0, out_n = 0;     // the K use and the item whose dQ is still to go
+  auto store_out = [&]() -> bool {
+    WAIT_OR_RETURN_W(bars->out_staged, out_n & 1);
+    if ((threadIdx.x & 31) == 0) {
+      store_tile(&tm.dq, smem + DQ_OFF_K + out_use % DQ_NK * TILE_BYTES, out_row, out_z);
+      tma_store_commit();
+      tma_store_wait_read();
+    }
+    __syncwarp();
+    out_use = -1;
+    return true;
+  };
   for (;; ++n) {
     int idx;
     if (!sched_draw(&bars->sched, a.counter, n_items, n, &bars->abort, &idx)) return false;
@@ -378,6 +391,7 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
       st = kc % DQ_NK;
       const int use = kc / DQ_NK;
       if (use >= 1) WAIT_OR_RETURN_W(bars->k_free[st], (use - 1) & 1);
+      if (out_use >= 0 && kc == out_use + DQ_NK && !store_out()) return false;
       ++kc;
       return true;
     };
@@ -395,22 +409,20 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
       ++gc;
       return true;
     };
-    // The barrier's previous phase must be over before this item arrives on it: after a short
-    // item the loader gets here while that item's Q is still in flight.
-    if (n >= 1) WAIT_OR_RETURN_W(bars->q_full, (n - 1) & 1);
+    if (n >= 1) WAIT_OR_RETURN_W(bars->q_free, (n - 1) & 1);
     mbar_arrive_expect_tx(&bars->q_full, TILE_BYTES);
-    // Q into the buffer last used two items ago: free once its dQ, staged there by that item's epilogue, has left.  (Not
-    // acc_free as well: the item in between may have completed that barrier a second time before this warp looks, and
-    // then the wait, which sees the parity alone, would be for a completion that needs this load.)
-    if (n >= 2) WAIT_OR_RETURN_W(bars->q_read, (n - 2) & 1);
-    load_tile(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q), &tm.q, &bars->q_full, it.q0, it.bh_q);
-    // in the order in which their places become free: V_i behind dP_(i-1), K_(i+1) behind dQ_(i-2)
+    load_tile(smem + DQ_OFF_Q, &tm.q, &bars->q_full, it.q0, it.bh_q);
     if (!load_k(0) || !load_g(&tm.gs)) return false;
+    int last_use = kc - 1;
     for (int i = 0; i < it.n_kt; ++i, ++vc) {
-      if (vc >= 1) WAIT_OR_RETURN_W(bars->v_free, (vc - 1) & 1);
-      mbar_arrive_expect_tx(&bars->v_full, TILE_BYTES);
-      load_tile(smem + DQ_OFF_V, &tm.v, &bars->v_full, it.q0 - i * TILE, it.bh_kv);
-      if (i + 1 < it.n_kt && !load_k(i + 1)) return false;
+      const int st = vc % DQ_NV, use = vc / DQ_NV;
+      if (use >= 1) WAIT_OR_RETURN_W(bars->v_free[st], (use - 1) & 1);
+      mbar_arrive_expect_tx(&bars->v_full[st], TILE_BYTES);
+      load_tile(smem + DQ_OFF_V + st * TILE_BYTES, &tm.v, &bars->v_full[st], it.q0 - i * TILE, it.bh_kv);
+      if (i + 1 < it.n_kt) {
+        if (!load_k(i + 1)) return false;
+        last_use = kc - 1;
+      }
     }
     if (it.has_rla) {
       if (it.has_state) {
@@ -421,12 +433,20 @@ __device__ bool dq_loader(const DqMaps& tm, const BwdArgs& a, unsigned char* sme
       }
       if (!load_g(&tm.gr)) return false;
     }
+    if (out_use >= 0 && !store_out()) return false;        // a short item has not come to that slot
+    out_use = last_use;
+    out_row = it.q0;
+    out_z = it.bh_q;
+    out_n = n;
   }
+  if (out_use >= 0 && !store_out()) return false;
+  if ((threadIdx.x & 31) == 0) tma_store_wait();           // the last store has completed
   return true;
 }
 
 __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int n_qt) {
-  const uint32_t sG = smem_u32(smem + DQ_OFF_G), sK = smem_u32(smem + DQ_OFF_K), sV = smem_u32(smem + DQ_OFF_V);
+  const uint32_t sQ = smem_u32(smem + DQ_OFF_Q), sG = smem_u32(smem + DQ_OFF_G);
+  const uint32_t sK = smem_u32(smem + DQ_OFF_K), sV = smem_u32(smem + DQ_OFF_V);
   const uint32_t tS = tmem, tP = tmem + 128, tQ = tmem + 256, tF = tmem + 384;
   constexpr uint32_t idesc_ts = instr_desc(128, 128, 0, 1);
   int kc = 0, vc = 0, gc = 0, n = 0, cs = 0, cr = 0;       // K, V and g uses, items, score hand-overs, residual items
@@ -435,17 +455,21 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
     if (!sched_read_warp(&bars->sched, n, &bars->abort, &idx)) return false;
     if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
-    const uint32_t sQ = smem_u32(smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q));
     auto k_landed = [&](int use) -> bool {
       WAIT_OR_RETURN_W(bars->k_full[use % DQ_NK], (use / DQ_NK) & 1);
       return true;
     };
+    auto v_landed = [&]() -> bool {
+      WAIT_OR_RETURN_W(bars->v_full[vc % DQ_NV], (vc / DQ_NV) & 1);
+      return true;
+    };
     // dP = g_s V^T of key tile i, with the releases behind it (the last tile's V is read once more by the residual part)
     auto dp_products = [&](int i) {
-      mma_kk(tP, sG, sV, false);
+      mma_kk(tP, sG, sV + vc % DQ_NV * TILE_BYTES, false);
       mma_commit(&bars->s_full);
-      if (!(it.has_rla && i + 1 == it.n_kt)) mma_commit(&bars->v_free);
+      if (!(it.has_rla && i + 1 == it.n_kt)) mma_commit(&bars->v_free[vc % DQ_NV]);
       if (i + 1 == it.n_kt) mma_commit(&bars->g_free);
+      ++vc;
     };
     WAIT_OR_RETURN_W(bars->q_full, n & 1);
     if (!k_landed(kc)) return false;
@@ -453,8 +477,7 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
     mma_kk(tS, sQ, sK + kc % DQ_NK * TILE_BYTES, false);   // S = Q K^T
     WAIT_OR_RETURN_W(bars->g_full, gc & 1);
     ++gc;
-    WAIT_OR_RETURN_W(bars->v_full, vc & 1);
-    ++vc;
+    if (!v_landed()) return false;
     tc_fence_after();
     dp_products(0);
     for (int i = 0; i < it.n_kt; ++i, ++kc, ++cs) {
@@ -466,8 +489,7 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
       if (more) {
         tc_fence_after();
         mma_kk(tSn, sQ, sK + (kc + 1) % DQ_NK * TILE_BYTES, false);   // the next tile's S, while the row threads work on this one's
-        WAIT_OR_RETURN_W(bars->v_full, vc & 1);
-        ++vc;
+        if (!v_landed()) return false;
       }
       WAIT_OR_RETURN_W(bars->ds_full, cs & 1);
       tc_fence_after();
@@ -480,14 +502,14 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
       // the products that overwrite what these read follow them in the tensor pipe, which runs in issue order
     }
     if (it.has_rla) {
-      const int last_st = (kc - 1) % DQ_NK, xs = kc % DQ_NK;   // K_cb; the stored state
+      const int last_st = (kc - 1) % DQ_NK, xs = kc % DQ_NK, vs = (vc - 1) % DQ_NV;   // K_cb; the stored state; V_cb
       mma_commit(&bars->o_done);                           // (interim) every window product done: K_cb may be rewritten
       WAIT_OR_RETURN_W(bars->g_full, gc & 1);              // g_r
       ++gc;
       tc_fence_after();
-      mma_kk(tS, sG, sV, false);                           // dA = g_r V_cb^T
+      mma_kk(tS, sG, sV + vs * TILE_BYTES, false);         // dA = g_r V_cb^T
       mma_commit(&bars->s_full);
-      mma_commit(&bars->v_free);
+      mma_commit(&bars->v_free[vs]);
       if (it.has_state) {
         if (!k_landed(kc)) return false;
         tc_fence_after();
@@ -511,13 +533,13 @@ __device__ bool dq_mma(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint
 }
 
 // Row thread (r, part): query row r = TMEM lane, columns 32 part .. 32 part + 31.
-__device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int part, int r,
+__device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uint32_t tmem, int part, int r,
                         int n_qt) {
   const uint32_t lane_off = ((uint32_t)((r & ~31) << 16)) + 32 * part;
   const uint32_t tS = tmem + lane_off, tP = tmem + 128 + lane_off, tQ = tmem + 256 + lane_off,
                  tF = tmem + 384 + lane_off;
   int kc = 0, n = 0, cs = 0, co = 0;                       // ring uses, items, score hand-overs, o_done completions
-  bool store_pending = false;                              // this thread issued a dQ store whose read-out it has not confirmed
+  const unsigned char* sQ = smem + DQ_OFF_Q;
   const bool soft = (a.phi == RATTN_PHI_SOFTMAX);
   const float2 sl2 = make_float2(a.scale_log2, a.scale_log2), sc2 = make_float2(a.scale, a.scale);
   // one value per thread, shared by the four threads of a row (the four warps of the same 32 rows meet; sync again before
@@ -536,7 +558,6 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
     if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     const int n_kt = it.n_kt;
-    unsigned char* sQ = smem + ((n & 1) ? DQ_OFF_Q1 : DQ_OFF_Q);
     const int t = it.q0 + r;
     const bool live = t < a.T;
     const size_t row = (size_t)it.bh_q * a.T + t;
@@ -565,17 +586,45 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&bars->ds_full);
-      if (i == 0 && store_pending) {                         // the previous item's dQ has left its Q buffer by now
-        tma_store_wait_read();
-        mbar_arrive(&bars->q_read);
-        store_pending = false;
-      }
     }
     const int last = (kc + n_kt - 1) % DQ_NK;                // the slot of K_cb
     kc += n_kt + (it.has_state ? 1 : 0);
 
     float ph[32];                                            // phi(q), this thread's columns
     if (it.has_rla) {
+      // phi(q), while the last window products run (for the element-wise maps q itself)
+#pragma unroll
+      for (int cc = 0; cc < 4; ++cc) {
+        const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, 4 * part + cc));
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          ph[8 * cc + 2 * e] = __uint_as_float(w[e] << 16);
+          ph[8 * cc + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+        }
+      }
+    }
+    mbar_arrive(&bars->q_free);                              // every S has been formed
+    if (it.has_rla) {
+      if (soft) {
+        float all[4];
+        exchange(max32(ph), all);
+        const float nml = -fmaxf(fmaxf(all[0], all[1]), fmaxf(all[2], all[3])) * LOG2E;
+        float2 s0 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+          const float2 y = __ffma2_rn(make_float2(ph[e], ph[e + 1]), make_float2(LOG2E, LOG2E), make_float2(nml, nml));
+          ph[e] = ex2(y.x);
+          ph[e + 1] = ex2(y.y);
+          s0 = __fadd2_rn(s0, make_float2(ph[e], ph[e + 1]));
+        }
+        row_sync();
+        exchange(s0.x + s0.y, all);
+        const float inv = 1.f / ((all[0] + all[1]) + (all[2] + all[3]));
+#pragma unroll
+        for (int e = 0; e < 32; ++e) ph[e] *= inv;
+        row_sync();
+      }
       WAIT_OR_RETURN(bars->o_done, co & 1);                    // every window product done: K_cb is no longer read raw
       ++co;
       {
@@ -602,36 +651,6 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
       tc_fence_before();
       mbar_arrive(&bars->ds_full);
       ++cs;
-      // phi(q), while the last products run (for the element-wise maps q itself)
-#pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        const uint4 u = *reinterpret_cast<const uint4*>(sQ + swz(r, 4 * part + cc));
-        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          ph[8 * cc + 2 * e] = __uint_as_float(w[e] << 16);
-          ph[8 * cc + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-        }
-      }
-      if (soft) {
-        float all[4];
-        exchange(max32(ph), all);
-        const float nml = -fmaxf(fmaxf(all[0], all[1]), fmaxf(all[2], all[3])) * LOG2E;
-        float2 s0 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          const float2 y = __ffma2_rn(make_float2(ph[e], ph[e + 1]), make_float2(LOG2E, LOG2E), make_float2(nml, nml));
-          ph[e] = ex2(y.x);
-          ph[e + 1] = ex2(y.y);
-          s0 = __fadd2_rn(s0, make_float2(ph[e], ph[e + 1]));
-        }
-        row_sync();
-        exchange(s0.x + s0.y, all);
-        const float inv = 1.f / ((all[0] + all[1]) + (all[2] + all[3]));
-#pragma unroll
-        for (int e = 0; e < 32; ++e) ph[e] *= inv;
-        row_sync();
-      }
     }
 
     // ---- dq = dQ + phi(q) * (dphi_q - <dphi_q, phi(q)>) -----------------------------------
@@ -652,8 +671,8 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
       exchange(dot, all);
       dot = (all[0] + all[1]) + (all[2] + all[3]);
     }
-    // every product has completed: this item's Q buffer stages the output, each thread
-    // rewriting its own columns in place, for one TMA store
+    // every product has completed: the slot of the last K tile stages the output, which the loader warp stores
+    unsigned char* sOut = smem + DQ_OFF_K + last * TILE_BYTES;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       float x[16];
@@ -673,23 +692,16 @@ __device__ bool dq_rows(const DqMaps& tm, const BwdArgs& a, unsigned char* smem,
       }
 #pragma unroll
       for (int e = 0; e < 2; ++e)
-        *reinterpret_cast<uint4*>(sQ + swz(r, 4 * part + 2 * c + e)) =
+        *reinterpret_cast<uint4*>(sOut + swz(r, 4 * part + 2 * c + e)) =
             make_uint4(pack_bf16(x[8 * e + 0], x[8 * e + 1]), pack_bf16(x[8 * e + 2], x[8 * e + 3]),
                        pack_bf16(x[8 * e + 4], x[8 * e + 5]), pack_bf16(x[8 * e + 6], x[8 * e + 7]));
     }
     tc_fence_before();
     mbar_arrive(&bars->acc_free);          // the dQ / dphi_q columns have been read
     fence_proxy_async_smem();
-    asm volatile("bar.sync 1, 512;" ::: "memory");
-    if (part == 0 && r == 0) {
-      // nobody waits for the store to read the Q buffer out: the loader refills that buffer two items
-      // on, after q_read, which this thread confirms once the next item's first key tile is behind it
-      store_tile(&tm.dq, sQ, it.q0, it.bh_q);
-      tma_store_commit();
-      store_pending = true;
-    }
+    mbar_arrive(&bars->out_staged);
+    if (it.has_rla && soft) row_sync();                      // the last exchanged value has been read
   }
-  if (store_pending) tma_store_wait();     // the last store has completed before the CTA may go
   return true;
 }
 
@@ -705,10 +717,13 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   if (tid == 0) {
     sched_init(&bars->sched, 32 * DQ_ROW_WARPS + 1);
     mbar_init(&bars->q_full, 1);
+    mbar_init(&bars->q_free, 32 * DQ_ROW_WARPS);
     mbar_init(&bars->g_full, 1);
     mbar_init(&bars->g_free, 1);
-    mbar_init(&bars->v_full, 1);
-    mbar_init(&bars->v_free, 1);
+    for (int i = 0; i < DQ_NV; ++i) {
+      mbar_init(&bars->v_full[i], 1);
+      mbar_init(&bars->v_free[i], 1);
+    }
     for (int i = 0; i < DQ_NK; ++i) {
       mbar_init(&bars->k_full[i], 1);
       mbar_init(&bars->k_free[i], 1);
@@ -718,7 +733,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     mbar_init(&bars->phik_ready, 32 * DQ_ROW_WARPS);
     mbar_init(&bars->o_done, 1);
     mbar_init(&bars->acc_free, 32 * DQ_ROW_WARPS);
-    mbar_init(&bars->q_read, 1);
+    mbar_init(&bars->out_staged, 32 * DQ_ROW_WARPS);
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
     fence_mbar_init();
@@ -750,7 +765,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
   if (warp < DQ_ROW_WARPS) setmaxnreg_inc<104>();
   else setmaxnreg_dec<64>();
   if (warp < DQ_ROW_WARPS) {
-    ok = dq_rows(tm, a, smem, bars, tmem, warp >> 2, tid & 127, n_qt);
+    ok = dq_rows(a, smem, bars, tmem, warp >> 2, tid & 127, n_qt);
   } else if (warp == DQ_ROW_WARPS) {
     ok = dq_mma(a, smem, bars, tmem, n_qt);
     if (!ok) {
