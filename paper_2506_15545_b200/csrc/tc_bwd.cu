@@ -1411,12 +1411,12 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   // sum that walks the query tiles from the last one down to wt+1.  The dq kernel does not read them, so the two share
   // the GPU.  A serial chain (one CTA per K/V head) goes first, and the dq kernel runs beside it on the other SMs; that
   // costs least as long as the chain is over by then (1.4 us per tile and query head, measured, against about
-  // 2 us per key tile + 5 us for a dq item; up to 15 % longer is still cheaper than the other way).  Where it would
+  // 1.45 us per key tile + 5 us for a dq item; up to 15 % longer is still cheaper than the other way).  Where it would
   // outlast the dq kernel, its terms are formed in parallel behind that kernel, on the SMs it runs out of items on: at
   // 1 x 16/4 heads, T = 1111, w = 128 the chain took 46 us on four SMs beside a dq kernel of 16 us, the terms and their
   // sum end 11 us behind it.  With a chain on more than half of the SMs there is nothing to share.
   const int n_r = rla_on && a.mode != RATTN_MODE_FULL_CAUSAL ? n_qt - wt - 1 : 0;
-  const long long chain_ns = 1400ll * n_r * a.group, dq_ns = 1000ll * n_qt * (long long)nq * (2 * (wt + 1) + 5) / n_sm;
+  const long long chain_ns = 1400ll * n_r * a.group, dq_ns = 10ll * n_qt * (long long)nq * (145 * (wt + 1) + 500) / n_sm;
   const bool few_heads = 2 * (int)nkv <= n_sm;
   const bool parallel_terms = n_r > 0 && a.rdelta != nullptr && few_heads && 100 * chain_ns > 115 * dq_ns;
   const bool chain_beside = n_r > 0 && !parallel_terms && few_heads;
