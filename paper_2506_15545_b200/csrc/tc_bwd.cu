@@ -71,7 +71,10 @@ struct BwdArgs {
 // per-row statistics; bound by HBM.  The unit is a chunk of 32 rows of one head (8 KB per tensor,
 // contiguous), which travels global -> shared -> global as bulk asynchronous copies through a ring
 // of stages, so the bytes in flight do not depend on where the warps are; the rows are transformed
-// in place in shared memory (g_s over o_swa, g_r over o_rla).  Eight neighbouring lanes hold a row:
+// in place in shared memory (g_s over o_swa, g_r over o_rla).  The warps meet only at the ring's barriers and take
+// turns with the copies: chunk n is stored, and its stage refilled, by warp n mod 8 (with all of that on one warp
+// behind a __syncthreads per chunk, that warp's path, 5500 cycles a chunk, was everybody's).  GAINS: without gains
+// neither they nor the sums of their gradients take registers.  Eight neighbouring lanes hold a row:
 // lane l has features [8l, 8l+8) and [64+8l, 64+8l+8).  Every CTA takes an equal contiguous share of
 // the chunks (head-major), so it meets few heads and keeps its gain-gradient sums in registers.
 // With n = o / r (r the rms incl. eps), gh = dy * gain, A = gh . o:
@@ -105,11 +108,13 @@ __device__ __forceinline__ void unpack8(const unsigned char* p, float (&x)[8]) {
   }
 }
 
+template <bool GAINS>
 __global__ void __launch_bounds__(PREP_THREADS, 2)
 tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ CUtensorMap dy_map) {
   extern __shared__ __align__(128) unsigned char psm[];
   uint64_t* full = reinterpret_cast<uint64_t*>(psm + PREP_STAGES * 3 * PREP_CHUNK);
-  volatile int* abort = reinterpret_cast<volatile int*>(full + PREP_STAGES);
+  uint64_t* done = full + PREP_STAGES;                              // the chunk in the stage has been transformed
+  volatile int* abort = reinterpret_cast<volatile int*>(done + PREP_STAGES);
   const int tid = threadIdx.x, l = tid & 7, row = tid >> 3;
   const int cph = a.t_pad / PREP_ROWS;                              // chunks per head
   const long long n_all = (long long)a.n_heads * cph;
@@ -118,7 +123,10 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
 
   if (tid == 0) {
     prefetch_tensormap(&dy_map);
-    for (int i = 0; i < PREP_STAGES; ++i) mbar_init(&full[i], 1);
+    for (int i = 0; i < PREP_STAGES; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&done[i], PREP_THREADS / 32);
+    }
     *abort = 0;
     fence_mbar_init();
   }
@@ -129,35 +137,40 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
 
   // chunk i: head i / cph, rows t0 .. t0 + 31 of it; rows at or beyond T are padding (nothing is copied)
   auto rows_of = [&](int i) { const int t0 = (i % cph) * PREP_ROWS; return a.T - t0 < 0 ? 0 : a.T - t0 < PREP_ROWS ? a.T - t0 : PREP_ROWS; };
-  // Thread 0 keeps the ring fed: the next chunk with data goes into stage (chunks issued so far) % stages.
-  int cursor = lo, n_issued = 0;
-  auto issue_next = [&]() {
-    while (cursor < hi && rows_of(cursor) == 0) ++cursor;
-    if (cursor >= hi) return;
-    const int i = cursor++, rows = rows_of(i);
-    const size_t at = ((size_t)(i / cph) * a.T + (size_t)(i % cph) * PREP_ROWS) * 128;
-    unsigned char* dst = psm + (size_t)(n_issued % PREP_STAGES) * 3 * PREP_CHUNK;
-    uint64_t* bar = &full[n_issued % PREP_STAGES];
-    ++n_issued;
+  // `ahead` is the next chunk with data to ask for, the n_ahead-th of this CTA's; every thread follows it
+  int ahead = lo, n_ahead = 0;
+  auto skip_padding = [&] { while (ahead < hi && rows_of(ahead) == 0) ++ahead; };
+  auto issue_ahead = [&]() {                                        // one thread
+    const int rows = rows_of(ahead), slot = n_ahead % PREP_STAGES;
+    const int bq = ahead / cph, t0 = (ahead - bq * cph) * PREP_ROWS, b = bq / a.H_q, h = bq - b * a.H_q;
+    const size_t at = ((size_t)bq * a.T + t0) * 128;
+    unsigned char* dst = psm + (size_t)slot * 3 * PREP_CHUNK;
+    uint64_t* bar = &full[slot];
     const uint32_t bytes = (uint32_t)rows * 256;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                  ::"r"(smem_u32(bar)), "r"((uint32_t)PREP_CHUNK + bytes * (n_in - 1)) : "memory");
     // dO is the caller's tensor (either head layout): a tiled copy of 32 whole rows, rows beyond T read as zero
-    const int bq_ = i / cph, b_ = bq_ / a.H_q, h_ = bq_ - b_ * a.H_q;
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(&dy_map), "r"(smem_u32(bar)), "r"(0), "r"((i % cph) * PREP_ROWS), "r"(h_), "r"(b_)
+                 ::"r"(smem_u32(dst)), "l"(&dy_map), "r"(smem_u32(bar)), "r"(0), "r"(t0), "r"(h), "r"(b)
                  : "memory");
     const __nv_bfloat16* src[3] = {nullptr, a.o_s, a.o_r};
     for (int k = 1; k < n_in; ++k)
       asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                    ::"r"(smem_u32(dst + k * PREP_CHUNK)), "l"(src[k] + at), "r"(bytes), "r"(smem_u32(bar)) : "memory");
   };
-  if (tid == 0)
-    for (int k = 0; k < PREP_STAGES - 1; ++k) issue_next();
+  for (int k = 0; k < PREP_STAGES; ++k) {
+    skip_padding();
+    if (ahead >= hi) break;
+    if (tid == 0) issue_ahead();
+    ++ahead;
+    ++n_ahead;
+  }
 
   float gs_lo[8], gs_hi[8], gr_lo[8], gr_hi[8], acc_s[16], acc_r[16];
 #pragma unroll
   for (int e = 0; e < 16; ++e) acc_s[e] = acc_r[e] = 0.f;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) gs_lo[e] = gs_hi[e] = gr_lo[e] = gr_hi[e] = 1.f;
   int cur_h = -1;
   auto flush = [&]() {                                              // this CTA's sums for head cur_h
     if (cur_h < 0) return;
@@ -186,7 +199,7 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
       continue;
     }
     const int h = bq % a.H_q;
-    if (h != cur_h) {
+    if (GAINS && h != cur_h) {
       if (a.dgamma_s || a.dgamma_r) flush();
       cur_h = h;
 #pragma unroll
@@ -203,7 +216,9 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
     // the row's log-sum-exp is asked for before the wait, so that its latency passes under it
     const float lse_row = (live && l == 0) ? __ldg(a.lse + (size_t)bq * a.T + t) : 0.f;
     const bool got = mbar_wait_warp(&full[slot], (uint32_t)(n_cons / PREP_STAGES) & 1u, abort);
-    if (got) {
+    ok = got;
+    if (!ok) break;
+    {
       float g_lo[8], g_hi[8], s_lo[8], s_hi[8], r_lo[8], r_hi[8];
       if (live) {
         unpack8(buf, g_lo); unpack8(buf + 128, g_hi);
@@ -254,7 +269,7 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
           *reinterpret_cast<uint4*>(buf + 2 * PREP_CHUNK + 128) = make_uint4(w_hi[0], w_hi[1], w_hi[2], w_hi[3]);
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
+        for (int e = 0; GAINS && e < 8; ++e) {
           acc_s[e] += g_lo[e] * s_lo[e] * is;
           acc_s[8 + e] += g_hi[e] * s_hi[e] * is;
           acc_r[e] += g_lo[e] * r_lo[e] * ir;
@@ -275,31 +290,40 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
       }
       fence_proxy_async_smem();
     }
-    ok = __syncthreads_and(got) != 0;
-    if (!ok) break;
-    if (tid == 0) {
-      const size_t at = ((size_t)bq * a.T + t0) * 128;
-      unsigned char* src = psm + (size_t)slot * 3 * PREP_CHUNK;
-      const uint32_t bytes = (uint32_t)rows * 256;
-      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(a.g_s + at), "r"(smem_u32(src + PREP_CHUNK)), "r"(bytes) : "memory");
-      if (a.rla_on)
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(a.g_r + at), "r"(smem_u32(src + 2 * PREP_CHUNK)), "r"(bytes) : "memory");
-      tma_store_commit();
-      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the stage of the chunk before this one has been read out
-      issue_next();
+    __syncwarp();
+    if ((tid & 31) == 0) mbar_arrive(&done[slot]);
+    skip_padding();
+    if ((tid >> 5) == n_cons % (PREP_THREADS / 32)) {               // this warp's turn with the copies
+      ok = mbar_wait_warp(&done[slot], (uint32_t)(n_cons / PREP_STAGES) & 1u, abort);
+      if (!ok) break;
+      if ((tid & 31) == 0) {
+        const size_t at = ((size_t)bq * a.T + t0) * 128;
+        unsigned char* src = psm + (size_t)slot * 3 * PREP_CHUNK;
+        const uint32_t bytes = (uint32_t)rows * 256;
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(a.g_s + at), "r"(smem_u32(src + PREP_CHUNK)), "r"(bytes) : "memory");
+        if (a.rla_on)
+          asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(a.g_r + at), "r"(smem_u32(src + 2 * PREP_CHUNK)), "r"(bytes) : "memory");
+        tma_store_commit();
+        if (ahead < hi) {
+          tma_store_wait_read();                                    // the stage has been read out
+          issue_ahead();
+        }
+      }
+      __syncwarp();
     }
+    if (ahead < hi) { ++ahead; ++n_ahead; }
     ++n_cons;
   }
-  if (tid == 0) {
-    tma_store_wait();
-    if (!ok) {
-      // give the copies still in flight a bounded time to land before the CTA's memory goes away
-      for (int n = n_cons; n < n_issued; ++n)
-        for (int it = 0; it < kWaitPolls && !mbar_try_wait(&full[n % PREP_STAGES], (uint32_t)(n / PREP_STAGES) & 1u); ++it) {}
-      atomicExch(a.status, RATTN_ERR_TIMEOUT);
+  if ((tid & 31) == 0) tma_store_wait();
+  if (!ok) {
+    // give the copies still in flight a bounded time to land before the CTA's memory goes away
+    if (tid == 0) {
+      for (int n = n_cons; n < n_cons + PREP_STAGES; ++n)
+        for (int it = 0; it < (1 << 14) && !mbar_try_wait(&full[n % PREP_STAGES], (uint32_t)(n / PREP_STAGES) & 1u); ++it) {}
     }
+    if ((tid & 31) == 0) atomicExch(a.status, RATTN_ERR_TIMEOUT);
   }
-  if (ok && (a.dgamma_s || a.dgamma_r)) flush();
+  if (GAINS && ok && (a.dgamma_s || a.dgamma_r)) flush();
 }
 
 // ================================================================================ dq
@@ -1370,14 +1394,15 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
     pa.status = a.status; pa.counters = a.work_counter + 1;
     pa.n_heads = a.B * a.H_q; pa.T = a.T; pa.t_pad = t_pad; pa.H_q = a.H_q; pa.rla_on = rla_on ? 1 : 0;
     pa.eps = a.eps; pa.scale = a.scale;
-    e = allow_smem<tc_bwd_prep_kernel>(PREP_SMEM);
+    const bool gains = a.gamma_swa || a.gamma_rla || a.dgamma_swa || a.dgamma_rla;
+    e = gains ? allow_smem<tc_bwd_prep_kernel<true>>(PREP_SMEM) : allow_smem<tc_bwd_prep_kernel<false>>(PREP_SMEM);
     if (e != cudaSuccess) return e;
     const long long n_chunks_all = (long long)pa.n_heads * (t_pad / PREP_ROWS);
     const int grid = (int)(n_chunks_all < 2ll * n_sm ? n_chunks_all : 2ll * n_sm);
     CUtensorMap dy_map;
     if (!make_row_map(&dy_map, a.dout, a.T, a.H_q, a.B, a.layout, PREP_ROWS)) return cudaErrorInvalidValue;
     KernelTimer kt("tc_bwd_prep", s);
-    e = launch_pdl(tc_bwd_prep_kernel, dim3(grid), dim3(PREP_THREADS), PREP_SMEM, s, !a.dgamma_swa && !a.dgamma_rla, pa, dy_map);
+    e = launch_pdl(gains ? tc_bwd_prep_kernel<true> : tc_bwd_prep_kernel<false>, dim3(grid), dim3(PREP_THREADS), PREP_SMEM, s, !a.dgamma_swa && !a.dgamma_rla, pa, dy_map);
     if (e != cudaSuccess) return e;
   }
   count_launches(1);
