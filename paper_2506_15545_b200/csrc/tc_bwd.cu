@@ -219,67 +219,56 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
     ok = got;
     if (!ok) break;
     {
-      float g_lo[8], g_hi[8], s_lo[8], s_hi[8], r_lo[8], r_hi[8];
+      float g_lo[8], g_hi[8];
       if (live) {
         unpack8(buf, g_lo); unpack8(buf + 128, g_hi);
-        unpack8(buf + PREP_CHUNK, s_lo); unpack8(buf + PREP_CHUNK + 128, s_hi);
-      }
-      if (live && a.rla_on) { unpack8(buf + 2 * PREP_CHUNK, r_lo); unpack8(buf + 2 * PREP_CHUNK + 128, r_hi); }
-      if (!live || !a.rla_on) {
+      } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) r_lo[e] = r_hi[e] = 0.f;
+        for (int e = 0; e < 8; ++e) g_lo[e] = g_hi[e] = 0.f;
       }
-      if (!live) {
+      // one branch after the other (both at once, with gains and sums, do not fit the registers); returns D = g . o
+      auto branch = [&](unsigned char* p, const float (&ga_lo)[8], const float (&ga_hi)[8], float (&acc)[16]) -> float {
+        float o_lo[8], o_hi[8];
+        if (live) {
+          unpack8(p, o_lo); unpack8(p + 128, o_hi);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) g_lo[e] = g_hi[e] = s_lo[e] = s_hi[e] = 0.f;
-      }
-      float ss = 0.f, sr = 0.f, As = 0.f, Ar = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        ss += s_lo[e] * s_lo[e] + s_hi[e] * s_hi[e];
-        sr += r_lo[e] * r_lo[e] + r_hi[e] * r_hi[e];
-        As += g_lo[e] * gs_lo[e] * s_lo[e] + g_hi[e] * gs_hi[e] * s_hi[e];
-        Ar += g_lo[e] * gr_lo[e] * r_lo[e] + g_hi[e] * gr_hi[e] * r_hi[e];
-      }
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-        ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        sr += __shfl_xor_sync(0xffffffffu, sr, o);
-        As += __shfl_xor_sync(0xffffffffu, As, o);
-        Ar += __shfl_xor_sync(0xffffffffu, Ar, o);
-      }
-      const float is = rsqrtf(ss * (1.f / 128.f) + a.eps), ir = rsqrtf(sr * (1.f / 128.f) + a.eps);
-      const float cs = As * is * is * (1.f / 128.f), cr = Ar * ir * ir * (1.f / 128.f);   // mean(gh n) / r
-      if (live) {
-        uint32_t w_lo[4], w_hi[4];
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-          w_lo[e >> 1] = pack_bf16((g_lo[e] * gs_lo[e] - s_lo[e] * cs) * is, (g_lo[e + 1] * gs_lo[e + 1] - s_lo[e + 1] * cs) * is);
-          w_hi[e >> 1] = pack_bf16((g_hi[e] * gs_hi[e] - s_hi[e] * cs) * is, (g_hi[e + 1] * gs_hi[e + 1] - s_hi[e + 1] * cs) * is);
+          for (int e = 0; e < 8; ++e) o_lo[e] = o_hi[e] = 0.f;
         }
-        *reinterpret_cast<uint4*>(buf + PREP_CHUNK) = make_uint4(w_lo[0], w_lo[1], w_lo[2], w_lo[3]);
-        *reinterpret_cast<uint4*>(buf + PREP_CHUNK + 128) = make_uint4(w_hi[0], w_hi[1], w_hi[2], w_hi[3]);
-        if (a.rla_on) {
+        float ss = 0.f, A = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          ss += o_lo[e] * o_lo[e] + o_hi[e] * o_hi[e];
+          A += g_lo[e] * ga_lo[e] * o_lo[e] + g_hi[e] * ga_hi[e] * o_hi[e];
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+          ss += __shfl_xor_sync(0xffffffffu, ss, o);
+          A += __shfl_xor_sync(0xffffffffu, A, o);
+        }
+        const float ir = rsqrtf(ss * (1.f / 128.f) + a.eps), c = A * ir * ir * (1.f / 128.f);   // c = mean(gh n) / r
+        if (live) {
+          uint32_t w_lo[4], w_hi[4];
 #pragma unroll
           for (int e = 0; e < 8; e += 2) {
-            w_lo[e >> 1] = pack_bf16((g_lo[e] * gr_lo[e] - r_lo[e] * cr) * ir, (g_lo[e + 1] * gr_lo[e + 1] - r_lo[e + 1] * cr) * ir);
-            w_hi[e >> 1] = pack_bf16((g_hi[e] * gr_hi[e] - r_hi[e] * cr) * ir, (g_hi[e + 1] * gr_hi[e + 1] - r_hi[e + 1] * cr) * ir);
+            w_lo[e >> 1] = pack_bf16((g_lo[e] * ga_lo[e] - o_lo[e] * c) * ir, (g_lo[e + 1] * ga_lo[e + 1] - o_lo[e + 1] * c) * ir);
+            w_hi[e >> 1] = pack_bf16((g_hi[e] * ga_hi[e] - o_hi[e] * c) * ir, (g_hi[e + 1] * ga_hi[e + 1] - o_hi[e + 1] * c) * ir);
           }
-          *reinterpret_cast<uint4*>(buf + 2 * PREP_CHUNK) = make_uint4(w_lo[0], w_lo[1], w_lo[2], w_lo[3]);
-          *reinterpret_cast<uint4*>(buf + 2 * PREP_CHUNK + 128) = make_uint4(w_hi[0], w_hi[1], w_hi[2], w_hi[3]);
-        }
+          *reinterpret_cast<uint4*>(p) = make_uint4(w_lo[0], w_lo[1], w_lo[2], w_lo[3]);
+          *reinterpret_cast<uint4*>(p + 128) = make_uint4(w_hi[0], w_hi[1], w_hi[2], w_hi[3]);
 #pragma unroll
-        for (int e = 0; GAINS && e < 8; ++e) {
-          acc_s[e] += g_lo[e] * s_lo[e] * is;
-          acc_s[8 + e] += g_hi[e] * s_hi[e] * is;
-          acc_r[e] += g_lo[e] * r_lo[e] * ir;
-          acc_r[8 + e] += g_hi[e] * r_hi[e] * ir;
+          for (int e = 0; GAINS && e < 8; ++e) {
+            acc[e] += g_lo[e] * o_lo[e] * ir;
+            acc[8 + e] += g_hi[e] * o_hi[e] * ir;
+          }
         }
-      }
+        return (A - c * ss) * ir;
+      };
+      const float dl = branch(buf + PREP_CHUNK, gs_lo, gs_hi, acc_s);            // D_t = g_s . o_swa
+      if (a.rla_on) branch(buf + 2 * PREP_CHUNK, gr_lo, gr_hi, acc_r);
       if (l == 0) {
         if (live) {
           const size_t grow = (size_t)bq * a.T + t;
-          const float dl = (As - cs * ss) * is;                     // D_t = g_s . o_swa
           a.delta[grow] = dl;
           a.lse2p[prow] = -lse_row * LOG2E;
           a.dscp[prow] = -dl * a.scale;
