@@ -28,8 +28,6 @@
 // accumulator row each (row = TMEM lane), a loader warp issues the TMA loads, an MMA warp the
 // tcgen05 products; all accumulation is fp32 in TMEM, and the weight matrices of each tile
 // pair (P, dS) are rounded to bf16 and handed to the tensor core through TMEM.
-#include <type_traits>
-
 #include "tc_common.cuh"
 
 namespace rattn {
@@ -889,9 +887,10 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
     WAIT_OR_RETURN_W(bars->out_staged, (c.it - 1) & 1);
     if ((threadIdx.x & 31) == 0) {
       store_tile(&tm.dv, smem + KV_OFF_STAGE + out_seq % KV_NS * TILE_BYTES, out_row, out_z);
+      tma_store_commit();
       store_tile(&tm.dk, smem + KV_OFF_STAGE + (out_seq + 1) % KV_NS * TILE_BYTES, out_row, out_z);
       tma_store_commit();
-      tma_store_wait_read();
+      asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // dV has left its slot; dK's is refilled next
     }
     __syncwarp();
     out_seq = -1;
@@ -913,7 +912,12 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
       st = c.seq % KV_NS;
       const int use = c.seq / KV_NS;
       if (use >= 1) WAIT_OR_RETURN_W(bars->acc_done[st], (use - 1) & 1);
-      if (c.seq == out_seq + KV_NS && out_seq >= 0 && !store_out()) return false;
+      if (c.seq == out_seq + KV_NS && out_seq >= 0) {
+        if (!store_out()) return false;
+      } else {
+        if ((threadIdx.x & 31) == 0) tma_store_wait_read();   // dK of the previous key tile has left its slot
+        __syncwarp();
+      }
       ++c.seq;
       return true;
     };
@@ -1122,26 +1126,21 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
       // diagonal tile: queries q >= r; oldest tile of the band: queries q <= r; no mask in between
       const uint32_t keep = (diag ? bits_ge(rd) : 0xffffffffu) & (bound ? bits_le(rd) : 0xffffffffu);
       const float2 sl2 = make_float2(a.scale_log2, a.scale_log2), sc2 = make_float2(a.scale, a.scale);
-      auto weights = [&](auto masked_t) {
-        constexpr bool masked = decltype(masked_t)::value;
+      if (diag || bound) mask32(s, keep);                      // exp2(-inf) = 0: weight and score gradient vanish
 #pragma unroll
-        for (int e4 = 0; e4 < 32; e4 += 4) {
-          const float4 lv = *reinterpret_cast<const float4*>(nl + e4);
-          const float4 dv = *reinterpret_cast<const float4*>(nl + 64 + e4);
+      for (int e4 = 0; e4 < 32; e4 += 4) {
+        const float4 lv = *reinterpret_cast<const float4*>(nl + e4);
+        const float4 dv = *reinterpret_cast<const float4*>(nl + 64 + e4);
 #pragma unroll
-          for (int u = 0; u < 4; u += 2) {
-            const int e = e4 + u;
-            const float2 y = __ffma2_rn(make_float2(s[e], s[e + 1]), sl2, u ? make_float2(lv.z, lv.w) : make_float2(lv.x, lv.y));
-            const float2 p = make_float2(ex2(y.x), ex2(y.y));
-            const float2 d = __fmul2_rn(p, __ffma2_rn(make_float2(dp[e], dp[e + 1]), sc2, u ? make_float2(dv.z, dv.w) : make_float2(dv.x, dv.y)));
-            const bool k0 = !masked || ((keep >> e) & 1u), k1 = !masked || ((keep >> (e + 1)) & 1u);
-            pk1[e >> 1] = pack_bf16(k0 ? p.x : 0.f, k1 ? p.y : 0.f);
-            pk2[e >> 1] = pack_bf16(k0 ? d.x : 0.f, k1 ? d.y : 0.f);
-          }
+        for (int u = 0; u < 4; u += 2) {
+          const int e = e4 + u;
+          const float2 y = __ffma2_rn(make_float2(s[e], s[e + 1]), sl2, u ? make_float2(lv.z, lv.w) : make_float2(lv.x, lv.y));
+          const float2 p = make_float2(ex2(y.x), ex2(y.y));
+          const float2 d = __fmul2_rn(p, __ffma2_rn(make_float2(dp[e], dp[e + 1]), sc2, u ? make_float2(dv.z, dv.w) : make_float2(dv.x, dv.y)));
+          pk1[e >> 1] = pack_bf16(p.x, p.y);
+          pk2[e >> 1] = pack_bf16(d.x, d.y);
         }
-      };
-      if (diag || bound) weights(std::true_type{});
-      else weights(std::false_type{});
+      }
     }
     // bf16 results (two per column) overwrite the first half of the columns just consumed
     tmem_st16(tS, pk1);
