@@ -24,9 +24,8 @@
 //   tc_bwd_dkv_kernel  a (K/V head, key tile) item loops over the group's query heads and, for
 //                      each, over the query half tiles whose band contains the key tile.
 // Both are persistent (one CTA per SM walks its items, the next item's loads in flight while
-// the current one's epilogue drains) and warp-specialised: row groups of 128 threads own one
-// accumulator row each (row = TMEM lane), a loader warp issues the TMA loads, an MMA warp the
-// tcgen05 products; all accumulation is fp32 in TMEM, and the weight matrices of each tile
+// the current one's epilogue drains) and warp-specialised: row threads share the accumulator
+// rows (row = TMEM lane), a loader warp issues the TMA copies, MMA warps the tcgen05 products; all accumulation is fp32 in TMEM, and the weight matrices of each tile
 // pair (P, dS) are rounded to bf16 and handed to the tensor core through TMEM.
 #include "tc_common.cuh"
 
@@ -800,12 +799,12 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
 // One CTA per (key tile j, K/V head).  K_j, V_j (and phi(K_j)) stay in shared memory, the dV
 // and dK accumulators in TMEM.  The work is a list of items, one per (query head of the
 // group, query half tile of 64 rows): first the residual-branch items (query tile j + wt),
-// then the window items (query tiles j .. j + wt).  Two row groups of 128 threads (thread =
-// key row = TMEM lane) take the items alternately, each with its own TMEM slot, so that one
+// then the window items (query tiles j .. j + wt).  Two row groups of 256 threads (two per key
+// row = TMEM lane) take the items alternately, each with its own TMEM slot, so that one
 // group's exponentials overlap the other group's products:
-//   loader thread   TMA: K, V, [R_j], then per item Q_h, g_h and the query-side row statistics
-//   MMA thread      per item: S^T = K Q_h^T and dP^T = V g_h^T into the slot (128 x 64 each);
-//                   after the row group has overwritten them with bf16 P^T and dS^T:
+//   loader warp     TMA: K, V, [R_j], then per item Q_h, g_h and the query-side row statistics; stores dV, dK
+//   score warp      per item: S^T = K Q_h^T and dP^T = V g_h^T into the slot (128 x 64 each)
+//   accumulate warp after the row group has overwritten them with bf16 P^T and dS^T:
 //                   dV += P^T g_h, dK += dS^T Q_h with the A operand read from TMEM
 //   row group       P^T = exp2(S^T * scale_log2 - lse2[q]), dS^T = P^T (dP^T scale - D[q] scale)
 // The residual items run first and leave dphi_k in the dK accumulator; the row groups then fold
