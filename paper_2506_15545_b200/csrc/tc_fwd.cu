@@ -41,18 +41,19 @@ static Plan make_plan(const Args& a, int n_sm) {
   // matters.  Where the chain of a long sequence on few heads would outlast the main kernel, its terms are formed in
   // parallel (1 x 8/1 heads, T = 16384, w = 512: 202 -> 113 us).
   const long long chain_ns = 2600ll * p.n_steps;
-  long long main_ns = (long long)n_qt * n_q * (30 + 12 * (wt + 1));
-  if (main_ns < 40000) main_ns = 40000;
+  const long long work_ns = (long long)n_qt * n_q * (30 + 12 * (wt + 1)), main_ns = work_ns < 40000 ? 40000 : work_ns;
   p.terms = p.chain && a.rdelta && knob == 0 && n_kt >= kMinTermChunks && (long long)n_kv * a.n_chunks <= kMaxForwardTerms &&
             chain_ns > main_ns;
   // The single-tile kernel wins where the window loop is not everything: 1.05 - 1.28 times at w <= 768 (8 x 32/8 heads,
   // T = 4397, w = 128, training: 748 -> 610 us; 4 x 16/16, T = 4096, w = 512: 215 -> 201), in training, where all states are
   // stored and three outputs leave per tile, up to w = 1536; at w = 1408 and 2048 the pair kernel is 8 - 10 % faster in
   // inference.  It needs every state, in bf16, where of a pair the second tile takes the chunk in between exactly: a chain
-  // that outlasts the main kernel by far decides against it (16 heads, T = 16384, w = 128), and the element-wise maps'
-  // signed sums feel the rounding (of the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
-  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) &&
-             (p.terms || 2 * chain_ns <= 3 * main_ns);
+  // that outlasts the main kernel by far decides against it (16 heads, T = 16384, w = 128), in inference, where the pair
+  // kernel's chain stores half of the states, from 1.2 - 1.4 times on (1 x 16/4 heads, T = 6298, w = 768: 203 us against
+  // 167; 1 x 16/16, T = 2200, w = 128: 88 against 73; but 1 x 40/8, T = 3541, w = 128, at 1.1: 92 against 116), and the element-wise maps' signed sums feel the rounding (of
+  // the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
+  const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
+  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) && (p.terms || chain_fits);
   // The pair kernel where pairs do not fill the GPU: a tile of its own per CTA ends sooner.
   p.single_tiles = !p.single && !rla && (long long)((n_qt + 1) / 2) * n_q < n_sm;
   // The main kernel can take the chunk states as the chain publishes them instead of waiting for the whole
