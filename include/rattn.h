@@ -296,7 +296,7 @@ size_t rattn_workspace_bytes_chunked(int B, int H_q, int H_kv, int T, int d, int
                                      unsigned flags);
 
 /* An upper bound of rattn_workspace_bytes_ex over every mode and every flag combination for
- * these sizes (the training layout of the larger kernel family). */
+ * these sizes (the largest of the training layouts). */
 size_t rattn_workspace_bytes(int B, int H_q, int H_kv, int T, int d, int w, int dtype);
 
 /* Reads the status word of a workspace (synchronises `stream` first, copies 4 bytes

@@ -500,12 +500,16 @@ size_t rattn_workspace_bytes_chunked(int B, int H_q, int H_kv, int T, int d, int
 }
 
 size_t rattn_workspace_bytes(int B, int H_q, int H_kv, int T, int d, int w, int dtype) {
-  // enough for any mode and any flags: the training layout of either kernel family
-  const unsigned train = RATTN_FLAG_SAVE_RESIDUALS;
-  const size_t a = rattn_workspace_bytes_ex(B, H_q, H_kv, T, d, w, dtype, RATTN_MODE_RATTN, train);
-  const size_t b = rattn_workspace_bytes_ex(B, H_q, H_kv, T, d, w, dtype, RATTN_MODE_RATTN,
-                                            train | RATTN_FLAG_FORCE_GENERIC);
-  return a > b ? a : b;
+  // Enough for any mode and any flags.  The training layouts cover inference; which of them is the largest depends on the
+  // sizes: a window that is no multiple of 128 puts mode RATTN on the portable kernels and full-causal mode, whose window
+  // is T, on the tensor-core ones, with the partial dK, dV of a split group that the others do not have.
+  size_t most = 0;
+  for (int mode = RATTN_MODE_RATTN; mode <= RATTN_MODE_FULL_CAUSAL; ++mode)
+    for (unsigned flags : {RATTN_FLAG_SAVE_RESIDUALS, RATTN_FLAG_SAVE_RESIDUALS | RATTN_FLAG_FORCE_GENERIC}) {
+      const size_t n = rattn_workspace_bytes_ex(B, H_q, H_kv, T, d, w, dtype, mode, flags);
+      if (n > most) most = n;
+    }
+  return most;
 }
 
 int rattn_read_status(const void* workspace, void* stream) {

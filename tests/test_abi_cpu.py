@@ -98,6 +98,20 @@ def test_workspace_size_follows_mode_and_flags(B):
     assert B.rattn_workspace_bytes_ex(*few, B.RATTN_BF16, B.MODE_RATTN, 0) == 256 + 256 + 2 * 8 * 128 * 128 * 2
 
 
+@pytest.mark.parametrize("B_,Hq,Hkv", [(1, 16, 4), (1, 8, 1), (1, 64, 1), (2, 24, 8), (3, 4, 4)])
+@pytest.mark.parametrize("d,dtype", [(128, 0), (64, 0), (128, 1)])
+def test_workspace_bound_covers_every_mode_and_flag(B, B_, Hq, Hkv, d, dtype):
+    """Short grouped sequences with windows on and off the 128-token grid: the layouts of the two kernel families, and
+    of full-causal mode (whose window is T), cross over there."""
+    for T in (1, 64, 129, 300, 500, 777, 1024, 1400, 8300):
+        for w in (1, 64, 100, 128, 129, 512, T):
+            bound = B.rattn_workspace_bytes(B_, Hq, Hkv, T, d, w, dtype)
+            for mode in (B.MODE_RATTN, B.MODE_SWA_ONLY, B.MODE_FULL_CAUSAL):
+                for flags in (0, B.FLAG_SAVE_RESIDUALS, B.FLAG_FORCE_GENERIC, B.FLAG_SAVE_RESIDUALS | B.FLAG_FORCE_GENERIC):
+                    need = B.rattn_workspace_bytes_ex(B_, Hq, Hkv, T, d, w, dtype, mode, flags)
+                    assert 0 < need <= bound, (T, w, mode, flags)
+
+
 def _p(bind, **kw):
     p = bind.RattnParams()
     fake = 0x10000                       # non-null, 16-byte aligned; never dereferenced
