@@ -18,10 +18,10 @@ namespace rattn {
 static std::atomic<uint64_t> g_launches{0};
 static thread_local int g_last_cuda_error = 0;
 
-static std::atomic<int> g_debug_skip_arrive{0};
-int debug_skip_arrive() {
+static std::atomic<int> g_debug_wait{0};
+int debug_wait() {
 #ifdef RATTN_DEBUG_KNOBS
-  return g_debug_skip_arrive.load(std::memory_order_relaxed);
+  return g_debug_wait.load(std::memory_order_relaxed);
 #else
   return 0;
 #endif
@@ -575,7 +575,7 @@ size_t rattn_timing_read(char* buf, size_t buf_bytes) {
 
 #ifdef RATTN_DEBUG_KNOBS
 int rattn_debug_withhold_arrival(int on) {
-  g_debug_skip_arrive.store(on ? 1 : 0, std::memory_order_relaxed);
+  g_debug_wait.store(on, std::memory_order_relaxed);
   return RATTN_OK;
 }
 #endif

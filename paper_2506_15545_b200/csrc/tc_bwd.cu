@@ -55,6 +55,7 @@ struct BwdArgs {
   float4* part;         // ... and where their dK, dV go in fp32 (null: one part, straight to the outputs)
   int phi;              // rattn_feature_map
   float scale, scale_log2;
+  int debug_wait;       // debug build only, 2: the first wait of some of the row threads counts as run out
 };
 
 #define WAIT_OR_RETURN(bar, parity) \
@@ -62,6 +63,9 @@ struct BwdArgs {
 // for roles run by a whole converged warp
 #define WAIT_OR_RETURN_W(bar, parity) \
   do { if (!mbar_wait_warp(&(bar), (parity), &bars->abort)) return false; } while (0)
+
+// of threads that share named barriers: see mbar_wait
+#define WAIT_ON(bar, parity) mbar_wait(&(bar), (parity), &bars->abort)
 
 // ------------------------------------------------------------------------------ prep
 // A pure stream: dO and the two un-normalised branch outputs in, g_s and g_r out (bf16), plus the
@@ -563,8 +567,7 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
     for (int k = 0; k < 4; ++k) all[k] = ex[k * TILE + r];
   };
   for (;; ++n) {
-    int idx;
-    if (!sched_read(&bars->sched, n, &bars->abort, &idx)) return false;
+    const int idx = sched_read_all(&bars->sched, n);
     if (idx < 0) break;
     const DqItem it = dq_item(a, idx, n_qt);
     const int n_kt = it.n_kt;
@@ -575,7 +578,10 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
     const float nD = live ? -a.delta[row] * a.scale : 0.f;
 
     for (int i = 0; i < n_kt; ++i, ++cs) {
-      WAIT_OR_RETURN(bars->s_full, cs & 1);
+      WAIT_ON(bars->s_full, cs & 1);
+#ifdef RATTN_DEBUG_KNOBS
+      if (a.debug_wait == 2 && part == 1 && n == 0 && i == 0) bars->abort = 1;
+#endif
       tc_fence_after();
       const bool diag = (i == 0), bound = it.has_boundary && (i == n_kt - 1);
       const uint32_t tSi = (i & 1) ? tF : tS;
@@ -635,7 +641,7 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
         for (int e = 0; e < 32; ++e) ph[e] *= inv;
         row_sync();
       }
-      WAIT_OR_RETURN(bars->o_done, co & 1);                    // every window product done: K_cb is no longer read raw
+      WAIT_ON(bars->o_done, co & 1);                    // every window product done: K_cb is no longer read raw
       ++co;
       {
         const int t4 = part * TILE + r, krow = t4 >> 2;        // four threads per key row
@@ -644,7 +650,7 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
       }
       fence_proxy_async_smem();
       mbar_arrive(&bars->phik_ready);
-      WAIT_OR_RETURN(bars->s_full, cs & 1);
+      WAIT_ON(bars->s_full, cs & 1);
       tc_fence_after();
       {
         float x[32];
@@ -664,7 +670,7 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
     }
 
     // ---- dq = dQ + phi(q) * (dphi_q - <dphi_q, phi(q)>) -----------------------------------
-    WAIT_OR_RETURN(bars->o_done, co & 1);
+    WAIT_ON(bars->o_done, co & 1);
     ++co;
     tc_fence_after();
     float dot = 0.f;
@@ -712,7 +718,7 @@ __device__ bool dq_rows(const BwdArgs& a, unsigned char* smem, DqBars* bars, uin
     mbar_arrive(&bars->out_staged);
     if (it.has_rla && soft) row_sync();                      // the last exchanged value has been read
   }
-  return true;
+  return *(volatile int*)&bars->abort == 0;
 }
 
 __global__ void __launch_bounds__(DQ_THREADS, 1)
@@ -784,6 +790,7 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
     }
   } else if (warp == DQ_ROW_WARPS + 1) {
     ok = dq_loader(tm, a, smem, bars, n_items, n_qt);
+    if (!ok && (tid & 31) == 0) sched_close(&bars->sched);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
   if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1070,14 +1077,13 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
   KvCount cnt = {0, 0, 0, 0};
 
   for (;;) {
-  int idx;
-  if (!sched_read(&bars->sched, cnt.it, &bars->abort, &idx)) return false;
+  const int idx = sched_read_all(&bars->sched, cnt.it);
   if (idx < 0) break;
   const KvPlan pl = kv_plan(a, idx);
   if (pl.n_R > 0) {
     // phi(K_j) into its own tile, four threads per row.  (Only here do these threads follow kv_full: without residual
     // items the next key tile's K and V may land before they look.)
-    WAIT_OR_RETURN(bars->kv_full, cnt.it & 1);
+    WAIT_ON(bars->kv_full, cnt.it & 1);
     const int row = (g * 256 + gt) >> 2;
     feature_map_quad(smem + KV_OFF_K + row * 128, smem + KV_OFF_KPHI + row * 128, HALF_BYTES, row, gt & 3, a.phi);
     fence_proxy_async_smem();
@@ -1093,8 +1099,8 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
     unsigned char* sQh = smem + KV_OFF_STAGE + st * TILE_BYTES;
     // A group sees every second item, so it follows a slot's uses with gaps, and a wait by parity cannot skip a phase:
     // the previous use of the slot must be known to be over.
-    if (use >= 1) WAIT_OR_RETURN(bars->acc_done[st], (use - 1) & 1);
-    WAIT_OR_RETURN(bars->full[st], use & 1);
+    if (use >= 1) WAIT_ON(bars->acc_done[st], (use - 1) & 1);
+    WAIT_ON(bars->full[st], use & 1);
     if (is_r) {
       // phi(Q_h) in place: 64 rows, four threads per row
       const int row = gt >> 2;
@@ -1102,7 +1108,10 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
       fence_proxy_async_smem();
       mbar_arrive(&bars->phiq_ready[g]);
     }
-    WAIT_OR_RETURN(bars->s_full[g], ((gi0 + n) >> 1) & 1);
+    WAIT_ON(bars->s_full[g], ((gi0 + n) >> 1) & 1);
+#ifdef RATTN_DEBUG_KNOBS
+    if (a.debug_wait == 2 && g == 1 && h == 1 && cnt.it == 0 && n < 2) bars->abort = 1;
+#endif
     tc_fence_after();
     const bool diag = !is_r && (i == pl.j), bound = !is_r && pl.windowed && (i == pl.j + pl.wt);
     float s[32], dp[32];
@@ -1151,7 +1160,7 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
     if (is_r && n + 2 >= pl.n_R) {                              // this group's last residual item of this key tile
       // end of the residual items: dK := dphi_k through the feature map's gradient (softmax map:
       // phi(k) (dphi_k - <dphi_k, phi(k)>)), a quarter of the columns per thread: every window item waits for it
-      WAIT_OR_RETURN(bars->r_acc_done, cnt.cr & 1);
+      WAIT_ON(bars->r_acc_done, cnt.cr & 1);
       tc_fence_after();
       // the identity map leaves dphi_k as it is
       if (a.phi != RATTN_PHI_IDENTITY) {
@@ -1205,7 +1214,7 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
   // every product has completed: group 1 stages dV and group 0 dK in the ring slots of this tile's last two items, from
   // where the loader warp stores them
   {
-    WAIT_OR_RETURN(bars->all_done, cnt.it & 1);
+    WAIT_ON(bars->all_done, cnt.it & 1);
     tc_fence_after();
     const uint32_t tOut = (g == 0 ? tK : tV) + 64 * h;
     float x[2][32];
@@ -1239,7 +1248,7 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
   if (pl.n_R > 0) ++cnt.cr;
   ++cnt.it;
   }
-  return true;
+  return *(volatile int*)&bars->abort == 0;
 }
 
 __global__ void __launch_bounds__(KV_THREADS, 1)
@@ -1311,6 +1320,7 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     }
   } else if (warp == KV_ROW_WARPS + 1) {
     ok = kv_loader(tm, a, smem, bars, n_items);
+    if (!ok && (tid & 31) == 0) sched_close(&bars->sched);
   }
   if (!ok && a.status) atomicExch(a.status, 1);
   tc_fence_before();
@@ -1414,6 +1424,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   t.T = a.T; t.w = a.w; t.H_q = a.H_q; t.group = a.group; t.mode = a.mode; t.n_chunks = a.n_chunks;
   t.scale = a.scale; t.scale_log2 = a.scale * LOG2E;
   t.phi = a.phi;
+  t.debug_wait = debug_wait();
   e = allow_smem<tc_bwd_dq_kernel>(DQ_SMEM);
   if (e != cudaSuccess) return e;
   e = allow_smem<tc_bwd_dkv_kernel>(KV_SMEM);

@@ -504,12 +504,18 @@ __device__ __forceinline__ float feature_map_row_any(unsigned char* tile, int r,
 // Of persistent kernels: a CTA's next item comes from a device-wide counter, so that CTAs that start late
 // (the SM was still running another kernel) or meet heavy items simply take fewer.  The loader warp draws it and
 // publishes it in a small ring that the other roles read in order; a slot is rewritten once every reader has read it.
+// A loader that gives up (a wait that ran out, here or in another role) notes how many items it has published.  The row
+// threads, which meet at named barriers, leave on the end of that list and on nothing else (see mbar_wait), and so all at
+// the same place.
 constexpr int SCHED_SLOTS = 4;
 struct SchedRing {
   uint64_t full[SCHED_SLOTS], free_[SCHED_SLOTS];
   int item[SCHED_SLOTS];
+  int published, closed;   // items so far; items in all, once the loader has given up
 };
 __device__ __forceinline__ void sched_init(SchedRing* r, int readers) {
+  r->published = 0;
+  r->closed = INT_MAX;
   for (int i = 0; i < SCHED_SLOTS; ++i) {
     mbar_init(&r->full[i], 1);
     mbar_init(&r->free_[i], readers);
@@ -521,11 +527,14 @@ __device__ __forceinline__ bool sched_publish(SchedRing* r, int n, int i, volati
   if (use >= 1) { if (!mbar_wait_warp(&r->free_[slot], (use - 1) & 1, abort)) return false; }
   if ((threadIdx.x & 31) == 0) {
     r->item[slot] = i;
+    r->published = n + 1;
     mbar_arrive(&r->full[slot]);
   }
   __syncwarp();
   return true;
 }
+// ... the end of the list, by one thread of a loader that gives up
+__device__ __forceinline__ void sched_close(SchedRing* r) { *(volatile int*)&r->closed = r->published; }
 // ... drawn from the counter
 __device__ __forceinline__ bool sched_draw(SchedRing* r, int* counter, int n_items, int n, volatile int* abort, int* out) {
   int i = 0;
@@ -541,6 +550,17 @@ __device__ __forceinline__ bool sched_read(SchedRing* r, int n, volatile int* ab
   *out = r->item[slot];
   mbar_arrive(&r->free_[slot]);
   return true;
+}
+// ... of the threads that share named barriers: item n, or -1 where the list has ended.  Whether item n has been published
+// does not depend on when a thread asks.  (The loader's own waits are bounded; the limit here is four of them.)
+__device__ __forceinline__ int sched_read_all(SchedRing* r, int n) {
+  const int slot = n % SCHED_SLOTS, use = n / SCHED_SLOTS;
+#pragma unroll 1
+  for (int it = 0; !mbar_try_wait(&r->full[slot], use & 1); ++it)
+    if (it == 4 * kWaitPolls || ((it & 63) == 63 && *(volatile int*)&r->closed <= n)) return -1;
+  const int i = r->item[slot];
+  mbar_arrive(&r->free_[slot]);
+  return i;
 }
 // ... and a whole warp's (one of its lanes is counted)
 __device__ __forceinline__ bool sched_read_warp(SchedRing* r, int n, volatile int* abort, int* out) {

@@ -79,7 +79,8 @@ struct FArgs {
   int wait_for_states;    // a chunk-state kernel runs ahead of this one: wait for it before the first state load
   const int* state_ready; // ... or, per K/V head, for the number of states it has published so far (null: the former)
   int ascending;          // units in sequence order, the order in which their states appear
-  int debug_skip_arrive;  // debug build only: the row threads withhold their first hand-over (a wait then runs out)
+  int debug_wait;         // debug build only, 1: the row threads withhold their first hand-over (a wait then runs out); 2: the
+                          // first wait of one half of them counts as run out
   float scale_log2, eps;
 };
 
@@ -149,6 +150,9 @@ struct UsePhase {
   do { if (!mbar_wait(&(bar), (parity), &bars->abort)) return false; } while (0)
 #define WAIT_OR_RETURN_W(bar, parity) \
   do { if (!mbar_wait_warp(&(bar), (parity), &bars->abort)) return false; } while (0)
+
+// of threads that share named barriers: see mbar_wait
+#define WAIT_ON(bar, parity) mbar_wait(&(bar), (parity), &bars->abort)
 
 // D[128x128] (+)= P[128 x 64 keys] (fp16 in TMEM, 32 columns) . V[64 keys x 128] (fp16, MN-major half tile)
 __device__ __forceinline__ void mma_pv(uint32_t d, uint32_t p_tmem, uint32_t v_base, bool acc) {
@@ -357,12 +361,7 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
 __device__ __forceinline__ uint32_t lane_base(int r) { return (uint32_t)((r & ~31) << 16); }
 // barrier of the two warps that hold the two column halves of the same 32 rows (ids 4 .. 7), and the same with a vote
 __device__ __forceinline__ void pair_sync(int wq) { asm volatile("bar.sync %0, 64;" ::"r"(4 + wq) : "memory"); }
-__device__ __forceinline__ bool pair_any(int wq, bool p) {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %2, 0;\n\tbarrier.cta.red.or.pred q, %1, 64, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
-               : "=r"(r) : "r"(4 + wq), "r"((uint32_t)p) : "memory");
-  return r != 0;
-}
+__device__ __forceinline__ bool pair_any(int wq, bool p) { return named_any(4 + wq, 64, p); }
 // One value per row, combined over the two column halves: half 1 hands its own over, half 0 combines and hands the
 // result back (one word per row).
 template <typename F>
@@ -391,8 +390,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
   auto add2 = [](float p, float q) { return p + q; };
 
   for (int n = 0;; ++n) {
-    int u;
-    if (!sched_read(&bars->sched, n, &bars->abort, &u)) return false;
+    const int u = sched_read_all(&bars->sched, n);
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t < 0) continue;
@@ -408,7 +406,10 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #pragma unroll 1
     for (int s = 0; s < L; ++s) {
       const int b = s & 1, chunk = 2 * b + h;
-      WAIT_OR_RETURN(bars->s_full[b], (cs + (s >> 1)) & 1);
+      WAIT_ON(bars->s_full[b], (cs + (s >> 1)) & 1);
+#ifdef RATTN_DEBUG_KNOBS
+      if (a.debug_wait == 2 && h == 1 && n == 0 && s == 0) bars->abort = 1;      // as if this half's wait had run out
+#endif
       tc_fence_after();
       const bool diag = s < 2, bound = un.c >= 0 && s >= L - 2;
       const bool kept = !(diag && chunk > wq) && !(bound && chunk < wq);
@@ -425,8 +426,8 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
         const float m_new = fmaxf(m_ref, pair_combine(ex, wq, h, mx, max2));
         // the product of the previous step must have completed: its V slot is released then (the one of the
         // last step but one of a residual unit is kept, and reported apart)
-        if (un.rla && s == L - 1) WAIT_OR_RETURN(bars->pv_done, cr & 1);
-        else WAIT_OR_RETURN(bars->free_[ring.slot(pos_v(s - 1, L, un.rla))], ring.phase(pos_v(s - 1, L, un.rla)));
+        if (un.rla && s == L - 1) WAIT_ON(bars->pv_done, cr & 1);
+        else WAIT_ON(bars->free_[ring.slot(pos_v(s - 1, L, un.rla))], ring.phase(pos_v(s - 1, L, un.rla)));
         tc_fence_after();
         const float f = ex2(m_ref - m_new);
 #pragma unroll 1
@@ -467,7 +468,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #ifdef RATTN_DEBUG_KNOBS
       // failure injection for the time-out test: an arrival that nothing else depends on is left
       // out, so the MMA warp's bounded wait expires and every role takes the abort path
-      if (!(a.debug_skip_arrive && n == 0 && s == 0))
+      if (!(a.debug_wait == 1 && n == 0 && s == 0))
 #endif
       mbar_arrive(&bars->p_ready[b]);
     }
@@ -498,7 +499,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     l = pair_combine(ex, wq, h, l, add2);
 
     // ---- park the normalised window output (Section 3.2, first norm) in registers ---------
-    WAIT_OR_RETURN(bars->o_ready, co & 1);
+    WAIT_ON(bars->o_ready, co & 1);
     ++co;
     tc_fence_after();
     const float inv_l = 1.f / l;
@@ -531,7 +532,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       mbar_arrive(&bars->stash_done);
 #pragma unroll 1
       for (int b = 0; b < 2; ++b) {
-        WAIT_OR_RETURN(bars->s_full[b], cs & 1);
+        WAIT_ON(bars->s_full[b], cs & 1);
         tc_fence_after();
         float x[32];
         tmem_ld32(tS + 64 * b + 32 * h, x);
@@ -551,7 +552,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       }
       ++cs;
       ++cr;
-      WAIT_OR_RETURN(bars->o_ready, co & 1);
+      WAIT_ON(bars->o_ready, co & 1);
       ++co;
       tc_fence_after();
       float sr = 0.f;
@@ -669,7 +670,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     if (h == 0 && t < a.T && a.lse) a.lse[(size_t)un.bh_q * a.T + t] = (m_ref + log2f(l)) * 0.6931471805599453f;
   }
   if (r == 0) tma_store_wait();          // this thread's stores have completed before the CTA may go
-  return true;
+  return *(volatile int*)&bars->abort == 0;
 }
 
 __global__ void __launch_bounds__(F_THREADS, 2)
@@ -739,6 +740,7 @@ tc_fwd1_kernel(const __grid_constant__ FMaps tm, FArgs a) {
     }
   } else if (warp == 9) {
     ok = fwd_loader(tm, a, smem, bars);
+    if (!ok && (tid & 31) == 0) sched_close(&bars->sched);
   } else {
     ok = fwd_convert(a, smem, bars, tid - 320);
   }
@@ -791,7 +793,7 @@ cudaError_t launch_tc_forward_single(const Args& a, cudaStream_t s, bool after_s
   t.wait_first = after_states ? 0 : 1;
   t.state_ready = after_states ? a.state_ready : nullptr;
   t.ascending = (t.state_ready && t.n_stateless > 0) ? 1 : 0;
-  t.debug_skip_arrive = debug_skip_arrive();
+  t.debug_wait = debug_wait();
   int grid = 2 * n_sm;
   if (tuning(RATTN_TUNE_GRID) > 0 && tuning(RATTN_TUNE_GRID) < grid) grid = tuning(RATTN_TUNE_GRID);
   if (t.n_units < grid) grid = t.n_units;

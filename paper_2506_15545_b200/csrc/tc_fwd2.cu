@@ -70,7 +70,8 @@ struct FArgs {
   int wait_for_states;    // a chunk-state kernel runs ahead of this one: wait for it before the first state load
   const int* state_ready; // ... or, per K/V head, for the number of states it has published so far (null: the former)
   int ascending;          // units in sequence order, the order in which their states appear
-  int debug_skip_arrive;  // debug build only: tile A's row group withholds its first hand-over (a wait then runs out)
+  int debug_wait;         // debug build only, 1: row group A withholds its first hand-over (a wait then runs out); 2: the first
+                          // wait of some of its threads counts as run out
   float scale_log2, eps;
 };
 
@@ -150,6 +151,9 @@ __device__ int g_timeline_n[4];
   do { if (!mbar_wait(&(bar), (parity), &bars->abort)) return false; } while (0)
 #define WAIT_OR_RETURN_W(bar, parity) \
   do { if (!mbar_wait_warp(&(bar), (parity), &bars->abort)) return false; } while (0)
+
+// of threads that share named barriers: see mbar_wait
+#define WAIT_ON(bar, parity) mbar_wait(&(bar), (parity), &bars->abort)
 
 // D[128x128] (+)= P[128 x 128 keys] (fp16 in TMEM, 64 columns) . V[128 keys x 128] (fp16, MN-major)
 __device__ __forceinline__ void mma_pv(uint32_t d, uint32_t p_tmem, uint32_t v_base, bool acc) {
@@ -411,8 +415,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
   TL_DECL(blockIdx.x == 7 && r == 0);
 
   for (int n = 0;; ++n) {
-    int u;
-    if (!sched_read(&bars->sched, n, &bars->abort, &u)) return false;
+    const int u = sched_read_all(&bars->sched, n);
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t[0] < 0) continue;
@@ -435,7 +438,10 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     for (int i = i0; i <= i1; ++i) {
       const int kt = un.kt_hi - i;
       TL(X, 100 + i);
-      WAIT_OR_RETURN(bars->s_full[X], cntS & 1);
+      if (!WAIT_ON(bars->s_full[X], cntS & 1)) break;    // (out of the loop, not out of the unit)
+#ifdef RATTN_DEBUG_KNOBS
+      if (a.debug_wait == 2 && X == 0 && r < 32 && n == 0 && i == i0) bars->abort = 1;
+#endif
       TL(X, 200 + i);
       ++cntS;
       tc_fence_after();
@@ -508,7 +514,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #ifdef RATTN_DEBUG_KNOBS
       // failure injection for the time-out test: an arrival that nothing else depends on is left
       // out, so the MMA warp's bounded wait expires and every role takes the abort path
-      if (!(a.debug_skip_arrive && X == 0 && n == 0 && i == i0))
+      if (!(a.debug_wait == 1 && X == 0 && n == 0 && i == i0))
 #endif
       mbar_arrive(&bars->p_ready[X]);
       TL(X, 400 + i);
@@ -537,7 +543,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 
     // ---- park the normalised window output (Section 3.2, first norm) in registers ---------
     TL(X, 500);
-    WAIT_OR_RETURN(bars->o_ready[X], cntO & 1);
+    WAIT_ON(bars->o_ready[X], cntO & 1);
     TL(X, 501);
     ++cntO;
     tc_fence_after();
@@ -572,7 +578,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #pragma unroll 1
       for (int term = 0; term < n_terms; ++term) {
         const bool masked = (term == n_terms - 1);                     // B's first term takes chunk cA whole
-        WAIT_OR_RETURN(bars->s_full[X], cntS & 1);
+        WAIT_ON(bars->s_full[X], cntS & 1);
         ++cntS;
         tc_fence_after();
 #pragma unroll 1
@@ -593,7 +599,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
         tc_fence_before();
         mbar_arrive(&bars->p_ready[X]);
       }
-      WAIT_OR_RETURN(bars->o_ready[X], cntO & 1);
+      WAIT_ON(bars->o_ready[X], cntO & 1);
       ++cntO;
       tc_fence_after();
 #pragma unroll 1
@@ -738,7 +744,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     mbar_arrive(&bars->y_done[X]);         // the staging buffer may take the next state tile
     TL(X, 540);
   }
-  return true;
+  return *(volatile int*)&bars->abort == 0;
 }
 
 __global__ void __launch_bounds__(F_THREADS, 1)
@@ -811,6 +817,7 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
     }
   } else if (warp == 9) {
     ok = fwd_loader(tm, a, smem, bars);
+    if (!ok && (tid & 31) == 0) sched_close(&bars->sched);
   } else {
     ok = fwd_convert(a, smem, bars, tid - 320);
   }
@@ -879,7 +886,7 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   // with per-head progress words the units can follow the chain; worth it where the order above would
   // have put the units without a state first anyway (few K/V heads, many SMs free beside the chain)
   t.ascending = (t.state_ready && t.n_stateless > 0) ? 1 : 0;
-  t.debug_skip_arrive = debug_skip_arrive();
+  t.debug_wait = debug_wait();
   t.work_counter = (order != 3 && t.n_units > n_sm) ? a.work_counter : nullptr;   // one unit per CTA needs no counter
   t.clear_status = after_states ? nullptr : a.clear_status;
   t.wait_first = after_states ? 0 : 1;

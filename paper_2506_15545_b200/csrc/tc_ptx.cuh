@@ -58,6 +58,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
 }
 // Bounded wait.  Returns false when the limit is hit (and raises *abort so that every other
 // waiter of the CTA gives up too) or when another thread has already raised it.
+// Threads that share a named barrier must not leave on that answer one by one: a barrier has no bound, and of two threads
+// that look at the flag while the awaited phase is just completing one may give up and the other go on, to a barrier that
+// the first will never reach.  They carry on with whatever they have (every address is formed from the work item, never
+// from what was awaited) until something that all of them learn alike ends the kernel: the end of the list of items, or
+// a vote at a barrier.
 // (The debug build, which exists to make a wait run out in a test, gives up much sooner.)
 #ifdef RATTN_DEBUG_KNOBS
 constexpr int kWaitPolls = 1 << 15;
@@ -142,6 +147,13 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // ... has at least finished reading its shared-memory source
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// Barrier among n threads (id) with a vote: whether any of them says yes.
+__device__ __forceinline__ bool named_any(int id, int n, bool p) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.or.pred q, %1, %2, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"(id), "r"(n), "r"((uint32_t)p) : "memory");
+  return r != 0;
+}
 // barrier among the 128 threads of row group g (0 or 1), ids 2 and 3
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(2 + g) : "memory"); }
 

@@ -55,6 +55,7 @@ struct StateArgs {
   int n_split;      // steps that the grid is split into (delta)
   int h_split;      // ... and the group's heads: term matrix ((kv * n_split + step) * h_split + part)
   int wait_before;  // 1: the kernel ahead may still be running; not to end before it
+  int debug_wait;   // debug build only, 2: the first wait of some of the flush threads counts as run out
 };
 
 struct StBars {
@@ -194,7 +195,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       st_release_gpu(a.ready + kv, pending);
       pending = 0;
     };
-    auto store_row = [&](const float (&x)[4][32], int mat) {
+    auto store_row = [&](const float (&x)[4][32], int mat) -> bool {
       if (issuer) {
         // The kernel that reads the states runs beside this one and takes them as they appear.  The
         // matrix stored last is published here, one flush later, when its store has long completed
@@ -202,7 +203,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
         if (a.ready && pending) publish();
         else tma_store_wait_read();                          // the staging tile has left
       }
-      asm volatile("bar.sync 4, 128;" ::: "memory");
+      if (named_any(4, 128, *(volatile int*)&bars->abort)) return false;       // the whole group or nobody
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
 #pragma unroll
@@ -222,6 +223,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
         tma_store_commit();
         pending = mat + 1;
       }
+      return true;
     };
     auto write_final = [&](const float (&x)[4][32]) {
       float* dst = a.final_out + ((size_t)kv * 128 + r) * 128;
@@ -252,15 +254,17 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(&bars->acc_free);
-        if (stored_step(a, -1)) store_row(x, a.out_first - a.dir);
+        if (stored_step(a, -1)) ok = store_row(x, a.out_first - a.dir);
       }
       if (a.final_out != nullptr && n_steps == 0) write_final(x);
     }
     for (int s = 0; s < n_steps && ok; ++s) {
       if (!flushed_step(a, s, n_steps)) continue;
-      ok = mbar_wait(&bars->done, n_flush & 1, &bars->abort);
+      mbar_wait(&bars->done, n_flush & 1, &bars->abort);       // (on a wait that ran out store_row has the vote)
+#ifdef RATTN_DEBUG_KNOBS
+      if (a.debug_wait == 2 && warp == 10 && n_flush == 0) bars->abort = 1;
+#endif
       ++n_flush;
-      if (!ok) break;
       tc_fence_after();
       float x[4][32];
 #pragma unroll
@@ -277,7 +281,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
             dst[(8 * c + e) * 128] = make_float4(x[c][4 * e], x[c][4 * e + 1], x[c][4 * e + 2], x[c][4 * e + 3]);
         continue;
       }
-      if (stored_step(a, s)) store_row(x, a.out_first + a.dir * s);
+      if (stored_step(a, s) && !store_row(x, a.out_first + a.dir * s)) ok = false;
       if (a.final_out != nullptr && s == n_steps - 1) write_final(x);
     }
     if (issuer) {
@@ -366,6 +370,7 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   a.n_split = L.delta ? L.n_steps : 1;
   a.h_split = L.delta ? L.h_split : 1;
   a.wait_before = L.after_independent ? 1 : 0;
+  a.debug_wait = debug_wait();
   cudaError_t e = allow_smem<tc_state_scan_kernel>(ST_SMEM);
   if (e != cudaSuccess) return e;
   {

@@ -98,3 +98,43 @@ def test_plain_forward_latches_its_status_before_freeing_its_scratch(dbg):
     # the product library's own word was never touched
     y = R.rattn_forward(qd, kd, vd, wl.w)
     assert R.rattn_forward_status() == 0 and torch.equal(y, out)
+
+
+@pytest.mark.parametrize("B_,Hq,Hkv,T,w,mode", [
+    (1, 2, 1, 384, 128, R.MODE_RATTN),          # single tiles behind a chain of states; all three backward kernels
+    (1, 2, 2, 128, 128, R.MODE_RATTN),          # ... without states: the forward kernel alone, one tile
+    (1, 2, 2, 700, 256, R.MODE_FULL_CAUSAL),    # the pair kernel
+    (1, 40, 40, 1000, 128, R.MODE_RATTN),       # more units than CTAs hold at once: threads leave between two of them
+])
+def test_threads_that_share_a_barrier_leave_together(dbg, B_, Hq, Hkv, T, w, mode):
+    """Some of the threads that meet at a named barrier (which has no bound) take a wait as run out that the others have
+    passed: the kernel must end and report, not wait for those that left."""
+    wl = small("fdb", B_, Hq, Hkv, T, 128, w, "bf16", 8300 + T, unit=True)
+    q, k, v = (t.cuda() for t in W.make_qkv(wl))
+    dy = W.make_dout(wl).cuda()
+    ws = R.alloc_workspace(q, k, w, mode, R.FLAG_SAVE_RESIDUALS)
+    out, dq, dk, dv = (torch.zeros_like(t) for t in (q, q, k, v))
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    dbg.rattn_backward_ex.argtypes = [ctypes.POINTER(R.RattnParams), ctypes.c_void_p]
+    dbg.rattn_backward_ex.restype = ctypes.c_int
+    p = R._params(q, k, v, out, w, wl.scale, 1e-6, None, None, mode, ws, R.FLAG_SAVE_RESIDUALS)
+    p.dout, p.dq, p.dk, p.dv = (t.data_ptr() for t in (dy, dq, dk, dv))
+    status = lambda: dbg.rattn_read_status(ctypes.c_void_p(ws.data_ptr()), stream)
+    try:
+        dbg.rattn_debug_withhold_arrival(2)
+        assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0
+        assert status() == RATTN_ERR_TIMEOUT
+        dbg.rattn_debug_withhold_arrival(0)
+        assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0 and status() == 0
+        dbg.rattn_debug_withhold_arrival(2)
+        assert dbg.rattn_backward_ex(ctypes.byref(p), stream) == 0
+        assert status() == RATTN_ERR_TIMEOUT
+    finally:
+        dbg.rattn_debug_withhold_arrival(0)
+    # the same context and buffers, normal operation: the product library's results
+    assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0
+    assert dbg.rattn_backward_ex(ctypes.byref(p), stream) == 0
+    assert status() == 0
+    y = R.rattn_forward_ex(q, k, v, w, scale=wl.scale, mode=mode, workspace=ws, save_residuals=True)
+    grads = R.rattn_backward_ex(q, k, v, dy, w, ws, scale=wl.scale, mode=mode, flags=R.FLAG_SAVE_RESIDUALS)
+    assert all(torch.equal(a, b) for a, b in zip((out, dq, dk, dv), (y, *grads)))
