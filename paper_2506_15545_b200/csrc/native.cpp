@@ -7,6 +7,7 @@
 //
 // The library is not linked: binding.py loads librattn.so (or another build of it) and hands over the addresses of its
 // entry points, so that both sides use one instance of it.
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ATen.h>
@@ -153,8 +154,8 @@ PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
   try {
     return F(Args{args, args + n});
   } catch (const Raised&) {
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
+  } catch (...) {                            // as torch's own functions raise it: callers catch torch.OutOfMemoryError
+    torch::translate_exception_to_python(std::current_exception());
   }
   return nullptr;
 }
