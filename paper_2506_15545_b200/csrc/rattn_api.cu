@@ -345,6 +345,20 @@ struct ForwardDevice {
 std::mutex g_forward_mu;
 ForwardDevice g_forward_device[kMaxDevices];
 
+// Set-up calls of a first use may fall into a stream capture of this thread, which forbids them (the address of a symbol
+// loads its module, a pool is created) unless the thread says that they have nothing to do with what is captured.
+class OutsideCapture {
+ public:
+  OutsideCapture() { ok_ = cudaThreadExchangeStreamCaptureMode(&mode_) == cudaSuccess; }
+  ~OutsideCapture() { if (ok_) cudaThreadExchangeStreamCaptureMode(&mode_); }
+  OutsideCapture(const OutsideCapture&) = delete;
+  OutsideCapture& operator=(const OutsideCapture&) = delete;
+
+ private:
+  cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+  bool ok_;
+};
+
 cudaError_t forward_device(ForwardDevice* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -352,13 +366,14 @@ cudaError_t forward_device(ForwardDevice* out) {
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lk(g_forward_mu);
   ForwardDevice& f = g_forward_device[dev];
-  if (!f.status) {
-    void* word = nullptr;
-    e = cudaGetSymbolAddress(&word, g_forward_status);
-    if (e != cudaSuccess) return e;
-    f.status = static_cast<int*>(word);
-  }
-  if (!f.pool) {
+  if (!f.status || !f.pool) {
+    OutsideCapture relaxed;
+    if (!f.status) {
+      void* word = nullptr;
+      e = cudaGetSymbolAddress(&word, g_forward_status);
+      if (e != cudaSuccess) return e;
+      f.status = static_cast<int*>(word);
+    }
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
