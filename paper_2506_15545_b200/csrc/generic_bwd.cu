@@ -353,6 +353,8 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
     tile_matrix<D, NA>(dfk, Vs, R, true, Qs, Gs, tid, ty, tx);           // dphi_k += V R^T
     tile_matrix<D, NA>(dv, Fk, R, false, Qs, Gs, tid, ty, tx);           // dv     += phi(k) R
   }
+  // Not to write before the dq kernel beside it has ended: dk and dv may take the place of k and v, which that one reads.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   TIO* dkg = reinterpret_cast<TIO*>(a.dk) + kv_head;
   TIO* dvg = reinterpret_cast<TIO*>(a.dv) + kv_head;
 #pragma unroll
@@ -383,7 +385,6 @@ __global__ void __launch_bounds__(NT) bwd_dkv_kernel(Args a, const float* __rest
       }
     }
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");                   // not to end before the dq kernel beside it
 }
 
 template <typename TIO, int D>

@@ -125,3 +125,22 @@ def test_portable_chunk_states(B, Hq, Hkv, T, d, w, dtype):
     for name, got, ref in zip(("dq", "dk", "dv"), grads, want):
         got = np64(got[:, heads])
         assert np.linalg.norm(got - ref) <= (1e-4 if dtype == "f32" else 5e-2) * np.linalg.norm(ref), name
+
+
+@pytest.mark.parametrize("Hq,Hkv,T,d,w,dtype", [
+    (1, 1, 1024, 64, 1000, "f32"),       # portable kernels, dk/dv beside dq: its last key tiles are done first
+    (2, 1, 700, 128, 500, "f32"),
+    (2, 1, 700, 128, 256, "bf16"),       # tensor-core kernels
+])
+def test_gradients_in_place_of_the_inputs(Hq, Hkv, T, d, w, dtype):
+    """dk, dv may be written over k, v and dq over dout: nothing reads those once the gradient is written."""
+    wl = small("alias", 1, Hq, Hkv, T, d, w, dtype, 9800 + T, unit=True)
+    q, k, v = (t.cuda() for t in W.make_qkv(wl))
+    dy = W.make_dout(wl).cuda()
+    ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, R.FLAG_SAVE_RESIDUALS)
+    R.rattn_forward_ex(q, k, v, w, scale=wl.scale, workspace=ws, save_residuals=True)
+    apart = R.rattn_backward_ex(q, k, v, dy, w, ws, scale=wl.scale, flags=R.FLAG_SAVE_RESIDUALS)
+    for _ in range(5):
+        k2, v2, dy2 = k.clone(), v.clone(), dy.clone()
+        R.rattn_backward_ex(q, k2, v2, dy2, w, ws, scale=wl.scale, flags=R.FLAG_SAVE_RESIDUALS, dq=dy2, dk=k2, dv=v2)
+        assert all(torch.equal(a, b) for a, b in zip(apart, (dy2, k2, v2)))
