@@ -265,8 +265,8 @@ int rattn_decode_step_ex(const rattn_params* p, void* k_ring, void* v_ring, floa
  * decode step stages the ring and the state through shared memory with asynchronous copies and
  * waits for them with a bound.  rattn_decode_status (synchronises the stream) returns
  * RATTN_ERR_TIMEOUT if such a wait has expired in any decode step on the current device since it
- * was last asked (the step then left its outputs, ring and state in an unspecified state), else
- * RATTN_OK. */
+ * was last asked (for the K/V heads concerned the step then wrote neither outputs nor rings; of
+ * their state some rows may have been updated), else RATTN_OK. */
 int rattn_decode_status(void* stream);
 
 /*

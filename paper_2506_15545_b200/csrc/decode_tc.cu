@@ -44,6 +44,7 @@ struct DecodeTcArgs {
   const float* gamma_swa; const float* gamma_rla;
   const int* pos_dev;
   int B, H_q, H_kv, w, pos, group, phi, stages, cluster;
+  int debug_wait;             // debug build only, 2: a wait of the last CTA of each cluster counts as run out
   float scale, eps;
 };
 
@@ -296,7 +297,6 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
     v_old[tid] = __bfloat162float(vo_);
   }
   __syncthreads();
-  if (CS > 1) cluster_arrive();                                  // the evicted slot has been read (every CTA needs it)
 
   // query fragments: rows 0..7 from q_b (rows 8..15 of the 16-row product are zero)
   uint32_t qa[8][2];
@@ -438,15 +438,6 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
       st_sum[hh] = l;
     }
   }
-  if (CS > 1) cluster_wait();
-  // the incoming token takes the evicted token's slot: the CTA whose piece that is has consumed it (a slot
-  // beyond the valid pieces is read by nobody), and every CTA has read the evicted token
-  if (ok && rank == min((slot >> 6) / max(ppr, 1), CS - 1)) {
-    if (tid < D) {
-      kr[(size_t)slot * D + tid] = kn;
-      vr[(size_t)slot * D + tid] = vn;
-    }
-  }
 
   // ---- the state: read-out phi(q) S and the update S += phi(k_old)^T v_old (Eq. 4), fp32 -----------
   // thread = two float4 column groups (c4, c4 + 16) and one of 8 row lanes (rl) that sit in the same warp; a piece
@@ -460,6 +451,12 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
     for (int u = 0; u < 2; ++u) vo[u] = *reinterpret_cast<const float4*>(v_old + (c4 + 16 * u) * 4);
     for (int p = n_kv; p < n_pieces && ok; ++p) {
       ok = wait_piece(p);
+#ifdef RATTN_DEBUG_KNOBS
+      if (a.debug_wait == 2 && rank == CS - 1 && warp == 0) {     // as if this wait had run out
+        ok = false;
+        *abort = 1;
+      }
+#endif
       if (!ok) break;
       const float* piece = reinterpret_cast<const float*>(sm + stage_of(p) * DT_PIECE);
       const int r0 = row0 + (grp + 2 * (p - n_kv)) * st_piece;
@@ -508,6 +505,14 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   if (CS > 1) {
     cluster_arrive();                                              // partial sums of every CTA are in place
     cluster_wait();
+    // a wait that ran out in one of the CTAs ends the step for all of them
+    ok = !__any_sync(0xffffffffu, lane < CS && __float_as_uint(ld_cluster(cluster_addr((const void*)abort, lane))) != 0u);
+  }
+  // The incoming token takes the evicted token's slot: every CTA has read the evicted token, and the one whose piece that
+  // is has consumed it (a slot beyond the valid pieces is read by nobody).
+  if (ok && tid < D && rank == min((slot >> 6) / max(ppr, 1), CS - 1)) {
+    kr[(size_t)slot * D + tid] = __float2bfloat16_rn(k_new[tid]);
+    vr[(size_t)slot * D + tid] = __float2bfloat16_rn(v_new[tid]);
   }
 
   // ---- combine, Section 3.2: two RMS norms and the sum: one warp per head, heads spread over the cluster -----
@@ -561,7 +566,7 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
                    pack_bf16(gs.z * x.z * is + gr.z * y.z * ir, gs.w * x.w * is + gr.w * y.w * ir));
   }
   if (!ok && tid == 0) {
-    // a wait ran out: give what is still in flight a bounded time to land, report (the step's results are unspecified)
+    // a wait ran out: give what is still in flight a bounded time to land, report (neither output nor rings are written)
     for (int i = 0; i < NS; ++i)
       for (int it = 0; it < kWaitPolls && issued[i] > 0 && !mbar_try_wait(&full[i], (uint32_t)(issued[i] - 1) & 1u); ++it) {}
     g_decode_status = RATTN_ERR_TIMEOUT;
@@ -634,6 +639,7 @@ cudaError_t launch_decode_tc(const Args& p, void* k_ring, void* v_ring, float* s
       !tc::make_map(&m.v, v_ring, (uint64_t)p.w, (uint64_t)p.B * p.H_kv, 64))
     return cudaErrorInvalidValue;
   a.stages = tuning(RATTN_TUNE_DECODE_STAGES);
+  a.debug_wait = debug_wait();
   int n_sm = 0;
   const cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;

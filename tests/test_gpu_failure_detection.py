@@ -138,3 +138,35 @@ def test_threads_that_share_a_barrier_leave_together(dbg, B_, Hq, Hkv, T, w, mod
     y = R.rattn_forward_ex(q, k, v, w, scale=wl.scale, mode=mode, workspace=ws, save_residuals=True)
     grads = R.rattn_backward_ex(q, k, v, dy, w, ws, scale=wl.scale, mode=mode, flags=R.FLAG_SAVE_RESIDUALS)
     assert all(torch.equal(a, b) for a, b in zip((out, dq, dk, dv), (y, *grads)))
+
+
+@pytest.mark.parametrize("B_,Hq,Hkv,w,pos", [
+    (1, 8, 2, 512, 1000),        # cluster of 8 CTAs, the last of which gives up
+    (40, 32, 8, 64, 100),        # one CTA per head
+])
+def test_a_decode_step_that_gives_up_writes_neither_output_nor_rings(dbg, B_, Hq, Hkv, w, pos):
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    rnd = lambda *s, dt=torch.bfloat16: torch.randn(s, generator=gen, device="cuda").to(dt)
+    q, k, v = rnd(B_, Hq, 128), rnd(B_, Hkv, 128), rnd(B_, Hkv, 128)
+    cache = [rnd(B_, Hkv, w, 128), rnd(B_, Hkv, w, 128), rnd(B_, Hkv, 128, 128, dt=torch.float32)]
+    out = torch.full_like(q, 7.0)
+    vp = ctypes.c_void_p
+    stream = vp(torch.cuda.current_stream().cuda_stream)
+    dbg.rattn_decode_step_ex.argtypes = [ctypes.POINTER(R.RattnParams), vp, vp, vp, ctypes.c_int, vp]
+    dbg.rattn_decode_status.argtypes = [vp]
+    p = R._params(q, k, v, out, w, 0.1, 1e-6, None, None, R.MODE_RATTN, None, 0)
+    step = lambda c: dbg.rattn_decode_step_ex(ctypes.byref(p), *(vp(t.data_ptr()) for t in c), pos, stream)
+    assert dbg.rattn_decode_status(stream) == 0
+    used = [t.clone() for t in cache]
+    try:
+        dbg.rattn_debug_withhold_arrival(2)
+        assert step(used) == 0
+        assert dbg.rattn_decode_status(stream) == RATTN_ERR_TIMEOUT
+    finally:
+        dbg.rattn_debug_withhold_arrival(0)
+    assert torch.equal(used[0], cache[0]) and torch.equal(used[1], cache[1]) and (out == 7.0).all()
+    # normal operation again: the product library's step
+    used = [t.clone() for t in cache]
+    assert step(used) == 0 and dbg.rattn_decode_status(stream) == 0
+    y = R.rattn_decode_step_ex(q, k, v, *cache, pos, scale=0.1)
+    assert torch.equal(y, out) and all(torch.equal(a, b) for a, b in zip(used, cache))
