@@ -13,6 +13,7 @@
  *      that a wait does run out;
  *   2  in every tensor-core kernel whose threads share named barriers, some of these threads
  *      treat their first wait as run out while the others have passed the same wait.
+ *   3  rattn_forward_status finds that the scratch pool cannot be given back.
  * The paper has no counterpart; this exists for the failure-detection test.
  */
 #ifndef RATTN_DEBUG_H_
@@ -22,7 +23,7 @@
 extern "C" {
 #endif
 
-/* on = 1 or 2: the tensor-core kernels launched from now on fail in that way; 0: normal operation.
+/* on = 1, 2 or 3: what is called from now on fails in that way; 0: normal operation.
  * Process-wide switch, host side only.  Returns RATTN_OK. */
 int rattn_debug_withhold_arrival(int on);
 

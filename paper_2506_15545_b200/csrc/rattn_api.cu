@@ -392,6 +392,17 @@ cudaError_t forward_device(ForwardDevice* out) {
   *out = f;
   return cudaSuccess;
 }
+
+// Gives the scratch that the current device's pool keeps back to the device; where no rattn_forward has run there is none.
+cudaError_t trim_forward_pool() {
+  if (debug_wait() == 3) return cudaErrorUnknown;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_forward_mu);
+  return g_forward_device[dev].pool ? cudaMemPoolTrimTo(g_forward_device[dev].pool, 0) : cudaSuccess;
+}
 }  // namespace
 
 extern "C" {
@@ -410,11 +421,10 @@ int rattn_forward_status(void* stream) {
     e = cudaMemcpyToSymbolAsync(g_forward_status, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  ForwardDevice f;
-  if (e == cudaSuccess) e = forward_device(&f);
-  if (e == cudaSuccess) e = cudaMemPoolTrimTo(f.pool, 0);
   if (e != cudaSuccess) return fail_cuda(e);
-  return word == 0 ? RATTN_OK : RATTN_ERR_TIMEOUT;
+  const cudaError_t trim = trim_forward_pool();
+  if (word != 0) return RATTN_ERR_TIMEOUT;      // it has just been cleared: whatever became of the scratch, the caller learns of it
+  return trim == cudaSuccess ? RATTN_OK : fail_cuda(trim);
 }
 
 int rattn_forward(const void* q, const void* k, const void* v, int B, int H_q, int H_kv, int T,

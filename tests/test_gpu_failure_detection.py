@@ -91,6 +91,10 @@ def test_plain_forward_latches_its_status_before_freeing_its_scratch(dbg):
     assert call() == 0
     assert dbg.rattn_forward_status(stream) == RATTN_ERR_TIMEOUT
     assert dbg.rattn_forward_status(stream) == 0          # reading clears it
+    assert call() == 0
+    dbg.rattn_debug_withhold_arrival(3)                   # the scratch cannot be given back: the expired wait is reported all the same
+    assert dbg.rattn_forward_status(stream) == RATTN_ERR_TIMEOUT
+    assert dbg.rattn_forward_status(stream) == -6         # RATTN_ERR_CUDA
     dbg.rattn_debug_withhold_arrival(0)
     assert call() == 0
     assert dbg.rattn_forward_status(stream) == 0
