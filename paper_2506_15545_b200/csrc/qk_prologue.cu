@@ -243,7 +243,6 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
     *abort = 0;
     ptx::fence_mbar_init();
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");        // the inputs may come from the kernel before
   if (BWD && a.partial != nullptr && tid < D) {
     a.partial[((size_t)0 * gridDim.x + blockIdx.x) * D + tid] = 0.f;
@@ -433,6 +432,9 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
     }
   }
 
+  // Only here, where its last chunks leave: CTAs of the next kernel that wait on the SM from the start took shared memory
+  // and issue slots from this one (1 x 40/8 heads, T = 4096, [B,T,H,d]: 38.7 us against 33.0).
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     ptx::tma_store_wait();
     if (!ok) {
@@ -450,10 +452,7 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
 
 // The forward pass for few head vectors (decoding), where latency counts and not bandwidth: a warp per head vector, lane
 // l holding its pairs (i, i + d/2) of PPL consecutive i.  No staging and no barriers: one load, the sines and cosines
-// under it, one store (1 sequence of 32/8 heads: 4.3 -> 2.7 us, 32 sequences: 8.4 -> 3.7).  From some thousand vectors
-// on the sines and cosines formed per vector cost more than the chunks of the kernel above (13 thousand: 9.0 against
-// 6.1 us).
-constexpr long long QK_SMALL_VECTORS = 4096;
+// under it, one store (1 sequence of 32/8 heads: 3.1 -> 2.2 us).
 template <typename T, int D>
 __global__ void __launch_bounds__(QK_THREADS) qk_small_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Freqs f,
                                                               int ctas_per_token) {
@@ -502,6 +501,19 @@ __global__ void __launch_bounds__(QK_THREADS) qk_small_kernel(const __grid_const
     y[i0 + j] = (T)(n_lo * c[j] - n_hi * s[j]);
     y[D / 2 + i0 + j] = (T)(n_hi * c[j] + n_lo * s[j]);
   }
+}
+
+// Up to how many head vectors that is the faster way: once there is more than about one CTA of eight of them per SM, the
+// sines and cosines that every vector forms for itself cost more than a table or a row block per position (32/8 heads, one
+// token each, d = 128: 960 vectors 2.6 against 3.3 us, 1280 alike, 2560 5.5 against 3.3; at d = 64 at twice as many).  With
+// one or two heads in a tensor a chunk of [B,T,H,d] spans so many positions that the line lies half as high again; of
+// [B,H,T,d] with few tokens most rows of a row block are empty (T = 2: 6000 vectors 1.7 times faster, T = 16: alike at 1600).
+constexpr long long QK_SMALL_VECTORS = 4096;               // and no more than these
+long long small_limit(const QkArgs& a, int d, int n_sm) {
+  const long long per = (long long)n_sm * 128 / d;
+  const int rpb = QK_THREADS / (d / 16), few = a.H[1] > 0 && a.H[1] < a.H[0] ? a.H[1] : a.H[0];
+  const long long n = a.layout == RATTN_LAYOUT_BHTD ? 6 * per * a.nblk_t * rpb / a.T : (few < 4 ? 12 : 8) * per;
+  return n < QK_SMALL_VECTORS ? n : QK_SMALL_VECTORS;
 }
 
 template <typename T, int D>
@@ -575,12 +587,15 @@ void fill(const rattn_qk_params* p, QkArgs* a, Freqs* f) {
   a->inv_H[0] = 1.f / (float)p->H_q; a->inv_H[1] = p->H_kv > 0 ? 1.f / (float)p->H_kv : 0.f;
   const int rpb = QK_THREADS / (p->d / 16);
   a->B = p->B; a->T = p->T; a->nblk_t = (p->T + rpb - 1) / rpb;
-  a->layout = p->layout;
+  // One token per entry: [B,H,1,d] and [B,1,H,d] are the same memory, and runs of head vectors serve it better than row
+  // blocks of one row each (103 x 32/8 heads: 14.8 us against 3.4).
+  const int layout = p->T == 1 && p->H_q <= 4096 && p->H_kv <= 4096 ? (int)RATTN_LAYOUT_BTHD : p->layout;
+  a->layout = layout;
   a->tbl_tokens = 0;
   for (int w = 0; w < 2; ++w) {     // [B,H,T,d]: row blocks x heads; [B,T,H,d]: runs of rpb head vectors
-    a->n_chunks[w] = p->layout == RATTN_LAYOUT_BHTD ? p->B * a->nblk_t * a->H[w]
-                                                    : (int)(((long long)p->B * p->T * a->H[w] + rpb - 1) / rpb);
-    if (p->layout != RATTN_LAYOUT_BHTD && a->H[w] > 0 && p->theta > 0.f) {
+    a->n_chunks[w] = layout == RATTN_LAYOUT_BHTD ? p->B * a->nblk_t * a->H[w]
+                                                 : (int)(((long long)p->B * p->T * a->H[w] + rpb - 1) / rpb);
+    if (layout != RATTN_LAYOUT_BHTD && a->H[w] > 0 && p->theta > 0.f) {
       const int tokens = (rpb + a->H[w] - 1) / a->H[w] + 1;      // positions a chunk can touch
       if (tokens > a->tbl_tokens) a->tbl_tokens = tokens;
     }
@@ -678,14 +693,16 @@ int rattn_qk_prologue(const rattn_qk_params* p, void* stream) {
   fill(p, &a, &f);
   a.y[0] = p->q_out; a.y[1] = p->k_out;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if ((long long)p->B * p->T * (p->H_q + p->H_kv) <= QK_SMALL_VECTORS) {
-    cudaError_t e;
+  int n_sm = 0;
+  cudaError_t e = sm_count(&n_sm);
+  if (e != cudaSuccess) return fail(e);
+  if ((long long)p->B * p->T * (p->H_q + p->H_kv) <= small_limit(a, p->d, n_sm)) {
     if (p->dtype == RATTN_BF16) e = p->d == 128 ? launch_small<__nv_bfloat16, 128>(a, f, s) : launch_small<__nv_bfloat16, 64>(a, f, s);
     else e = p->d == 128 ? launch_small<float, 128>(a, f, s) : launch_small<float, 64>(a, f, s);
     return e == cudaSuccess ? RATTN_OK : fail(e);
   }
   int n_cta = 0;
-  cudaError_t e = grid_size(a, QK_CTAS_PER_SM, &n_cta);
+  e = grid_size(a, QK_CTAS_PER_SM, &n_cta);
   if (e == cudaSuccess) e = launch<false>(a, f, p->d, p->dtype, n_cta, s);
   return e == cudaSuccess ? RATTN_OK : fail(e);
 }

@@ -247,3 +247,29 @@ def test_prologue_in_bthd_layout(B, Hq, Hkv, T, d, dtype, theta):
     for b in range(B):
         p = int(pos[b]) + np.arange(T)
         close(tr(qb)[b], P.qk_prologue(np64(q[b]), np64(gq), p, theta), dtype, f"q entry {b}")
+
+
+@pytest.mark.parametrize("d,B,Hq,Hkv,T,layout", [
+    (128, 29, 32, 8, 1, R.LAYOUT_BHTD),      # 1160 vectors: a warp each; 1200: chunks
+    (64, 59, 32, 8, 1, R.LAYOUT_BTHD),       # 2360 and 2400 of half the size
+    (128, 197, 8, 1, 1, R.LAYOUT_BHTD),      # 1773 and 1782: one key head
+    (128, 51, 32, 8, 2, R.LAYOUT_BHTD),      # 4080 and 4160: row blocks of two rows
+    (128, 1, 40, 16, 33, R.LAYOUT_BHTD),     # 1848 (chunks already at one entry) and 3696: two row blocks, the second of one row
+])
+def test_sides_of_the_limit_between_the_kernels(d, B, Hq, Hkv, T, layout):
+    """One batch entry more takes the other kernel: the entries that both calls have come out alike."""
+    gen = torch.Generator(device="cuda").manual_seed(B + T)
+    make = lambda H: torch.randn((B + 1, H, T, d) if layout == R.LAYOUT_BHTD else (B + 1, T, H, d), generator=gen, device="cuda").bfloat16()
+    q, k = make(Hq), make(Hkv)
+    gain = torch.rand(d, generator=gen, device="cuda") + 0.5
+    pos = torch.randint(0, 100000, (B + 1,), generator=gen, device="cuda", dtype=torch.int32)
+    call = lambda n: R.rattn_qk_prologue(q[:n], k[:n], q_gain=gain, k_gain=gain, pos=pos[:n], layout=layout)
+    for a, b in zip(call(B + 1), call(B)):
+        a, b = a[:B].float(), b.float()
+        # the same fp32 arithmetic with sums in another order, rounded once
+        assert (a - b).abs().max().item() <= a.abs().max().item() * 2.0 ** -8
+    if T == 1:                                # [B,H,1,d] is [B,1,H,d]
+        for a, b in zip(call(B + 1), R.rattn_qk_prologue(q.reshape(B + 1, 1, Hq, d), k.reshape(B + 1, 1, Hkv, d), q_gain=gain, k_gain=gain,
+                                                         pos=pos, layout=R.LAYOUT_BTHD)):
+            assert torch.equal(a.reshape(-1), b.reshape(-1))
+    assert R.rattn_qk_prologue_status() == 0
