@@ -406,7 +406,7 @@ cudaError_t launch_bwd(const Args& a, cudaStream_t s) {
     bwd_preprocess_kernel<TIO, D><<<(unsigned)((n_rows + 7) / 8), 256, 0, s>>>(a, do_s, do_r, delta); }
   count_launches(1);
   if (a.grstate) {
-    e = launch_chunk_states<TIO, float, D>(static_cast<const TIO*>(a.q), do_r, a.grstate, a.B, a.T, a.H_kv, a.group, a.layout,
+    e = launch_chunk_states<TIO, float, D>(static_cast<const TIO*>(a.q), do_r, a.grstate, a.B, a.T, a.w, a.H_kv, a.group, a.layout,
                                            RATTN_LAYOUT_BHTD, a.phi, 1, s);
     if (e != cudaSuccess) return e;
   }

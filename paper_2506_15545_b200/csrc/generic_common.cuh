@@ -171,18 +171,19 @@ __device__ __forceinline__ void tile_pv(float4 (&acc)[NA][D / 64], const float* 
 // key tiles, one after another, where it now walks five and a matrix.
 constexpr int GC = 64;        // tokens of a chunk
 
-// term[bh, c] = sum over the output's `group` heads of phi(X_c)^T Y_c; X (type TX) is mapped through phi, Y (type TY) taken
-// as it is; both have H_out * group heads per batch entry.
+// term[bh, c] = sum over the output's `group` heads of phi(X_c)^T Y_c for the chunks c = first .. first + gridDim.x - 1 of n;
+// X (type TX) is mapped through phi, Y (type TY) taken as it is; both have H_out * group heads per batch entry.
 template <typename TX, typename TY, int D>
 __global__ void __launch_bounds__(NT) chunk_term_kernel(const TX* __restrict__ x, const TY* __restrict__ y, float* __restrict__ out,
-                                                        int T, int H_out, int group, int x_layout, int y_layout, int phi) {
+                                                        int T, int H_out, int group, int x_layout, int y_layout, int phi,
+                                                        int first, int n) {
   constexpr int LD = D + PAD, M = D / 16;
   extern __shared__ __align__(16) float smem[];
   float* Xs = smem;
   float* Fs = Xs + GC * LD;
   float* Ys = Fs + GC * LD;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int c = blockIdx.x, bh = blockIdx.y, b = bh / H_out, ho = bh - b * H_out, H = H_out * group;
+  const int c = first + blockIdx.x, bh = blockIdx.y, b = bh / H_out, ho = bh - b * H_out, H = H_out * group;
   float acc[M][M];
 #pragma unroll
   for (int i = 0; i < M; ++i)
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(NT) chunk_term_kernel(const TX* __restrict__ x
         for (int j = 0; j < M; ++j) acc[i][j] += f[i] * v[j];
     }
   }
-  float* o = out + ((size_t)bh * gridDim.x + c) * D * D;
+  float* o = out + ((size_t)bh * n + c) * D * D;
 #pragma unroll
   for (int i = 0; i < M; ++i)
 #pragma unroll
@@ -219,19 +220,20 @@ __global__ void __launch_bounds__(NT) chunk_term_kernel(const TX* __restrict__ x
           make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
 }
 
-// In place along the chunks of each head: suffix = 0: slot c := sum of the slots before it; 1: sum of the slots from it on.
-// A thread walks one float4 of the matrix, eight loads in flight.
-static __global__ void __launch_bounds__(256) chunk_sum_kernel(float4* __restrict__ s, int n_chunks, int vecs, int suffix) {
+// In place along the first (suffix = 0) or last (1) n_chunks of each head's n slots: suffix = 0: slot c := sum of the slots
+// before it (the last slot has no term of its own); 1: sum of the slots from it on.  A thread walks one float4 of the
+// matrix, eight loads in flight.
+static __global__ void __launch_bounds__(256) chunk_sum_kernel(float4* __restrict__ s, int n_chunks, int n, int vecs, int suffix) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= vecs) return;
-  float4* p = s + (size_t)blockIdx.y * n_chunks * vecs + i + (suffix ? (size_t)(n_chunks - 1) * vecs : 0);
+  float4* p = s + (size_t)blockIdx.y * n * vecs + i + (suffix ? (size_t)(n - 1) * vecs : 0);
+  const int n_terms = suffix ? n_chunks : n_chunks - 1;
   const ptrdiff_t step = suffix ? -(ptrdiff_t)vecs : (ptrdiff_t)vecs;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int c0 = 0; c0 < n_chunks; c0 += 8) {
     float4 d[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (c0 + k < n_chunks) d[k] = p[(c0 + k) * step];
+    for (int k = 0; k < 8; ++k) d[k] = c0 + k < n_terms ? p[(c0 + k) * step] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (c0 + k >= n_chunks) break;
@@ -242,17 +244,26 @@ static __global__ void __launch_bounds__(256) chunk_sum_kernel(float4* __restric
   }
 }
 
+// Forms the states that some tile reads, where the sizes leave any: a tile of 32 (or 64) query rows from q0 on reads S_c for
+// c = (q0 - w) / 64, one of 32 (or 64) key rows from j0 on R_c for c = (j0 + 32 + w) / 64 rounded up, or a later one.  With a
+// window about as long as the sequence that is next to nothing (64/16 heads of 64, T = 100, w = 512: the states of all
+// chunks took 16 of a training step's 178 us for nobody).
 template <typename TX, typename TY, int D>
-cudaError_t launch_chunk_states(const TX* x, const TY* y, float* out, int B, int T, int H_out, int group, int x_layout,
+cudaError_t launch_chunk_states(const TX* x, const TY* y, float* out, int B, int T, int w, int H_out, int group, int x_layout,
                                 int y_layout, int phi, int suffix, cudaStream_t s) {
+  const int n = (T + GC - 1) / GC, q_last = (T - 1) / 32 * 32;
+  const int n_sums = suffix ? n - (int)(((long long)w + 32 + GC - 1) / GC) : q_last > w ? (q_last - w) / GC + 1 : 0;
+  const int n_terms = suffix ? n_sums : n_sums - 1, first = suffix ? n - n_terms : 0;      // (S_c takes the chunks before c)
+  if (n_terms <= 0) return cudaSuccess;
   constexpr int smem = 3 * GC * (D + PAD) * (int)sizeof(float);
   const cudaError_t e = allow_smem<chunk_term_kernel<TX, TY, D>>(smem);
   if (e != cudaSuccess) return e;
-  const int n = (T + GC - 1) / GC;
   { KernelTimer kt("generic_terms", s);
-    chunk_term_kernel<TX, TY, D><<<dim3(n, B * H_out), NT, smem, s>>>(x, y, out, T, H_out, group, x_layout, y_layout, phi); }
+    chunk_term_kernel<TX, TY, D><<<dim3(n_terms, B * H_out), NT, smem, s>>>(x, y, out, T, H_out, group, x_layout, y_layout, phi,
+                                                                            first, n); }
   { KernelTimer kt("generic_sums", s);
-    chunk_sum_kernel<<<dim3((D * D / 4 + 255) / 256, B * H_out), 256, 0, s>>>(reinterpret_cast<float4*>(out), n, D * D / 4, suffix); }
+    chunk_sum_kernel<<<dim3((D * D / 4 + 255) / 256, B * H_out), 256, 0, s>>>(reinterpret_cast<float4*>(out), n_sums, n, D * D / 4,
+                                                                              suffix); }
   count_launches(2);
   return cudaGetLastError();
 }

@@ -12,7 +12,7 @@ namespace {
 using namespace generic;
 constexpr int BN = 64;        // keys per tile
 
-// BM: query rows per CTA (64, or 32 where tiles of 64 would leave most of the GPU idle)
+// BM: query rows per CTA (64, or 32 where tiles of 64 would leave half of the GPU idle)
 template <typename TIO, int D, int BM>
 __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
   constexpr int NA = BM / 16;
@@ -185,8 +185,9 @@ __global__ void __launch_bounds__(NT) generic_fwd_kernel(Args a) {
 }
 
 template <typename TIO, int D, int BM>
-cudaError_t launch_tiles(const Args& a, cudaStream_t s) {
-  constexpr int smem = (2 * BM * (D + PAD) + 3 * BN * (D + PAD) + BM * (BN + PAD)) * (int)sizeof(float);
+cudaError_t launch_tiles(const Args& a, cudaStream_t s, bool one_per_sm) {
+  constexpr int used = (2 * BM * (D + PAD) + 3 * BN * (D + PAD) + BM * (BN + PAD)) * (int)sizeof(float);
+  const int smem = one_per_sm && used < 116 * 1024 ? 116 * 1024 : used;         // more than half of an SM's
   const cudaError_t e = allow_smem<generic_fwd_kernel<TIO, D, BM>>(smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.T + BM - 1) / BM, a.B * a.H_q);
@@ -201,11 +202,16 @@ cudaError_t launch_fwd(const Args& a, cudaStream_t s) {
   cudaError_t e = sm_count(&n_sm);
   if (e != cudaSuccess) return e;
   if (a.gstate) {
-    e = launch_chunk_states<TIO, TIO, D>(static_cast<const TIO*>(a.k), static_cast<const TIO*>(a.v), a.gstate, a.B, a.T, a.H_kv, 1,
+    e = launch_chunk_states<TIO, TIO, D>(static_cast<const TIO*>(a.k), static_cast<const TIO*>(a.v), a.gstate, a.B, a.T, a.w, a.H_kv, 1,
                                          a.kv_layout, a.kv_layout, a.phi, 0, s);
     if (e != cudaSuccess) return e;
   }
-  return (long long)((a.T + 63) / 64) * a.B * a.H_q < n_sm ? launch_tiles<TIO, D, 32>(a, s) : launch_tiles<TIO, D, 64>(a, s);
+  // Tiles of 32 rows where tiles of 64 would leave half of the SMs idle (8 heads of 64, T = 300: 72 -> 64 us; with 128 tiles
+  // of 64, T = 1000, 32 rows take 219 us and 64 take 214).  Of tiles of 64 two share an SM; up to one and a half per SM they
+  // take one each, because the first, longest ones end last and would share theirs (T = 1500, 192 tiles: 372 us against 336).
+  const long long tiles = (long long)((a.T + 63) / 64) * a.B * a.H_q;
+  if (2 * tiles <= n_sm) return launch_tiles<TIO, D, 32>(a, s, false);
+  return launch_tiles<TIO, D, 64>(a, s, 2 * tiles <= 3 * n_sm);
 }
 
 }  // namespace

@@ -227,3 +227,31 @@ def test_plain_backward_entry_point():
     ref = O.backward(np64(q), np64(k), np64(v), np64(dy), wl.w, 1.0)
     for got, want in zip((dq, dk, dv), ref):
         assert rel_fro(np64(got), want) <= GRAD_TOL
+
+
+@pytest.mark.parametrize("T,w,states", [
+    (100, 512, 0),          # window longer than the sequence: nothing lies beyond it
+    (192, 96, 4),           # one chunk to the left of the last tile, one to the right of the first
+    (160, 96, 2),           # ... to the right only
+])
+def test_portable_training_forms_the_states_that_are_read(T, w, states):
+    """Launches of a portable training step: forward, preprocess, dq, dk/dv and two kernels per direction with states."""
+    wl = small("gsl", 1, 2, 1, T, 64, w, "f32", 9600 + T, unit=True)
+    q, k, v = (t.cuda() for t in W.make_qkv(wl))
+    dy = W.make_dout(wl).cuda()
+    ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, R.FLAG_SAVE_RESIDUALS)
+    ws.fill_(0xff)
+    before = R.rattn_launch_count()
+    y = R.rattn_forward_ex(q, k, v, w, scale=wl.scale, workspace=ws, save_residuals=True)
+    grads = R.rattn_backward_ex(q, k, v, dy, w, ws, scale=wl.scale, flags=R.FLAG_SAVE_RESIDUALS)
+    assert R.rattn_launch_count() - before == 4 + states
+    check(y, O.forward(np64(q), np64(k), np64(v), w, wl.scale), "f32", "forward")
+    for got, ref in zip(grads, O.backward(np64(q), np64(k), np64(v), np64(dy), w, wl.scale)):
+        assert rel_fro(np64(got), ref) <= 1e-4
+
+
+@pytest.mark.parametrize("T", [512, 577, 1281, 1500, 1825])
+def test_portable_forward_tile_choice(T):
+    """64 tiles of 64 rows (32 rows are taken), 80 (64 from here on), 168 and 192 (one per SM), 232 (two)."""
+    y, ref, _ = run_fwd(small("gft", 1, 8, 2, T, 64, 200, "f32", 9700 + T, unit=True))
+    check(y, ref, "f32", T)
