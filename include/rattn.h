@@ -341,8 +341,9 @@ typedef enum rattn_knob {
                                     throughout; 3 the same, dealt round-robin instead of drawn from a counter.
                                     Automatic = 1 when the state kernel leaves at least half of the SMs free. */
   RATTN_TUNE_GRID = 3,           /* CTAs of the persistent forward kernel: 0 (default) = one per SM */
-  RATTN_TUNE_DECODE_STAGES = 4,  /* 16 KB stages of the staged decode step: 0 (default) = as many as let two
-                                    CTAs share an SM; 4, 6 or 8 (odd values are rounded down, 3 counts as 0) */
+  RATTN_TUNE_DECODE_STAGES = 4,  /* 16 KB stages of the staged decode step: 0 (default) eight where every CTA has an SM to
+                                    itself, else as many as let two CTAs share one; 4, 6 or 8 (odd values are rounded
+                                    down, 3 counts as 0) */
   RATTN_TUNE_STATE_PROGRESS = 5  /* the main kernel takes the chunk states as the chunk-state kernel publishes them
                                     (one progress word per K/V head, work units in sequence order) instead of
                                     waiting for that whole kernel: 0 (default) automatic = on for long chains on

@@ -7,7 +7,7 @@
 // shared by a cluster of 1, 2, 4 or 8 CTAs: each takes a run of ring pieces and of state rows, forms the partial
 // softmax sums and read-outs of them, and the cluster combines these through distributed shared memory.  Everything a
 // CTA will read is requested up front as 16 KB pieces (64 ring slots, or up to 32 state rows) that pass through a
-// ring of stages (as many as let two CTAs share an SM), refilled by whichever warp reads a stage last, so the memory
+// ring of stages (eight, or as many as let two CTAs share an SM), refilled by whichever warp reads a stage last, so the memory
 // system always has the next pieces in flight, whatever the warps are doing.
 //
 // The ring is one pass over K and V pieces together: four warps take the even pieces and four the odd ones, 16 slots
@@ -43,7 +43,7 @@ struct DecodeTcArgs {
   __nv_bfloat16* k_ring; __nv_bfloat16* v_ring; float* state; __nv_bfloat16* out;
   const float* gamma_swa; const float* gamma_rla;
   const int* pos_dev;
-  int B, H_q, H_kv, w, pos, group, phi, stages, cluster;
+  int B, H_q, H_kv, w, pos, group, phi, cluster;
   int debug_wait;             // debug build only, 2: a wait of the last CTA of each cluster counts as run out
   float scale, eps;
 };
@@ -122,24 +122,22 @@ __host__ __device__ inline Plan plan_with(int g, int stages) {
   int off = stages * DT_PIECE;
   auto take = [&](int bytes) { const int at = off; off += (bytes + 15) & ~15; return at; };
   p.q_b = take(8 * QB_STRIDE * 2);         // bf16 [8][136]: the group's queries, rows >= g zero
-  p.q_f = take(g * D * 4);                 // fp32 raw q
+  p.q_f = p.o_swa = take(g * D * 4);       // fp32 raw q; the ring's output once that has been used
   p.fq = take(g * D * 4);                  // phi(q)
   p.vec = take(5 * D * 4);                 // k_new, v_new, k_old, v_old, phi(k_old)
   p.o_warp = take(DT_WARPS * g * D * 4);   // per warp: un-normalised output over its slots
-  p.o_swa = take(g * D * 4);
-  p.o_rla = take(2 * g * D * 4);           // per group of warps
+  // read-out of the state, per group of warps.  For 7 and 8 heads it takes the place of o_warp, behind a barrier of its
+  // own: otherwise one CTA per SM is all that fits (148 heads of 8: 30.8 us a step against 22.0).
+  p.o_rla = g > 6 ? p.o_warp : take(2 * g * D * 4);
   p.w_stat = take(2 * DT_WARPS * 8 * 4);   // per warp and head: maximum, sum
   p.stat = take(3 * 8 * 4);                // per head: this CTA's maximum and sum, logit of the incoming token
   p.bars = take(8 * DT_MAX_STAGES + 4 * DT_MAX_STAGES + 4 * DT_MAX_STAGES + 16);
   p.total = off + 1024;                    // room to align the stages
   return p;
 }
-// As many stages (an even number) as let two CTAs share an SM (each may use (227 KB - 2 KB) / 2), at least four.
-__host__ __device__ inline Plan plan(int g, int forced = 0) {
-  forced &= ~1;
-  if (forced >= 4 && forced <= DT_MAX_STAGES && plan_with(g, forced).total <= 227 * 1024) return plan_with(g, forced);
-  return plan_with(g, plan_with(g, 6).total <= (227 * 1024 - 2048) / 2 ? 6 : 4);
-}
+constexpr int DT_SMEM = 227 * 1024, DT_SMEM_SHARED = (DT_SMEM - 2048) / 2;      // of a CTA alone on its SM; of each of two
+// As many stages as let two CTAs share an SM, at least four.
+inline int lean_stages(int g) { return plan_with(g, 6).total <= DT_SMEM_SHARED ? 6 : 4; }
 
 // ---- cluster: barrier halves, and a read from another CTA's shared memory
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
@@ -162,15 +160,17 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
 // pieces of the ring that one CTA of a cluster of cs takes, of np
 __host__ __device__ inline int pieces_per_rank(int np, int cs) { return (np + cs - 1) / cs; }
 
-template <int G>
-__global__ void __launch_bounds__(DT_THREADS, 2)
+// G: query heads of a group, at most; NS: stages (known when compiled: a piece's stage and the phase of its barrier are
+// divisions by it)
+template <int G, int NS>
+__global__ void __launch_bounds__(DT_THREADS, NS == DT_MAX_STAGES ? 1 : 2)
 decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__ DecodeTcMaps maps) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int g = a.group, w = a.w;
   const int CS = a.cluster, rank = CS > 1 ? (int)(blockIdx.x % CS) : 0;
-  const Plan P = plan(g, a.stages);
-  const int NS = P.stages, NG = NS / 2;                         // stages in all, and of each group of warps
+  const Plan P = plan_with(g, NS);
+  constexpr int NG = NS / 2;                                    // stages of each group of warps
   __nv_bfloat16* q_b = reinterpret_cast<__nv_bfloat16*>(sm + P.q_b);
   float* q_f = reinterpret_cast<float*>(sm + P.q_f);
   float* fq_s = reinterpret_cast<float*>(sm + P.fq);
@@ -486,6 +486,7 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
       }
       release(p);
     }
+    if (P.o_rla == P.o_warp) __syncthreads();                    // everybody has read the warps' shares of the ring
 #pragma unroll
     for (int hh = 0; hh < G; ++hh) {
 #pragma unroll
@@ -578,40 +579,98 @@ decode_tc_kernel(const __grid_constant__ DecodeTcArgs a, const __grid_constant__
   }
 }
 
-template <int G>
-cudaError_t launch_g(const DecodeTcArgs& a, const DecodeTcMaps& m, int smem, cudaStream_t s) {
-  cudaError_t e = allow_smem<decode_tc_kernel<G>>(smem);
-  if (e != cudaSuccess) return e;
-  {
-    KernelTimer kt("decode_step", s);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.B * a.H_kv * a.cluster));
+struct Launch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  Launch(int n_heads, int cluster, int smem, cudaStream_t s) {
+    cfg.gridDim = dim3((unsigned)(n_heads * cluster));
     cfg.blockDim = dim3(DT_THREADS);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
     // the kernel waits for its predecessor itself (griddepcontrol.wait), after its set-up
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)a.cluster;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.cluster > 1 ? 2 : 1;
-    e = cudaLaunchKernelEx(&cfg, decode_tc_kernel<G>, a, m);
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+  }
+  Launch(const Launch&) = delete;
+  Launch& operator=(const Launch&) = delete;
+};
+
+// Clusters of `cluster` CTAs that the current device runs at once, asked of the driver when a device meets another size of
+// shared memory than before (0: it would not say).
+template <int G, int NS>
+int clusters_at_once(int cluster, int smem) {
+  static std::atomic<uint64_t> known[kMaxDevices][4][4];             // smem << 32 | clusters
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  std::atomic<uint64_t>& k = known[dev][cluster == 1 ? 0 : cluster == 2 ? 1 : cluster == 4 ? 2 : 3][(smem >> 12) & 3];
+  const uint64_t seen = k.load(std::memory_order_relaxed);
+  if ((int)(seen >> 32) == smem) return (int)(seen & 0xffffffffu);
+  int n = 0, n_sm = 0;
+  cudaError_t e = allow_smem<decode_tc_kernel<G, NS>>(smem);
+  if (e == cudaSuccess && cluster == 1) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_tc_kernel<G, NS>, DT_THREADS, (size_t)smem);
+    if (e == cudaSuccess) e = sm_count(&n_sm);
+    n *= n_sm;
+  } else if (e == cudaSuccess) {
+    Launch l(1, cluster, smem, nullptr);
+    e = cudaOccupancyMaxActiveClusters(&n, decode_tc_kernel<G, NS>, &l.cfg);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  k.store((uint64_t)smem << 32 | (uint32_t)n, std::memory_order_relaxed);
+  return n;
+}
+
+// CTAs per (batch entry, K/V head), for a ring of `pieces` pieces: as many as still find room on the GPU at once -- a second
+// wave costs more than the shorter shares save, and room for the CTAs is not yet room for their clusters, which do not span
+// GPCs (4 heads a group, w = 512: 64 heads by 4 take 11.1 us a step, 72 heads by 4 20.5 and by 2 13.4) -- and no more than
+// there are pieces to share out: a share of the state alone costs as much as it saves (w = 128, 64 heads: 8.9 us undivided,
+// 9.1 by 2).  0: not even one CTA each finds room.
+template <int G, int NS>
+int cluster_size(int n_heads, int pieces, int g) {
+  const int smem = plan_with(g, NS).total;
+  if (clusters_at_once<G, NS>(1, smem) < n_heads) return 0;
+  int cs = 1;
+  while (cs < 8 && pieces > 2 && 2 * cs <= pieces && clusters_at_once<G, NS>(2 * cs, smem) >= n_heads) cs *= 2;
+  return cs;
+}
+
+template <int G, int NS>
+cudaError_t launch_with(DecodeTcArgs a, const DecodeTcMaps& m, int cluster, cudaStream_t s) {
+  const int smem = plan_with(a.group, NS).total;
+  cudaError_t e = allow_smem<decode_tc_kernel<G, NS>>(smem);
+  if (e != cudaSuccess) return e;
+  a.cluster = cluster > 0 ? cluster : 1;
+  {
+    KernelTimer kt("decode_step", s);
+    const Launch l(a.B * a.H_kv, a.cluster, smem, s);
+    e = cudaLaunchKernelEx(&l.cfg, decode_tc_kernel<G, NS>, a, m);
     if (e != cudaSuccess) return e;
   }
   count_launches(1);
   return cudaGetLastError();
 }
 
-// CTAs per (batch entry, K/V head): as many as still find room on the GPU at once (two per SM).  A second wave costs more
-// than the shorter shares save: at w = 512 and 64 heads clusters of 2 / 4 / 8 take 12.0 / 12.0 / 20.8 us a step, at 256
-// heads 1 / 2 / 4 take 23.6 / 35.7 / 54.6.
-int cluster_size(int n_heads, int n_sm) {
-  int cs = 1;
-  while (cs < 8 && cs * n_heads <= n_sm) cs *= 2;
-  return cs;
+template <int G>
+cudaError_t launch_g(const DecodeTcArgs& a, const DecodeTcMaps& m, int pieces, cudaStream_t s) {
+  const int n_heads = a.B * a.H_kv, knob = tuning(RATTN_TUNE_DECODE_STAGES) & ~1;
+  const int stages = knob >= 4 ? knob : lean_stages(a.group);
+  const int shared = stages == 4 ? cluster_size<G, 4>(n_heads, pieces, a.group)
+                   : stages == 6 ? cluster_size<G, 6>(n_heads, pieces, a.group) : 0;
+  // Where the CTAs find room one to an SM, each takes eight stages: nearly everything it reads is then under way from the
+  // start, and the scheduler cannot put two of them on one SM while others idle (16 sequences of 32/8 heads, w = 64: 11.1 ->
+  // 9.0 us; 8 of w = 256 10.4 -> 9.3; 9 of w = 512 13.4 -> 11.2).  Not where that halves the cluster and leaves eight
+  // pieces or more to a CTA (12 sequences of w = 1024: 22.3 us, shared by two 19.6).
+  const int alone = knob == 8 || knob < 4 ? cluster_size<G, 8>(n_heads, pieces, a.group) : 0;
+  if (knob == 8 || (alone > 0 && (alone >= shared || pieces < 8 * alone))) return launch_with<G, 8>(a, m, alone, s);
+  return stages == 4 ? launch_with<G, 4>(a, m, shared, s) : launch_with<G, 6>(a, m, shared, s);
 }
 
 }  // namespace
@@ -638,17 +697,13 @@ cudaError_t launch_decode_tc(const Args& p, void* k_ring, void* v_ring, float* s
   if (!tc::make_map(&m.k, k_ring, (uint64_t)p.w, (uint64_t)p.B * p.H_kv, 64) ||
       !tc::make_map(&m.v, v_ring, (uint64_t)p.w, (uint64_t)p.B * p.H_kv, 64))
     return cudaErrorInvalidValue;
-  a.stages = tuning(RATTN_TUNE_DECODE_STAGES);
   a.debug_wait = debug_wait();
-  int n_sm = 0;
-  const cudaError_t e = sm_count(&n_sm);
-  if (e != cudaSuccess) return e;
-  a.cluster = cluster_size(p.B * p.H_kv, n_sm);
-  const int smem = plan(p.group, a.stages).total;
-  if (p.group == 1) return launch_g<1>(a, m, smem, s);
-  if (p.group == 2) return launch_g<2>(a, m, smem, s);
-  if (p.group <= 4) return launch_g<4>(a, m, smem, s);
-  return launch_g<8>(a, m, smem, s);
+  a.cluster = 0;                            // launch_g
+  const int pieces = ((pos_dev || pos >= p.w ? p.w : pos) + 63) / 64;
+  if (p.group == 1) return launch_g<1>(a, m, pieces, s);
+  if (p.group == 2) return launch_g<2>(a, m, pieces, s);
+  if (p.group <= 4) return launch_g<4>(a, m, pieces, s);
+  return launch_g<8>(a, m, pieces, s);
 }
 
 int decode_tc_status(cudaStream_t s, cudaError_t* err) {

@@ -19,6 +19,11 @@ pytestmark = pytest.mark.gpu
     (11, 8, 3, 128, 100),        # 2 CTAs, the last piece partly filled
     (19, 8, 8, 192, 1000),       # one CTA per head, an odd number of pieces
     (40, 4, 2, 64, 0),           # one CTA per head, no token yet
+    (2, 8, 8, 512, 700),         # 8 heads a group, whose read-out takes the ring's place: clusters of 4, eight stages
+    (9, 8, 7, 128, 500),         # ... 7 heads, two pieces: one CTA each
+    (9, 8, 4, 512, 5000),        # 72 K/V heads: clusters of 4 would not all fit
+    (12, 8, 4, 1024, 3000),      # 16 pieces: clusters of 2, two CTAs per SM
+    (37, 8, 6, 192, 250),        # 296 heads, two CTAs per SM, four stages
 ])
 def test_decode_clusters_against_the_portable_kernel(B, Hkv, g, w, pos):
     gen = torch.Generator(device="cuda").manual_seed(77 + B)
