@@ -797,7 +797,9 @@ cudaError_t launch_tc_forward_single(const Args& a, cudaStream_t s, bool after_s
   int grid = 2 * n_sm;
   if (tuning(RATTN_TUNE_GRID) > 0 && tuning(RATTN_TUNE_GRID) < grid) grid = tuning(RATTN_TUNE_GRID);
   if (t.n_units < grid) grid = t.n_units;
-  t.work_counter = (order != 3 && t.n_units > 2 * n_sm) ? a.work_counter : nullptr;   // one unit per CTA needs no counter
+  // One unit per CTA needs no counter; behind a chunk-state kernel, whose CTAs keep whole SMs for a while, it does: the CTAs
+  // that find no room until then would start their units last.
+  t.work_counter = (order != 3 && (after_states || t.n_units > 2 * n_sm)) ? a.work_counter : nullptr;
   t.clear_status = after_states ? nullptr : a.clear_status;
   e = allow_smem<tc_fwd1_kernel>(F_SMEM);
   if (e != cudaSuccess) return e;
