@@ -54,8 +54,9 @@ static Plan make_plan(const Args& a, int n_sm) {
   // the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
   const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
   p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) && (p.terms || chain_fits);
-  // The pair kernel where pairs do not fill the GPU: a tile of its own per CTA ends sooner.
-  p.single_tiles = !p.single && !rla && (long long)((n_qt + 1) / 2) * n_q < n_sm;
+  // The pair kernel where there are no more tiles than SMs: a tile of its own per CTA ends sooner.  (With more, the second
+  // wave costs more than that: 32 heads, T = 1000, w = 256, window only: 26.7 us as 256 tiles, 18.6 as 128 pairs.)
+  p.single_tiles = !p.single && !rla && (long long)n_qt * n_q <= n_sm;
   // The main kernel can take the chunk states as the chain publishes them instead of waiting for the whole
   // chain.  That pays where the chain is long and leaves most SMs to the main kernel, which otherwise runs out
   // of work that needs no state (2 x 32/8 heads, T = 8192, w = 512: 422 -> 357 us; 1 x 32/8, T = 2048: 64 -> 58); elsewhere
