@@ -126,7 +126,8 @@ WorkspaceLayout workspace_layout(int B, int H_q, int H_kv, int T, int d, int w, 
   L.rstate = take(tc && rla && train, states * sizeof(__nv_bfloat16));
   const long long terms = (long long)B * H_kv * L.n_chunks;
   const int parts = head_split(terms, H_q / H_kv);
-  L.rdelta = take(tc && rla && ((train && terms <= kMaxParallelTerms) || (L.n_chunks >= kMinTermChunks && terms <= kMaxForwardTerms)),
+  L.rdelta = take(tc && rla && ((train && terms <= (L.n_chunks < kMinTermChunks ? 1 : 2) * kMaxParallelTerms) ||
+                                 (L.n_chunks >= kMinTermChunks && terms <= kMaxForwardTerms)),
                   states * sizeof(float) * (size_t)parts);
   L.kvpart = take(tc && train && parts > 1, 2 * states * sizeof(float) * (size_t)parts);
   // (not for a shape that is merely kept off the tensor-core kernels: that is for comparisons)

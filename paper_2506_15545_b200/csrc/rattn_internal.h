@@ -43,15 +43,17 @@ struct WorkspaceLayout {
 
 // The reverse states of the backward are a running sum over the query tiles of each K/V head.  Walked by one CTA per
 // head (tc_state.cu) the chain takes a microsecond per tile and query head of the group on as few SMs as there are
-// heads.  Up to this many terms (64 KB each) they are formed by a CTA each and summed by a second kernel instead; with
-// more of them the chain runs beside the dq kernel, which hides it.
+// heads.  Up to this many terms (64 KB each; twice as many of long chains) they are formed by a CTA each and summed by a
+// second kernel instead; with more of them the chain runs beside the dq kernel, which hides it.
 constexpr long long kMaxParallelTerms = 512;
 
 // The forward's chain, one CTA per K/V head, takes 2.6 us per chunk when every state is stored.  For long sequences of few
 // heads that is longer than everything else; the workspace then has room for the terms, so that they too can be formed in
-// parallel.  (From 64 chunks on: shorter chains hide under the main kernel.)
+// parallel.  (From 64 chunks on: shorter chains hide under the main kernel.  Up to 384 terms: with more of them, 80 ns each,
+// the chain whose states the main kernel takes as they appear is over sooner: 1 x 16/16 heads, T = 8192, w = 512, 960 terms:
+// 170 us against 119; 1 x 32/8, w = 128, 496: 165 against 155; 1 x 16/4, 240: 92 against 115.)
 constexpr int kMinTermChunks = 64;
-constexpr long long kMaxForwardTerms = 1024;
+constexpr long long kMaxForwardTerms = 384;
 
 // Grouped heads: where the (key tile, K/V head) items of the dk/dv kernel leave most of the GPU idle, an item is split
 // over the group's query heads, whose contributions (fp32) a second kernel adds.  The largest divisor of the group for

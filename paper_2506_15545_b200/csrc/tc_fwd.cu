@@ -53,7 +53,13 @@ static Plan make_plan(const Args& a, int n_sm) {
   // 167; 1 x 16/16, T = 2200, w = 128: 88 against 73; but 1 x 40/8, T = 3541, w = 128, at 1.1: 92 against 116), and the element-wise maps' signed sums feel the rounding (of
   // the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
   const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
-  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) && (p.terms || chain_fits);
+  // Where the pairs all run at once, everything else is over within a unit's time, about 20 us: a chain much
+  // longer than that decides, and the pair kernel's is the shorter one (inference: 1.65 us a step) or leaves it less to do at
+  // the end (1 x 16/4 heads, T = 2200, w = 512: 47 us as single tiles, 37 as pairs; w = 768, two steps fewer: 42 and 41;
+  // training, w = 128: 55 and 50).
+  const bool chain_decides = (long long)((n_qt + 1) / 2) * n_q <= n_sm && chain_ns > (a.training ? 36000 : 30000);
+  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) &&
+             (p.terms || (chain_fits && !chain_decides));
   // The pair kernel where there are no more tiles than SMs: a tile of its own per CTA ends sooner.  (With more, the second
   // wave costs more than that: 32 heads, T = 1000, w = 256, window only: 26.7 us as 256 tiles, 18.6 as 128 pairs.)
   p.single_tiles = !p.single && !rla && (long long)n_qt * n_q <= n_sm;

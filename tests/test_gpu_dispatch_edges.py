@@ -66,10 +66,10 @@ def test_prologue_per_vector_and_chunked_agree(layout, d, dtype):
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,T,w", [
-    (4, 18, 18, 384, 128),       # 144 pairs: single tiles, three per head
-    (10, 16, 4, 300, 128),       # 320 pairs, the second one half empty, one unit drawn after another
-    (1, 37, 37, 1000, 256),      # exactly 148 pairs: no single tiles, one pair per CTA
-    (1, 147, 49, 200, 128),      # 147 pairs: single tiles, two waves
+    (4, 18, 18, 384, 128),       # 216 tiles on two CTAs per SM
+    (10, 16, 4, 300, 128),       # 480, the last of each head half empty, some CTAs taking two
+    (1, 37, 37, 1000, 256),      # 296: one per CTA
+    (1, 147, 49, 200, 128),      # 294
 ])
 def test_forward_single_tiles_and_pairs(B, Hq, Hkv, T, w):
     wl = small("units", B, Hq, Hkv, T, 128, w, "bf16", 9500 + T, unit=True)
@@ -83,6 +83,36 @@ def test_forward_single_tiles_and_pairs(B, Hq, Hkv, T, w):
     g, heads = Hq // Hkv, sorted({0, Hq // 2, Hq - 1})
     for h in heads:
         ref = O.forward(np64(q[-1:, h:h + 1]), np64(k[-1:, h // g:h // g + 1]), np64(v[-1:, h // g:h // g + 1]), w, wl.scale)
+        check(y[-1:, h:h + 1], ref, "bf16", f"head {h}")
+    assert np.isfinite(np64(y)).all()
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,T,w,mode,train", [
+    (1, 4, 1, 1100, 896, R.MODE_RATTN, False),     # the widest window of the single-tile kernel in inference
+    (1, 4, 1, 1300, 1024, R.MODE_RATTN, False),    # ... pairs, the last one half empty
+    (1, 4, 1, 1800, 1536, R.MODE_RATTN, True),     # ... single tiles in training
+    (1, 4, 1, 1900, 1664, R.MODE_RATTN, True),     # ... pairs
+    (1, 16, 4, 1400, 128, R.MODE_RATTN, False),    # 96 pairs, a chain of 9 steps: single tiles
+    (1, 16, 4, 2200, 128, R.MODE_RATTN, False),    # 144 pairs, a chain of 16 steps that decides: pairs, one per CTA behind it
+    (1, 16, 16, 2200, 128, R.MODE_RATTN, True),    # ... in training
+    (1, 37, 37, 512, 128, R.MODE_SWA_ONLY, False),     # 148 tiles: one per SM
+    (1, 37, 37, 513, 128, R.MODE_SWA_ONLY, False),     # 185 tiles: 111 pairs
+    (2, 18, 9, 500, 128, R.MODE_FULL_CAUSAL, False),   # 144 tiles
+    (1, 60, 20, 700, 128, R.MODE_FULL_CAUSAL, True),   # 360 tiles: 180 pairs, drawn from the counter
+])
+def test_forward_kernel_by_window_chain_and_mode(B, Hq, Hkv, T, w, mode, train):
+    wl = small("rule", B, Hq, Hkv, T, 128, w, "bf16", 9400 + T, unit=True)
+    q, k, v = W.make_qkv(wl)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    ws = R.alloc_workspace(qd, kd, w, mode, R.FLAG_SAVE_RESIDUALS if train else 0)
+    ws.fill_(0xff)
+    y = R.rattn_forward_ex(qd, kd, vd, w, scale=wl.scale, mode=mode, workspace=ws, save_residuals=train)
+    torch.cuda.synchronize()
+    assert R.rattn_read_status(ws) == 0
+    g = Hq // Hkv
+    for h in sorted({0, Hq // 2, Hq - 1}):
+        ref = O.forward(np64(q[-1:, h:h + 1]), np64(k[-1:, h // g:h // g + 1]), np64(v[-1:, h // g:h // g + 1]), w, wl.scale,
+                        mode=mode)
         check(y[-1:, h:h + 1], ref, "bf16", f"head {h}")
     assert np.isfinite(np64(y)).all()
 
