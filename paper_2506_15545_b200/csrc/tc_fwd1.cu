@@ -631,26 +631,31 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
           tmem_ld16(tO + 16 * c, orl);
           tmem_wait_ld();
         }
-        float y[16];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&stash[8 * c + e]));
-          y[2 * e] = f.x;
-          y[2 * e + 1] = f.y;
-        }
-        if constexpr (has_gains) {
-          if (gs) apply_gain16(y, gs + 16 * c);
-        }
-        if constexpr (has_rla) {
-          if constexpr (has_gains) {
-            if (gr) apply_gain16(orl, gr + 16 * c);
-          }
-#pragma unroll
-          for (int e = 0; e < 16; ++e) y[e] += orl[e] * rr;
-        }
         uint32_t yk[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) yk[e] = pack_bf16(y[2 * e], y[2 * e + 1]);
+        for (int e = 0; e < 4; ++e) {                                  // four of them: sixteen outputs and gains at once spill
+          const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&stash[8 * c + 2 * e]));
+          const float2 f1 = __half22float2(*reinterpret_cast<const __half2*>(&stash[8 * c + 2 * e + 1]));
+          float4 y = make_float4(f0.x, f0.y, f1.x, f1.y);
+          if constexpr (has_gains) {
+            if (gs) {
+              const float4 g = __ldg(reinterpret_cast<const float4*>(gs + 16 * c) + e);
+              y.x *= g.x; y.y *= g.y; y.z *= g.z; y.w *= g.w;
+            }
+          }
+          if constexpr (has_rla) {
+            float4 x = make_float4(orl[4 * e] * rr, orl[4 * e + 1] * rr, orl[4 * e + 2] * rr, orl[4 * e + 3] * rr);
+            if constexpr (has_gains) {
+              if (gr) {
+                const float4 g = __ldg(reinterpret_cast<const float4*>(gr + 16 * c) + e);
+                x.x *= g.x; x.y *= g.y; x.z *= g.z; x.w *= g.w;
+              }
+            }
+            y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
+          }
+          yk[2 * e] = pack_bf16(y.x, y.y);
+          yk[2 * e + 1] = pack_bf16(y.z, y.w);
+        }
         *reinterpret_cast<uint4*>(stage + swz(r, 2 * c)) = make_uint4(yk[0], yk[1], yk[2], yk[3]);
         *reinterpret_cast<uint4*>(stage + swz(r, 2 * c + 1)) = make_uint4(yk[4], yk[5], yk[6], yk[7]);
       }
