@@ -686,10 +686,12 @@ def run_timeline(args):
     """Where one CTA of the forward kernel spends a work unit: the library is rebuilt with its clock
     stamps compiled in (librattn_tl.so), one forward of the small case (B=2 of config 2; --train for
     the training-mode forward of config 4) is run, and the stamps of CTA 7's two row groups are
-    printed as cycles since the unit began.  Stamp ids: 200+i first scores of stream position i
-    seen, 300+i row maxima done, 400+i weights handed over, 503 phi(Q) done, 504 phi(K) done,
-    501 window accumulator complete, 502 window output parked, 530 residual products complete,
-    535 residuals for the backward stored, 540 output stored."""
+    printed as cycles since the unit began: of the pair kernel a unit's two tiles, of the
+    single-tile kernel the two column halves of its tile.  Stamp ids: 200+i first scores of stream
+    position i (pairs: key tiles, single tiles: half tiles) seen, 300+i row maxima done, 400+i
+    weights handed over, 503 phi(Q) done (single tiles: both maps), 504 phi(K) done, 501 window
+    accumulator complete, 502 window output parked, 530 residual products complete, 535 residuals
+    for the backward stored, 540 output stored."""
     import ctypes
     from paper_2506_15545_b200 import binding as R
     from paper_2506_15545_b200 import build as B
@@ -706,7 +708,7 @@ def run_timeline(args):
     for _ in range(3):
         R.rattn_forward_ex(q, k, v, wl.w, scale=wl.scale, workspace=ws, out=out, save_residuals=args.train)
         torch.cuda.synchronize()
-        L.rattn_timeline_read(buf, n)
+        tiles = L.rattn_timeline_read(buf, n)
     units = []
     for role in range(2):
         ev = [(int(buf[role * 2048 + 2 * i]), int(buf[role * 2048 + 2 * i + 1])) for i in range(n[role])]
@@ -719,7 +721,7 @@ def run_timeline(args):
                 if e == 540:
                     units.append({"row_group": "AB"[role], **marks})
     print(json.dumps({"case": "timeline", "workload": workload_name(wl), "training_mode": bool(args.train),
-                      "units_of_cta_7": units}))
+                      "query_tiles_per_unit": tiles, "units_of_cta_7": units}))
 
 
 def run_sweep(args):

@@ -500,6 +500,28 @@ __device__ __forceinline__ float feature_map_row_any(unsigned char* tile, int r,
   return 1.f;
 }
 
+// ------------------------------------------------------------------------ timeline
+// For tuning (compiled in only with -DRATTN_TIMELINE): one CTA of the kernel in this file records (event id, clock) pairs
+// per role.
+#ifdef RATTN_TIMELINE
+static __device__ unsigned long long g_timeline[4][2048];
+static __device__ int g_timeline_n[4];
+#define TL_DECL(on_expr) const bool tl_on = (on_expr); int tl_i = 0; (void)tl_on; (void)tl_i
+#define TL(role, id) do { if (tl_on && tl_i < 1000) { unsigned long long c_; asm volatile("mov.u64 %0, %%clock64;" : "=l"(c_) :: "memory"); \
+    g_timeline[role][2 * tl_i] = (unsigned long long)(id); g_timeline[role][2 * tl_i + 1] = c_; ++tl_i; g_timeline_n[role] = tl_i; } } while (0)
+// the records so far, which are cleared; whether there were any
+static bool read_timeline(unsigned long long* out, int* n) {
+  const int none[4] = {0, 0, 0, 0};
+  cudaMemcpyFromSymbol(out, g_timeline, sizeof(g_timeline));
+  cudaMemcpyFromSymbol(n, g_timeline_n, sizeof(g_timeline_n));
+  cudaMemcpyToSymbol(g_timeline_n, none, sizeof(none));
+  return n[0] + n[1] + n[2] + n[3] > 0;
+}
+#else
+#define TL_DECL(on_expr) do { } while (0)
+#define TL(role, id) do { } while (0)
+#endif
+
 // ------------------------------------------------------------------------ work items
 // Of persistent kernels: a CTA's next item comes from a device-wide counter, so that CTAs that start late
 // (the SM was still running another kernel) or meet heavy items simply take fewer.  The loader warp draws it and

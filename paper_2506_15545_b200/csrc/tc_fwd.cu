@@ -124,4 +124,16 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
   return p.single ? launch_tc_forward_single(m, s, p.chain) : launch_tc_forward_main(m, s, p.chain);
 }
 
+#ifdef RATTN_TIMELINE
+bool read_timeline_single(unsigned long long* out, int* n);
+bool read_timeline_pair(unsigned long long* out, int* n);
+#endif
+
 }  // namespace rattn
+
+#ifdef RATTN_TIMELINE
+// Records of the forward kernel that has run since the last call; how many query tiles its units have (0: no record).
+extern "C" int rattn_timeline_read(unsigned long long* out, int* n) {
+  return rattn::read_timeline_single(out, n) ? 1 : rattn::read_timeline_pair(out, n) ? 2 : 0;
+}
+#endif

@@ -389,11 +389,13 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
   auto max2 = [](float p, float q) { return fmaxf(p, q); };
   auto add2 = [](float p, float q) { return p + q; };
 
+  TL_DECL(blockIdx.x == 7 && r == 0);
   for (int n = 0;; ++n) {
     const int u = sched_read_all(&bars->sched, n);
     if (u < 0) break;
     const Unit un = make_unit(a, u);
     if (un.t < 0) continue;
+    TL(h, 1000 + u);
     const int L = 2 * un.n;
     const int q0 = (un.t - a.off) * TILE;          // first query row of the tile (un.t is its key-space index)
 
@@ -410,6 +412,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #ifdef RATTN_DEBUG_KNOBS
       if (a.debug_wait == 2 && h == 1 && n == 0 && s == 0) bars->abort = 1;      // as if this half's wait had run out
 #endif
+      TL(h, 200 + s);
       tc_fence_after();
       const bool diag = s < 2, bound = un.c >= 0 && s >= L - 2;
       const bool kept = !(diag && chunk > wq) && !(bound && chunk < wq);
@@ -444,6 +447,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
         m_ref = m_new;
       }
       tc_fence_after();
+      TL(h, 300 + s);
       // weights, written back (fp16, two per column) over the score columns
       uint32_t pk[16];
       if (kept) {
@@ -471,6 +475,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       if (!(a.debug_wait == 1 && n == 0 && s == 0))
 #endif
       mbar_arrive(&bars->p_ready[b]);
+      TL(h, 400 + s);
     }
     cs += un.n;
 
@@ -492,6 +497,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       }
       fence_proxy_async_smem();
       mbar_arrive(&bars->phi_ready);
+      TL(h, 503);
       pair_sync(wq);
       inv_q = *ex;
       pair_sync(wq);
@@ -501,6 +507,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     // ---- park the normalised window output (Section 3.2, first norm) in registers ---------
     WAIT_ON(bars->o_ready, co & 1);
     ++co;
+    TL(h, 501);
     tc_fence_after();
     const float inv_l = 1.f / l;
     uint32_t stash[32];
@@ -526,6 +533,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     }
 
     // ---- residual branch, second part -------------------------------------------------------
+    TL(h, 502);
     float rr = 0.f;
     if (un.rla) {
       tc_fence_before();
@@ -568,6 +576,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       rr = inv_q * rsqrtf(sr * inv_q * inv_q * (1.f / 128.f) + a.eps);     // o_rla = inv_q * accumulator
     }
     ring.base += unit_uses(un);
+    TL(h, 530);
 
     // ---- Section 3.2: gains, sum; outputs leave through the tile's Q buffer ---------------
     // (every product that reads Q has completed) by TMA: plain 16-byte global stores from row owners keep
@@ -619,6 +628,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       }
       send(&tm.o_rla, false);
     }
+    TL(h, 535);
     const float* gs = a.gamma_swa ? a.gamma_swa + (size_t)un.h * 128 + 64 * h : nullptr;
     const float* gr = a.gamma_rla ? a.gamma_rla + (size_t)un.h * 128 + 64 * h : nullptr;
     // The branches on "gains given" and "tile has a residual branch" are taken once, outside the loops.
@@ -672,6 +682,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
     }
     send(&tm.out, true);
     const int t = q0 + r;
+    TL(h, 540);
     if (h == 0 && t < a.T && a.lse) a.lse[(size_t)un.bh_q * a.T + t] = (m_ref + log2f(l)) * 0.6931471805599453f;
   }
   if (r == 0) tma_store_wait();          // this thread's stores have completed before the CTA may go
@@ -762,6 +773,10 @@ tc_fwd1_kernel(const __grid_constant__ FMaps tm, FArgs a) {
 }
 
 }  // namespace
+
+#ifdef RATTN_TIMELINE
+bool read_timeline_single(unsigned long long* out, int* n) { return tc::read_timeline(out, n); }
+#endif
 
 cudaError_t launch_tc_forward_single(const Args& a, cudaStream_t s, bool after_states) {
   FMaps tm;

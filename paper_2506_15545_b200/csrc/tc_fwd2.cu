@@ -127,19 +127,6 @@ __device__ __forceinline__ Unit make_unit(const FArgs& a, int u) {
 
 __device__ __forceinline__ bool active(const Unit& un, int X, int i) { return un.t[X] >= 0 && i >= un.i0[X] && i <= un.i1[X]; }
 
-// Optional timeline for tuning (compiled in only with -DRATTN_TIMELINE): one CTA records
-// (event id, clock) pairs per role.
-#ifdef RATTN_TIMELINE
-__device__ unsigned long long g_timeline[4][2048];
-__device__ int g_timeline_n[4];
-#define TL_DECL(on_expr) const bool tl_on = (on_expr); int tl_i = 0; (void)tl_on; (void)tl_i
-#define TL(role, id) do { if (tl_on && tl_i < 1000) { unsigned long long c_; asm volatile("mov.u64 %0, %%clock64;" : "=l"(c_) :: "memory"); \
-    g_timeline[role][2 * tl_i] = (unsigned long long)(id); g_timeline[role][2 * tl_i + 1] = c_; ++tl_i; g_timeline_n[role] = tl_i; } } while (0)
-#else
-#define TL_DECL(on_expr) do { } while (0)
-#define TL(role, id) do { } while (0)
-#endif
-
 // the MMA warp's own events cost it issue slots: they are a second switch (-DRATTN_TIMELINE_MMA)
 #ifdef RATTN_TIMELINE_MMA
 #define TLM(role, id) TL(role, id)
@@ -836,13 +823,7 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
 }  // namespace
 
 #ifdef RATTN_TIMELINE
-extern "C" int rattn_timeline_read(unsigned long long* out, int* n) {
-  cudaMemcpyFromSymbol(out, g_timeline, sizeof(g_timeline));
-  cudaMemcpyFromSymbol(n, g_timeline_n, sizeof(g_timeline_n));
-  int z[4] = {0, 0, 0, 0};
-  cudaMemcpyToSymbol(g_timeline_n, z, sizeof(z));
-  return 0;
-}
+bool read_timeline_pair(unsigned long long* out, int* n) { return tc::read_timeline(out, n); }
 #endif
 
 cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_states) {
