@@ -28,7 +28,6 @@ __device__ __forceinline__ uint64_t kmajor_base(uint32_t base) { return smem_des
 __device__ __forceinline__ uint64_t mnmajor_base(uint32_t base) { return smem_desc(base, HALF_BYTES, 1024); }
 __host__ __device__ constexpr uint32_t kstep_k(int k, int half_bytes) { return (uint32_t)(((k >> 2) * half_bytes + (k & 3) * 32) >> 4); }
 __host__ __device__ constexpr uint32_t kstep_mn(int k) { return (uint32_t)((k * 2048) >> 4); }
-__device__ __forceinline__ uint64_t kmajor_desc(uint32_t base, int kstep) { return kmajor_base(base) + kstep_k(kstep, HALF_BYTES); }
 __device__ __forceinline__ uint64_t mnmajor_desc(uint32_t base, int kstep) { return mnmajor_base(base) + kstep_mn(kstep); }
 
 // D[128x128] (+)= A B^T-style products over a reduction of 128, 8 MMAs of K = 16.  (Unrolled on
@@ -105,26 +104,6 @@ __device__ __forceinline__ void load_tile(unsigned char* dst, const CUtensorMap*
 __device__ __forceinline__ void load_half_tile(unsigned char* dst, const CUtensorMap* tm, uint64_t* bar, int row, int z) {
   tma_load_3d(dst, tm, bar, 0, row, z);
   tma_load_3d(dst + HT_HALF, tm, bar, 64, row, z);
-}
-
-// The same for bf16 output: 32 values of row r become one 64-byte row of an 8 KB region
-// (16-byte chunks XOR-swizzled by row pair), flushed in 64-byte segments, eight rows per
-// instruction.  dst points at column 32*c of the tile's first row (row pitch 128 bf16).
-__device__ __forceinline__ void stage_bf16_block(unsigned char* stage, int r, const float (&x)[32]) {
-#pragma unroll
-  for (int e = 0; e < 4; ++e)
-    *reinterpret_cast<uint4*>(stage + r * 64 + ((e ^ ((r >> 1) & 3)) << 4)) =
-        make_uint4(pack_bf16(x[8 * e], x[8 * e + 1]), pack_bf16(x[8 * e + 2], x[8 * e + 3]),
-                   pack_bf16(x[8 * e + 4], x[8 * e + 5]), pack_bf16(x[8 * e + 6], x[8 * e + 7]));
-}
-__device__ __forceinline__ void flush_bf16_block(const unsigned char* stage, int r, __nv_bfloat16* dst, int n_rows) {
-  const int sub = r & 3;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = (r >> 5) * 32 + 8 * k + ((r & 31) >> 2);
-    const uint4 v = *reinterpret_cast<const uint4*>(stage + row * 64 + ((sub ^ ((row >> 1) & 3)) << 4));
-    if (row < n_rows) *reinterpret_cast<uint4*>(dst + (size_t)row * 128 + 8 * sub) = v;
-  }
 }
 
 // The element-wise maps of the paper's ablation (Table 6) on packed bf16 pairs: ReLU; the
@@ -296,26 +275,6 @@ __device__ __forceinline__ void store_tile(const CUtensorMap* tm, const unsigned
   tma_store_3d(tm, tile + HALF_BYTES, 64, row0, z);
 }
 
-// Row-owner r holds 32 fp32 values (columns 32*c .. 32*c+31 of its row).  Stages them in a
-// 16 KB region ([128 rows x 128 bytes], 16-byte chunks XOR-swizzled by row) so that the 128
-// row owners can then write the [128 x 32] block to global memory with full 128-byte segments.
-__device__ __forceinline__ void stage_f32_block(unsigned char* stage, int r, const float (&x)[32]) {
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    *reinterpret_cast<float4*>(stage + r * 128 + ((e ^ (r & 7)) << 4)) =
-        make_float4(x[4 * e], x[4 * e + 1], x[4 * e + 2], x[4 * e + 3]);
-}
-// dst points at column 32*c of the tile's first row (row pitch 128 floats); rows >= n_rows are skipped.
-__device__ __forceinline__ void flush_f32_block(const unsigned char* stage, int r, float* dst, int n_rows) {
-  const int sub = r & 7;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int row = (r >> 5) * 32 + 4 * k + ((r & 31) >> 3);
-    const float4 v = *reinterpret_cast<const float4*>(stage + row * 128 + ((sub ^ (row & 7)) << 4));
-    if (row < n_rows) *reinterpret_cast<float4*>(dst + (size_t)row * 128 + 4 * sub) = v;
-  }
-}
-
 // Bit e of the result says whether column 32*c + e of a [128 x 128] score tile is kept for row
 // r: on the diagonal tile the keys j <= r, on the oldest tile of the band the keys j >= r.
 __device__ __forceinline__ uint32_t keep_bits(int r, int c, bool diag, bool bound) {
@@ -350,18 +309,6 @@ __device__ __forceinline__ void mask32(float (&x)[32], uint32_t keep) {
 #pragma unroll
   for (int e = 0; e < 32; ++e) x[e] = (keep >> e) & 1u ? x[e] : -INFINITY;
 }
-__device__ __forceinline__ float max32_masked(const float (&x)[32], uint32_t keep) {
-  float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
-#pragma unroll
-  for (int e = 0; e < 32; e += 4) {
-    m0 = fmaxf(m0, (keep >> e) & 1u ? x[e] : -INFINITY);
-    m1 = fmaxf(m1, (keep >> (e + 1)) & 1u ? x[e + 1] : -INFINITY);
-    m2 = fmaxf(m2, (keep >> (e + 2)) & 1u ? x[e + 2] : -INFINITY);
-    m3 = fmaxf(m3, (keep >> (e + 3)) & 1u ? x[e + 3] : -INFINITY);
-  }
-  return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
-}
-
 // The helpers below walk a row in sixteen 16-byte steps with a rolled loop: compact code
 // matters more than loop overhead here (large unrolled kernels are instruction-fetch bound).
 // Row maximum of row r of a swizzled bf16 tile.

@@ -859,7 +859,7 @@ cudaError_t launch_tc_forward_main(const Args& a, cudaStream_t s, bool after_sta
   const int order = tuning(RATTN_TUNE_UNIT_ORDER);
   const bool stateless_first = order == 1 || (order == 0 && 2 * a.B * a.H_kv <= n_sm);
   if (a.mode == RATTN_MODE_RATTN && after_states && !a.state_in && stateless_first) {
-    t.n_stateless = (a.w / TILE) / t.per_unit + 1;
+    t.n_stateless = (a.w / TILE) / 2 + 1;                            // (units of this mode are pairs)
     if (t.n_stateless > t.n_pairs) t.n_stateless = t.n_pairs;
   }
   t.wait_for_states = after_states ? 1 : 0;
