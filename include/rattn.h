@@ -331,8 +331,9 @@ size_t rattn_timing_read(char* buf, size_t buf_bytes);
  * sweep in profiles/ found best on B200.
  */
 typedef enum rattn_knob {
-  RATTN_TUNE_STATE_STRIDE = 0,   /* m: 0 = automatic (2 for an inference forward, whose query-tile pairs read every
-                                    second chunk state; 1 when the backward will read them all), 1, 2 */
+  RATTN_TUNE_STATE_STRIDE = 0,   /* m: 0 = automatic (1 when the backward will read every chunk state and for the kernel of
+                                    single query tiles, which does too; 2 for the kernel of query-tile pairs, which reads
+                                    every second one), 1; 2: an inference forward takes the pair kernel */
   RATTN_TUNE_OVERLAP = 1,        /* 1 (default): the main kernel starts under the chunk-state kernel
                                     (programmatic dependent launch); 0: strictly one after the other */
   RATTN_TUNE_UNIT_ORDER = 2,     /* order in which the persistent forward kernel hands out its work units:
@@ -340,14 +341,17 @@ typedef enum rattn_knob {
                                     under the chunk-state kernel), then heaviest first; 2 heaviest first
                                     throughout; 3 the same, dealt round-robin instead of drawn from a counter.
                                     Automatic = 1 when the state kernel leaves at least half of the SMs free. */
-  RATTN_TUNE_GRID = 3,           /* CTAs of the persistent forward kernel: 0 (default) = one per SM */
+  RATTN_TUNE_GRID = 3,           /* CTAs of the persistent forward kernel: 0 (default) = one per SM (pairs of query tiles)
+                                    or two (single tiles) */
   RATTN_TUNE_DECODE_STAGES = 4,  /* 16 KB stages of the staged decode step: 0 (default) eight where every CTA has an SM to
                                     itself, else as many as let two CTAs share one; 4, 6 or 8 (odd values are rounded
                                     down, 3 counts as 0) */
   RATTN_TUNE_STATE_PROGRESS = 5  /* the main kernel takes the chunk states as the chunk-state kernel publishes them
                                     (one progress word per K/V head, work units in sequence order) instead of
-                                    waiting for that whole kernel: 0 (default) automatic = on for long chains on
-                                    few K/V heads with windows up to 512 (T >= 6144, 4 B H_kv <= SMs); 1 on; 2 off */
+                                    waiting for that whole kernel: 0 (default) automatic = on for long chains on few K/V
+                                    heads (at least 48 key tiles, 4 B H_kv <= SMs, windows up to 512 or, single tiles,
+                                    1024; single tiles also from 16 key tiles on for 8 B H_kv <= SMs); 1 on; 2 off.
+                                    With 1 or 2 the states are never formed as parallel terms */
 } rattn_knob;
 int rattn_tune(int knob, int value);
 

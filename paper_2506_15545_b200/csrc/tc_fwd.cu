@@ -59,7 +59,8 @@ static Plan make_plan(const Args& a, int n_sm) {
   // training, w = 128: 55 and 50).
   const bool chain_decides = (long long)((n_qt + 1) / 2) * n_q <= n_sm && chain_ns > (a.training ? 36000 : 30000);
   p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) &&
-             (p.terms || (chain_fits && !chain_decides));
+             (p.terms || (chain_fits && !chain_decides)) &&
+             !(p.chain && !a.training && tuning(RATTN_TUNE_STATE_STRIDE) == 2);
   // The pair kernel where there are no more tiles than SMs: a tile of its own per CTA ends sooner.  (With more, the second
   // wave costs more than that: 32 heads, T = 1000, w = 256, window only: 26.7 us as 256 tiles, 18.6 as 128 pairs.)
   p.single_tiles = !p.single && !rla && (long long)n_qt * n_q <= n_sm;

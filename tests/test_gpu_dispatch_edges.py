@@ -117,6 +117,27 @@ def test_forward_kernel_by_window_chain_and_mode(B, Hq, Hkv, T, w, mode, train):
     assert np.isfinite(np64(y)).all()
 
 
+def test_state_stride_knob():
+    """m = 2 takes the pair kernel where single tiles would run: another kernel, the same operator."""
+    wl = small("stride", 1, 8, 2, 1000, 128, 256, "bf16", 9450, unit=True)
+    q, k, v = W.make_qkv(wl)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    ws = R.alloc_workspace(qd, kd, wl.w, R.MODE_RATTN, 0)
+    out = {}
+    try:
+        for m in (0, 1, 2):
+            R.rattn_tune(R.TUNE_STATE_STRIDE, m)
+            ws.fill_(0xff)
+            out[m] = R.rattn_forward_ex(qd, kd, vd, wl.w, scale=wl.scale, workspace=ws)
+            assert R.rattn_read_status(ws) == 0
+    finally:
+        R.rattn_tune(R.TUNE_STATE_STRIDE, 0)
+    assert torch.equal(out[0], out[1]) and not torch.equal(out[0], out[2])
+    ref = O.forward(np64(q[:, 3:4]), np64(k[:, 0:1]), np64(v[:, 0:1]), wl.w, wl.scale)
+    for y in out.values():
+        check(y[:, 3:4], ref, "bf16")
+
+
 @pytest.mark.parametrize("B,Hq,Hkv,T,w", [
     (8, 16, 16, 4096, 512),      # every key tile comes from HBM: loads in flight land out of order
     (1, 40, 8, 2048, 256),       # ... mostly from L2
