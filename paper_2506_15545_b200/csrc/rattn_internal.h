@@ -57,7 +57,8 @@ constexpr long long kMaxForwardTerms = 384;
 
 // Grouped heads: where the (key tile, K/V head) items of the dk/dv kernel leave most of the GPU idle, an item is split
 // over the group's query heads, whose contributions (fp32) a second kernel adds.  The largest divisor of the group for
-// which the parts still run at once, one per SM of a B200.
+// which the parts still run at once, one per SM of a B200: 148 is written in because the workspace's layout depends on
+// this and is computed without a device.
 inline int head_split(long long items, int group) {
   for (int n = group; n > 1; --n)
     if (group % n == 0 && items * n <= 148) return n;

@@ -36,23 +36,26 @@ static Plan make_plan(const Args& a, int n_sm) {
   if (p.n_steps < 0) p.n_steps = 0;
   p.chain = n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
   const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
-  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one), the main
-  // kernel 30 ns per query tile and 12 ns per tile and key tile with all SMs at work, and no less than 40 us as far as this
-  // matters.  Where the chain of a long sequence on few heads would outlast the main kernel, its terms are formed in
-  // parallel (1 x 8/1 heads, T = 16384, w = 512: 202 -> 113 us).
+  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one), the main kernel
+  // 30 ns per query tile and 12 ns per tile and key tile, and no less than 40 us as far as this matters.  (Fitted on a B200
+  // with all of its 148 SMs at work and every window full: short sequences, whose first tiles read less, and ragged batches
+  // have less work than this says.)  Where the chain of a long sequence on few heads would outlast the main kernel, its terms
+  // are formed in parallel (1 x 8/1 heads, T = 16384, w = 512: 202 -> 113 us).
   const long long chain_ns = 2600ll * p.n_steps;
   const long long work_ns = (long long)n_qt * n_q * (30 + 12 * (wt + 1)), main_ns = work_ns < 40000 ? 40000 : work_ns;
   p.terms = p.chain && a.rdelta && knob == 0 && n_kt >= kMinTermChunks && (long long)n_kv * a.n_chunks <= kMaxForwardTerms &&
             chain_ns > main_ns;
-  // The single-tile kernel wins where the window loop is not everything: 1.05 - 1.28 times at w <= 768 (8 x 32/8 heads,
-  // T = 4397, w = 128, training: 748 -> 610 us; 4 x 16/16, T = 4096, w = 512: 215 -> 201), in training, where all states are
-  // stored and three outputs leave per tile, up to w = 1536; at w = 1408 and 2048 the pair kernel is 8 - 10 % faster in
-  // inference.  It needs every state, in bf16, where of a pair the second tile takes the chunk in between exactly: a chain
-  // that outlasts the main kernel by far decides against it (16 heads, T = 16384, w = 128), in inference, where the pair
-  // kernel's chain stores half of the states, from 1.2 - 1.4 times on (1 x 16/4 heads, T = 6298, w = 768: 203 us against
-  // 167; 1 x 16/16, T = 2200, w = 128: 88 against 73; but 1 x 40/8, T = 3541, w = 128, at 1.1: 92 against 116), and the element-wise maps' signed sums feel the rounding (of
-  // the output's bound of 2e-2 the last rounding alone takes 1.6e-2 above 4).
-  const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
+  // The single-tile kernel wins where the window loop is not everything: 1.05 - 1.28 times where measured up to w = 768 (8 x
+  // 32/8 heads, T = 4397, w = 128, training: 748 -> 610 us; 4 x 16/16, T = 4096, w = 512: 215 -> 201), in training, where all
+  // states are stored and three outputs leave per tile, up to w = 1536; at w = 1408 and 2048 the pair kernel is 8 - 10 % faster
+  // in inference.  The lines are drawn at 7 key tiles (w = 896) and, in training, at 12.  It needs every state, in bf16, where
+  // of a pair the second tile takes the chunk in between exactly: a chain that outlasts the main kernel by far decides against
+  // it (16 heads, T = 16384, w = 128), in inference, where the pair kernel's chain stores half of the states, from 1.2 - 1.4
+  // times on (1 x 16/4 heads, T = 6298, w = 768: 203 us against 167; 1 x 16/16, T = 2200, w = 128: 88 against 73; but 1 x 40/8,
+  // T = 3541, w = 128, at 1.1: 92 against 116), and the element-wise maps' signed sums feel the rounding (of the output's bound
+  // of 2e-2 the last rounding alone takes 1.6e-2 above 4).
+  const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns
+                                     : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
   // Where the pairs all run at once, everything else is over within a unit's time, about 20 us: a chain much
   // longer than that decides, and the pair kernel's is the shorter one (inference: 1.65 us a step) or leaves it less to do at
   // the end (1 x 16/4 heads, T = 2200, w = 512: 47 us as single tiles, 37 as pairs; w = 768, two steps fewer: 42 and 41;

@@ -19,17 +19,18 @@
 //   goes to HBM.
 //   Section 3.2: y = g_s * o_swa / rms(o_swa) + g_r * o_rla / rms(o_rla), staged in the tile's Q buffer and written by TMA.
 //
-// Why two small CTAs.  A unit is a chain of dependent phases (scores -> row threads -> products, then the feature maps,
-// the residual products, the epilogue), none of which fills the SM alone, and the window loop is less than half of it.  The
-// pair kernel (tc_fwd2.cu: one CTA per SM, two adjacent tiles sharing each K/V tile) has both tiles in the same phase most
-// of the time: 47.5k cycles per pair at w = 512, of which the tensor pipe works 14k and the exponential unit 13k.  Two
-// independent CTAs drift apart, so that one's feature maps and epilogue pass under the other's window loop: 38k cycles per
-// tile and CTA, i.e. 19k per tile against 23.7k.  Half of TMEM (256 columns) holds the accumulator and two 64-column score
-// buffers, so the scores of the next step are ready when the row threads come for them.  The price: every K/V tile is
+// Why two small CTAs. A unit is a chain of dependent phases (scores -> row threads -> products, then the feature maps, the
+// residual products, the epilogue), none of which fills the SM alone, and the window loop is less than half of it. The pair
+// kernel (tc_fwd2.cu: one CTA per SM, two adjacent tiles sharing each K/V tile) has both tiles in the same phase most of
+// the time: 41k cycles per pair at w = 512 for the late units (up to 60k for earlier ones), of which the tensor pipe works
+// 14k and the exponential unit 13k. Two independent CTAs drift apart, so that one's feature maps and epilogue pass under
+// the other's window loop: 34 - 42k cycles per tile and CTA, i.e. 17 - 21k per tile against 20.5k and more (2 x 16/16
+// heads, T = 4096; clock stamps of single units). Half of TMEM (256 columns) holds the accumulator and two 64-column score
+// buffers, so the scores of the next step are ready when the row threads come for them. The price: every K/V tile is
 // fetched once per query tile (L2 delivers that: measured 70 bytes per clock and SM to two CTAs with copies in flight, half
 // of it used), the N = 64 score products read Q from shared memory twice as often (shared memory carries 2.0k cycles per
 // tile and key tile against the pair's 1.3k, about what the row threads take), and every tile reads a state of its own, so
-// all of them are stored.  Without the residual part (control modes) the pair kernel is the faster one.
+// all of them are stored. Without the residual part (control modes) the pair kernel is the faster one.
 #include <type_traits>
 
 #include "tc_common.cuh"
