@@ -155,8 +155,8 @@ template <typename T, bool BWD> struct Ring {
 //                 row block, head, so consecutive chunks share their positions and a thread forms its 8
 //                 sines and cosines once per row block.
 //   [B, T, H, d]: memory is a sequence of head vectors in (b, t, h) order; a chunk = RPB consecutive ones
-//                 (a few positions' worth).  The sines and cosines of a chunk's positions are formed once
-//                 per CTA, one chunk ahead, in a small shared-memory table.
+//                 (a few positions' worth).  The sines and cosines are formed once per CTA, for sixteen or more
+//                 positions at a time, in a shared-memory table.
 // A cursor is set once and then stepped.
 struct Cursor {
   int which;            // 0: q, 1: k
@@ -232,7 +232,7 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
   float* red = reinterpret_cast<float*>(smem + S * R::kBufs * R::kChunk);         // [RPB][D] (backward)
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * R::kBufs * R::kChunk + R::kRed);
   volatile int* abort = reinterpret_cast<volatile int*>(full + S);
-  float2* tbl = reinterpret_cast<float2*>(smem + R::kBytes);                      // [2][tbl_tokens][D/2] (cos, sin)
+  float2* tbl = reinterpret_cast<float2*>(smem + R::kBytes);                      // [tbl_tokens][D/2] (cos, sin)
 
   const int tid = threadIdx.x, l = tid % LPR, row = tid / LPR;
   const long long n_all = (long long)a.n_chunks[0] + a.n_chunks[1];           // < 2^31, checked on the host
@@ -290,15 +290,22 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
     __syncthreads();
   };
 
-  // [B, T, H, d]: cos and sin of every (position, pair) of the cursor's chunk into table `buf`, one entry per
-  // thread and round (a chunk of RPB head vectors spans RPB / H positions, plus one when it straddles)
+  // [B, T, H, d]: cos and sin of every (position, pair) of the tokens from chunk i on, as many as the table holds or this CTA
+  // still meets in the tensor.  Pairs 8l + j, 8l + j + 1 of a token lie together, those of neighbouring lanes l side by
+  // side, so that a chunk's loads meet every bank once.
+  // Formed for every chunk anew, by a quarter to half of the threads and ahead of a barrier, they were most of a chunk's time
+  // (1 x 40/8 heads, T = 8192: forward 71 -> 57 us, backward 94 -> 80).
   const bool tabled = BTHD && a.rotate;
-  auto fill_table = [&](const Cursor& cx, int buf) {
+  int tbl_first = 0, tbl_end = 0;                       // the tokens (entry b, position t: number b T + t) in the table
+  auto tbl_at = [&](int tok, int pair) { return tok * (D / 2) + (((pair & 7) >> 1) * LPR + (pair >> 3)) * 2 + (pair & 1); };
+  auto fill_table = [&](const Cursor& cx, int i) {
     constexpr double kTwoPi = 6.283185307179586476925286766559;
-    size_t at_;
-    int rows_;
-    where<RPB, ROW, BTHD>(a, cx, &at_, &rows_);
-    const int n_tok = small_div(cx.h0 + rows_ - 1, a.inv_H[cx.which]) + 1;
+    const int H = a.H[cx.which];
+    long long v_end = ((long long)cx.c + (hi - i)) * RPB;
+    if (v_end > (long long)a.B * a.T * H) v_end = (long long)a.B * a.T * H;
+    tbl_first = cx.b0 * a.T + cx.t0;
+    const int n_tok = min((int)((v_end - 1) / H) - tbl_first + 1, a.tbl_tokens);
+    tbl_end = tbl_first + n_tok;
     for (int e = tid; e < n_tok * (D / 2); e += QK_THREADS) {
       const int tok = e / (D / 2), pair = e % (D / 2);
       int t = cx.t0 + tok, b = cx.b0;
@@ -308,11 +315,10 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
       ang -= kTwoPi * rint(ang * (1.0 / kTwoPi));
       float sn, cs;
       sincosf((float)ang, &sn, &cs);
-      tbl[((size_t)buf * a.tbl_tokens + tok) * (D / 2) + pair] = make_float2(cs, sn);
+      tbl[tbl_at(tok, pair)] = make_float2(cs, sn);
     }
   };
   Cursor ch = cursor_at<RPB>(a, lo);
-  if (tabled && lo < hi) fill_table(ch, 0);
   if (!a.rotate) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) { c[j] = 1.f; s[j] = 0.f; }
@@ -340,17 +346,20 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
         cur_rb = rb;
       }
     } else if (tabled) {
-      // the next chunk's table while this chunk's data is on its way; this chunk's was written one
-      // iteration ago (or before the loop) and the barrier in between made it visible
-      if (i + 1 < hi) {
-        Cursor nx = ch;
-        step<BTHD, RPB>(a, nx);
-        fill_table(nx, (n + 1) & 1);
+      // Table fills are rare (a table holds the positions of many chunks) and pass under the copies in flight.  The
+      // barrier at the end of an iteration has everybody's last reads behind it.
+      const int tok0 = ch.b0 * a.T + ch.t0;
+      if (tok0 < tbl_first || tok0 + small_div(ch.h0 + ch_rows - 1, a.inv_H[ch.which]) >= tbl_end) {
+        fill_table(ch, i);
+        __syncthreads();
       }
-      const int tok = small_div(ch.h0 + row, a.inv_H[ch.which]);
-      const float2* e = tbl + ((size_t)(n & 1) * a.tbl_tokens + (row < ch_rows ? tok : 0)) * (D / 2) + 8 * l;
+      const int tok = tok0 - tbl_first + (row < ch_rows ? small_div(ch.h0 + row, a.inv_H[ch.which]) : 0);
+      const float4* e = reinterpret_cast<const float4*>(tbl + tbl_at(tok, 8 * l));
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { c[j] = e[j].x; s[j] = e[j].y; }
+      for (int j = 0; j < 8; j += 2) {
+        const float4 v = e[(j >> 1) * LPR];
+        c[j] = v.x; s[j] = v.y; c[j + 1] = v.z; s[j + 1] = v.w;
+      }
     }
     const bool live = row < ch_rows;
     unsigned char* buf = stage + (size_t)slot * R::kBufs * R::kChunk + (size_t)row * ROW;
@@ -596,8 +605,9 @@ void fill(const rattn_qk_params* p, QkArgs* a, Freqs* f) {
     a->n_chunks[w] = layout == RATTN_LAYOUT_BHTD ? p->B * a->nblk_t * a->H[w]
                                                  : (int)(((long long)p->B * p->T * a->H[w] + rpb - 1) / rpb);
     if (layout != RATTN_LAYOUT_BHTD && a->H[w] > 0 && p->theta > 0.f) {
-      const int tokens = (rpb + a->H[w] - 1) / a->H[w] + 1;      // positions a chunk can touch
-      if (tokens > a->tbl_tokens) a->tbl_tokens = tokens;
+      // at least the positions a chunk can touch; of sixteen, 8 KB, three CTAs share an SM with the eight stages of bf16
+      const int tokens = (rpb + a->H[w] - 1) / a->H[w] + 1;
+      if (a->tbl_tokens < (tokens > 16 ? tokens : 16)) a->tbl_tokens = tokens > 16 ? tokens : 16;
     }
   }
   a->eps = p->eps;
@@ -633,7 +643,7 @@ cudaError_t grid_size(const QkArgs& a, int per_sm, int* n_cta) {
 
 template <typename T, int D, bool BWD, bool BTHD>
 cudaError_t launch_layout(const QkArgs& a, const Freqs& f, int n_cta, cudaStream_t s) {
-  const int smem = Ring<T, BWD>::kBytes + 2 * a.tbl_tokens * (D / 2) * (int)sizeof(float2);
+  const int smem = Ring<T, BWD>::kBytes + a.tbl_tokens * (D / 2) * (int)sizeof(float2);
   cudaError_t e = allow_smem<qk_prologue_kernel<T, D, BWD, BTHD>>(smem);
   if (e != cudaSuccess) return e;
   KernelTimer kt(BWD ? "qk_prologue_bwd" : "qk_prologue", s);

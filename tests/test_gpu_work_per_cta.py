@@ -1,0 +1,36 @@
+"""Work that a persistent CTA does after its first piece: the rotation table of the prologue refilled."""
+import pytest
+import torch
+
+from paper_2506_15545_b200 import binding as R
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,T,d,dtype,entry_pos", [
+    (1, 40, 8, 3000, 128, torch.bfloat16, False),    # a CTA's share of q: tens of positions
+    (2, 3, 2, 7001, 128, torch.bfloat16, True),      # several refills, a batch entry's end inside a table
+    (3, 2, 1, 9000, 64, torch.bfloat16, False),      # one head: more positions in a chunk than the usual table holds
+    (700, 5, 3, 7, 128, torch.float32, True),        # many short entries
+    (2500, 4, 1, 1, 64, torch.float32, True),        # one token each
+])
+def test_prologue_rotation_table(B, Hq, Hkv, T, d, dtype, entry_pos):
+    """[B, T, H, d] takes sines and cosines from a table, [B, H, T, d] forms them per row: the same numbers."""
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda").to(dtype)
+    q, k, dq, dk = rnd(B, T, Hq, d), rnd(B, T, Hkv, d), rnd(B, T, Hq, d), rnd(B, T, Hkv, d)
+    gains = dict(q_gain=1 + 0.1 * rnd(d).float(), k_gain=1 + 0.1 * rnd(d).float())
+    if entry_pos:
+        gains["pos"] = torch.randint(0, 100000, (B,), generator=g, device="cuda", dtype=torch.int32)
+    t = lambda x: x.transpose(1, 2).contiguous()
+    a = R.rattn_qk_prologue(q, k, layout=R.LAYOUT_BTHD, **gains)
+    b = R.rattn_qk_prologue(t(q), t(k), **gains)
+    for x, y in zip(a, b):
+        assert torch.equal(t(x), y)
+    a = R.rattn_qk_prologue_backward(q, k, dq, dk, layout=R.LAYOUT_BTHD, **gains)
+    b = R.rattn_qk_prologue_backward(t(q), t(k), t(dq), t(dk), **gains)
+    for x, y in zip(a[:2], b[:2]):
+        assert torch.equal(t(x), y)
+    for x, y in zip(a[2:], b[2:]):                   # fp32 sums of B T H terms in another order
+        assert (x - y).abs().max() <= 1e-4 * y.abs().max()
+    assert R.rattn_qk_prologue_status() == 0, "a device-side wait expired"
