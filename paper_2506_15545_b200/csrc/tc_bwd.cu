@@ -173,18 +173,21 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
 #pragma unroll
   for (int e = 0; e < 8; ++e) gs_lo[e] = gs_hi[e] = gr_lo[e] = gr_hi[e] = 1.f;
   int cur_h = -1;
-  auto flush = [&]() {                                              // this CTA's sums for head cur_h
+  // This CTA's sums for head cur_h.  The four rows of a warp are added first and share the additions to memory: with every
+  // row adding for itself these were 4.8 million at 40 heads, T = 8192 (145 -> 113 us with gains).
+  auto flush = [&]() {
     if (cur_h < 0) return;
+    const int part = (tid >> 3) & 3;                                // 0, 1: the window branch's halves, 2, 3: the other's
+    float* dst = part < 2 ? a.dgamma_s : a.rla_on ? a.dgamma_r : nullptr;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      if (a.dgamma_s) {
-        atomicAdd(a.dgamma_s + (size_t)cur_h * 128 + 8 * l + e, acc_s[e]);
-        atomicAdd(a.dgamma_s + (size_t)cur_h * 128 + 64 + 8 * l + e, acc_s[8 + e]);
+      float v[4] = {acc_s[e], acc_s[8 + e], acc_r[e], acc_r[8 + e]};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], 8);
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
       }
-      if (a.dgamma_r && a.rla_on) {
-        atomicAdd(a.dgamma_r + (size_t)cur_h * 128 + 8 * l + e, acc_r[e]);
-        atomicAdd(a.dgamma_r + (size_t)cur_h * 128 + 64 + 8 * l + e, acc_r[8 + e]);
-      }
+      if (dst) atomicAdd(dst + (size_t)cur_h * 128 + 64 * (part & 1) + 8 * l + e, part & 2 ? (part & 1 ? v[3] : v[2]) : (part & 1 ? v[1] : v[0]));
       acc_s[e] = acc_s[8 + e] = acc_r[e] = acc_r[8 + e] = 0.f;
     }
   };
