@@ -810,11 +810,14 @@ tc_bwd_dq_kernel(const __grid_constant__ DqMaps tm, BwdArgs a, int n_items, int 
 // and dK accumulators in TMEM.  The work is a list of items, one per (query head of the
 // group, query half tile of 64 rows): first the residual-branch items (query tile j + wt),
 // then the window items (query tiles j .. j + wt).  Two row groups of 256 threads (two per key
-// row = TMEM lane) take the items alternately, each with its own TMEM slot, so that one
-// group's exponentials overlap the other group's products:
+// row = TMEM lane) take the items alternately, so that one group's exponentials overlap the
+// other group's products.  One TMEM buffer holds the scores of an item: they are read into registers at once, and the
+// next item's replace them; each group has columns of its own for its weights.  (With scores and weights in a slot per
+// group, the scores of an item waited for the products of the one two before: 488 -> 476 us at 8 x 16/16 heads, T = 4096,
+// w = 512.)
 //   loader warp     TMA: K, V, [R_j], then per item Q_h, g_h and the query-side row statistics; stores dV, dK
-//   score warp      per item: S^T = K Q_h^T and dP^T = V g_h^T into the slot (128 x 64 each)
-//   accumulate warp after the row group has overwritten them with bf16 P^T and dS^T:
+//   score warp      per item: S^T = K Q_h^T and dP^T = V g_h^T (128 x 64 each)
+//   accumulate warp from the row group's bf16 P^T and dS^T:
 //                   dV += P^T g_h, dK += dS^T Q_h with the A operand read from TMEM
 //   row group       P^T = exp2(S^T * scale_log2 - lse2[q]), dS^T = P^T (dP^T scale - D[q] scale)
 // The residual items run first and leave dphi_k in the dK accumulator; the row groups then fold
@@ -832,7 +835,7 @@ constexpr int KV_ROW_WARPS = 16;
 constexpr int KV_THREADS = 32 * (KV_ROW_WARPS + 4);        // 2 row groups; score, loader and accumulate warp (and one idle)
 
 struct KvBars {
-  uint64_t kv_full, kphi_ready, full[KV_NS], acc_done[KV_NS], s_full[2], p_ready[2], phiq_ready[2],
+  uint64_t kv_full, kphi_ready, full[KV_NS], acc_done[KV_NS], s_full[2], s_read, p_ready[2], p_free[2], phiq_ready[2],
       r_acc_done, fold_done, all_done, acc_free, kv_free, out_staged, drain, drain2;
   SchedRing sched;
   uint32_t tmem_base;
@@ -970,19 +973,16 @@ __device__ bool kv_loader(const KvMaps& tm, const BwdArgs& a, unsigned char* sme
 // The products are issued by two warps: the score warp issues S^T and dP^T of every item, the accumulate
 // warp everything that writes the dV / dK accumulators, so that the waits of one (a wait that is already
 // satisfied still costs an issuing warp some 300 cycles) pass under the products of the other.  A third
-// issuer (S^T and dP^T apart) measured no faster: what then limits an item is the chain scores -> row
-// group -> accumulate on its TMEM slot, of which there are two.  Order between the two warps:
+// issuer (S^T and dP^T apart) measured no faster.  Order between the two warps:
 //   scores(n) -> row group -> p_ready -> accumulate(n)        (existing barriers)
-//   accumulate(n - 2) complete -> scores(n) may overwrite the TMEM slot they share   (acc_done of n - 2's stage)
+//   scores(n - 1) in registers -> scores(n)                   (s_read)
+//   accumulate(n - 2) complete -> the group's next weights     (p_free)
 __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem) {
   const uint32_t sK = smem_u32(smem + KV_OFF_K), sV = smem_u32(smem + KV_OFF_V), sKphi = smem_u32(smem + KV_OFF_KPHI);
   const uint32_t sStage = smem_u32(smem + KV_OFF_STAGE);
-  // slot s: [S^T | dP^T] at columns 256 + 128 s and 320 + 128 s (computed, not looked up: an array
-  // indexed by the slot would live in local memory)
-  const uint32_t tS0 = tmem + 256, tP0 = tmem + 320;
+  const uint32_t tS = tmem + 256, tP = tmem + 320;
   KvCount c = {0, 0, 0, 0};
-  int cq0 = 0, cq1 = 0;                                    // phi(Q_h) hand-overs per TMEM slot
-  int seq_m1 = -1, seq_m2 = -1;                            // ring uses of the last two items (the previous key tile's at first)
+  int cq0 = 0, cq1 = 0;                                    // phi(Q_h) hand-overs per row group
 
   for (;; ++c.it) {
     int idx;
@@ -999,16 +999,14 @@ __device__ bool kv_mma_scores(const BwdArgs& a, unsigned char* smem, KvBars* bar
       // the reverse state's use of this slot is over (this warp has not followed it, and may not skip a phase)
       if (n == KV_NS - 1 && pl.has_inter) WAIT_OR_RETURN_W(bars->acc_done[st], (use - 1) & 1);
       WAIT_OR_RETURN_W(bars->full[st], use & 1);
-      if (seq_m2 >= 0) WAIT_OR_RETURN_W(bars->acc_done[seq_m2 % KV_NS], (seq_m2 / KV_NS) & 1);   // the TMEM slot's previous item is over
-      seq_m2 = seq_m1;
-      seq_m1 = seq0 + n;
+      if (gi0 + n >= 1) WAIT_OR_RETURN_W(bars->s_read, (gi0 + n - 1) & 1);   // the item before is in registers
       if (pl.is_r(n)) {
         WAIT_OR_RETURN_W(bars->phiq_ready[slot], (slot ? cq1 : cq0) & 1);
         if (slot) ++cq1; else ++cq0;
       }
       tc_fence_after();
-      mma_k_kh(tS0 + 128 * slot, pl.is_r(n) ? sKphi : sK, sQh);   // S^T  = K Q_h^T   (phi(K) phi(Q_h)^T)
-      mma_k_kh(tP0 + 128 * slot, sV, sGh);                         // dP^T = V g_h^T
+      mma_k_kh(tS, pl.is_r(n) ? sKphi : sK, sQh);          // S^T  = K Q_h^T   (phi(K) phi(Q_h)^T)
+      mma_k_kh(tP, sV, sGh);                               // dP^T = V g_h^T
       mma_commit(&bars->s_full[slot]);
       if (n == pl.N - 1) mma_commit(&bars->kv_free);
     }
@@ -1023,7 +1021,7 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
   const uint32_t sV = smem_u32(smem + KV_OFF_V), sKphi = smem_u32(smem + KV_OFF_KPHI);
   const uint32_t sStage = smem_u32(smem + KV_OFF_STAGE);
   const uint32_t tV = tmem, tK = tmem + 128;
-  const uint32_t tS0 = tmem + 256, tP0 = tmem + 320;
+  const uint32_t tW = tmem + 384;                          // the weights of row group g at columns 64 g: P^T, then dS^T
   KvCount c = {0, 0, 0, 0};
 
   for (;; ++c.it) {
@@ -1055,9 +1053,10 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
       if (m == pl.n_R && pl.n_R > 0) WAIT_OR_RETURN_W(bars->fold_done, c.cr & 1);
       if (!acc_ok) { WAIT_OR_RETURN_W(bars->acc_free, (c.it - 1) & 1); acc_ok = true; }
       tc_fence_after();
-      mma_ts_h(tV, tS0 + 128 * slot, sGh, accV);           // dV += P^T g_h
-      mma_ts_h(tK, tP0 + 128 * slot, sQh, accK);           // dK += dS^T Q_h   (dphi_k += dA^T phi(Q_h))
+      mma_ts_h(tV, tW + 64 * slot, sGh, accV);             // dV += P^T g_h
+      mma_ts_h(tK, tW + 64 * slot + 32, sQh, accK);        // dK += dS^T Q_h   (dphi_k += dA^T phi(Q_h))
       accV = accK = true;
+      mma_commit(&bars->p_free[slot]);
       mma_commit(&bars->acc_done[st]);
       if (m == pl.n_R - 1) mma_commit(&bars->r_acc_done);
     }
@@ -1070,12 +1069,12 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
 }
 
 __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int g, int h, int r) {
-  // Two groups of 256 threads, one per TMEM slot.  A thread is key row r = TMEM lane and half h of its item's 64 query
+  // Two groups of 256 threads.  A thread is key row r = TMEM lane and half h of its item's 64 query
   // columns: with all 64 on one thread a warp had a scheduler almost to itself and an item's arithmetic took 1530 cycles of
   // the 4400 from scores to scores on a slot.
   const uint32_t lane_off = (uint32_t)((r & ~31) << 16);
   const uint32_t tV = tmem + lane_off, tK = tmem + 128 + lane_off;
-  const uint32_t tS = tmem + 256 + 128 * g + 32 * h + lane_off, tP = tS + 64;
+  const uint32_t tS = tmem + 256 + 32 * h + lane_off, tP = tS + 64, tW = tmem + 384 + 64 * g + 16 * h + lane_off;
   const int gt = h * 128 + r;                                  // thread of the group
   KvCount cnt = {0, 0, 0, 0};
 
@@ -1095,7 +1094,7 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
   const int seq0 = cnt.seq + (pl.has_inter ? 1 : 0), gi0 = cnt.gi;
 
   for (int n = 0; n < pl.N; ++n) {
-    if (((gi0 + n) & 1) != g) continue;                       // the other TMEM slot's item
+    if (((gi0 + n) & 1) != g) continue;                       // the other group's item
     const int st = (seq0 + n) % KV_NS, use = (seq0 + n) / KV_NS;
     const bool is_r = pl.is_r(n);
     const int i = pl.qtile(n), hf = pl.half(n);
@@ -1121,6 +1120,8 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
     tmem_ld32(tS, s);
     tmem_ld32(tP, dp);
     tmem_wait_ld();
+    tc_fence_before();
+    mbar_arrive(&bars->s_read);                                // the next item's scores may come
     const int rd = r - (64 * hf + 32 * h);                     // key row relative to this thread's first query
     uint32_t pk1[16], pk2[16];
     if (is_r) {
@@ -1153,9 +1154,12 @@ __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uin
         }
       }
     }
-    // bf16 results (two per column) overwrite the first half of the columns just consumed
-    tmem_st16(tS, pk1);
-    tmem_st16(tP, pk2);
+    // bf16 results, two per column, once the group's previous ones have been consumed
+    const int gn = (gi0 + n) >> 1;
+    if (gn >= 1) WAIT_ON(bars->p_free[g], (gn - 1) & 1);
+    tc_fence_after();
+    tmem_st16(tW, pk1);
+    tmem_st16(tW + 32, pk2);
     tmem_wait_st();
     tc_fence_before();
     mbar_arrive(&bars->p_ready[g]);
@@ -1274,8 +1278,10 @@ tc_bwd_dkv_kernel(const __grid_constant__ KvMaps tm, BwdArgs a, int n_items) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->s_full[i], 1);
       mbar_init(&bars->p_ready[i], 16 * KV_ROW_WARPS);
+      mbar_init(&bars->p_free[i], 1);
       mbar_init(&bars->phiq_ready[i], 16 * KV_ROW_WARPS);
     }
+    mbar_init(&bars->s_read, 16 * KV_ROW_WARPS);
     mbar_init(&bars->r_acc_done, 1);
     mbar_init(&bars->fold_done, 32 * KV_ROW_WARPS);
     mbar_init(&bars->all_done, 1);
