@@ -9,13 +9,16 @@
 // caller wants the decode state, once more in fp32 at the end.  phi (softmax over the head
 // features, Section 3.1) is applied to the loaded tile in shared memory.
 //
-// The chain is a pipeline of four roles, so that a step costs little more than its slowest
+// The chain is a pipeline of five roles, so that a step costs little more than its slowest
 // stage (the feature map, bound by the exponential unit):
 //   loader warp    TMA: X and Y tiles of the next chunks into a ring of three stages
-//   8 phi warps    feature map of the X tile in place, two lanes per row
+//   16 phi warps   feature map of the X tile in place, four lanes per row
 //   MMA warp       acc += phi(X)^T Y as soon as the tile is mapped
-//   4 flush warps  after a stored step: accumulator -> registers (the MMA warp goes on as soon as
-//                  the TMEM loads have landed) -> bf16 -> staging tile -> TMA store
+//   8 flush warps  after a stored step: accumulator -> registers (the MMA warp goes on as soon as
+//                  the TMEM loads have landed) -> bf16 -> staging tile; two threads per row
+//   store warp     staging tile -> TMA store, and the number of stored states where they are published
+// With eight phi and four flush warps, which looked for the staging tile only once they held the sum, a step took 2.6 us
+// where every sum is stored and 1.65 where every second one is.
 #include <climits>
 
 #include "tc_common.cuh"
@@ -31,7 +34,8 @@ constexpr int ST_STAGE = 2 * TILE_BYTES;                   // X tile + Y tile
 constexpr int ST_OFF_OUT = ST_NS * ST_STAGE;               // staging for one [128 x 128] bf16 matrix
 constexpr int ST_OFF_BAR = ST_OFF_OUT + TILE_BYTES;
 constexpr int ST_SMEM = ST_OFF_BAR + 128;
-constexpr int ST_THREADS = 448;                            // 8 phi warps, MMA warp, loader warp, 4 flush warps
+constexpr int ST_PHI_WARPS = 16, ST_FLUSH_WARP = 20;      // 16: MMA warp, 17: loader warp, 18: store warp (19 is idle)
+constexpr int ST_THREADS = 32 * (ST_FLUSH_WARP + 8);
 
 struct StateArgs {
   int n_steps;      // chunks to walk
@@ -59,7 +63,7 @@ struct StateArgs {
 };
 
 struct StBars {
-  uint64_t full[ST_NS], phi_ready[ST_NS], free_[ST_NS], done, acc_free;
+  uint64_t full[ST_NS], phi_ready[ST_NS], free_[ST_NS], done, acc_free, staged, stage_free;
   uint32_t tmem_base;
   int abort;
 };
@@ -101,19 +105,21 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   if (tid == 0) {
     for (int i = 0; i < ST_NS; ++i) {
       mbar_init(&bars->full[i], 1);
-      mbar_init(&bars->phi_ready[i], 256);
+      mbar_init(&bars->phi_ready[i], 32 * ST_PHI_WARPS);
       mbar_init(&bars->free_[i], 1);
     }
     mbar_init(&bars->done, 1);
-    mbar_init(&bars->acc_free, 128);
+    mbar_init(&bars->acc_free, 256);
+    mbar_init(&bars->staged, 256);
+    mbar_init(&bars->stage_free, 1);
     bars->abort = 0;
     fence_mbar_init();
   }
-  if (warp == 8) {
+  if (warp == ST_PHI_WARPS) {
     tmem_alloc(&bars->tmem_base, 128);
     tmem_relinquish();
   }
-  if (tid == 288) {
+  if (tid == 32 * (ST_PHI_WARPS + 1)) {
     prefetch_map(&tm_x);
     prefetch_map(&tm_y);
     prefetch_tensormap(&tm_out);
@@ -129,83 +135,44 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   const int n_items = n_steps * group;
   bool ok = true;
 
-  if (warp < 8) {
-    // ---- feature map of the X tile, in place: two adjacent lanes per row ------------------
+  // registers follow the work: 512 x 64 + 128 x 48 + 256 x 96, within the CTA's 896 x 72
+  if (warp < ST_PHI_WARPS) {
+    setmaxnreg_dec<64>();
+    // ---- feature map of the X tile, in place: four adjacent lanes per row -----------------
     for (int it = 0; it < n_items && ok; ++it) {
       const int st = it % ST_NS, use = it / ST_NS;
-      ok = mbar_wait(&bars->full[st], use & 1, &bars->abort);
+      ok = mbar_wait_warp(&bars->full[st], use & 1, &bars->abort);
       if (!ok) break;
-      unsigned char* xh = smem + st * ST_STAGE + (tid & 1) * HALF_BYTES;
-      const int row = tid >> 1;
+      const int row = tid >> 2, q = tid & 3;
+      unsigned char* x = smem + st * ST_STAGE + row * 128;
       const int token = (first + a.dir * (it / group)) * TILE + row;
-      // every lane maps its row (the softmax map exchanges partial results between the two lanes
+      // every lane maps its row (the softmax map exchanges partial results between the lanes
       // of a row with full-warp shuffles, so no lane may skip it); rows past the limit are then cleared
-      feature_map_pair_any(xh, xh, row, a.phi);
+      feature_map_quad(x, x, HALF_BYTES, row, q, a.phi);
+      __syncwarp();
       if (token >= row_limit) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) *reinterpret_cast<uint4*>(xh + row * 128 + (c << 4)) = make_uint4(0, 0, 0, 0);
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(x + (q >> 1) * HALF_BYTES + ((4 * (q & 1) + c) << 4)) = make_uint4(0, 0, 0, 0);
       }
       fence_proxy_async_smem();
       mbar_arrive(&bars->phi_ready[st]);
     }
-  } else if (warp == 8) {
-    // ---- acc[128 features x 128] += phi(X)^T Y   (both operands MN-major: rows are the tokens)
-    int n_wait = 0;                                          // hand-backs of the accumulator so far
-    for (int it = 0; it < n_items && ok; ++it) {
-      const int st = it % ST_NS, use = it / ST_NS;
-      const int s = it / group, hh = it - s * group;
-      ok = mbar_wait_warp(&bars->phi_ready[st], use & 1, &bars->abort);
-      // the flush warps hold the previous sum, or are still writing the incoming state into the accumulator
-      if (ok && hh == 0 && ((s > 0 && flushed_step(a, s - 1, n_steps)) || (s == 0 && has_init))) {
-        ok = mbar_wait_warp(&bars->acc_free, n_wait & 1, &bars->abort);
-        ++n_wait;
-      }
-      if (!ok) break;
-      tc_fence_after();
-      mma_mnmn(tmem, smem_u32(smem + st * ST_STAGE), smem_u32(smem + st * ST_STAGE + TILE_BYTES), it > 0 || has_init);
-      mma_commit(&bars->free_[st]);
-      if (hh == group - 1 && flushed_step(a, s, n_steps)) mma_commit(&bars->done);
-    }
-  } else if (warp == 9) {
-    // ---- loader ---------------------------------------------------------------------------
-    for (int it = 0; it < n_items && ok; ++it) {
-      const int st = it % ST_NS, use = it / ST_NS;
-      const int s = it / group, hh = it - s * group;
-      if (use >= 1) ok = mbar_wait_warp(&bars->free_[st], (use - 1) & 1, &bars->abort);
-      if (!ok) break;
-      const int row = (first + a.dir * s) * TILE, z = kv * a.group + head0 + hh;
-      unsigned char* dst = smem + st * ST_STAGE;
-      mbar_arrive_expect_tx(&bars->full[st], ST_STAGE);
-      load_tile(dst, &tm_x, &bars->full[st], row, z);
-      load_tile(dst + TILE_BYTES, &tm_y, &bars->full[st], row, z);
-    }
-  } else {
-    // ---- flush: thread = accumulator row (its warp's TMEM lane quarter) --------------------
-    const int r = (warp & 3) * 32 + (tid & 31);
-    const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  } else if (warp >= ST_FLUSH_WARP) {
+    setmaxnreg_inc<96>();
+    // ---- flush: thread = accumulator row (its warp's TMEM lane quarter) and one half of the columns
+    const int r = (warp & 3) * 32 + (tid & 31), half = (warp - ST_FLUSH_WARP) >> 2;
+    const uint32_t t_row = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 64 * half;
     unsigned char* s_out = smem + ST_OFF_OUT;
-    const bool issuer = (tid == 320);
-    int n_flush = 0;
-    // bf16 copy of this thread's row of the sum -> staging -> matrix `mat` of the head, one TMA store
-    int pending = 0;                                         // matrices stored, not yet published
-    auto publish = [&]() {
-      tma_store_wait();
-      fence_proxy_async_all();
-      __threadfence();
-      st_release_gpu(a.ready + kv, pending);
-      pending = 0;
+    int n_flush = 0, n_stored = 0;
+    // The staging tile has left; all of these warps or none of them go on.
+    auto stage_free = [&]() -> bool {
+      if (n_stored >= 1) mbar_wait(&bars->stage_free, (n_stored - 1) & 1, &bars->abort);
+      return !named_any(4, 256, *(volatile int*)&bars->abort);
     };
-    auto store_row = [&](const float (&x)[4][32], int mat) -> bool {
-      if (issuer) {
-        // The kernel that reads the states runs beside this one and takes them as they appear.  The
-        // matrix stored last is published here, one flush later, when its store has long completed
-        // (it must be in memory, not merely read out of the staging tile, before its index is shown).
-        if (a.ready && pending) publish();
-        else tma_store_wait_read();                          // the staging tile has left
-      }
-      if (named_any(4, 128, *(volatile int*)&bars->abort)) return false;       // the whole group or nobody
+    // bf16 copy of this thread's half row of the sum -> staging; the store warp sends it off
+    auto store_row = [&](const float (&x)[2][32]) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < 2; ++c) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           uint4 u;
@@ -213,22 +180,17 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
           u.y = pack_bf16(x[c][8 * e + 2], x[c][8 * e + 3]);
           u.z = pack_bf16(x[c][8 * e + 4], x[c][8 * e + 5]);
           u.w = pack_bf16(x[c][8 * e + 6], x[c][8 * e + 7]);
-          *reinterpret_cast<uint4*>(s_out + swz(r, 4 * c + e)) = u;
+          *reinterpret_cast<uint4*>(s_out + swz(r, 8 * half + 4 * c + e)) = u;
         }
       }
       fence_proxy_async_smem();
-      asm volatile("bar.sync 4, 128;" ::: "memory");
-      if (issuer) {
-        store_tile(&tm_out, s_out, 0, kv * a.n_chunks + mat);
-        tma_store_commit();
-        pending = mat + 1;
-      }
-      return true;
+      mbar_arrive(&bars->staged);
+      ++n_stored;
     };
-    auto write_final = [&](const float (&x)[4][32]) {
-      float* dst = a.final_out + ((size_t)kv * 128 + r) * 128;
+    auto write_final = [&](const float (&x)[2][32]) {
+      float* dst = a.final_out + ((size_t)kv * 128 + r) * 128 + 64 * half;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < 2; ++c) {
 #pragma unroll
         for (int e = 0; e < 8; ++e)
           *reinterpret_cast<float4*>(dst + 32 * c + 4 * e) =
@@ -238,10 +200,10 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     if (has_init || (a.final_out != nullptr && n_steps == 0 && !a.delta)) {
       // the chain starts from the incoming state (zero without one): into the accumulator, into the
       // matrix in front of the first step's, and -- when no token leaves the window -- straight out
-      float x[4][32];
-      const float* src = has_init ? a.state_in + ((size_t)kv * 128 + r) * 128 : nullptr;
+      float x[2][32];
+      const float* src = has_init ? a.state_in + ((size_t)kv * 128 + r) * 128 + 64 * half : nullptr;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < 2; ++c) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float4 f = src ? *reinterpret_cast<const float4*>(src + 32 * c + 4 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -250,50 +212,109 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       }
       if (has_init) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_st32(t_row + 32 * c, x[c]);
+        for (int c = 0; c < 2; ++c) tmem_st32(t_row + 32 * c, x[c]);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(&bars->acc_free);
-        if (stored_step(a, -1)) ok = store_row(x, a.out_first - a.dir);
+        if (stored_step(a, -1)) store_row(x);
       }
       if (a.final_out != nullptr && n_steps == 0) write_final(x);
     }
     for (int s = 0; s < n_steps && ok; ++s) {
       if (!flushed_step(a, s, n_steps)) continue;
-      mbar_wait(&bars->done, n_flush & 1, &bars->abort);       // (on a wait that ran out store_row has the vote)
+      // (ahead of the wait, so that the last store passes under it; a wait that runs out shows in the next vote)
+      if (!a.delta && stored_step(a, s) && !stage_free()) { ok = false; break; }
+      mbar_wait(&bars->done, n_flush & 1, &bars->abort);
 #ifdef RATTN_DEBUG_KNOBS
-      if (a.debug_wait == 2 && warp == 10 && n_flush == 0) bars->abort = 1;
+      if (a.debug_wait == 2 && warp == ST_FLUSH_WARP && n_flush == 0) bars->abort = 1;
 #endif
       ++n_flush;
       tc_fence_after();
-      float x[4][32];
+      float x[2][32];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) tmem_ld32(t_row + 32 * c, x[c]);
+      for (int c = 0; c < 2; ++c) tmem_ld32(t_row + 32 * c, x[c]);
       tmem_wait_ld();
       tc_fence_before();
       mbar_arrive(&bars->acc_free);                            // the next step may accumulate
       if (a.delta) {                                           // rows are neighbours in memory: whole 512-byte runs per store
-        float4* dst = reinterpret_cast<float4*>(a.delta) + (size_t)blockIdx.x * 4096 + r;
+        float4* dst = reinterpret_cast<float4*>(a.delta) + (size_t)blockIdx.x * 4096 + 16 * half * 128 + r;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
           for (int e = 0; e < 8; ++e)
             dst[(8 * c + e) * 128] = make_float4(x[c][4 * e], x[c][4 * e + 1], x[c][4 * e + 2], x[c][4 * e + 3]);
         continue;
       }
-      if (stored_step(a, s) && !store_row(x, a.out_first + a.dir * s)) ok = false;
+      if (stored_step(a, s)) store_row(x);
       if (a.final_out != nullptr && s == n_steps - 1) write_final(x);
     }
-    if (issuer) {
-      if (a.ready && pending) publish();
-      else tma_store_wait();
+  } else {
+    setmaxnreg_dec<48>();
+    if (warp == ST_PHI_WARPS) {
+      // ---- acc[128 features x 128] += phi(X)^T Y   (both operands MN-major: rows are the tokens)
+      int n_wait = 0;                                          // hand-backs of the accumulator so far
+      for (int it = 0; it < n_items && ok; ++it) {
+        const int st = it % ST_NS, use = it / ST_NS;
+        const int s = it / group, hh = it - s * group;
+        ok = mbar_wait_warp(&bars->phi_ready[st], use & 1, &bars->abort);
+        // the flush warps hold the previous sum, or are still writing the incoming state into the accumulator
+        if (ok && hh == 0 && ((s > 0 && flushed_step(a, s - 1, n_steps)) || (s == 0 && has_init))) {
+          ok = mbar_wait_warp(&bars->acc_free, n_wait & 1, &bars->abort);
+          ++n_wait;
+        }
+        if (!ok) break;
+        tc_fence_after();
+        mma_mnmn(tmem, smem_u32(smem + st * ST_STAGE), smem_u32(smem + st * ST_STAGE + TILE_BYTES), it > 0 || has_init);
+        mma_commit(&bars->free_[st]);
+        if (hh == group - 1 && flushed_step(a, s, n_steps)) mma_commit(&bars->done);
+      }
+    } else if (warp == ST_PHI_WARPS + 2) {
+      // ---- store: staged sums to memory, in order -----------------------------------------------
+      int n = 0;
+      for (int s = (has_init ? -1 : 0); s < n_steps && ok && !a.delta; ++s) {
+        if (!stored_step(a, s)) continue;
+        const int mat = a.out_first + a.dir * s;
+        ok = mbar_wait_warp(&bars->staged, n & 1, &bars->abort);
+        if (!ok) break;
+        ++n;
+        if ((tid & 31) == 0) {
+          store_tile(&tm_out, smem + ST_OFF_OUT, 0, kv * a.n_chunks + mat);
+          tma_store_commit();
+          tma_store_wait_read();
+          mbar_arrive(&bars->stage_free);
+          if (a.ready) {
+            // The kernel that reads the states runs beside this one and takes them as they appear: the matrix must be in
+            // memory, not merely read out of the staging tile, before its index is shown.  (Shown one store later, without
+            // this wait, the reader lost more than the chain gained: 129.5 -> 131 us for a chunk of 2 x 32/8 heads, T = 2048.)
+            tma_store_wait();
+            fence_proxy_async_all();
+            __threadfence();
+            st_release_gpu(a.ready + kv, mat + 1);
+          }
+        }
+        __syncwarp();
+      }
+      if ((tid & 31) == 0) tma_store_wait();
+    } else if (warp == ST_PHI_WARPS + 1) {
+      // ---- loader ---------------------------------------------------------------------------
+      for (int it = 0; it < n_items && ok; ++it) {
+        const int st = it % ST_NS, use = it / ST_NS;
+        const int s = it / group, hh = it - s * group;
+        if (use >= 1) ok = mbar_wait_warp(&bars->free_[st], (use - 1) & 1, &bars->abort);
+        if (!ok) break;
+        const int row = (first + a.dir * s) * TILE, z = kv * a.group + head0 + hh;
+        unsigned char* dst = smem + st * ST_STAGE;
+        mbar_arrive_expect_tx(&bars->full[st], ST_STAGE);
+        load_tile(dst, &tm_x, &bars->full[st], row, z);
+        load_tile(dst + TILE_BYTES, &tm_y, &bars->full[st], row, z);
+      }
     }
   }
   if (!ok && a.status) atomicExch(a.status, 1);
   if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == ST_PHI_WARPS) {
     tc_fence_after();
     tmem_dealloc(tmem, 128);
   }
