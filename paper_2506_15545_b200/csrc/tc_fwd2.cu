@@ -5,9 +5,13 @@
 // key tiles (2p+1 down to 2p - w/128), so every K/V tile is fetched once for both.
 //
 //   row group A / B (4 warps each, thread = query row = TMEM lane)
-//       SWA (Section 2.1): online softmax straight out of TMEM; P (fp16) is written back over
-//       the score columns and read from there by the P V product, so it never touches shared
-//       memory.  While one group exponentiates, the tensor pipe works for the other group.
+//       SWA (Section 2.1): online softmax straight out of TMEM; P (fp16) goes to TMEM columns of
+//       its own and is read from there by the P V product, so it never touches shared memory.
+//       The tiles' scores take turns in one TMEM buffer: a group reads its row into registers at
+//       once, and the other tile's scores replace it, so the next scores are there when a group
+//       has handed its weights over.  (With a buffer per tile, which held the weights too, they
+//       waited for the product in front: 2 x 32/8 heads, T = 8192, w = 2048 640 -> 628 us,
+//       w = 1024 486 -> 475.)
 //   MMA warp      S = Q K^T, O += P V (A operand from TMEM), the residual-branch products
 //   loader warp   TMA: Q tiles, K/V stages, the stored chunk state
 //   2 helper warps re-encode each V tile bf16 -> fp16 in place (tcgen05 needs A and B of one type)
@@ -44,7 +48,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 
 struct FBars {
   uint64_t q_full[2], q_free[2], k_full[2], v_full[2], v_ready[2], k_free[2], v_free[2], x_full, x_free;
-  uint64_t s_full[2], p_ready[2], o_ready[2], stash_done[2], phiq_ready[2], phik_ready[2], o_free[2], y_done[2], drain;
+  uint64_t s_full[2], s_read[2], p_ready[2], pv_done[2], o_ready[2], stash_done[2], phiq_ready[2], phik_ready[2], o_free[2], y_done[2], drain;
   SchedRing sched;
   uint32_t tmem_base;
   int abort;
@@ -245,8 +249,10 @@ __device__ bool fwd_convert(const FArgs& a, unsigned char* smem, FBars* bars, in
 __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32_t tmem) {
   const uint32_t sQ[2] = {smem_u32(smem + F_OFF_Q), smem_u32(smem + F_OFF_Q + TILE_BYTES)};
   const uint32_t sKV = smem_u32(smem + F_OFF_KV), sX = smem_u32(smem + F_OFF_X);
-  const uint32_t tS[2] = {tmem, tmem + 128}, tO[2] = {tmem + 256, tmem + 384};
+  // scores of the window; its weights; scores and weights of the residual branch; outputs
+  const uint32_t tS = tmem, tP[2] = {tmem + 128, tmem + 192}, tR[2] = {tmem, tmem + 128}, tO[2] = {tmem + 256, tmem + 384};
   int kv_count = 0, cntU[2] = {0, 0}, cntX = 0, cntP[2] = {0, 0}, cntR[2] = {0, 0}, cntK[2] = {0, 0};
+  int cntL0 = 0, cntL1 = 0;                        // window scores of tiles A, B so far
   TL_DECL(blockIdx.x == 7 && (threadIdx.x & 31) == 0);
 
   for (int n = 0;; ++n) {
@@ -272,37 +278,41 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
     auto kept = [&](int i) { return (un.rla[0] && i == un.n - 1) || (un.rla[1] && i == un.i1[1]); };
     WAIT_OR_RETURN_W(bars->k_full[stage_of(0)], use_of(0) & 1);
     tc_fence_after();
+    // Scores of tile X at position i, once the scores before them, of whichever tile, are in registers.
+    int last = -1;
+    auto scores = [&](int X, int i) -> bool {
+      if (last >= 0) WAIT_OR_RETURN_W(bars->s_read[last], ((last ? cntL1 : cntL0) - 1) & 1);
+      tc_fence_after();
+      mma_kk(tS, sQ[X], sK(i), false);                                         // S_X = Q_X K^T
+      mma_commit(&bars->s_full[X]);
+      last = X;
+      if (X) ++cntL1; else ++cntL0;
+      return true;
+    };
 #pragma unroll
-    for (int X = 1; X >= 0; --X) {
-      if (active(un, X, 0)) {
-        mma_kk(tS[X], sQ[X], sK(0), false);
-        mma_commit(&bars->s_full[X]);
-      }
-    }
+    for (int X = 1; X >= 0; --X)
+      if (active(un, X, 0) && !scores(X, 0)) return false;
     if (!kept(0)) mma_commit(&bars->k_free[stage_of(0)]);
     for (int i = 0; i < un.n; ++i) {
-      // The operands of this position are awaited once and ahead of the weights, so that the
-      // products and the next scores go out the moment a row group hands its weights over
-      // (a wait costs this warp a few hundred cycles even when it is already satisfied).
-      WAIT_OR_RETURN_W(bars->v_ready[stage_of(i)], use_of(i) & 1);
       if (i + 1 < un.n) WAIT_OR_RETURN_W(bars->k_full[stage_of(i + 1)], use_of(i + 1) & 1);
 #pragma unroll
       for (int X = 0; X < 2; ++X) {
+        // the next position's scores ahead of this one's product: the row group comes for them once it has handed over
+        if (i + 1 < un.n && active(un, X, i + 1)) {
+          if (!scores(X, i + 1)) return false;
+          TLM(2, 500 + 10 * i + X);
+        }
+        if (X == 0) WAIT_OR_RETURN_W(bars->v_ready[stage_of(i)], use_of(i) & 1);
         if (active(un, X, i)) {
           TLM(2, 10 * i + X);
           WAIT_OR_RETURN_W(bars->p_ready[X], cntP[X] & 1);
           ++cntP[X];
           TLM(2, 200 + 10 * i + X);
           tc_fence_after();
-          mma_pv(tO[X], tS[X], sV(i), i > un.i0[X]);                             // O_X += P V
+          mma_pv(tO[X], tP[X], sV(i), i > un.i0[X]);                             // O_X += P V
+          mma_commit(&bars->pv_done[X]);
           if (i == un.i1[X]) mma_commit(&bars->o_ready[X]);
           TLM(2, 300 + 10 * i + X);
-        }
-        if (i + 1 < un.n && active(un, X, i + 1)) {
-          tc_fence_after();
-          mma_kk(tS[X], sQ[X], sK(i + 1), false);                                // S_X = Q_X K^T (after P V in pipe order)
-          mma_commit(&bars->s_full[X]);
-          TLM(2, 500 + 10 * i + X);
         }
       }
       // K of the next position has served all its scores, V of this one all its products
@@ -322,13 +332,13 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
         WAIT_OR_RETURN_W(bars->phiq_ready[0], cntR[0] & 1);
         WAIT_OR_RETURN_W(bars->phik_ready[0], cntK[0] & 1);
         tc_fence_after();
-        mma_kk(tS[0], sQ[0], sK(iA), false);                                     // phi(Q_A) phi(K_cA)^T
+        mma_kk(tR[0], sQ[0], sK(iA), false);                                     // phi(Q_A) phi(K_cA)^T
         mma_commit(&bars->s_full[0]);
       }
       if (un.rla[1] && un.rla[0]) {
         WAIT_OR_RETURN_W(bars->phiq_ready[1], cntR[1] & 1);
         tc_fence_after();
-        mma_kk(tS[1], sQ[1], sK(iA), false);                                     // phi(Q_B) phi(K_cA)^T, whole chunk
+        mma_kk(tR[1], sQ[1], sK(iA), false);                                     // phi(Q_B) phi(K_cA)^T, whole chunk
         mma_commit(&bars->s_full[1]);
       }
       if (un.rla[0] && un.has_state) {
@@ -349,7 +359,7 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
         WAIT_OR_RETURN_W(bars->p_ready[0], cntP[0] & 1);
         ++cntP[0];
         tc_fence_after();
-        mma_pv(tO[0], tS[0], sV(iA), un.has_state);
+        mma_pv(tO[0], tR[0], sV(iA), un.has_state);
         mma_commit(&bars->o_ready[0]);
       }
       if (un.rla[1]) {
@@ -358,16 +368,16 @@ __device__ bool fwd_mma(const FArgs& a, unsigned char* smem, FBars* bars, uint32
           WAIT_OR_RETURN_W(bars->p_ready[1], cntP[1] & 1);
           ++cntP[1];
           tc_fence_after();
-          mma_pv(tO[1], tS[1], sV(iA), un.has_state);
+          mma_pv(tO[1], tR[1], sV(iA), un.has_state);
         }
         WAIT_OR_RETURN_W(bars->phik_ready[1], cntK[1] & 1);
         tc_fence_after();
-        mma_kk(tS[1], sQ[1], sK(iB), false);                                     // phi(Q_B) phi(K_cB)^T
+        mma_kk(tR[1], sQ[1], sK(iB), false);                                     // phi(Q_B) phi(K_cB)^T
         mma_commit(&bars->s_full[1]);
         WAIT_OR_RETURN_W(bars->p_ready[1], cntP[1] & 1);
         ++cntP[1];
         tc_fence_after();
-        mma_pv(tO[1], tS[1], sV(iB), un.rla[0]);
+        mma_pv(tO[1], tR[1], sV(iB), un.rla[0]);
         mma_commit(&bars->o_ready[1]);
       }
       if (un.has_state) mma_commit(&bars->x_free);
@@ -396,9 +406,9 @@ __device__ __forceinline__ uint32_t lane_base(int r) { return (uint32_t)((r & ~3
 // unrolled the kernel was ~390 KB of code and ran instruction-fetch bound.
 __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, FBars* bars, uint32_t tmem, int X,
                          int r) {
-  const uint32_t tS = tmem + 128 * X + lane_base(r), tO = tmem + 256 + 128 * X + lane_base(r);
+  const uint32_t tS = tmem + lane_base(r), tP = tS + 128 + 64 * X, tR = tS + 128 * X, tO = tS + 256 + 128 * X;
   unsigned char* sQ = smem + F_OFF_Q + X * TILE_BYTES;
-  int kv_count = 0, cntS = 0, cntO = 0;
+  int kv_count = 0, cntS = 0, cntW = 0, cntO = 0;  // ...; score hand-overs, weights of the window handed over, o_ready completions
   TL_DECL(blockIdx.x == 7 && r == 0);
 
   for (int n = 0;; ++n) {
@@ -440,6 +450,8 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #pragma unroll
       for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, x[c]);      // dropped chunks too: four loads in flight
       tmem_wait_ld();
+      tc_fence_before();
+      mbar_arrive(&bars->s_read[X]);                                 // the other tile's scores may replace them
       if (diag || bound) {
         // the one chunk this warp keeps partly: dropped columns become -inf (weight zero)
         const uint32_t keep = keep_bits(r, wq, diag, bound);
@@ -458,7 +470,8 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
       if (i == i0) m_ref = m_new;
       else rescale = __any_sync(0xffffffffu, m_new > m_ref + 8.f);
       if (rescale) {
-        // P V of the previous tile has completed (the commit behind these scores covers it)
+        WAIT_ON(bars->pv_done[X], (cntW - 1) & 1);   // P V of the previous position
+        tc_fence_after();
         const float f = ex2(m_ref - m_new);
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
@@ -473,7 +486,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
         m_ref = m_new;
       }
       TL(X, 300 + i);
-      // weights, written back (fp16, two per column) over the score columns
+      // weights (fp16, two per column), once the previous ones have been consumed
       const float2 sc2 = make_float2(a.scale_log2, a.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
       float2 ps0 = make_float2(0.f, 0.f), ps1 = make_float2(0.f, 0.f);
 #pragma unroll
@@ -492,8 +505,13 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
             pk[e] = pack_f16(pp.x, pp.y);
           }
         }
-        tmem_st16(tS + 16 * c, pk);
+        if (c == 0) {
+          if (i > i0) WAIT_ON(bars->pv_done[X], (cntW - 1) & 1);
+          tc_fence_after();
+        }
+        tmem_st16(tP + 16 * c, pk);
       }
+      ++cntW;
       const float psum = (ps0.x + ps0.y) + (ps1.x + ps1.y);
       l += psum;
       tmem_wait_st();
@@ -571,7 +589,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           float x[32];
-          tmem_ld32(tS + 32 * c, x);
+          tmem_ld32(tR + 32 * c, x);
           tmem_wait_ld();
           // residual keys of row r in its chunk: j < r
           const int rd = r - 32 * c;
@@ -580,7 +598,7 @@ __device__ bool fwd_rows(const FMaps& tm, const FArgs& a, unsigned char* smem, F
 #pragma unroll
           for (int e = 0; e < 16; ++e)
             pk[e] = pack_f16((keep >> (2 * e)) & 1u ? x[2 * e] : 0.f, (keep >> (2 * e + 1)) & 1u ? x[2 * e + 1] : 0.f);
-          tmem_st16(tS + 16 * c, pk);                                  // columns already consumed
+          tmem_st16(tR + 16 * c, pk);                                  // columns already consumed
         }
         tmem_wait_st();
         tc_fence_before();
@@ -754,7 +772,9 @@ tc_fwd2_kernel(const __grid_constant__ FMaps tm, FArgs a) {
       mbar_init(&bars->k_free[i], 1);
       mbar_init(&bars->v_free[i], 1);
       mbar_init(&bars->s_full[i], 1);
+      mbar_init(&bars->s_read[i], 128);
       mbar_init(&bars->p_ready[i], 128);
+      mbar_init(&bars->pv_done[i], 1);
       mbar_init(&bars->o_ready[i], 1);
       mbar_init(&bars->stash_done[i], 128);
       mbar_init(&bars->phiq_ready[i], 128);
