@@ -494,25 +494,35 @@ cudaError_t launch_handoff_t(const Args& a, cudaStream_t s, bool state_too, int*
   return cudaGetLastError();
 }
 
-// k_ext[bh, e] = e < w ? ring[bh, (pos0 - w + e) % w] : chunk[bh, e - w]   (16-byte vectors)
-__global__ void gather_history_kernel(const uint4* __restrict__ k_chunk, const uint4* __restrict__ v_chunk,
-                                      const uint4* __restrict__ k_ring, const uint4* __restrict__ v_ring,
-                                      uint4* __restrict__ k_ext, uint4* __restrict__ v_ext, int T, int w, int pos0,
-                                      int vec_per_row, int H_kv, int layout, int* __restrict__ clear, int clear_ints) {
+// k_ext[bh, e] = e < w ? ring[bh, (pos0 - w + e) % w] : chunk[bh, e - w]   (16-byte vectors), and, where ring outputs are
+// given, what the rings hold behind the chunk: the thread that reads a slot also writes its successor, so that the rings may
+// be written in place (with a kernel of its own for that the two copies took 19 us of a chunk of 2048 tokens on 16 heads).
+__global__ void __launch_bounds__(256) gather_history_kernel(const uint4* __restrict__ k_chunk, const uint4* __restrict__ v_chunk,
+                                                             const uint4* k_ring, const uint4* v_ring, uint4* __restrict__ k_ext,
+                                                             uint4* __restrict__ v_ext, uint4* k_out, uint4* v_out, int T, int w,
+                                                             int pos0, int vec_shift, int H_kv, int layout,
+                                                             int* __restrict__ clear, int clear_ints) {
   const int bh = blockIdx.y;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (bh == 0)
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < clear_ints; e += gridDim.x * blockDim.x) clear[e] = 0;
   // the chunk is the caller's tensor: [B, H_kv, T, d] (layout 0) or [B, T, H_kv, d] (layout 1), in 16-byte vectors
-  const size_t head0 = layout ? ((size_t)(bh / H_kv) * T * H_kv + bh % H_kv) * vec_per_row : (size_t)bh * T * vec_per_row;
-  const size_t pitch = layout ? (size_t)H_kv * vec_per_row : (size_t)vec_per_row;
-  const size_t n_ext = (size_t)(w + T) * vec_per_row;
+  const size_t head0 = (layout ? (size_t)(bh / H_kv) * T * H_kv + bh % H_kv : (size_t)bh * T) << vec_shift;
+  const size_t pitch = (size_t)(layout ? H_kv : 1) << vec_shift;
+  const size_t n_ext = (size_t)(w + T) << vec_shift;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_ext; i += (size_t)gridDim.x * blockDim.x) {
-    const int e = (int)(i / vec_per_row), c = (int)(i % vec_per_row);
+    const int e = (int)(i >> vec_shift), c = (int)i & ((1 << vec_shift) - 1);
     uint4 kk, vv;
     if (e < w) {
-      const int slot = (pos0 - w + e) % w;
-      kk = k_ring[((size_t)bh * w + slot) * vec_per_row + c];
-      vv = v_ring[((size_t)bh * w + slot) * vec_per_row + c];
+      const size_t at = (((size_t)bh * w + (pos0 - w + e) % w) << vec_shift) + c;
+      kk = k_ring[at];
+      vv = v_ring[at];
+      if (k_out) {
+        const int j = e - w + (T - 1 + w - e) / w * w;       // the chunk's last token for this slot; negative: none
+        k_out[at] = j >= 0 ? k_chunk[head0 + (size_t)j * pitch + c] : kk;
+        v_out[at] = j >= 0 ? v_chunk[head0 + (size_t)j * pitch + c] : vv;
+      }
     } else {
       kk = k_chunk[head0 + (size_t)(e - w) * pitch + c];
       vv = v_chunk[head0 + (size_t)(e - w) * pitch + c];
@@ -525,18 +535,18 @@ __global__ void gather_history_kernel(const uint4* __restrict__ k_chunk, const u
 }  // namespace
 
 cudaError_t launch_gather_history(const Args& a, const void* k_chunk, const void* v_chunk, const void* k_ring,
-                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, int* clear, int clear_ints,
-                                  cudaStream_t s) {
-  const int elem = a.dtype == RATTN_F32 ? 4 : 2;
-  const int vec_per_row = a.d * elem / 16;
-  const size_t n_ext = (size_t)(a.w + a.T) * vec_per_row;
+                                  const void* v_ring, void* k_ext, void* v_ext, void* k_ring_out, void* v_ring_out, int pos0,
+                                  int* clear, int clear_ints, cudaStream_t s) {
+  const int vec_shift = (a.d == 128 ? 4 : 3) + (a.dtype == RATTN_F32 ? 1 : 0);        // 16-byte vectors per row: 1 << shift
+  const size_t n_ext = (size_t)(a.w + a.T) << vec_shift;
   dim3 grid((unsigned)((n_ext + 255) / 256 < 1024 ? (n_ext + 255) / 256 : 1024), a.B * a.H_kv);
   KernelTimer kt("gather_history", s);
-  gather_history_kernel<<<grid, 256, 0, s>>>(
-      reinterpret_cast<const uint4*>(k_chunk), reinterpret_cast<const uint4*>(v_chunk),
-      reinterpret_cast<const uint4*>(k_ring), reinterpret_cast<const uint4*>(v_ring),
-      reinterpret_cast<uint4*>(k_ext), reinterpret_cast<uint4*>(v_ext), a.T, a.w, pos0, vec_per_row, a.H_kv, a.layout, clear,
-      clear_ints);
+  const cudaError_t e = launch_pdl(
+      gather_history_kernel, grid, dim3(256), 0, s, true, reinterpret_cast<const uint4*>(k_chunk),
+      reinterpret_cast<const uint4*>(v_chunk), reinterpret_cast<const uint4*>(k_ring), reinterpret_cast<const uint4*>(v_ring),
+      reinterpret_cast<uint4*>(k_ext), reinterpret_cast<uint4*>(v_ext), reinterpret_cast<uint4*>(k_ring_out),
+      reinterpret_cast<uint4*>(v_ring_out), a.T, a.w, pos0, vec_shift, a.H_kv, a.layout, clear, clear_ints);
+  if (e != cudaSuccess) return e;
   count_launches(1);
   return cudaGetLastError();
 }

@@ -254,13 +254,28 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
   int* const block = a.status;
   const int block_ints = (int)(L.status_bytes / sizeof(int));
   const bool rings = want_handoff && p->k_ring_out;
-  bool cleared = block == nullptr;
+  bool cleared = block == nullptr, rings_done = false;
   if (block && status_word) a.status = status_word;
   if (resume) {
     char* base = reinterpret_cast<char*>(p->workspace);
     void* k_ext = base + L.k_ext;
     void* v_ext = base + L.v_ext;
-    e = launch_gather_history(a, p->k, p->v, p->k_ring_in, p->v_ring_in, k_ext, v_ext, p->pos0, block, block_ints, s);
+    // The gather hands the rings out on the way, over the incoming ones or to memory of their own: it reads a slot once and
+    // writes that slot.  Outputs that overlap its inputs in any other way are written behind it.
+    const size_t elem = p->dtype == RATTN_F32 ? 4 : 2, ring_bytes = (size_t)p->B * p->H_kv * p->w * p->d * elem,
+                 chunk_bytes = (size_t)p->B * p->H_kv * p->T * p->d * elem;
+    auto apart = [](const void* x, size_t nx, const void* y, size_t ny) {
+      return (uintptr_t)x + nx <= (uintptr_t)y || (uintptr_t)y + ny <= (uintptr_t)x;
+    };
+    auto fits = [&](const void* out, const void* in, const void* other_in, const void* other_out) {
+      return (out == in || apart(out, ring_bytes, in, ring_bytes)) && apart(out, ring_bytes, other_in, ring_bytes) &&
+             apart(out, ring_bytes, other_out, ring_bytes) && apart(out, ring_bytes, p->k, chunk_bytes) &&
+             apart(out, ring_bytes, p->v, chunk_bytes);
+    };
+    rings_done = tc && rings && fits(p->k_ring_out, p->k_ring_in, p->v_ring_in, p->v_ring_out) &&
+                 fits(p->v_ring_out, p->v_ring_in, p->k_ring_in, p->k_ring_out);
+    e = launch_gather_history(a, p->k, p->v, p->k_ring_in, p->v_ring_in, k_ext, v_ext, rings_done ? p->k_ring_out : nullptr,
+                              rings_done ? p->v_ring_out : nullptr, p->pos0, block, block_ints, s);
     if (e != cudaSuccess) return fail_cuda(e);
     cleared = true;
     a.k = k_ext; a.v = v_ext;
@@ -268,7 +283,7 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
     a.Tk = p->w + p->T; a.q_off = p->w; a.state_in = p->state_in; a.pos_shift = p->pos0 - p->w;
   }
   // the rings may be written over in place (a resumed sequence hands out where it came from): after the gather
-  const bool rings_first = rings && tc;
+  const bool rings_first = rings && tc && !rings_done;
   if (rings_first) {
     e = launch_handoff(a, s, false, cleared ? nullptr : block, cleared ? 0 : block_ints);
     if (e != cudaSuccess) return fail_cuda(e);

@@ -189,8 +189,8 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s);
 cudaError_t launch_tc_backward(const Args& a, cudaStream_t s);
 // chunked prefill: k_ext/v_ext[b,hk] = the ring's tokens pos0-w .. pos0-1 in time order, then the chunk
 cudaError_t launch_gather_history(const Args& a, const void* k_chunk, const void* v_chunk, const void* k_ring,
-                                  const void* v_ring, void* k_ext, void* v_ext, int pos0, int* clear, int clear_ints,
-                                  cudaStream_t s);
+                                  const void* v_ring, void* k_ext, void* v_ext, void* k_ring_out, void* v_ring_out, int pos0,
+                                  int* clear, int clear_ints, cudaStream_t s);
 
 int debug_wait();                    // always 0 outside the debug build
 int tuning(int knob);                       // current value of a rattn_knob

@@ -36,7 +36,8 @@ static Plan make_plan(const Args& a, int n_sm) {
   if (p.n_steps < 0) p.n_steps = 0;
   p.chain = n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
   const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
-  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one), the main kernel
+  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one; it has become
+  // faster since, 2.5 where it publishes them and 2 where not, and the lines below stand where these drew them), the main kernel
   // 30 ns per query tile and 12 ns per tile and key tile, and no less than 40 us as far as this matters.  (Fitted on a B200
   // with all of its 148 SMs at work and every window full: short sequences, whose first tiles read less, and ragged batches
   // have less work than this says.)  Where the chain of a long sequence on few heads would outlast the main kernel, its terms

@@ -200,3 +200,35 @@ def test_gradients_in_place_of_the_inputs(Hq, Hkv, T, d, w, dtype):
         k2, v2, dy2 = k.clone(), v.clone(), dy.clone()
         R.rattn_backward_ex(q, k2, v2, dy2, w, ws, scale=wl.scale, flags=R.FLAG_SAVE_RESIDUALS, dq=dy2, dk=k2, dv=v2)
         assert all(torch.equal(a, b) for a, b in zip(apart, (dy2, k2, v2)))
+
+
+@pytest.mark.parametrize("T,w,pos0", [(128, 512, 700), (512, 512, 512), (1000, 256, 3333), (300, 128, 1280)])
+@pytest.mark.parametrize("place", ["apart", "in place", "shifted", "crossed"])
+def test_rings_of_a_resumed_chunk(T, w, pos0, place):
+    """The rings behind a chunk hold its tokens (and, of a chunk shorter than the window, older ones) wherever they are written:
+    to memory of their own, over the incoming rings, over half of them, or each over the other's place."""
+    gen = torch.Generator(device="cuda").manual_seed(T + w)
+    B, Hq, Hkv, d = 2, 4, 2, 128
+    rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rnd(B, Hq, T, d), rnd(B, Hkv, T, d), rnd(B, Hkv, T, d)
+    rings = [rnd(B, Hkv, w, d) for _ in range(2)]
+    want = []
+    for ring, x in zip(rings, (k, v)):
+        r = ring.clone()
+        for j in range(max(0, T - w), T):
+            r[:, :, (pos0 + j) % w] = x[:, :, j]
+        want.append(r)
+    n = B * Hkv * w * d
+    pool = torch.zeros(4 * n, device="cuda", dtype=torch.bfloat16)
+    at = lambda i: pool[i:i + n].view(B, Hkv, w, d)
+    k_in, v_in = at(0), at(n)
+    k_in.copy_(rings[0])
+    v_in.copy_(rings[1])
+    k_out, v_out = {"apart": (at(2 * n), at(3 * n)), "in place": (k_in, v_in), "shifted": (at(n // 2), at(2 * n)),
+                    "crossed": (v_in, k_in)}[place]
+    state = torch.zeros(B, Hkv, d, d, device="cuda")
+    ws = R.alloc_workspace_chunked(q, k, w)
+    R.rattn_forward_ex(q, k, v, w, scale=0.1, workspace=ws, pos0=pos0, state_in=state, k_ring_in=k_in, v_ring_in=v_in,
+                       state_out=torch.empty_like(state), k_ring_out=k_out, v_ring_out=v_out)
+    assert R.rattn_read_status(ws) == 0
+    assert torch.equal(k_out, want[0]) and torch.equal(v_out, want[1])
