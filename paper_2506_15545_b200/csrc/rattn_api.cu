@@ -278,6 +278,7 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
                               rings_done ? p->v_ring_out : nullptr, p->pos0, block, block_ints, s);
     if (e != cudaSuccess) return fail_cuda(e);
     cleared = true;
+    a.kernel_ahead = true;
     a.k = k_ext; a.v = v_ext;
     a.kv_layout = RATTN_LAYOUT_BHTD;                       // the gathered history + chunk is dense per head
     a.Tk = p->w + p->T; a.q_off = p->w; a.state_in = p->state_in; a.pos_shift = p->pos0 - p->w;
@@ -288,6 +289,7 @@ static int forward_impl(const rattn_params* p, cudaStream_t s, int* status_word 
     e = launch_handoff(a, s, false, cleared ? nullptr : block, cleared ? 0 : block_ints);
     if (e != cudaSuccess) return fail_cuda(e);
     cleared = true;
+    a.kernel_ahead = true;
   }
 #ifdef RATTN_HAVE_TC
   // a forward that is one kernel with one unit per CTA uses nothing but the status word, which it clears itself

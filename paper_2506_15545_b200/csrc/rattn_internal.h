@@ -112,6 +112,7 @@ struct Args {
   int n_chunks;
   int* status;                 // device status word (may be null when no workspace)
   int* clear_status;           // the status word, where no kernel ahead of the forward's first one has cleared it
+  bool kernel_ahead;           // the last thing put on the stream is a kernel of this call that signals its successor
   bool single_tiles;           // the pair kernel's work units are single query tiles
   int* work_counter;           // the forward's work counter, zero at launch (null: units are dealt round-robin);
                                // the backward's two kernels use the two words behind it
@@ -182,6 +183,7 @@ struct StateLaunch {
   float* delta;             // optional fp32 scratch, n_kv * n_steps * h_split matrices: the terms are formed in parallel
                             // and summed by a second kernel
   int h_split;              // ... each by this many CTAs, a share of the group's heads each
+  bool wait_first;          // the kernel before on the stream signals its successor: this one is set up under it, and waits
   bool after_independent;   // the kernel before on the stream neither feeds this one nor is fed by it: they may overlap
   const char* name;         // label of the timing record
 };

@@ -1466,6 +1466,7 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   L.delta = parallel_terms ? a.rdelta : nullptr;
   L.h_split = parts;
   L.after_independent = parallel_terms;
+  L.wait_first = false;                                    // (under prep: no difference)
   if (!parallel_terms) {
     e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;

@@ -120,6 +120,10 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.delta = p.terms ? a.rdelta : nullptr;
     L.h_split = 1;
     L.after_independent = false;
+    // Behind the call's own copies (gather, ring hand-off) the chain is set up under them where it has few CTAs: 1 x 40/8
+    // heads, T = 300, w = 256 26.7 -> 24.4 us, 2 x 32/8, T = 2048 124.8 -> 122.0; with 64 of them, which hold SMs while they
+    // wait, 198.5 -> 203, with 128 159.6 -> 162.4.
+    L.wait_first = a.kernel_ahead && 4 * n_kv <= n_sm;
     e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;
   }

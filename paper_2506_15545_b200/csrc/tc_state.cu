@@ -59,6 +59,7 @@ struct StateArgs {
   int n_split;      // steps that the grid is split into (delta)
   int h_split;      // ... and the group's heads: term matrix ((kv * n_split + step) * h_split + part)
   int wait_before;  // 1: the kernel ahead may still be running; not to end before it
+  int wait_first;   // 1: set up under the kernel ahead, whose results this one reads
   int debug_wait;   // debug build only, 2: the first wait of some of the flush threads counts as run out
 };
 
@@ -96,8 +97,9 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   const int kv = a.delta ? unit / a.n_split : unit;
   const int first = a.delta ? a.first + a.dir * (unit - kv * a.n_split) : a.first;
   const int group = a.delta ? a.group / a.h_split : a.group, head0 = a.delta ? group * ((int)blockIdx.x - unit * a.h_split) : 0;
-  // the kernel that follows may start its own prologue (and whatever does not read the states)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The kernel that follows may start its own prologue, and whatever does not read the states; where this kernel itself is set
+  // up under the one ahead, behind its wait, because the next one relies on what is ahead of this one.
+  if (!a.wait_first) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0 && a.status) atomicExch(a.status, 2);
     return;
@@ -123,6 +125,10 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     prefetch_map(&tm_x);
     prefetch_map(&tm_y);
     prefetch_tensormap(&tm_out);
+  }
+  if (a.wait_first) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -391,13 +397,14 @@ cudaError_t launch_tc_states(const StateLaunch& L, cudaStream_t s) {
   a.n_split = L.delta ? L.n_steps : 1;
   a.h_split = L.delta ? L.h_split : 1;
   a.wait_before = L.after_independent ? 1 : 0;
+  a.wait_first = L.wait_first ? 1 : 0;
   a.debug_wait = debug_wait();
   cudaError_t e = allow_smem<tc_state_scan_kernel>(ST_SMEM);
   if (e != cudaSuccess) return e;
   {
     KernelTimer kt(L.name, s);
     e = launch_pdl(tc_state_scan_kernel, dim3((unsigned)(L.n_kv * a.n_split * a.h_split)), dim3(ST_THREADS), ST_SMEM, s,
-                   L.after_independent, tm_x, tm_y, tm_out, a);
+                   L.after_independent || L.wait_first, tm_x, tm_y, tm_out, a);
     if (e != cudaSuccess) return e;
   }
   count_launches(1);

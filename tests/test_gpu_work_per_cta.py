@@ -1,10 +1,45 @@
-"""Work that a persistent CTA does after its first piece: the rotation table of the prologue refilled."""
+"""Work that a persistent CTA does after its first piece: pairs of query tiles one behind the other, the rotation table of the
+prologue refilled.  The arithmetic of a result does not depend on which CTA has it or what that CTA did before, so a few CTAs
+with all of the work give the bits that many give."""
 import pytest
 import torch
 
 from paper_2506_15545_b200 import binding as R
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("grid", [1, 3])
+@pytest.mark.parametrize("mode,T,w,lens", [
+    (R.MODE_RATTN, 2300, 1024, None),                # an odd number of tiles: a unit of one at the end
+    (R.MODE_RATTN, 2400, 1024, [2400, 130, 1200]),   # units beyond an entry's end are passed over, some have a tile less
+    (R.MODE_SWA_ONLY, 900, 256, None),               # no residual part between the windows
+    (R.MODE_FULL_CAUSAL, 700, 700, None),
+])
+def test_pairs_one_behind_the_other(mode, T, w, lens, grid):
+    """Scores of two tiles in one buffer, the next unit's behind the residual part that had its columns."""
+    g = torch.Generator(device="cuda").manual_seed(T + w)
+    B = len(lens) if lens else 2
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    q, k, v = (rnd(B, h, T, 128).bfloat16() for h in (4, 2, 2))
+    more = dict(scale=0.25, mode=mode, gamma_swa=1 + 0.1 * rnd(4, 128), gamma_rla=1 + 0.1 * rnd(4, 128))
+    if lens:
+        more["seq_lens"] = torch.tensor(lens, dtype=torch.int32, device="cuda")
+
+    def run():
+        ws = R.alloc_workspace(q, k, w)
+        out = R.rattn_forward_ex(q, k, v, w, workspace=ws, **more)
+        assert R.rattn_read_status(ws) == 0, "a device-side wait expired"
+        return [out[b, :, :n] for b, n in enumerate(lens)] if lens else [out]
+
+    many = run()
+    prev = R.rattn_tune(R.TUNE_GRID, grid)
+    try:
+        few = run()
+    finally:
+        R.rattn_tune(R.TUNE_GRID, prev)
+    for x, y in zip(many, few):
+        assert torch.isfinite(x.float()).all() and torch.equal(x, y)
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,T,d,dtype,entry_pos", [
