@@ -62,7 +62,10 @@ static Plan make_plan(const Args& a, int n_sm) {
   // the end (1 x 16/4 heads, T = 2200, w = 512: 47 us as single tiles, 37 as pairs; w = 768, two steps fewer: 42 and 41;
   // training, w = 128: 55 and 50).
   const bool chain_decides = (long long)((n_qt + 1) / 2) * n_q <= n_sm && chain_ns > (a.training ? 36000 : 30000);
-  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && wt <= (a.training ? 12 : 7) &&
+  // A head of one tile has no pairs, whatever its window: two tiles per SM instead of one (T = 116, w = 1024, 100 / 160 / 290 / 600
+  // tiles: 10.6 / 19.0 / 21.9 / 38.9 us as units of the pair kernel, 9.8 / 10.6 / 10.7 / 24.7 as single tiles; of two tiles a head
+  // the two are alike, from four on the pairs are faster).
+  p.single = rla && (a.phi == RATTN_PHI_SOFTMAX || !p.chain) && (wt <= (a.training ? 12 : 7) || (!a.training && n_kt == 1)) &&
              (p.terms || (chain_fits && !chain_decides)) &&
              !(p.chain && !a.training && tuning(RATTN_TUNE_STATE_STRIDE) == 2);
   // The pair kernel where there are no more tiles than SMs: a tile of its own per CTA ends sooner.  (With more, the second

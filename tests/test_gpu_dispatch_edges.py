@@ -232,3 +232,25 @@ def test_rings_of_a_resumed_chunk(T, w, pos0, place):
                        state_out=torch.empty_like(state), k_ring_out=k_out, v_ring_out=v_out)
     assert R.rattn_read_status(ws) == 0
     assert torch.equal(k_out, want[0]) and torch.equal(v_out, want[1])
+
+
+@pytest.mark.parametrize("T,lens", [(1, None), (77, None), (128, None), (116, [116, 1, 50])])
+@pytest.mark.parametrize("w", [1024, 2048])
+def test_prompts_of_one_tile_in_wide_windows(T, w, lens):
+    """A prompt that every window covers: one operator whatever the window, and the same kernel as with a narrower one."""
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    B = len(lens) if lens else 3
+    rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rnd(B, 8, T, 128), rnd(B, 2, T, 128), rnd(B, 2, T, 128)
+
+    def run(w):
+        ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, 0)
+        rings = [torch.empty(B, 2, w, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2)]
+        state = torch.full((B, 2, 128, 128), 7.0, device="cuda")
+        more = dict(seq_lens=torch.tensor(lens, dtype=torch.int32, device="cuda")) if lens else {}
+        out = R.rattn_forward_ex(q, k, v, w, scale=0.1, workspace=ws, state_out=state, k_ring_out=rings[0], v_ring_out=rings[1], **more)
+        assert R.rattn_read_status(ws) == 0
+        return [out[b, :, :n] for b, n in enumerate(lens or [T] * B)] + [r[:, :, :T] for r in rings] + [state]
+
+    for x, y in zip(run(w), run(768)):
+        assert torch.isfinite(x.float()).all() and torch.equal(x, y)
