@@ -171,12 +171,17 @@ __device__ __forceinline__ void feature_map_pair_any(const unsigned char* src_ha
   feature_map_half_row(src_half + row * 128, dst_half + row * 128, row, (int)(threadIdx.x & 1), phi, true);
 }
 
-// ... by four adjacent lanes per row, of which this one (q = lane & 3) owns 32 columns; `src` and `dst` point at the row in
-// the first column half's box, the second half's lies `half_stride` behind.  A quarter-warp (two rows) touches every bank
-// once: the lanes of the second half walk their chunks two apart from the first's.
+// ... by four lanes per row, of which this one (q) owns 32 columns; `src` and `dst` point at the row in the first column
+// half's box, the second half's lies `half_stride` behind.
+// PAIR_SUMS = false: q = lane & 3.  A quarter-warp (two rows) touches every bank once: the lanes of the second half walk
+// their chunks two apart from the first's.
+// PAIR_SUMS = true: the softmax map's sums are formed in feature_map_half_row's order, so that both leave the same bits:
+// of a half's two lanes (q, q ^ 1: neighbours; the other half's lie 8 lanes away) the second carries on from the first's
+// partial sums.  A quarter-warp touches every bank once with one half of four rows.
+template <bool PAIR_SUMS = false>
 __device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsigned char* dst, int half_stride, int row, int q,
                                                  int phi) {
-  const int sw = (row & 7) ^ ((q & 1) << 2) ^ (q & 2);
+  const int sw = (row & 7) ^ ((q & 1) << 2) ^ (PAIR_SUMS ? 0 : q & 2);
   src += (q >> 1) * half_stride;
   dst += (q >> 1) * half_stride;
   if (phi != RATTN_PHI_SOFTMAX) {
@@ -203,7 +208,7 @@ __device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsig
   }
   float m = fmaxf(m0, m1);
   m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, PAIR_SUMS ? 8 : 2));
   const float ml = m * 1.4426950408889634f;
   const float2 l2e = make_float2(1.4426950408889634f, 1.4426950408889634f), nml = make_float2(-ml, -ml);
   float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
@@ -216,9 +221,24 @@ __device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsig
     if (i & 2) s1 = __fadd2_rn(s1, p);
     else s0 = __fadd2_rn(s0, p);
   }
-  float sum = (s0.x + s0.y) + (s1.x + s1.y);
-  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  float sum;
+  if (PAIR_SUMS) {
+    // a pair's lane walks the first half's chunks 0 .. 7, the second half's 4 .. 7, 0 .. 3: first are q = 0 and q = 3
+    s0.x = __shfl_xor_sync(0xffffffffu, s0.x, 1); s0.y = __shfl_xor_sync(0xffffffffu, s0.y, 1);
+    s1.x = __shfl_xor_sync(0xffffffffu, s1.x, 1); s1.y = __shfl_xor_sync(0xffffffffu, s1.y, 1);
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+      s0 = __fadd2_rn(s0, make_float2(x[i], x[i + 1]));
+      s1 = __fadd2_rn(s1, make_float2(x[i + 2], x[i + 3]));
+    }
+    sum = (s0.x + s0.y) + (s1.x + s1.y);                  // of a half, in q = 1 and q = 2
+    const int lane0 = (int)(threadIdx.x & 31) & ~9;       // q = 0 of this row
+    sum = __shfl_sync(0xffffffffu, sum, lane0 + 1) + __shfl_sync(0xffffffffu, sum, lane0 + 8);
+  } else {
+    sum = (s0.x + s0.y) + (s1.x + s1.y);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+  }
   const float sc = 1.f / sum;
 #pragma unroll
   for (int c = 0; c < 4; ++c)

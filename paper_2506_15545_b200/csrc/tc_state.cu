@@ -144,17 +144,17 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
   // registers follow the work: 512 x 64 + 128 x 48 + 256 x 96, within the CTA's 896 x 72
   if (warp < ST_PHI_WARPS) {
     setmaxnreg_dec<64>();
-    // ---- feature map of the X tile, in place: four adjacent lanes per row -----------------
+    // ---- feature map of the X tile, in place: four lanes per row ---------------------------
+    const int row = 8 * warp + 4 * ((tid >> 4) & 1) + ((tid >> 1) & 3), q = 2 * ((tid >> 3) & 1) + (tid & 1);
     for (int it = 0; it < n_items && ok; ++it) {
       const int st = it % ST_NS, use = it / ST_NS;
       ok = mbar_wait_warp(&bars->full[st], use & 1, &bars->abort);
       if (!ok) break;
-      const int row = tid >> 2, q = tid & 3;
       unsigned char* x = smem + st * ST_STAGE + row * 128;
       const int token = (first + a.dir * (it / group)) * TILE + row;
       // every lane maps its row (the softmax map exchanges partial results between the lanes
       // of a row with full-warp shuffles, so no lane may skip it); rows past the limit are then cleared
-      feature_map_quad(x, x, HALF_BYTES, row, q, a.phi);
+      feature_map_quad<true>(x, x, HALF_BYTES, row, q, a.phi);
       __syncwarp();
       if (token >= row_limit) {
 #pragma unroll
