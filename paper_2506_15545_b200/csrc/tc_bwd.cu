@@ -231,7 +231,7 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
         for (int e = 0; e < 8; ++e) g_lo[e] = g_hi[e] = 0.f;
       }
       // one branch after the other (both at once, with gains and sums, do not fit the registers); returns D = g . o
-      auto branch = [&](unsigned char* p, const float (&ga_lo)[8], const float (&ga_hi)[8], float (&acc)[16]) -> float {
+      auto branch = [&](unsigned char* p, const float (&ga_lo)[8], const float (&ga_hi)[8], float (&acc)[16], bool window) -> float {
         float o_lo[8], o_hi[8];
         if (live) {
           unpack8(p, o_lo); unpack8(p + 128, o_hi);
@@ -251,12 +251,17 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
           A += __shfl_xor_sync(0xffffffffu, A, o);
         }
         const float ir = rsqrtf(ss * (1.f / 128.f) + a.eps), c = A * ir * ir * (1.f / 128.f);   // c = mean(gh n) / r
+        // gh - n A / (128 r): which of the two products is rounded on its own is said here and not left to the compiler, whose
+        // choice, and with it the last bit of some g, changed with the code around
+        auto diff = [&](float g, float ga, float o) {
+          return GAINS && window ? fmaf(g, ga, -__fmul_rn(o, c)) : fmaf(-o, c, __fmul_rn(g, ga));
+        };
         if (live) {
           uint32_t w_lo[4], w_hi[4];
 #pragma unroll
           for (int e = 0; e < 8; e += 2) {
-            w_lo[e >> 1] = pack_bf16((g_lo[e] * ga_lo[e] - o_lo[e] * c) * ir, (g_lo[e + 1] * ga_lo[e + 1] - o_lo[e + 1] * c) * ir);
-            w_hi[e >> 1] = pack_bf16((g_hi[e] * ga_hi[e] - o_hi[e] * c) * ir, (g_hi[e + 1] * ga_hi[e + 1] - o_hi[e + 1] * c) * ir);
+            w_lo[e >> 1] = pack_bf16(diff(g_lo[e], ga_lo[e], o_lo[e]) * ir, diff(g_lo[e + 1], ga_lo[e + 1], o_lo[e + 1]) * ir);
+            w_hi[e >> 1] = pack_bf16(diff(g_hi[e], ga_hi[e], o_hi[e]) * ir, diff(g_hi[e + 1], ga_hi[e + 1], o_hi[e + 1]) * ir);
           }
           *reinterpret_cast<uint4*>(p) = make_uint4(w_lo[0], w_lo[1], w_lo[2], w_lo[3]);
           *reinterpret_cast<uint4*>(p + 128) = make_uint4(w_hi[0], w_hi[1], w_hi[2], w_hi[3]);
@@ -268,8 +273,8 @@ tc_bwd_prep_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ C
         }
         return (A - c * ss) * ir;
       };
-      const float dl = branch(buf + PREP_CHUNK, gs_lo, gs_hi, acc_s);            // D_t = g_s . o_swa
-      if (a.rla_on) branch(buf + 2 * PREP_CHUNK, gr_lo, gr_hi, acc_r);
+      const float dl = branch(buf + PREP_CHUNK, gs_lo, gs_hi, acc_s, true);            // D_t = g_s . o_swa
+      if (a.rla_on) branch(buf + 2 * PREP_CHUNK, gr_lo, gr_hi, acc_r, false);
       if (l == 0) {
         if (live) {
           const size_t grow = (size_t)bq * a.T + t;

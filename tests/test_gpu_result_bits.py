@@ -53,3 +53,39 @@ def test_feature_map_of_the_chunk_states(resumed):
     R.rattn_forward_ex(q, k, v, w, scale=0.1, workspace=ws, state_out=state, **more)
     assert R.rattn_read_status(ws) == 0
     assert torch.equal(state.transpose(-1, -2), phi_pair_sums(left).float())
+
+
+def test_output_norm_gradient_with_gains():
+    """Of a single token the window's weight is one: dv is the gradient that went through the norm and its gain."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    B, H, w = 256, 64, 128
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda")
+    q, k, dy = (rnd(B, H, 1, 128).bfloat16() for _ in range(3))
+    v = (rnd(B, H, 1, 128) * 16).round() / 16            # the same in fp16
+    v = v.bfloat16()
+    v = torch.where(v.abs() < 1e-3, torch.full_like(v, 0.0625), v)
+    gain = 1 + 0.1 * rnd(H, 128)
+    ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, R.FLAG_SAVE_RESIDUALS)
+    more = dict(scale=0.1, workspace=ws, gamma_swa=gain, gamma_rla=torch.ones_like(gain))
+    R.rattn_forward_ex(q, k, v, w, save_residuals=True, **more)
+    _, _, dv = R.rattn_backward_ex(q, k, v, dy, w, flags=R.FLAG_SAVE_RESIDUALS, **more)
+    assert R.rattn_read_status(ws) == 0
+
+    o, gy = v.float()[:, :, 0], dy.float()[:, :, 0]
+    t = gy * gain
+    lanes = lambda x, half: x[..., 64 * half:64 * half + 64].unflatten(-1, (8, 8))
+    ss = torch.zeros_like(lanes(o, 0)[..., 0])
+    A = torch.zeros_like(ss)
+    for e in range(8):
+        lo, hi = lanes(o, 0)[..., e], lanes(o, 1)[..., e]
+        ss = ss + fma(lo, lo, hi * hi)
+        A = A + fma(lanes(t, 0)[..., e], lo, lanes(t, 1)[..., e] * hi)
+    for step in (1, 2, 4):
+        other = torch.arange(8, device="cuda") ^ step
+        ss, A = ss + ss[..., other], A + A[..., other]
+    ss, A = ss[..., :1], A[..., :1]
+    full = lambda c: torch.full_like(ss, c)
+    ir = torch.rsqrt(fma(ss, full(1 / 128), full(1e-6)))
+    c = A * ir * ir * (1 / 128)
+    want = (fma(gy, gain.expand_as(gy), -(o * c)) * ir).bfloat16()
+    assert torch.equal(dv[:, :, 0], want)
