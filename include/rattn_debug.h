@@ -13,7 +13,9 @@
  *      that a wait does run out;
  *   2  in every tensor-core kernel whose threads share named barriers, some of these threads
  *      treat their first wait as run out while the others have passed the same wait.
- *   3  rattn_forward_status finds that the scratch pool cannot be given back.
+ *   3  rattn_forward_status finds that the scratch pool cannot be given back;
+ *   4  in the chunk-state kernel alone, some of the threads that take the sums treat their wait
+ *      for the last one as run out.
  * The paper has no counterpart; this exists for the failure-detection test.
  */
 #ifndef RATTN_DEBUG_H_
@@ -23,7 +25,7 @@
 extern "C" {
 #endif
 
-/* on = 1, 2 or 3: what is called from now on fails in that way; 0: normal operation.
+/* on = 1 .. 4: what is called from now on fails in that way; 0: normal operation.
  * Process-wide switch, host side only.  Returns RATTN_OK. */
 int rattn_debug_withhold_arrival(int on);
 

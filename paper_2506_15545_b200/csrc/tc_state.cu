@@ -60,7 +60,7 @@ struct StateArgs {
   int h_split;      // ... and the group's heads: term matrix ((kv * n_split + step) * h_split + part)
   int wait_before;  // 1: the kernel ahead may still be running; not to end before it
   int wait_first;   // 1: set up under the kernel ahead, whose results this one reads
-  int debug_wait;   // debug build only, 2: the first wait of some of the flush threads counts as run out
+  int debug_wait;   // debug build only, 2 (4): the first (last) wait for a sum of some of the flush threads counts as run out
 };
 
 struct StBars {
@@ -228,11 +228,12 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
     }
     for (int s = 0; s < n_steps && ok; ++s) {
       if (!flushed_step(a, s, n_steps)) continue;
-      // (ahead of the wait, so that the last store passes under it; a wait that runs out shows in the next vote)
+      // (ahead of the wait, so that the last store passes under it; of a wait that runs out the store warp learns before it sends
+      // the sum off)
       if (!a.delta && stored_step(a, s) && !stage_free()) { ok = false; break; }
       mbar_wait(&bars->done, n_flush & 1, &bars->abort);
 #ifdef RATTN_DEBUG_KNOBS
-      if (a.debug_wait == 2 && warp == ST_FLUSH_WARP && n_flush == 0) bars->abort = 1;
+      if (warp == ST_FLUSH_WARP && (a.debug_wait == 2 ? n_flush == 0 : a.debug_wait == 4 && s == n_steps - 1)) bars->abort = 1;
 #endif
       ++n_flush;
       tc_fence_after();
@@ -280,7 +281,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       for (int s = (has_init ? -1 : 0); s < n_steps && ok && !a.delta; ++s) {
         if (!stored_step(a, s)) continue;
         const int mat = a.out_first + a.dir * s;
-        ok = mbar_wait_warp(&bars->staged, n & 1, &bars->abort);
+        ok = mbar_wait_warp(&bars->staged, n & 1, &bars->abort) && !__any_sync(0xffffffffu, *(volatile int*)&bars->abort);
         if (!ok) break;
         ++n;
         if ((tid & 31) == 0) {
@@ -316,10 +317,11 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       }
     }
   }
-  if (!ok && a.status) atomicExch(a.status, 1);
   if (a.wait_before) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
+  // every wait that has run out has raised the flag, the last one of a role too
+  if (tid == 0 && bars->abort && a.status) atomicExch(a.status, 1);
   if (warp == ST_PHI_WARPS) {
     tc_fence_after();
     tmem_dealloc(tmem, 128);

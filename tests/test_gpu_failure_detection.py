@@ -144,6 +144,49 @@ def test_threads_that_share_a_barrier_leave_together(dbg, B_, Hq, Hkv, T, w, mod
     assert all(torch.equal(a, b) for a, b in zip((out, dq, dk, dv), (y, *grads)))
 
 
+@pytest.mark.parametrize("Hq,Hkv,T,w,train,handoff", [
+    (2, 1, 384, 128, False, False),             # a chain of one step: nothing behind its only sum
+    (2, 1, 384, 128, True, False),              # ... and the backward's
+    (2, 2, 1000, 128, False, True),             # several steps, the last one for the decode state alone
+    (8, 1, 8200, 512, False, True),             # terms formed in parallel
+])
+def test_a_chunk_state_that_gives_up_is_reported(dbg, Hq, Hkv, T, w, train, handoff):
+    """The wait for a sum runs out in some threads of the chunk-state kernel and nowhere else: the status says so, also where
+    no further step follows that could notice, and the sum does not leave."""
+    gen = torch.Generator(device="cuda").manual_seed(13)
+    rnd = lambda h: torch.randn(1, h, T, 128, generator=gen, device="cuda").bfloat16()
+    q, k, v, dy = rnd(Hq), rnd(Hkv), rnd(Hkv), rnd(Hq)
+    flags = R.FLAG_SAVE_RESIDUALS if train else 0
+    ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, flags)
+    ws.fill_(0xAB)
+    out, dq, dk, dv = (torch.zeros_like(t) for t in (q, q, k, v))
+    state = torch.zeros(1, Hkv, 128, 128, device="cuda")
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    dbg.rattn_backward_ex.argtypes = [ctypes.POINTER(R.RattnParams), ctypes.c_void_p]
+    p = R._params(q, k, v, out, w, 0.1, 1e-6, None, None, R.MODE_RATTN, ws, flags)
+    p.dout, p.dq, p.dk, p.dv = (t.data_ptr() for t in (dy, dq, dk, dv))
+    if handoff:
+        p.state_out = state.data_ptr()
+    status = lambda: dbg.rattn_read_status(ctypes.c_void_p(ws.data_ptr()), stream)
+    try:
+        dbg.rattn_debug_withhold_arrival(4)
+        assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0
+        assert status() == RATTN_ERR_TIMEOUT
+        if T == 384 and not train:
+            assert (ws[512:] == 0xAB).all()     # behind the status block the chunk states: the only one has not been stored
+        if train:
+            dbg.rattn_debug_withhold_arrival(0)
+            assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0 and status() == 0
+            dbg.rattn_debug_withhold_arrival(4)
+            assert dbg.rattn_backward_ex(ctypes.byref(p), stream) == 0
+            assert status() == RATTN_ERR_TIMEOUT
+    finally:
+        dbg.rattn_debug_withhold_arrival(0)
+    assert dbg.rattn_forward_ex(ctypes.byref(p), stream) == 0 and status() == 0
+    y = R.rattn_forward_ex(q, k, v, w, scale=0.1, workspace=ws, save_residuals=train, state_out=torch.empty_like(state) if handoff else None)
+    assert torch.equal(out, y)
+
+
 @pytest.mark.parametrize("B_,Hq,Hkv,w,pos", [
     (1, 8, 2, 512, 1000),        # cluster of 8 CTAs, the last of which gives up
     (40, 32, 8, 64, 100),        # one CTA per head
