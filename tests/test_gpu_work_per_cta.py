@@ -1,23 +1,29 @@
 """Work that a persistent CTA does after its first piece: pairs of query tiles one behind the other, the rotation table of the
 prologue refilled.  The arithmetic of a result does not depend on which CTA has it or what that CTA did before, so a few CTAs
 with all of the work give the bits that many give."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import rattn_oracle as O
 from paper_2506_15545_b200 import binding as R
+from test_gpu_full_size import sample_rows
+from test_gpu_parity import TOL, np64
 
 pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("grid", [1, 3])
 @pytest.mark.parametrize("mode,T,w,lens", [
-    (R.MODE_RATTN, 2300, 1024, None),                # an odd number of tiles: a unit of one at the end
+    (R.MODE_RATTN, 2300, 1024, None),                # nine pairs
+    (R.MODE_RATTN, 2100, 1024, None),                # an odd number of tiles: a unit of one at the end
     (R.MODE_RATTN, 2400, 1024, [2400, 130, 1200]),   # units beyond an entry's end are passed over, some have a tile less
-    (R.MODE_SWA_ONLY, 900, 256, None),               # no residual part between the windows
-    (R.MODE_FULL_CAUSAL, 700, 700, None),
+    (R.MODE_SWA_ONLY, 2600, 256, None),              # no residual part between the windows, an odd number of tiles
+    (R.MODE_FULL_CAUSAL, 2600, 2600, None),
 ])
 def test_pairs_one_behind_the_other(mode, T, w, lens, grid):
-    """Scores of two tiles in one buffer, the next unit's behind the residual part that had its columns."""
+    """Scores of two tiles in one buffer, the next unit's behind the residual part that had its columns.  Without a residual
+    branch the units are pairs only where there are more tiles than SMs."""
     g = torch.Generator(device="cuda").manual_seed(T + w)
     B = len(lens) if lens else 2
     rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
@@ -32,6 +38,7 @@ def test_pairs_one_behind_the_other(mode, T, w, lens, grid):
         assert R.rattn_read_status(ws) == 0, "a device-side wait expired"
         return [out[b, :, :n] for b, n in enumerate(lens)] if lens else [out]
 
+    assert mode == R.MODE_RATTN or (T + 127) // 128 * 4 * B > torch.cuda.get_device_properties(0).multi_processor_count
     many = run()
     prev = R.rattn_tune(R.TUNE_GRID, grid)
     try:
@@ -40,6 +47,16 @@ def test_pairs_one_behind_the_other(mode, T, w, lens, grid):
         R.rattn_tune(R.TUNE_GRID, prev)
     for x, y in zip(many, few):
         assert torch.isfinite(x.float()).all() and torch.equal(x, y)
+    if grid != 1:
+        return
+    for b, h in ((0, 0), (B - 1, 3)):                # ... and they are the right ones
+        n = lens[b] if lens else T
+        rows = sample_rows(n, min(w, n - 1), 24, T + h)
+        ref = O.forward_rows(np64(q[b, h, :n]), np64(k[b, h // 2, :n]), np64(v[b, h // 2, :n]), rows, w, 0.25, mode=mode,
+                             gamma_swa=np64(more["gamma_swa"][h]), gamma_rla=np64(more["gamma_rla"][h]))
+        err = np.abs(np64(many[b][h] if lens else many[0][b, h])[rows] - ref)
+        bound = TOL["bf16"]["max_abs"] + 2.0 ** -8 * np.maximum(np.abs(ref) - 4.0, 0.0)   # beyond 4 the output's own spacing grows
+        assert (err <= bound).all() and err.mean() <= TOL["bf16"]["mean_abs"], (err.max(), err.mean())
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,T,d,dtype,entry_pos", [
