@@ -175,8 +175,9 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       if (n_stored >= 1) mbar_wait(&bars->stage_free, (n_stored - 1) & 1, &bars->abort);
       return !named_any(4, 256, *(volatile int*)&bars->abort);
     };
-    // bf16 copy of this thread's half row of the sum -> staging; the store warp sends it off
-    auto store_row = [&](const float (&x)[2][32]) {
+    // bf16 copy of this thread's half row of the sum -> staging; the store warp sends it off, unless a thread has given up
+    // waiting for the sum and does not say that its share is there
+    auto store_row = [&](const float (&x)[2][32], bool arrived) {
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
 #pragma unroll
@@ -190,7 +191,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
         }
       }
       fence_proxy_async_smem();
-      mbar_arrive(&bars->staged);
+      if (arrived) mbar_arrive(&bars->staged);
       ++n_stored;
     };
     auto write_final = [&](const float (&x)[2][32]) {
@@ -222,18 +223,20 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(&bars->acc_free);
-        if (stored_step(a, -1)) store_row(x);
+        if (stored_step(a, -1)) store_row(x, true);
       }
       if (a.final_out != nullptr && n_steps == 0) write_final(x);
     }
     for (int s = 0; s < n_steps && ok; ++s) {
       if (!flushed_step(a, s, n_steps)) continue;
-      // (ahead of the wait, so that the last store passes under it; of a wait that runs out the store warp learns before it sends
-      // the sum off)
+      // (ahead of the wait, so that the last store passes under it)
       if (!a.delta && stored_step(a, s) && !stage_free()) { ok = false; break; }
-      mbar_wait(&bars->done, n_flush & 1, &bars->abort);
+      bool arrived = mbar_wait(&bars->done, n_flush & 1, &bars->abort);
 #ifdef RATTN_DEBUG_KNOBS
-      if (warp == ST_FLUSH_WARP && (a.debug_wait == 2 ? n_flush == 0 : a.debug_wait == 4 && s == n_steps - 1)) bars->abort = 1;
+      if (warp == ST_FLUSH_WARP && (a.debug_wait == 2 ? n_flush == 0 : a.debug_wait == 4 && s == n_steps - 1)) {
+        bars->abort = 1;
+        arrived = false;
+      }
 #endif
       ++n_flush;
       tc_fence_after();
@@ -252,7 +255,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
             dst[(8 * c + e) * 128] = make_float4(x[c][4 * e], x[c][4 * e + 1], x[c][4 * e + 2], x[c][4 * e + 3]);
         continue;
       }
-      if (stored_step(a, s)) store_row(x);
+      if (stored_step(a, s)) store_row(x, arrived);
       if (a.final_out != nullptr && s == n_steps - 1) write_final(x);
     }
   } else {
@@ -281,7 +284,7 @@ tc_state_scan_kernel(const __grid_constant__ UMap tm_x, const __grid_constant__ 
       for (int s = (has_init ? -1 : 0); s < n_steps && ok && !a.delta; ++s) {
         if (!stored_step(a, s)) continue;
         const int mat = a.out_first + a.dir * s;
-        ok = mbar_wait_warp(&bars->staged, n & 1, &bars->abort) && !__any_sync(0xffffffffu, *(volatile int*)&bars->abort);
+        ok = mbar_wait_warp(&bars->staged, n & 1, &bars->abort);
         if (!ok) break;
         ++n;
         if ((tid & 31) == 0) {
