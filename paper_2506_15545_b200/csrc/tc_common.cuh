@@ -166,13 +166,8 @@ __device__ __forceinline__ float feature_map_half_row(const unsigned char* src, 
                    pack_bf16(x[c * 8 + 4] * sc, x[c * 8 + 5] * sc), pack_bf16(x[c * 8 + 6] * sc, x[c * 8 + 7] * sc));
   return inv;
 }
-// ... normalised; src_half / dst_half point at the [rows x 64] box of this lane's column half
-__device__ __forceinline__ void feature_map_pair_any(const unsigned char* src_half, unsigned char* dst_half, int row, int phi) {
-  feature_map_half_row(src_half + row * 128, dst_half + row * 128, row, (int)(threadIdx.x & 1), phi, true);
-}
-
-// ... by four lanes per row, of which this one (q) owns 32 columns; `src` and `dst` point at the row in the first column
-// half's box, the second half's lies `half_stride` behind.
+// ... normalised, by four lanes per row, of which this one (q) owns 32 columns; `src` and `dst` point at the row in the
+// first column half's box, the second half's lies `half_stride` behind.
 // PAIR_SUMS = false: q = lane & 3.  A quarter-warp (two rows) touches every bank once: the lanes of the second half walk
 // their chunks two apart from the first's.
 // PAIR_SUMS = true: the softmax map's sums are formed in feature_map_half_row's order, so that both leave the same bits:
@@ -193,20 +188,22 @@ __device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsig
     }
     return;
   }
-  float x[32], m0 = -INFINITY, m1 = -INFINITY;
+  float x[32];
+  __nv_bfloat162 mx[4];                                   // packed: two values per instruction
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const uint4 u = *reinterpret_cast<const uint4*>(src + ((c ^ sw) << 4));
     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(w);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       x[c * 8 + 2 * e] = __uint_as_float(w[e] << 16);
       x[c * 8 + 2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-      m0 = fmaxf(m0, x[c * 8 + 2 * e]);
-      m1 = fmaxf(m1, x[c * 8 + 2 * e + 1]);
+      mx[e] = c == 0 ? h[e] : __hmax2(mx[e], h[e]);
     }
   }
-  float m = fmaxf(m0, m1);
+  const float2 m2 = __bfloat1622float2(__hmax2(__hmax2(mx[0], mx[1]), __hmax2(mx[2], mx[3])));
+  float m = fmaxf(m2.x, m2.y);
   m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
   m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, PAIR_SUMS ? 8 : 2));
   const float ml = m * 1.4426950408889634f;
@@ -240,11 +237,17 @@ __device__ __forceinline__ void feature_map_quad(const unsigned char* src, unsig
     sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   }
   const float sc = 1.f / sum;
+  const float2 sc2 = make_float2(sc, sc);
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
-    *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) =
-        make_uint4(pack_bf16(x[c * 8 + 0] * sc, x[c * 8 + 1] * sc), pack_bf16(x[c * 8 + 2] * sc, x[c * 8 + 3] * sc),
-                   pack_bf16(x[c * 8 + 4] * sc, x[c * 8 + 5] * sc), pack_bf16(x[c * 8 + 6] * sc, x[c * 8 + 7] * sc));
+  for (int c = 0; c < 4; ++c) {
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 y = __fmul2_rn(make_float2(x[c * 8 + 2 * e], x[c * 8 + 2 * e + 1]), sc2);
+      w[e] = pack_bf16(y.x, y.y);
+    }
+    *reinterpret_cast<uint4*>(dst + ((c ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
 }
 
 // byte offset of 16-byte chunk c (0..15) of row r inside a swizzled [128 x 128] bf16 tile
