@@ -223,19 +223,28 @@ cudaError_t allow_smem(int bytes) {
 // Launch with or without programmatic stream serialisation: with it the kernel may be set up while the one ahead of it on
 // the stream still runs, and has to wait for that one itself (griddepcontrol.wait) before it reads or overwrites anything
 // the other uses -- and in any case before it ends, so that whatever follows may rely on both.
+// cluster > 1: in clusters of that many CTAs, of which the grid is a multiple.
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap, A&&... args) {
+cudaError_t launch_pdl_cluster(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap, int cluster,
+                               A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool overlap, A&&... args) {
+  return launch_pdl_cluster(kernel, grid, block, smem, s, overlap, 1, std::forward<A>(args)...);
 }
 
 // Records a CUDA event pair around one kernel launch on its stream while per-kernel

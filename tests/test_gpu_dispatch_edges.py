@@ -254,3 +254,33 @@ def test_prompts_of_one_tile_in_wide_windows(T, w, lens):
 
     for x, y in zip(run(w), run(768)):
         assert torch.isfinite(x.float()).all() and torch.equal(x, y)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,T,w", [
+    (1, 2, 1, 700, 128),         # one head: a CTA alone
+    (3, 2, 1, 700, 128),         # odd: a pair has a CTA without work
+    (1, 14, 7, 1500, 256),
+    (4, 8, 8, 900, 1024),        # nothing leaves the window but the decode state is formed
+    (37, 1, 1, 300, 128),        # the most heads that go under the copy
+    (38, 1, 1, 300, 128),        # behind it
+    (1, 3, 3, 8200, 128),        # parallel terms: 3 x 64 CTAs
+    (1, 5, 5, 8321, 1024),       # 5 x 58
+])
+def test_chain_under_the_hand_off(B, Hq, Hkv, T, w):
+    """Behind the call's own copy the chunk states' CTAs are set up early and in pairs; without it the same kernel starts
+    in full order: the same bits."""
+    gen = torch.Generator(device="cuda").manual_seed(T + B)
+    rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").bfloat16()
+    q, k, v = rnd(B, Hq, T, 128), rnd(B, Hkv, T, 128), rnd(B, Hkv, T, 128)
+    ws = R.alloc_workspace(q, k, w, R.MODE_RATTN, 0)
+    rings = dict(k_ring_out=torch.empty(B, Hkv, w, 128, device="cuda", dtype=torch.bfloat16))
+    rings["v_ring_out"] = torch.empty_like(rings["k_ring_out"])
+    got = []
+    for more in ({}, rings, rings):
+        ws.fill_(0xAB)
+        state = torch.full((B, Hkv, 128, 128), 7.0, device="cuda")
+        out = R.rattn_forward_ex(q, k, v, w, scale=0.1, workspace=ws, state_out=state, **more)
+        assert R.rattn_read_status(ws) == 0
+        got.append((out, state))
+    for out, state in got[1:]:
+        assert torch.isfinite(out.float()).all() and torch.equal(out, got[0][0]) and torch.equal(state, got[0][1])
