@@ -164,7 +164,8 @@ struct Cursor {
   int c;                // [B, T, H, d]: chunk inside the tensor; its first head vector is head h0 of
   int h0, t0, b0;       //               position t0 of batch entry b0
 };
-// x / H for 0 <= x < 8192 without an integer division ((x + 0.5) / H is at least 0.5 / H away from an integer)
+// x / H for 0 <= x < 2^21 without an integer division ((x + 0.5) / H is at least 0.5 / H away from an integer, and two
+// roundings by 2^-24 of it are less)
 __device__ __forceinline__ int small_div(int x, float inv_H) { return __float2int_rd(((float)x + 0.5f) * inv_H); }
 template <int RPB>
 __device__ __forceinline__ Cursor cursor_at(const QkArgs& a, int i) {
@@ -301,10 +302,12 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
   auto fill_table = [&](const Cursor& cx, int i) {
     constexpr double kTwoPi = 6.283185307179586476925286766559;
     const int H = a.H[cx.which];
-    long long v_end = ((long long)cx.c + (hi - i)) * RPB;
-    if (v_end > (long long)a.B * a.T * H) v_end = (long long)a.B * a.T * H;
+    // head vectors from the chunk's first on: this CTA's, the tensor's, as many as a full table's tokens have
+    const long long mine = (long long)(hi - i) * RPB, all = (long long)a.B * a.T * H - (long long)cx.c * RPB;
+    const long long left = mine < all ? mine : all;
+    const int n = left < (long long)a.tbl_tokens * H ? (int)left : a.tbl_tokens * H;
     tbl_first = cx.b0 * a.T + cx.t0;
-    const int n_tok = min((int)((v_end - 1) / H) - tbl_first + 1, a.tbl_tokens);
+    const int n_tok = min(small_div(cx.h0 + n - 1, a.inv_H[cx.which]) + 1, a.tbl_tokens);
     tbl_end = tbl_first + n_tok;
     for (int e = tid; e < n_tok * (D / 2); e += QK_THREADS) {
       const int tok = e / (D / 2), pair = e % (D / 2);
@@ -319,6 +322,13 @@ qk_prologue_kernel(const __grid_constant__ QkArgs a, const __grid_constant__ Fre
     }
   };
   Cursor ch = cursor_at<RPB>(a, lo);
+  // the first table shares the barrier below, with the gains asked for ahead of it (a decode step of 25 x 40/8 heads, w = 768,
+  // with its prologue: 15.5 -> 15.3 us)
+  if (tabled && lo < hi) {
+    load_gain(a.gain[ch.which], 8 * l, D / 2, g_lo, g_hi);
+    cur_which = ch.which;
+    fill_table(ch, lo);
+  }
   if (!a.rotate) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) { c[j] = 1.f; s[j] = 0.f; }
