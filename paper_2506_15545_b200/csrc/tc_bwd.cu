@@ -855,7 +855,7 @@ struct KvMaps {
 };
 
 // One key tile (j, K/V head) of the persistent CTA's work list, and how its half-tile items
-// are numbered.  Counters that run on across key tiles (ring slots, TMEM slots, barrier
+// are numbered.  Counters that run on across key tiles (ring slots, items, barrier
 // phases) are kept by every role in the same way.
 struct KvPlan {
   int j, bh_kv, head0, part_index, rs_index, n_qt, wt, group, n_R, n_s_tiles, N;
@@ -1075,8 +1075,7 @@ __device__ bool kv_mma_accum(const BwdArgs& a, unsigned char* smem, KvBars* bars
 
 __device__ bool kv_rows(const BwdArgs& a, unsigned char* smem, KvBars* bars, uint32_t tmem, int g, int h, int r) {
   // Two groups of 256 threads.  A thread is key row r = TMEM lane and half h of its item's 64 query
-  // columns: with all 64 on one thread a warp had a scheduler almost to itself and an item's arithmetic took 1530 cycles of
-  // the 4400 from scores to scores on a slot.
+  // columns: with all 64 on one thread a warp had a scheduler almost to itself and an item's arithmetic took 1530 cycles.
   const uint32_t lane_off = (uint32_t)((r & ~31) << 16);
   const uint32_t tV = tmem + lane_off, tK = tmem + 128 + lane_off;
   const uint32_t tS = tmem + 256 + 32 * h + lane_off, tP = tS + 64, tW = tmem + 384 + 64 * g + 16 * h + lane_off;
@@ -1447,8 +1446,8 @@ cudaError_t launch_tc_backward(const Args& a, cudaStream_t s) {
   // Reverse states of the residual branch: R_c for c = 0 .. n_r-1 (chunks with a query tile beyond c + wt), a running
   // sum that walks the query tiles from the last one down to wt+1.  The dq kernel does not read them, so the two share
   // the GPU.  A serial chain (one CTA per K/V head) goes first, and the dq kernel runs beside it on the other SMs; that
-  // costs least as long as the chain is over by then (1.4 us per tile and query head, measured, against about
-  // 1.45 us per key tile + 5 us for a dq item; up to 15 % longer is still cheaper than the other way).  Where it would
+  // costs least as long as the chain is over by then (1.4 us per tile and query head -- alone 1.7 with one head to a K/V
+  // head, 1.34 with two, 1.20 with eight -- against about 1.45 us per key tile + 5 us for a dq item; up to 15 % longer is still cheaper than the other way).  Where it would
   // outlast the dq kernel, its terms are formed in parallel behind that kernel, on the SMs it runs out of items on: at
   // 1 x 16/4 heads, T = 1111, w = 128 the chain took 46 us on four SMs beside a dq kernel of 16 us, the terms and their
   // sum end 11 us behind it.  With a chain on more than half of the SMs there is nothing to share.

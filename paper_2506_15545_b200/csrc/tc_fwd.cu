@@ -36,9 +36,9 @@ static Plan make_plan(const Args& a, int n_sm) {
   if (p.n_steps < 0) p.n_steps = 0;
   p.chain = n_delta > 0 || (want_state && (a.Tk > a.w || a.seq_lens)) || (a.state_in && rla);
   const int knob = tuning(RATTN_TUNE_STATE_PROGRESS);
-  // Estimates (measured on B200): the chain 2.6 us per step when it stores every state (1.65 every second one; it has become
-  // faster since, 2.5 where it publishes them and 2 where not, and the lines below stand where these drew them), the main kernel
-  // 30 ns per query tile and 12 ns per tile and key tile, and no less than 40 us as far as this matters.  (Fitted on a B200
+  // Estimates, for which the lines below are drawn: the chain 2.6 us per step, the main kernel 30 ns per query tile and 12 ns
+  // per tile and key tile, and no less than 40 us as far as this matters.  (A step with the GPU to itself takes 1.64 us where
+  // every state is stored, 1.30 where every second one is, 2.3 where they are published.)  (Fitted on a B200
   // with all of its 148 SMs at work and every window full: short sequences, whose first tiles read less, and ragged batches
   // have less work than this says.)  Where the chain of a long sequence on few heads would outlast the main kernel, its terms
   // are formed in parallel (1 x 8/1 heads, T = 16384, w = 512: 202 -> 113 us).
@@ -58,7 +58,7 @@ static Plan make_plan(const Args& a, int n_sm) {
   const bool chain_fits = a.training ? 2 * chain_ns <= 3 * main_ns
                                      : 5 * chain_ns <= (wt <= 4 ? 7 : 6) * (work_ns < 16000 ? 16000 : work_ns);
   // Where the pairs all run at once, everything else is over within a unit's time, about 20 us: a chain much
-  // longer than that decides, and the pair kernel's is the shorter one (inference: 1.65 us a step) or leaves it less to do at
+  // longer than that decides, and the pair kernel's is the shorter one (inference) or leaves it less to do at
   // the end (1 x 16/4 heads, T = 2200, w = 512: 47 us as single tiles, 37 as pairs; w = 768, two steps fewer: 42 and 41;
   // training, w = 128: 55 and 50).
   const bool chain_decides = (long long)((n_qt + 1) / 2) * n_q <= n_sm && chain_ns > (a.training ? 36000 : 30000);
@@ -123,9 +123,12 @@ cudaError_t launch_tc_forward(const Args& a, cudaStream_t s) {
     L.delta = p.terms ? a.rdelta : nullptr;
     L.h_split = 1;
     L.after_independent = false;
-    // Behind the call's own copies (gather, ring hand-off) the chain is set up under them where it has few CTAs: 1 x 40/8
-    // heads, T = 300, w = 256 26.7 -> 24.4 us, 2 x 32/8, T = 2048 124.8 -> 122.0; with 64 of them, which hold SMs while they
-    // wait, 198.5 -> 203, with 128 159.6 -> 162.4.
+    // Behind the call's own copies (gather, ring hand-off) the chain is set up under them where it has few heads.  Resumed
+    // chunks in full order and so: 1 x 40/8 heads, T = 300, w = 256 26.6 and 24.6 us; w = 512: 2 x 32/8, T = 2048 126.8 and 121.9,
+    // 4 x 32/8, T = 1024 120.5 and 115.3.  Heads are counted and not CTAs, of which parallel terms have one per head and step:
+    // 1 x 8/1, T = 8192 63.2 and 60.2, 1 x 16/4 127.4 and 122.5.  (The line lies where the chain's CTAs lost when they did not yet
+    // come in pairs, 5 x 32/8, T = 1024 139.8 and 144.9; as pairs they gain beyond it too, 139.1 and 136.1, 8 x 32/8 217.3 and
+    // 214.1.)
     L.wait_first = a.kernel_ahead && 4 * n_kv <= n_sm;
     e = launch_tc_states(L, s);
     if (e != cudaSuccess) return e;

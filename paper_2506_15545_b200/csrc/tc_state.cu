@@ -17,8 +17,9 @@
 //   8 flush warps  after a stored step: accumulator -> registers (the MMA warp goes on as soon as
 //                  the TMEM loads have landed) -> bf16 -> staging tile; two threads per row
 //   store warp     staging tile -> TMA store, and the number of stored states where they are published
-// With eight phi and four flush warps, which looked for the staging tile only once they held the sum, a step took 2.6 us
-// where every sum is stored and 1.65 where every second one is.
+// A step takes 1.64 us where every sum is stored, 1.30 where every second one is and 2.3 where they are published (4 to 16
+// heads on a GPU to itself; with eight phi and four flush warps, which looked for the staging tile only once they held the
+// sum, 2.6 and 1.65).
 #include <climits>
 
 #include "tc_common.cuh"
